@@ -3,6 +3,7 @@
 #include <algorithm>
 
 #include "idw_dev.cuh"
+#include "knn_warp.cuh"
 
 namespace bg {
 namespace {
@@ -42,6 +43,81 @@ __global__ void __launch_bounds__(128) k_idw(HashView h, GridView g, int k, floa
     knn_strip<128, decltype(emit), true, kLen>(h, g, K, o.i, o.j, hp, flag, emit);
 }
 
+struct KnnFar {
+    int cnt;
+    float d1, dk;
+};
+
+// Per-thread search and IDW of a node that the patch search did not serve
+template <int K>
+__device__ __noinline__ KnnFar knn_lane_idw(const HashView& h, int qx, int qy, uint64_t* hp, int k, float power,
+                                            float* depth, int32_t* nbr) {
+    const int cnt = knn_lane<K>(h, qx, qy, hp);
+    if (cnt < 0) return KnnFar{cnt, 0.0f, 0.0f};
+    const int bits = h.idx_bits, keff = min(cnt, k);
+    const uint64_t mask = (1ull << bits) - 1;
+    *depth = idw_from(h, keff, power, [&](int n, uint64_t& dd, int& ii) {
+        const uint64_t v = hp[n * 32];
+        dd = v >> bits;
+        ii = (int)(v & mask);
+    });
+    if (nbr) emit_ids<32>(nbr, hp, k, keff, mask);
+    return KnnFar{cnt, sqrtf((float)(hp[0] >> bits)), cnt == K ? sqrtf((float)(hp[(K - 1) * 32] >> bits)) : 0.0f};
+}
+
+// The same by patches of 8 x 4 nodes per warp (knn_warp.cuh), a strip of `len`
+// patches along x each; spr strips per patch row.
+template <int K>
+__global__ void __launch_bounds__(64, KnnWarp<K>::kBlocksPerSM) k_idw_patch(HashView h, GridView g, int k, float power,
+                                                  float* __restrict__ depth,
+                                                  int32_t* __restrict__ nbr, int* __restrict__ flag,
+                                                  int len, int spr) {
+    __shared__ typename KnnWarp<K>::Smem smem[2];
+    typename KnnWarp<K>::Smem& sm = smem[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
+    const unsigned w = blockIdx.x * 2 + (threadIdx.x >> 5);
+    const int py = (int)(w / (unsigned)spr), p0 = (int)(w % (unsigned)spr) * len;
+    if (py * 4 >= g.ny) return;
+    const int j = py * 4 + (lane >> 3), qy = g.y0 + j * g.cell + g.cell / 2;
+    KnnChain ch;
+    for (int p = p0; p < p0 + len && p * 8 < g.nx; ++p) {
+        const int i = p * 8 + (lane & 7), qx = g.x0 + i * g.cell + g.cell / 2;
+        const bool on = i < g.nx && j < g.ny;
+        const int ox = g.x0 + p * 8 * g.cell + g.cell / 2, oy = g.y0 + py * 4 * g.cell + g.cell / 2;
+        uint32_t base;
+        const float r = knn_first_radius<K>(h, ch, on, qx, qy, 8.0f * (float)g.cell, base);
+        const unsigned served = knn_patch<K>(h, sm, on, qx, qy, ox, oy, r, base, ch);
+        const int64_t node = (int64_t)j * g.nx + i;
+        int32_t* o = nbr ? nbr + node * k : nullptr;
+        if (served >> lane & 1) {
+            const int ux = qx - ox, uy = qy - oy;
+            depth[node] = idw_sum(k, power, [&](int n, float& d, float& z) {
+                const uint32_t q = sm.buf[n * 32 + lane] & kPlaceMask;
+                const int4 c = sm.st[q];
+                const int dx = c.x - ux, dy = c.y - uy;
+                d = __int2float_rn(dx * dx + dy * dy);
+                z = __int_as_float(__ldg(&h.rec[sm.pos[q]].z));
+            });
+            if (o)
+                for (int n = 0; n < k; ++n) o[n] = __ldg(&h.rec[sm.pos[sm.buf[n * 32 + lane] & kPlaceMask]].w);
+        }
+        if (served != kFull) {
+            __syncwarp();
+            if (on && !(served >> lane & 1)) {
+                ch.dk = -1.0f;
+                const KnnFar f = knn_lane_idw<K>(h, qx, qy, reinterpret_cast<uint64_t*>(sm.buf) + lane, k, power,
+                                                 depth + node, o);
+                if (f.cnt < 0) *flag = 1;  // the wide pass picks this node up
+                if (f.cnt == K) {
+                    ch.d1 = f.d1;
+                    ch.dk = f.dk;
+                }
+            }
+        }
+        __syncwarp();
+    }
+}
+
 // Wide-key pass over the nodes the packed pass could not take; it returns at
 // once when the packed pass flagged none.
 template <int K>
@@ -58,15 +134,20 @@ __global__ void __launch_bounds__(128) k_idw_wide(HashView h, GridView g, int k,
 }
 
 template <int K>
-bg_status launch_k(const HashView& h, const GridView& g, int k, float power, float* depth,
-                   int32_t* nbr, int* d_flag, cudaStream_t st, bg_ctx_s* prof_ctx) {
+bg_status launch_k(const bg_soundings_s* s, const HashView& h, const GridView& g, int k, float power,
+                   float* depth, int32_t* nbr, int* d_flag, cudaStream_t st, bg_ctx_s* prof_ctx) {
     const int64_t nb = (int64_t)((g.nx + 15) / 16) * ((g.ny + 7) / 8);
     const int len = strip_len_for((int64_t)g.nx * g.ny);
     const int64_t nbs = (int64_t)((g.nx + 16 * len - 1) / (16 * len)) * ((g.ny + 7) / 8);
     BG_CUDA(cudaMemsetAsync(d_flag, 0, sizeof(int), st));
     {
         ProfScope ps(prof_ctx, kProfIdw, (int64_t)g.nx * g.ny, st);
-        if (len == 1)
+        const int pnx = (g.nx + 7) / 8, pny = (g.ny + 3) / 4;
+        const int plen = patch_strip_len((int64_t)pnx * pny), spr = (pnx + plen - 1) / plen;
+        if (knn_patch_fits<K>(s->info, g.cell, g.nx, g.ny) && (int64_t)spr * pny < ((int64_t)1 << 31))
+            k_idw_patch<K><<<(unsigned)(((int64_t)spr * pny + 1) / 2), 64, 0, st>>>(
+                h, g, k, power, depth, nbr, d_flag, plen, spr);
+        else if (len == 1)
             k_idw<K, 1><<<(unsigned)nbs, 128, 0, st>>>(h, g, k, power, depth, nbr, d_flag);
         else if (len == 2)
             k_idw<K, 2><<<(unsigned)nbs, 128, 0, st>>>(h, g, k, power, depth, nbr, d_flag);
@@ -181,10 +262,10 @@ bg_status launch_idw(const bg_soundings_s* s, const GridView& g, int k, float po
     bg_status rc = dalloc(s->ctx, (void**)&flag, sizeof(int), st);
     if (rc != BG_OK) return rc;
     switch (K) {
-        case 4: rc = launch_k<4>(h, g, k, power, depth, nbr, flag, st, s->ctx); break;
-        case 8: rc = launch_k<8>(h, g, k, power, depth, nbr, flag, st, s->ctx); break;
-        case 16: rc = launch_k<16>(h, g, k, power, depth, nbr, flag, st, s->ctx); break;
-        default: rc = launch_k<32>(h, g, k, power, depth, nbr, flag, st, s->ctx); break;
+        case 4: rc = launch_k<4>(s, h, g, k, power, depth, nbr, flag, st, s->ctx); break;
+        case 8: rc = launch_k<8>(s, h, g, k, power, depth, nbr, flag, st, s->ctx); break;
+        case 16: rc = launch_k<16>(s, h, g, k, power, depth, nbr, flag, st, s->ctx); break;
+        default: rc = launch_k<32>(s, h, g, k, power, depth, nbr, flag, st, s->ctx); break;
     }
     dfree(s->ctx, flag, sizeof(int), st);
     return rc;
@@ -196,10 +277,10 @@ bg_status launch_idw_with_flag(const bg_soundings_s* s, const GridView& g, int k
     const int K = k <= 4 ? 4 : k <= 8 ? 8 : k <= 16 ? 16 : 32;
     h.r0 = start_halfwidth(s, K);
     switch (K) {
-        case 4: return launch_k<4>(h, g, k, power, depth, nbr, d_flag, st, s->ctx);
-        case 8: return launch_k<8>(h, g, k, power, depth, nbr, d_flag, st, s->ctx);
-        case 16: return launch_k<16>(h, g, k, power, depth, nbr, d_flag, st, s->ctx);
-        default: return launch_k<32>(h, g, k, power, depth, nbr, d_flag, st, s->ctx);
+        case 4: return launch_k<4>(s, h, g, k, power, depth, nbr, d_flag, st, s->ctx);
+        case 8: return launch_k<8>(s, h, g, k, power, depth, nbr, d_flag, st, s->ctx);
+        case 16: return launch_k<16>(s, h, g, k, power, depth, nbr, d_flag, st, s->ctx);
+        default: return launch_k<32>(s, h, g, k, power, depth, nbr, d_flag, st, s->ctx);
     }
 }
 

@@ -48,37 +48,55 @@ __device__ __forceinline__ float idw_tree8(const float (&p)[kIdwLanes]) {
     return ((p[0] + p[1]) + (p[2] + p[3])) + ((p[4] + p[5]) + (p[6] + p[7]));
 }
 
-// IDW from the neighbours in ascending (d2, index) order; get(i) returns
-// (d2, upload index) of the i-th.
+// IDW from keff neighbours in ascending (d2, index) order; get(i) returns
+// (idw_d2f of the squared distance, depth) of the i-th.
 template <class Get>
-__device__ __forceinline__ float idw_from(const HashView& h, int keff, float power, Get get) {
+__device__ __forceinline__ float idw_sum(int keff, float power, Get get) {
     if (keff == 0) return __int_as_float(0x7fc00000);  // NaN: no valid sounding
-    const int* zb = reinterpret_cast<const int*>(h.orig) + 2;  // z bits of record i at zb[4*i]
-    uint64_t d0;
-    int i0;
-    get(0, d0, i0);
-    const float z1 = __int_as_float(__ldg(zb + 4 * (int64_t)i0));
-    if (d0 == 0) return z1;  // node on top of a sounding
-    const float d1 = idw_d2f(d0);
+    float d1, z1;
+    get(0, d1, z1);
+    if (d1 == 0.0f) return z1;  // node on top of a sounding
     float l1 = 0.0f;  // log2(d1), for powers other than 2
     if (power != 2.0f) l1 = log2f(d1);
     const float hp = 0.5f * power;
     float num[kIdwLanes], den[kIdwLanes];
 #pragma unroll
     for (int q = 0; q < kIdwLanes; ++q) num[q] = den[q] = 0.0f;
+    // eight neighbours per turn (one per partial), each model its own loop: short
+    // enough to stay in the instruction cache beside a search
+    auto turns = [&](auto weight) {
+#pragma unroll 1
+        for (int n0 = 1; n0 < keff; n0 += kIdwLanes) {
 #pragma unroll
-    for (int n = 1; n < 32; ++n) {
-        if (n >= keff) break;
-        uint64_t di2;
-        int ii;
-        get(n, di2, ii);
-        const float zi = __int_as_float(__ldg(zb + 4 * (int64_t)ii));
-        const float w = idw_weight(d1, l1, hp, power, idw_d2f(di2));
-        num[(n - 1) % kIdwLanes] = fmaf(w, zi - z1, num[(n - 1) % kIdwLanes]);
-        den[(n - 1) % kIdwLanes] += w;
-    }
+            for (int q = 0; q < kIdwLanes; ++q) {
+                if (n0 + q >= keff) break;
+                float di, zi;
+                get(n0 + q, di, zi);
+                const float w = weight(di);
+                num[q] = fmaf(w, zi - z1, num[q]);
+                den[q] += w;
+            }
+        }
+    };
+    if (power == 2.0f)
+        turns([&](float d) { return idw_weight(d1, l1, hp, 2.0f, d); });
+    else
+        turns([&](float d) { return idw_weight(d1, l1, hp, power, d); });
     // neighbour 0 contributes weight 1 and anomaly 0
     return z1 + idw_tree8(num) / (1.0f + idw_tree8(den));
+}
+
+// The same with get(i) returning (d2, upload index).
+template <class Get>
+__device__ __forceinline__ float idw_from(const HashView& h, int keff, float power, Get get) {
+    const int* zb = reinterpret_cast<const int*>(h.orig) + 2;  // z bits of record i at zb[4*i]
+    return idw_sum(keff, power, [&](int n, float& d, float& z) {
+        uint64_t d2;
+        int i;
+        get(n, d2, i);
+        d = idw_d2f(d2);
+        z = __int_as_float(__ldg(zb + 4 * (int64_t)i));
+    });
 }
 
 template <int K, bool kWide>

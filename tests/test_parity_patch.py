@@ -1,0 +1,74 @@
+"""GPU parity of the patch search (one warp per 8 x 4 nodes) against the FP64
+oracle, at the sizes where it changes course: patch remainders, equal distances
+everywhere, more soundings than its list holds, gaps wider than its first
+radius, distances beyond its keys, clusters at one position.
+
+Neighbour lists are bit-exact, depths within the IDW tolerance of
+tests/gpu_util.py.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from gpu_util import Lib, assert_idw
+from synth import GridSpec
+
+pytestmark = pytest.mark.gpu
+
+
+def _uniform(seed, n, w_cm, h_cm):
+    r = np.random.Generator(np.random.PCG64(seed))
+    return (r.integers(0, w_cm, n).astype(np.int32), r.integers(0, h_cm, n).astype(np.int32),
+            (3500 + r.normal(0, 5, n)).astype(np.float32))
+
+
+def _lattice(nx, ny, step):
+    x, y = np.meshgrid(np.arange(nx) * step, np.arange(ny) * step)
+    z = 3500 + 0.01 * x + 0.02 * y
+    return x.ravel().astype(np.int32), y.ravel().astype(np.int32), z.ravel().astype(np.float32)
+
+
+def _gap(seed):
+    """Two strips of soundings, 40 m deep and 130 m apart."""
+    x, y, z = _uniform(seed, 12_000, 30_000, 8_000)
+    return x, np.where(y < 4_000, y, y + 13_000).astype(np.int32), z
+
+
+def _cluster(seed):
+    """A scatter with 300 soundings at one position and 40 at another."""
+    x, y, z = _uniform(seed, 4_000, 6_000, 6_000)
+    x[:300], y[:300] = 3_000, 3_000
+    x[300:340], y[300:340] = 1_111, 4_444
+    return x, y, z
+
+
+CASES = {
+    "one_node": (lambda: _uniform(1, 3_000, 6_000, 6_000), GridSpec(2_000, 2_000, 100, 1, 1)),
+    "whole_patch": (lambda: _uniform(2, 3_000, 6_000, 6_000), GridSpec(1_000, 1_000, 100, 8, 4)),
+    "remainders": (lambda: _uniform(3, 3_000, 6_000, 6_000), GridSpec(500, 700, 150, 33, 17)),
+    "past_the_edge": (lambda: _uniform(4, 3_000, 6_000, 6_000), GridSpec(-9_000, -3_000, 250, 70, 30)),
+    "lattice": (lambda: _lattice(60, 60, 100), GridSpec(-50, -50, 100, 57, 59)),
+    "half_lattice": (lambda: _lattice(60, 60, 100), GridSpec(0, 0, 100, 41, 23)),
+    "many_per_node": (lambda: _uniform(5, 60_000, 4_000, 4_000), GridSpec(0, 0, 200, 20, 19)),
+    "near_capacity": (lambda: _uniform(6, 12_000, 4_000, 4_000), GridSpec(0, 0, 100, 40, 39)),
+    "gap": (lambda: _gap(7), GridSpec(0, 0, 200, 150, 105)),
+    "sparse": (lambda: _uniform(8, 3_000, 200_000, 200_000), GridSpec(50_000, 50_000, 600, 45, 33)),
+    "cluster": (lambda: _cluster(9), GridSpec(0, 0, 150, 40, 40)),
+    "few": (lambda: _uniform(10, 40, 6_000, 6_000), GridSpec(0, 0, 300, 20, 20)),
+}
+
+
+@pytest.mark.parametrize("k", [3, 8, 16, 32])
+@pytest.mark.parametrize("name", CASES)
+def test_idw_neighbours_and_depths(name, k):
+    make, g = CASES[name]
+    x, y, z = make()
+    lib = Lib(x, y, z, g)
+    try:
+        d, nb = lib.idw(k, 2.0)
+    finally:
+        lib.close()
+    qx, qy = oracle.grid_nodes(g.x0_cm, g.y0_cm, g.cell_cm, g.nx, g.ny)
+    ref, ridx = oracle.idw(x, y, z, qx, qy, k, 2.0, want_idx=True)
+    assert np.array_equal(nb, ridx)
+    assert_idw(d, ref)
