@@ -336,7 +336,7 @@ bg_status bg_batch_create(bg_ctx_t ctx, const bg_tile* tiles, int n_tiles, bg_ba
 /* Grid every tile of the batch, ordered after prior work on cuda_stream and
  * before later work on it. The first run records the launch sequence (hash
  * build for all tiles, one persistent k-NN/IDW kernel, one persistent solve
- * kernel per kriging system size) as a CUDA graph; later runs replay it, with
+ * kernel per kriging system size and model) as a CUDA graph; later runs replay it, with
  * no host synchronization. */
 bg_status bg_batch_run(bg_batch_t b, void* cuda_stream);
 
@@ -348,8 +348,9 @@ bg_status bg_batch_set_cell_target(bg_batch_t b, float soundings_per_cell);
  *   knn_strip: grid nodes a k-NN thread takes one after another along x (1, 2
  *     or 4; from the second on, the previous node's k-th distance plus the
  *     step bounds the search), i.e. (16 knn_strip) x 8 nodes per k-NN item;
- *   solve_item: block batches of kriging systems per claimed solve item (1, 2,
- *     4, 8 or 16; 256 systems at K = 32 for 8, the default).
+ *   solve_item: kriging systems per claimed solve item, in units of 32 at
+ *     K = 32 (64 at K = 16, ...), rounded up to 128 systems (1, 2, 4, 8 or 16;
+ *     256 systems at K = 32 for 8, the default).
  * Results never depend on the shape. Other values: BG_ERR_INVALID_ARG. */
 bg_status bg_batch_set_shape(bg_batch_t b, int knn_strip, int solve_item);
 

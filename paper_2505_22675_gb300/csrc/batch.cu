@@ -17,9 +17,8 @@
 //      length; from the second node on, the previous node's K-th distance
 //      plus the step bounds the search): IDW tiles are gridded in place,
 //      kriging tiles get their neighbour ids;
-//   6. a persistent kernel per kriging system size drains (tile, nb x 16
-//      warps' systems) items (okrige_solve_block), nb block batches per
-//      claimed item;
+//   6. a persistent kernel per kriging system size and variogram model drains
+//      (tile, batches of 128 systems) items (okrige_solve_range);
 //   7. a wide-key pass, which returns at once unless a node's bound needed
 //      more than the packed key's bits.
 // Items are claimed with a global atomic counter, so uneven tiles balance
@@ -62,14 +61,11 @@ constexpr int kChunk = 4096;      // soundings per block in the per-sounding ker
 constexpr int kBT = 256;          // threads of those kernels
 constexpr int kItemThreads = 128;
 constexpr int kKnnThreads = 64;  // k-NN blocks: a 16 KB heap, 13 blocks (26 warps) per SM
-constexpr int kBatchSolveBlocks = 8;  // default block batches per claimed item (256 systems at K = 32)
+constexpr int kBatchSolveBlocks = 8;  // default solve_item (256 systems at K = 32)
 constexpr int kStrips[3] = {1, 2, 4};  // k-NN strip lengths the batch offers
-// The persistent solve runs 8-warp blocks, 2 per SM (128 registers, dynamic
-// shared memory), like the per-grid kernels: two blocks in different phases
-// of the long unrolled solve wait far less for instruction fetch than 3 or 4
-// smaller ones (measured 291 ms per batch against 325 ms for 3 x 4 warps).
-constexpr int kBatchSolveWarps = 8;
-constexpr int kBatchSolveBlocksPerSM = 2;
+// kriging systems per claimed solve item: 32 per unit of solve_item at K = 32
+// (more of smaller systems), in whole 128-system batches
+inline int64_t solve_item_systems(int K, int nb) { return std::max<int64_t>(128, 1024 / K * nb); }
 
 __device__ __forceinline__ int upper_tile(const int64_t* off, int T, int64_t v) {
     // largest t with off[t] <= v  (off ascending, off[0] = 0)
@@ -329,16 +325,18 @@ __global__ void __launch_bounds__(kKnnThreads) k_batch_knn(
     }
 }
 
-// 6. persistent kriging solves for the tiles of one system size K; the tile's
-// descriptor is staged in shared memory so its fields are read where needed
-// instead of being held in registers across the solve
-template <int K>
-__global__ void __launch_bounds__(kBatchSolveWarps * 32, kBatchSolveBlocksPerSM) k_batch_solve(
+// 6. persistent kriging solves for the tiles of one system size K and variogram
+// model; the tile's descriptor is staged in shared memory so its fields are read
+// where needed instead of being held in registers across the solve. nb: batches of 128
+// systems per item. Dynamic shared memory: Geo<K>::SMEM bytes.
+template <int K, bool kSph>
+__global__ void __launch_bounds__(Geo<K>::THREADS, Geo<K>::BLOCKS) k_batch_solve(
     const TileDesc* __restrict__ td, const int* __restrict__ tiles, int nt,
     const int64_t* __restrict__ off, int64_t items, unsigned long long* __restrict__ ctr,
     const int4* __restrict__ orig, const int4* __restrict__ rec, const int* __restrict__ cell_start,
     const int* __restrict__ sat, int nb) {
-    extern __shared__ __align__(16) float smem[];
+    extern __shared__ __align__(16) float4 smem[];
+    __shared__ uint32_t slot;
     __shared__ long long s_item;
     __shared__ int s_j;
     __shared__ HashView s_h;
@@ -347,7 +345,8 @@ __global__ void __launch_bounds__(kBatchSolveWarps * 32, kBatchSolveBlocksPerSM)
     __shared__ int s_k;
     __shared__ float* s_depth;
     __shared__ float* s_var;
-    __shared__ const int32_t* s_ids;
+    __shared__ IdsView s_ids;
+    const uint32_t tm = tmem_take<Geo<K>::COLS>(&slot);
     for (;;) {
         if (threadIdx.x == 0) {
             s_item = (long long)atomicAdd(ctr, 1ull);
@@ -360,18 +359,19 @@ __global__ void __launch_bounds__(kBatchSolveWarps * 32, kBatchSolveBlocksPerSM)
                 s_k = d.k;
                 s_depth = d.depth;
                 s_var = d.var;
-                s_ids = d.ids;
+                s_ids = IdsView{d.ids, 0, 0, 0, 0};
             }
         }
         __syncthreads();
         const long long item = s_item;
         if (item >= items) break;
-        const int64_t b0 = (item - __ldg(off + s_j)) * nb;
-        for (int b = 0; b < nb; ++b)
-            okrige_solve_block<K, false, false, kBatchSolveWarps>(
-                s_h, s_g, s_k, s_p, 0, (int64_t)s_g.nx * s_g.ny, s_ids, s_depth, s_var, b0 + b, smem);
+        const int64_t b0 = (item - __ldg(off + s_j)) * nb, nodes = (int64_t)s_g.nx * s_g.ny;
+        const int64_t b1 = min(b0 + nb, (nodes + kSolveSystems - 1) / kSolveSystems);
+        okrige_solve_range<K, kSph, false, false>(s_h, s_g, s_k, s_p, 0, nodes, s_ids, s_depth, s_var, b0, b1,
+                                                  smem, tm);
         __syncthreads();  // the next item overwrites the staged descriptor
     }
+    tmem_give<Geo<K>::COLS>(&slot);
 }
 
 // 7. wide-key pass over every item of every tile; returns at once unless flagged
@@ -440,6 +440,7 @@ struct bg_batch_s {
     int64_t knn_items_s[3] = {0, 0, 0};    // k-NN items per strip length 1, 2, 4
     struct Group {
         int K;
+        int model;        // bg_variogram_model
         int nt;
         int64_t items;
         int* tiles;       // device: tile indices
@@ -519,18 +520,25 @@ void enqueue_batch(bg_batch_s* b, cudaStream_t st) {
     for (int gi = 0; gi < ng; ++gi) {
         const auto& G = b->groups[gi];
         if (G.items == 0) continue;
-        const unsigned grid = (unsigned)std::min<int64_t>(G.items, 152 * kBatchSolveBlocksPerSM);
         unsigned long long* ctr = b->d_ctr + 1 + gi;
-#define BG_SOLVE(KK)                                                                              \
-    k_batch_solve<KK><<<grid, kBatchSolveWarps * 32, kBatchSolveWarps * Geo<KK>::WARP_FLOATS * 4, st>>>(b->d_desc, G.tiles, G.nt, G.off, G.items, \
-                                                        ctr, b->d_orig, b->d_rec,                 \
-                                                        b->d_cell_start, b->d_sat, b->solve_nb)
+        const int nb = (int)(solve_item_systems(G.K, b->solve_nb) / kSolveSystems);
+#define BG_SOLVE_M(KK, SPH)                                                                     \
+    k_batch_solve<KK, SPH><<<(unsigned)std::min<int64_t>(G.items, 152 * Geo<KK>::BLOCKS),       \
+                             Geo<KK>::THREADS, Geo<KK>::SMEM, st>>>(                               \
+        b->d_desc, G.tiles, G.nt, G.off, G.items, ctr, b->d_orig, b->d_rec, b->d_cell_start,    \
+        b->d_sat, nb)
+#define BG_SOLVE(KK)                               \
+    if (G.model == BG_VARIOGRAM_SPHERICAL)         \
+        BG_SOLVE_M(KK, true);                      \
+    else                                           \
+        BG_SOLVE_M(KK, false)
         switch (G.K) {
             case 4: BG_SOLVE(4); break;
             case 8: BG_SOLVE(8); break;
             case 16: BG_SOLVE(16); break;
             default: BG_SOLVE(32); break;
         }
+#undef BG_SOLVE_M
 #undef BG_SOLVE
         note_launches(1);
     }
@@ -540,8 +548,11 @@ cudaError_t set_batch_solve_smem() {
     cudaError_t e = cudaSuccess;
 #define BG_SMEM(KK)                                                                          \
     if (e == cudaSuccess)                                                                    \
-        e = cudaFuncSetAttribute(k_batch_solve<KK>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                 kBatchSolveWarps * Geo<KK>::WARP_FLOATS * 4);
+        e = cudaFuncSetAttribute(k_batch_solve<KK, true>,                                    \
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, Geo<KK>::SMEM); \
+    if (e == cudaSuccess)                                                                    \
+        e = cudaFuncSetAttribute(k_batch_solve<KK, false>,                                   \
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, Geo<KK>::SMEM);
     BG_SMEM(4) BG_SMEM(8) BG_SMEM(16) BG_SMEM(32)
 #undef BG_SMEM
     return e;
@@ -553,7 +564,7 @@ cudaError_t set_batch_solve_smem() {
 bg_status set_solve_offsets(bg_batch_s* b) {
     if (b->off_nb == b->solve_nb) return BG_OK;
     for (auto& G : b->groups) {
-        const int sys_per_item = kBatchSolveWarps * (32 / (G.K / kR)) * kRounds * b->solve_nb;
+        const int64_t sys_per_item = solve_item_systems(G.K, b->solve_nb);
         std::vector<int64_t> go(G.nodes.size() + 1, 0);
         for (size_t j = 0; j < G.nodes.size(); ++j)
             go[j + 1] = go[j] + (G.nodes[j] + sys_per_item - 1) / sys_per_item;
@@ -621,7 +632,7 @@ bg_status bg_batch_create(bg_ctx_t ctx, const bg_tile* tiles, int n_tiles, bg_ba
     std::vector<int64_t> soff(n_tiles + 1, 0), item_off(n_tiles + 1, 0);
     std::vector<std::vector<int64_t>> item_off_s(3, std::vector<int64_t>(n_tiles + 1, 0));
     const int Ks[4] = {4, 8, 16, 32};
-    std::vector<std::vector<int>> gt(4);
+    std::vector<std::vector<int>> gt(8);  // by system size and variogram model: 2 q + model
     for (int t = 0; t < n_tiles; ++t) {
         const bg_tile& r = tiles[t];
         TileDesc& d = b->host_desc[t];
@@ -662,7 +673,7 @@ bg_status bg_batch_create(bg_ctx_t ctx, const bg_tile* tiles, int n_tiles, bg_ba
         if (r.method == 1) {
             b->total_ids += m * r.k;
             for (int q = 0; q < 4; ++q)
-                if (Ks[q] == d.K) gt[q].push_back(t);
+                if (Ks[q] == d.K) gt[2 * q + (r.variogram.model != 0)].push_back(t);
         }
     }
     b->knn_items = item_off[n_tiles];
@@ -690,7 +701,7 @@ bg_status bg_batch_create(bg_ctx_t ctx, const bg_tile* tiles, int n_tiles, bg_ba
     const size_t o_ctr = take(8 * 16);  // [0] k-NN items, [1 + g] solve groups
     const size_t o_ids = take(4 * (size_t)b->total_ids);
     std::vector<size_t> o_gt, o_go;
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < 8; ++q) {
         o_gt.push_back(take(4 * (gt[q].size() + 1)));
         o_go.push_back(take(8 * (gt[q].size() + 1)));
     }
@@ -734,9 +745,9 @@ bg_status bg_batch_create(bg_ctx_t ctx, const bg_tile* tiles, int n_tiles, bg_ba
             ids_at += (int64_t)d.g.nx * d.g.ny * d.k;
         }
     }
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < 8; ++q) {
         if (gt[q].empty()) continue;
-        bg_batch_s::Group G{Ks[q], (int)gt[q].size(), 0, (int*)(base + o_gt[q]),
+        bg_batch_s::Group G{Ks[q / 2], q & 1, (int)gt[q].size(), 0, (int*)(base + o_gt[q]),
                             (int64_t*)(base + o_go[q]), {}};
         for (int t : gt[q])
             G.nodes.push_back((int64_t)b->host_desc[t].g.nx * b->host_desc[t].g.ny);

@@ -3,6 +3,7 @@
 // is in okrige_dev.cuh; see there for the formulation.
 #include <algorithm>
 
+#include "knn_warp.cuh"
 #include "okrige_dev.cuh"
 
 namespace bg {
@@ -50,33 +51,107 @@ __global__ void __launch_bounds__(64) k_knn_ids(HashView h, GridView g, int k, i
     knn_strip<64, decltype(emit), false, kLen>(h, g, K, o.i, o.j, hp, flag, emit);
 }
 
+// The same by patches of 8 x 4 nodes per warp (knn_warp.cuh), a strip of `len`
+// patches along x each, spr strips per patch row, into the patch layout (and,
+// as upload indices, to nbr [node][k], if any).
 template <int K>
-__global__ void __launch_bounds__(128) k_knn_ids_wide(HashView h, GridView g, int k, int j0,
-                                                      int j1, int32_t* __restrict__ ids,
-                                                      int* __restrict__ flag) {
+__global__ void __launch_bounds__(64, KnnWarp<K>::kBlocksPerSM) k_knn_ids_patch(HashView h, GridView g, int k,
+                                                                                IdsView ids, int32_t* __restrict__ nbr,
+                                                                                int* __restrict__ flag,
+                                                                                int len, int spr) {
+    __shared__ typename KnnWarp<K>::Smem smem[2];
+    typename KnnWarp<K>::Smem& sm = smem[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
+    const unsigned w = blockIdx.x * 2 + (threadIdx.x >> 5);
+    const int py = (int)(w / (unsigned)spr), p0 = (int)(w % (unsigned)spr) * len;
+    const int jb = ids.j0 + py * 4, j = jb + (lane >> 3), qy = g.y0 + j * g.cell + g.cell / 2;
+    if (jb >= ids.j1) return;
+    KnnChain ch;
+    for (int p = p0; p < p0 + len && p < ids.pnx; ++p) {
+        const int i = p * 8 + (lane & 7), qx = g.x0 + i * g.cell + g.cell / 2;
+        const bool on = i < g.nx && j < ids.j1;
+        const int ox = g.x0 + p * 8 * g.cell + g.cell / 2, oy = g.y0 + jb * g.cell + g.cell / 2;
+        uint32_t base;
+        const float r = knn_first_radius<K>(h, ch, on, qx, qy, 8.0f * (float)g.cell, base);
+        const unsigned served = knn_patch<K>(h, sm, on, qx, qy, ox, oy, r, base, ch);
+        int32_t* o = ids.p + ((int64_t)py * ids.pnx + p) * 32 + lane;
+        if (served >> lane & 1) {
+#pragma unroll 8
+            for (int n = 0; n < k; ++n) o[n * ids.stride] = sm.pos[sm.buf[n * 32 + lane] & kPlaceMask];
+            if (nbr)
+                for (int n = 0; n < k; ++n)
+                    nbr[((int64_t)j * g.nx + i) * k + n] =
+                        __ldg(&h.rec[sm.pos[sm.buf[n * 32 + lane] & kPlaceMask]].w);
+        }
+        if (served != kFull) {
+            __syncwarp();
+            if (on && !(served >> lane & 1)) {
+                ch.dk = -1.0f;
+                uint64_t* hp = reinterpret_cast<uint64_t*>(sm.buf) + lane;
+                const int cnt = knn_lane<K>(h, qx, qy, hp);
+                if (cnt < 0) *flag = 1;  // the wide pass picks this node up
+                const uint64_t mask = (1ull << h.idx_bits) - 1;
+#pragma unroll 1
+                for (int n = 0; n < k; ++n) {
+                    const int u = n < cnt ? (int)(hp[n * 32] & mask) : -1;
+                    o[n * ids.stride] = u < 0 ? -1 : -2 - u;
+                    if (nbr) nbr[((int64_t)j * g.nx + i) * k + n] = u;
+                }
+                if (cnt == K) {
+                    ch.d1 = sqrtf((float)(hp[0] >> h.idx_bits));
+                    ch.dk = sqrtf((float)(hp[(K - 1) * 32] >> h.idx_bits));
+                }
+            }
+        }
+        __syncwarp();
+    }
+}
+
+template <int K>
+__global__ void __launch_bounds__(128) k_knn_ids_wide(HashView h, GridView g, int k, IdsView ids,
+                                                      int32_t* __restrict__ nbr, int* __restrict__ flag) {
     if (*(volatile int*)flag == 0) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int gx = (g.nx + 15) / 16;
-    const int64_t nb = (int64_t)gx * ((j1 - j0 + 7) / 8);
+    const int64_t nb = (int64_t)gx * ((ids.j1 - ids.j0 + 7) / 8);
     for (int64_t b = blockIdx.x; b < nb; b += gridDim.x)
-        knn_ids_node<K, true>(h, g, k, (int64_t)j0 * g.nx, ids, flag,
-                              patch_node((int)(b % gx), j0 / 8 + (int)(b / gx), warp, lane), j1,
-                              nullptr);
+        knn_ids_node_wide<K>(h, g, k, ids, nbr, patch_node((int)(b % gx), ids.j0 / 8 + (int)(b / gx), warp, lane));
 }
 
-// dynamic shared memory: kGridSolveWarps * Geo<K>::WARP_FLOATS floats
-template <int K, bool kIdw>
-__global__ void __launch_bounds__(kGridSolveWarps * 32, kGridSolveBlocksPerSM) k_okrige_solve(
-    HashView h, GridView g, int k, OkParams p, int64_t node0, int64_t nodes,
-    const int32_t* __restrict__ ids, float* __restrict__ depth, float* __restrict__ var,
-    IdwFuse fz) {
-    extern __shared__ __align__(16) float smem[];
-    // the ids of a block two waves on (2 blocks per SM): the k-NN kernel wrote
-    // them a launch ago and they have left L2 since
-    prefetch_ids_l2(ids, nodes, k, (int64_t)blockIdx.x + kIdsPrefetchBlocks,
-                    kGridSolveWarps * Geo<K>::SYS * kRounds);
-    okrige_solve_block<K, false, kIdw, kGridSolveWarps>(h, g, k, p, node0, nodes, ids, depth, var,
-                                                        blockIdx.x, smem, nullptr, nullptr, fz);
+// Solve blocks take `per` consecutive batches of 128 systems: one take of the
+// tensor memory and one block start for several batches (about 10 us each),
+// but at least four waves of blocks, so that the last wave stays short and
+// small grids spread over the SMs.
+template <int K>
+int solve_batches_per_block(int64_t batches) {
+    return (int)std::min<int64_t>(8, std::max<int64_t>(1, batches / (4 * 152 * Geo<K>::BLOCKS)));
+}
+
+template <int K, class Fn>
+__device__ __forceinline__ void solve_batches(const IdsView& ids, int64_t nsys, int k, int per, Fn fn) {
+    __shared__ uint32_t slot;
+    const uint32_t tm = tmem_take<Geo<K>::COLS>(&slot);
+    const int64_t batches = (nsys + kSolveSystems - 1) / kSolveSystems;
+    const int64_t b0 = (int64_t)blockIdx.x * per, b1 = min(b0 + per, batches);
+    // the ids of this block's other batches and of the block that will follow it
+    // on its SM: the k-NN kernel wrote them a launch ago and they have left L2
+    // since
+    for (int64_t b = b0 + 1; b < b1; ++b) prefetch_ids_l2(ids, nsys, k, b);
+    prefetch_ids_l2(ids, nsys, k, b0 + (int64_t)152 * Geo<K>::BLOCKS * per);
+    fn(b0, b1, tm);
+    tmem_give<Geo<K>::COLS>(&slot);
+}
+
+// dynamic shared memory: Geo<K>::SMEM bytes
+template <int K, bool kSph, bool kIdw>
+__global__ void __launch_bounds__(Geo<K>::THREADS, Geo<K>::BLOCKS) k_okrige_solve(
+    HashView h, GridView g, int k, OkParams p, int64_t node0, int64_t nsys, IdsView ids,
+    float* __restrict__ depth, float* __restrict__ var, IdwFuse fz, int per) {
+    extern __shared__ __align__(16) float4 smem[];
+    solve_batches<K>(ids, nsys, k, per, [&](int64_t b0, int64_t b1, uint32_t tm) {
+        okrige_solve_range<K, kSph, false, kIdw>(h, g, k, p, node0, nsys, ids, depth, var, b0, b1, smem,
+                                                 tm, nullptr, nullptr, fz);
+    });
 }
 
 // Copy rows [off, off + n) of the outputs to their host destinations on
@@ -95,31 +170,42 @@ bg_status copy_rows_to_host(const HostOut* ho, int64_t off, int64_t n, const flo
     return e == cudaSuccess ? BG_OK : cuda_fail(e, "device-to-host copy");
 }
 
-template <int K>
-bg_status launch_k(const HashView& h, const GridView& g, int k, const OkParams& p, float* depth,
+template <int K, bool kSph>
+bg_status launch_k(const bg_soundings_s* snd, const HashView& h, const GridView& g, int k, const OkParams& p, float* depth,
                    float* var, int32_t* nbr, bg_ctx_s* ctx, cudaStream_t st, const IdwFuse* fz,
                    const HostOut* ho) {
     using Gm = Geo<K>;
-    // grid rows per chunk: the id buffer stays near 1 GiB unless the caller
-    // passed nbr_out, which then holds all ids
-    int64_t rows = g.ny;
-    if (!nbr) rows = std::max<int64_t>(8, ((((int64_t)1 << 28) / ((int64_t)k * g.nx)) / 8) * 8);
-    if (rows > g.ny) rows = g.ny;
+    // grid rows per chunk: the id buffer stays near 1 GiB. The patch layout rounds
+    // the rows up to whole patches; where the search by patches does not serve, or
+    // the budget has no room for that, the rows layout does, in nbr_out itself
+    // when the caller passed it (then whole).
+    const int64_t most = std::max<int64_t>(8, ((((int64_t)1 << 28) / ((int64_t)k * g.nx)) / 8) * 8);
+    int64_t rows = std::min<int64_t>(g.ny, most);
     const size_t flag_bytes = 256;
-    const size_t id_bytes = nbr ? 0 : (size_t)rows * g.nx * k * sizeof(int32_t);
+    const int pnx = (g.nx + 7) / 8;
+    bool patches = knn_patch_fits<K>(snd->info, g.cell, g.nx, g.ny);
+    const int64_t slots = (int64_t)pnx * ((rows + 3) / 4) * 32;
+    size_t id_bytes = patches ? (size_t)slots * k * sizeof(int32_t) : 0;
     void* scratch = nullptr;
-    bg_status rc = dalloc(ctx, &scratch, flag_bytes + id_bytes, st);
-    if (rc != BG_OK) return rc;
+    bg_status rc = BG_OK;
+    if (patches) {
+        rc = dalloc(ctx, &scratch, flag_bytes + id_bytes, st);
+        patches = rc == BG_OK;
+    }
+    if (!patches) {
+        if (nbr) rows = g.ny;
+        id_bytes = nbr ? 0 : (size_t)rows * g.nx * k * sizeof(int32_t);
+        rc = dalloc(ctx, &scratch, flag_bytes + id_bytes, st);
+        if (rc != BG_OK) return rc;
+    }
     int* flag = (int*)scratch;
     const int gx = (g.nx + 15) / 16;
-    const int64_t sys_per_block = (int64_t)kGridSolveWarps * Gm::SYS * kRounds;
-    const int smem_bytes = kGridSolveWarps * Gm::WARP_FLOATS * (int)sizeof(float);
-    cudaError_t ea = cudaFuncSetAttribute(k_okrige_solve<K, false>,
-                                          cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
+    cudaError_t ea = cudaFuncSetAttribute(k_okrige_solve<K, kSph, false>,
+                                          cudaFuncAttributeMaxDynamicSharedMemorySize, Gm::SMEM);
     if constexpr (K == 32)
         if (ea == cudaSuccess)
-            ea = cudaFuncSetAttribute(k_okrige_solve<K, true>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
+            ea = cudaFuncSetAttribute(k_okrige_solve<K, kSph, true>,
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, Gm::SMEM);
     if (ea != cudaSuccess) {
         dfree(ctx, scratch, flag_bytes + id_bytes, st);
         return cuda_fail(ea, "solve shared-memory size");
@@ -129,16 +215,24 @@ bg_status launch_k(const HashView& h, const GridView& g, int k, const OkParams& 
         const int64_t nb = (int64_t)gx * ((j1 - j0 + 7) / 8);
         const int len = strip_len_for((j1 - j0) * (int64_t)g.nx);
         const int64_t nbs = (int64_t)((g.nx + 16 * len - 1) / (16 * len)) * ((j1 - j0 + 3) / 4);
-        int32_t* chunk_ids = nbr ? nbr + j0 * g.nx * k : (int32_t*)((char*)scratch + flag_bytes);
+        int32_t* chunk_ids =
+            nbr && !patches ? nbr + j0 * g.nx * k : (int32_t*)((char*)scratch + flag_bytes);
         cudaError_t e = cudaMemsetAsync(flag, 0, sizeof(int), st);
         if (e != cudaSuccess) {
             rc = cuda_fail(e, "memset");
             break;
         }
         const int64_t nodes = (j1 - j0) * g.nx;
+        const int pny = (int)((j1 - j0 + 3) / 4);
+        const IdsView ids{chunk_ids, patches ? slots : 0, pnx, (int)j0, (int)j1};
+        const int64_t nsys = patches ? (int64_t)pnx * pny * 32 : nodes;
         {
             ProfScope ps(ctx, kProfKnnIds, nodes, st);
-            if (len == 1)
+            const int plen = patch_strip_len((int64_t)pnx * pny), spr = (pnx + plen - 1) / plen;
+            if (patches)
+                k_knn_ids_patch<K><<<(unsigned)(((int64_t)spr * pny + 1) / 2), 64, 0, st>>>(h, g, k, ids, nbr, flag,
+                                                                                           plen, spr);
+            else if (len == 1)
                 k_knn_ids<K, 1><<<(unsigned)nbs, 64, 0, st>>>(h, g, k, (int)j0, (int)j1, chunk_ids, flag);
             else if (len == 2)
                 k_knn_ids<K, 2><<<(unsigned)nbs, 64, 0, st>>>(h, g, k, (int)j0, (int)j1, chunk_ids, flag);
@@ -146,21 +240,23 @@ bg_status launch_k(const HashView& h, const GridView& g, int k, const OkParams& 
                 k_knn_ids<K, 4><<<(unsigned)nbs, 64, 0, st>>>(h, g, k, (int)j0, (int)j1, chunk_ids, flag);
         }
         k_knn_ids_wide<K><<<(unsigned)std::min<int64_t>(nb, 152 * 4), 128, 0, st>>>(
-            h, g, k, (int)j0, (int)j1, chunk_ids, flag);
-        const int64_t sb = (nodes + sys_per_block - 1) / sys_per_block;
+            h, g, k, ids, patches ? nbr : nullptr, flag);
+        const int64_t batches = (nsys + kSolveSystems - 1) / kSolveSystems;
+        const int per = solve_batches_per_block<K>(batches);
+        const unsigned sb = (unsigned)((batches + per - 1) / per);
         {
             ProfScope ps(ctx, kProfSolve, nodes, st);
             bool fused = false;
-            if constexpr (K == 32) {  // the fused IDW runs with 8 threads per system
+            if constexpr (K == 32) {
                 if (fz) {
-                    k_okrige_solve<K, true><<<(unsigned)sb, kGridSolveWarps * 32, smem_bytes, st>>>(
-                        h, g, k, p, j0 * g.nx, nodes, chunk_ids, depth, var, *fz);
+                    k_okrige_solve<K, kSph, true><<<sb, Gm::THREADS, Gm::SMEM, st>>>(
+                        h, g, k, p, j0 * g.nx, nsys, ids, depth, var, *fz, per);
                     fused = true;
                 }
             }
             if (!fused)
-                k_okrige_solve<K, false><<<(unsigned)sb, kGridSolveWarps * 32, smem_bytes, st>>>(
-                    h, g, k, p, j0 * g.nx, nodes, chunk_ids, depth, var, IdwFuse{});
+                k_okrige_solve<K, kSph, false><<<sb, Gm::THREADS, Gm::SMEM, st>>>(
+                    h, g, k, p, j0 * g.nx, nsys, ids, depth, var, IdwFuse{}, per);
         }
         note_launches(3);
         e = cudaGetLastError();
@@ -214,19 +310,19 @@ __global__ void __launch_bounds__(128) k_knn_ids_pts_wide(HashView h, PointsView
         knn_ids_point_wide<K>(h, __ldg(q.x + p), __ldg(q.y + p), k, ids + (p - p0) * k);
 }
 
-// dynamic shared memory: kGridSolveWarps * Geo<K>::WARP_FLOATS floats
-template <int K>
-__global__ void __launch_bounds__(kGridSolveWarps * 32, kGridSolveBlocksPerSM) k_okrige_solve_pts(
-    HashView h, PointsView q, int k, OkParams p, int64_t p0, int64_t nodes,
-    const int32_t* __restrict__ ids, float* __restrict__ depth, float* __restrict__ var) {
-    extern __shared__ __align__(16) float smem[];
-    prefetch_ids_l2(ids, nodes, k, (int64_t)blockIdx.x + kIdsPrefetchBlocks,
-                    kGridSolveWarps * Geo<K>::SYS * kRounds);
-    okrige_solve_block<K, true, false, kGridSolveWarps>(h, GridView{}, k, p, p0, nodes, ids, depth,
-                                                        var, blockIdx.x, smem, q.x, q.y);
+// dynamic shared memory: Geo<K>::SMEM bytes
+template <int K, bool kSph>
+__global__ void __launch_bounds__(Geo<K>::THREADS, Geo<K>::BLOCKS) k_okrige_solve_pts(
+    HashView h, PointsView q, int k, OkParams p, int64_t p0, int64_t nsys, IdsView ids,
+    float* __restrict__ depth, float* __restrict__ var, int per) {
+    extern __shared__ __align__(16) float4 smem[];
+    solve_batches<K>(ids, nsys, k, per, [&](int64_t b0, int64_t b1, uint32_t tm) {
+        okrige_solve_range<K, kSph, true, false>(h, GridView{}, k, p, p0, nsys, ids, depth, var, b0, b1,
+                                                 smem, tm, q.x, q.y);
+    });
 }
 
-template <int K>
+template <int K, bool kSph>
 bg_status launch_pts_k(const HashView& h, const PointsView& q, int k, const OkParams& p,
                        float* depth, float* var, int32_t* nbr, bg_ctx_s* ctx, cudaStream_t st) {
     using Gm = Geo<K>;
@@ -240,10 +336,8 @@ bg_status launch_pts_k(const HashView& h, const PointsView& q, int k, const OkPa
     bg_status rc = dalloc(ctx, &scratch, flag_bytes + id_bytes, st);
     if (rc != BG_OK) return rc;
     int* flag = (int*)scratch;
-    const int64_t sys_per_block = (int64_t)kGridSolveWarps * Gm::SYS * kRounds;
-    const int smem_bytes = kGridSolveWarps * Gm::WARP_FLOATS * (int)sizeof(float);
     const cudaError_t ea = cudaFuncSetAttribute(
-        k_okrige_solve_pts<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
+        k_okrige_solve_pts<K, kSph>, cudaFuncAttributeMaxDynamicSharedMemorySize, Gm::SMEM);
     if (ea != cudaSuccess) {
         dfree(ctx, scratch, flag_bytes + id_bytes, st);
         return cuda_fail(ea, "solve shared-memory size");
@@ -270,11 +364,13 @@ bg_status launch_pts_k(const HashView& h, const PointsView& q, int k, const OkPa
         }
         k_knn_ids_pts_wide<K><<<(unsigned)std::min<int64_t>((n + 127) / 128, 152 * 4), 128, 0, st>>>(
             h, q, k, p0, p1, chunk_ids, flag);
-        const int64_t sb = (n + sys_per_block - 1) / sys_per_block;
+        const int64_t batches = (n + kSolveSystems - 1) / kSolveSystems;
+        const int bper = solve_batches_per_block<K>(batches);
         {
             ProfScope ps(ctx, kProfSolve, n, st);
-            k_okrige_solve_pts<K><<<(unsigned)sb, kGridSolveWarps * 32, smem_bytes, st>>>(
-                h, q, k, p, p0, n, chunk_ids, depth, var);
+            k_okrige_solve_pts<K, kSph>
+                <<<(unsigned)((batches + bper - 1) / bper), Gm::THREADS, Gm::SMEM, st>>>(
+                    h, q, k, p, p0, n, IdsView{chunk_ids, 0, 0, 0, 0}, depth, var, bper);
         }
         note_launches(3);
         e = cudaGetLastError();
@@ -296,12 +392,17 @@ bg_status launch_okrige_points(const bg_soundings_s* s, const PointsView& q, int
     HashView h = s->h;
     const int K = k <= 4 ? 4 : k <= 8 ? 8 : k <= 16 ? 16 : 32;
     h.r0 = start_halfwidth(s, K);
+    const bool sph = p.model == BG_VARIOGRAM_SPHERICAL;
+#define BG_OK_CASE(KK) \
+    (sph ? launch_pts_k<KK, true>(h, q, k, p, depth, var, nbr, s->ctx, st) \
+         : launch_pts_k<KK, false>(h, q, k, p, depth, var, nbr, s->ctx, st))
     switch (K) {
-        case 4: return launch_pts_k<4>(h, q, k, p, depth, var, nbr, s->ctx, st);
-        case 8: return launch_pts_k<8>(h, q, k, p, depth, var, nbr, s->ctx, st);
-        case 16: return launch_pts_k<16>(h, q, k, p, depth, var, nbr, s->ctx, st);
-        default: return launch_pts_k<32>(h, q, k, p, depth, var, nbr, s->ctx, st);
+        case 4: return BG_OK_CASE(4);
+        case 8: return BG_OK_CASE(8);
+        case 16: return BG_OK_CASE(16);
+        default: return BG_OK_CASE(32);
     }
+#undef BG_OK_CASE
 }
 
 bg_status launch_okrige(const bg_soundings_s* s, const GridView& g, int k, const OkParams& p,
@@ -310,8 +411,8 @@ bg_status launch_okrige(const bg_soundings_s* s, const GridView& g, int k, const
     HashView h = s->h;
     const int K = k <= 4 ? 4 : k <= 8 ? 8 : k <= 16 ? 16 : 32;
     if (fz && K != 32) {
-        // smaller systems run 2 or 4 threads each: the IDW takes its own pass
-        // (the same depths: idw_from sums in the same fixed order)
+        // the fused kernel is built for the largest system only: the IDW takes its
+        // own pass (the same depths: idw_from sums in the same fixed order)
         bg_status rc = launch_idw(s, g, fz->k, fz->power, fz->out, nullptr, st);
         if (rc != BG_OK) return rc;
         if (ho && ho->idw) {  // the whole IDW grid is done: copy it now
@@ -323,12 +424,17 @@ bg_status launch_okrige(const bg_soundings_s* s, const GridView& g, int k, const
         fz = nullptr;
     }
     h.r0 = start_halfwidth(s, K);
+    const bool sph = p.model == BG_VARIOGRAM_SPHERICAL;
+#define BG_OK_CASE(KK) \
+    (sph ? launch_k<KK, true>(s, h, g, k, p, depth, var, nbr, s->ctx, st, fz, ho) \
+         : launch_k<KK, false>(s, h, g, k, p, depth, var, nbr, s->ctx, st, fz, ho))
     switch (K) {
-        case 4: return launch_k<4>(h, g, k, p, depth, var, nbr, s->ctx, st, fz, ho);
-        case 8: return launch_k<8>(h, g, k, p, depth, var, nbr, s->ctx, st, fz, ho);
-        case 16: return launch_k<16>(h, g, k, p, depth, var, nbr, s->ctx, st, fz, ho);
-        default: return launch_k<32>(h, g, k, p, depth, var, nbr, s->ctx, st, fz, ho);
+        case 4: return BG_OK_CASE(4);
+        case 8: return BG_OK_CASE(8);
+        case 16: return BG_OK_CASE(16);
+        default: return BG_OK_CASE(32);
     }
+#undef BG_OK_CASE
 }
 
 }  // namespace bg

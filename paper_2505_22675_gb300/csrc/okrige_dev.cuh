@@ -2,9 +2,8 @@
 // soundings, shared by the per-grid kernels (okrige.cu) and the batched
 // persistent kernels (batch.cu).
 //
-// Per grid node: exact k-NN to neighbour ids (knn_ids_node, one thread per
-// node); then the kriging system, solved by G = K/4 threads that each own
-// R = 4 rows, so a warp solves 32/G systems at once (okrige_solve_block).
+// Per grid node: exact k-NN to neighbour ids (knn_warp.cuh, knn.cuh); then the
+// kriging systems (okrige_solve_range).
 //
 // The bordered variogram system [Gamma 1; 1^T 0][lambda; mu] = [gamma_0; 1]
 // is reduced with sum(lambda) = 1 by eliminating lambda_0 (the nearest
@@ -13,29 +12,48 @@
 //     A lambda' = b,  lambda_0 = 1 - sum(lambda'),  mu = gamma_00 - sum_a Gamma_0a lambda_a.
 // A is symmetric positive definite for a conditionally negative definite
 // variogram (spherical and exponential are, in 2-D), so |A[r][c]| is bounded
-// by its largest diagonal entry. It is assembled once per entry straight into
-// a 30-bit fixed-point copy in shared memory (packed lower triangle), factored
-// by Cholesky in FP32 with each thread's rows in registers (thread t, slot s
-// holds row G*s + t, columns 0 .. G*(s+1)-1; pivots move between the G
-// threads by warp shuffles, column entries through a small column buffer in
-// shared memory). The back sweeps also run on the register rows, one column at
-// a time with a group sum (no transposed copy of the factor), so shared
-// memory per system stays near 2.8 KB (K = 32) and,
-// with the registers held to 128, a GB300 SM keeps 16 warps resident. One
-// step of iterative refinement follows: x is rounded to 24-bit fixed point x'
-// (exact in FP32), the residual b - A' x' is accumulated exactly in 64-bit
-// integers, and the correction reuses the factor. The weight sum closes in FP64:
-// lambda_0 = 1 - sum(lambda'). Outputs:
+// by its largest diagonal entry.
+//
+// Layout: a warp's 32 lanes run 32 systems in step, so nothing is exchanged
+// between lanes. Two threads share a system (one for K <= 8): the same lane of
+// warps w and w + 4, each owning four rows of every tile; 8 warps per SM at
+// K = 32, 16 at K = 16. The triangle is worked in tiles of 8 x 8 (left-looking
+// block Cholesky): a tile is assembled from the rows' records into registers,
+// updated with the factor's earlier columns, factored (by both threads alike,
+// after an exchange through shared memory) or solved against the diagonal tile,
+// and stored. The factor lives in tensor memory, used as a plain 128-lane store:
+// lane l holds system l's 512 columns, exactly the 6 off-diagonal tiles of 64
+// words and the 4 packed diagonal tiles of 28 (+ 4) of a K = 32 system, and both
+// of its warps reach it. Shared memory could not hold it (2 KB x 128 systems
+// + the records), and would serve one 128-byte wavefront per cycle to the
+// whole SM where tensor memory serves each scheduler its own; the loads are
+// issued four columns ahead of the multiplies. The records, right-hand sides
+// and integer sums stay in shared memory, system-interleaved 16-byte vectors.
+// The multiplies run as packed two-lane instructions (add/sub/mul/fma.rn.f32x2:
+// one instruction, two IEEE single operations), two rows per instruction
+// against one column's scalar in both lanes (which costs no extra
+// instruction). The factor works on -A (the tile sums then need no negations).
+// What bounds it: issue and latency at two warps per scheduler (half of the
+// issue slots; FP32 pipe half busy in the factor, the square roots and
+// conversions half busy in the residual), K = 32 with the fused IDW: 52,000
+// cycles per 128 systems, of them factor 21,000, residual 16,000, gathers 3,500.
+// Measured on one survey line (3,001 x 692 nodes, k = 32, fused IDW): 2.76 ms
+// against 3.84 ms for 8 threads per system with the factor in registers (1,500
+// warp instructions per system there, 780 here; one thread per system: 630, but
+// one warp per scheduler and 3.5 ms); 256 x 256 tile, k = 16: 29 against 37 us.
+// Loading the next batch's ids and records during the last solve, and keeping
+// one tile of A' in the shared memory that is left at K = 32, changed nothing.
+//
+// One step of iterative refinement follows the solve: A' is A rounded to a
+// 30-bit fixed point, x is rounded to 24-bit fixed point x' (exact in FP32),
+// and the residual b - A' x' is accumulated exactly in 64-bit integers; at K =
+// 32 the tiles of A are evaluated again rather than kept (on-chip memory holds
+// one of the two triangles), at K = 16 most are kept in tensor memory. The correction reuses the factor. The weight sum
+// closes in FP64: lambda_0 = 1 - sum(lambda'). Outputs:
 //     zhat    = z_0 + sum_a lambda_a (z_a - z_0)          (= sum lambda_i z_i)
 //     sigma^2 = lambda_0 gamma_00 + sum_a lambda_a gamma_a0 + mu.
 // Rows beyond k_eff - 1 are identity rows with zero right-hand side, so every
-// system has the fixed size K and all loops over rows and columns unroll.
-// Much of the FP32 work runs as packed two-lane instructions (add/sub/mul/fma
-// .rn.f32x2: one instruction, two IEEE single operations, each lane rounded
-// as its scalar form): the variogram assembly two rows at a time, the per-row
-// variograms of the prologue, and column pairs of the Cholesky update. The
-// solve is issue- and latency-bound, so halving those instructions pays, and
-// the results are bitwise those of the scalar code.
+// system has the fixed size K.
 #pragma once
 
 #include <algorithm>
@@ -49,35 +67,38 @@
 namespace bg {
 
 
-constexpr int kR = 4;            // rows per thread
-constexpr int kRounds = 1;       // system batches per warp (one: more, shorter blocks balance best)
-constexpr int kBwdLook = 2;      // back-sweep pipeline depth (see bwd_step)
-// The grid and point-list solve kernels run 8-warp blocks, 2 per SM (the same
-// 16 warps): with the unrolled solve's long instruction stream, two blocks in
-// different phases fetch far fewer distinct instructions than four.
-constexpr int kGridSolveWarps = 8;
-constexpr int kGridSolveBlocksPerSM = 2;
-// solve blocks ahead whose neighbour ids a block prefetches into L2: two
-// waves of the 152 SMs (one to eight waves measured the same)
-constexpr int kIdsPrefetchBlocks = 2 * 152 * kGridSolveBlocksPerSM;
+constexpr int kSolveSystems = 128;  // systems per block, one lane of tensor memory each
 
 template <int K>
 struct Geo {
-    static constexpr int G = K / kR;                      // threads per system
-    static constexpr int SYS = 32 / G;                    // systems per warp
-    static constexpr int LEN = G * kR * (kR + 1) / 2;     // register floats of L
-    static constexpr int TRI = K * (K + 1) / 2;           // packed lower triangle of A
-    static constexpr int TRIP = (TRI + 3) / 4 * 4;        // the triangle padded to 16 bytes
-    // per system: the fixed-point A as a packed lower triangle (row r at
-    // r (r + 1) / 2), the rows' records (three arrays of K floats: x, y,
-    // Gamma_r0, in a region of 4 K), and two column buffers for the Cholesky
-    // broadcasts (16-byte aligned); the stride is = G (mod 32) so that the
-    // G-thread groups of a warp spread over the banks
-    static constexpr int CB = TRIP + 4 * K;
-    static constexpr int RAW = CB + 2 * K;
-    static constexpr int SYS_FLOATS = RAW + ((G - RAW % 32) + 32) % 32;
-    static constexpr int WARP_FLOATS = SYS * SYS_FLOATS;
-    static __host__ __device__ constexpr int off(int s) { return G * s * (s + 1) / 2; }
+    static constexpr int TB = K < 8 ? K : 8;             // tile side
+    static constexpr int NB = K / TB;                    // tile rows
+    static constexpr int P = TB / 2;                     // row pairs of a tile
+    static constexpr int TRI = TB * (TB - 1) / 2;        // strictly lower entries of a diagonal tile
+    static constexpr int OFF = NB * (NB - 1) / 2;        // off-diagonal tiles
+    static constexpr int TILE = TB * TB;                 // words of an off-diagonal tile
+    static constexpr int DTILE = 32;                     // words of a packed diagonal tile
+    static constexpr int TPS = NB > 1 ? 2 : 1;           // threads per system
+    static constexpr int THREADS = TPS * kSolveSystems;
+    // tensor-memory columns of a block (0: the factor stays in registers). At K =
+    // 16 the two blocks of an SM have room for most of A' too: the off-diagonal
+    // and the first diagonal tile, 32 words a thread each, from KEEP on.
+    static constexpr int KEEP = OFF * TILE + NB * DTILE;
+    static constexpr int COLS = NB == 1 ? 0 : K == 16 ? KEEP + 128 : KEEP;
+    // shared memory, in 16-byte vectors per system: vectors of four rows
+    static constexpr int Q = K / 4;
+    static constexpr int X = 0, Y = Q, Z = 2 * Q;        // the rows' records
+    static constexpr int DZ = 3 * Q, G0 = 4 * Q;         // z_a - z_0, gamma_0a
+    static constexpr int V = 5 * Q;                      // L^-1 b, then x' (integers)
+    static constexpr int DI = 6 * Q;                     // -1 / L[r][r]
+    static constexpr int XB = 7 * Q;                     // exchange of eight rows, two buffers
+    static constexpr int EX = XB + 4;                    // exchange of the prologue
+    static constexpr int ACC = EX + 2;                   // 64-bit residual sums, one set a thread
+    static constexpr int DG = ACC;                       // diagonal tile (16 vectors), before them
+    static constexpr int VECS = NB == 1 ? ACC : ACC + 4 * Q;
+    static constexpr int SMEM = VECS * 16 * kSolveSystems;
+    // resident blocks per SM the registers are held to
+    static constexpr int BLOCKS = K == 32 ? 1 : K == 16 ? 2 : 4;
 };
 
 __device__ __forceinline__ float variogram(const OkParams& p, float h_m) {
@@ -113,10 +134,10 @@ __device__ __forceinline__ float gamma_pair_f(const OkParams& p, float dx, float
     return fmaf(p.c, -expm1f(-h_cm * p.inv_a * 0.01f), p.c0);
 }
 
-// one hardware square-root approximation (sqrt.approx.f32: a few ulp, 0 at 0)
+// one hardware square-root approximation (a few ulp, 0 at 0 and below 2^-126)
 __device__ __forceinline__ float sqrt_approx(float x) {
     float y;
-    asm("sqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
 
@@ -134,17 +155,6 @@ __device__ __forceinline__ ScaledVgm scaled_vgm(const OkParams& p, float sa) {
     const float kinv = p.inv_a * 0.01f;
     const float cs = p.c * sa;
     return ScaledVgm{kinv * kinv, p.c0 * sa, cs, -0.5f * cs, 1.5f * cs};
-}
-
-template <bool kSpherical>
-__device__ __forceinline__ float gamma_pair_scaled(const ScaledVgm& v, float dx, float dy) {
-    const float t2 = fmaf(dx, dx, dy * dy) * v.kinv2;
-    if constexpr (kSpherical) {
-        const float t = fminf(sqrt_approx(t2), 1.0f);  // the polynomial is the sill at t = 1
-        return fmaf(t, fmaf(v.k2, t * t, v.k3), v.c0s);
-    } else {
-        return fmaf(v.cs, -expm1f(-sqrt_approx(t2)), v.c0s);
-    }
 }
 
 // Packed two-lane FP32 arithmetic (one instruction for two IEEE single
@@ -178,25 +188,6 @@ __device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigne
     unsigned long long r;
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
     return r;
-}
-
-// Two assembly entries of one column (x0, y0, gcc) from rows a and b at once,
-// in the fixed-point scale, spherical model: each lane takes exactly the
-// operations of (z + gcc) - gamma_pair_scaled<true>(sv, x - x0, y - y0).
-__device__ __forceinline__ void gamma_rows2_sph(const ScaledVgm& v, float xa, float xb, float ya,
-                                                float yb, float za, float zb, float x0, float y0,
-                                                float gcc, float& oa, float& ob) {
-    const unsigned long long dx = sub2(pk2(xa, xb), pk2(x0, x0));
-    const unsigned long long dy = sub2(pk2(ya, yb), pk2(y0, y0));
-    const unsigned long long t2 = mul2(fma2(dx, dx, mul2(dy, dy)), pk2(v.kinv2, v.kinv2));
-    float ta, tb;
-    upk2(t2, ta, tb);
-    ta = fminf(sqrt_approx(ta), 1.0f);  // the polynomial is the sill at t = 1
-    tb = fminf(sqrt_approx(tb), 1.0f);
-    const unsigned long long t = pk2(ta, tb);
-    const unsigned long long gm = fma2(t, fma2(pk2(v.k2, v.k2), mul2(t, t), pk2(v.k3, v.k3)),
-                                       pk2(v.c0s, v.c0s));
-    upk2(sub2(add2(pk2(za, zb), pk2(gcc, gcc)), gm), oa, ob);
 }
 
 // gamma_pair_f, spherical model, for two rows at once (packed FP32, each lane
@@ -235,39 +226,59 @@ __device__ __forceinline__ void gamma_cm_sph2(const OkParams& p, int dxa, int dy
 
 // ------------------------------------------------------------ k-NN -> ids
 
-template <int K, bool kWide>
-__device__ __forceinline__ void knn_ids_node(const HashView& h, const GridView& g, int k,
-                                             int64_t node0, int32_t* __restrict__ ids,
-                                             int* __restrict__ flag, NodeIdx nd, int j1,
-                                             uint64_t* hp) {
-    if (nd.i >= g.nx || nd.j >= j1) return;
-    const int64_t node = (int64_t)nd.j * g.nx + nd.i;
+// The neighbour ids of a range of systems, in one of two layouts.
+//   rows (stride 0): system i's k ids at p[i k], upload indices, -1 past k_eff;
+//     system i is the i-th node (row-major) or point of the range.
+//   patches (stride > 0): id n of system i at p[n stride + i], so that a warp's
+//     loads and stores are whole lines; systems are the slots of 8 x 4 node
+//     patches (32 per patch, patches row-major, the ones outside the grid
+//     unused). A value >= 0 is a position in the cell-sorted records, whose
+//     neighbours in space are neighbours in memory; -1 none; -2 - u the upload
+//     index u (a node that the per-thread search served).
+struct IdsView {
+    int32_t* p;
+    int64_t stride;
+    int pnx;     // patches: per row of patches
+    int j0, j1;  // patches: the range's grid rows
+};
+// grid node of a patch slot; false outside the grid
+__device__ __forceinline__ bool slot_node(const IdsView& v, const GridView& g, int64_t slot, int& i, int& j) {
+    const unsigned patch = (unsigned)(slot >> 5), py = patch / (unsigned)v.pnx;
+    const int l = (int)(slot & 31);
+    i = (int)(patch - py * (unsigned)v.pnx) * 8 + (l & 7);
+    j = v.j0 + (int)py * 4 + (l >> 3);
+    return i < g.nx && j < v.j1;
+}
+__device__ __forceinline__ int64_t node_slot(const IdsView& v, int i, int j) {
+    return ((int64_t)((j - v.j0) >> 2) * v.pnx + (i >> 3)) * 32 + ((j - v.j0) & 3) * 8 + (i & 7);
+}
+
+// Wide-key neighbour ids of one grid node whose table bound does not fit the
+// packed key (patches layout: also to nbr, if any); other nodes return.
+template <int K>
+__device__ __forceinline__ void knn_ids_node_wide(const HashView& h, const GridView& g, int k, const IdsView& ids,
+                                                  int32_t* __restrict__ nbr, NodeIdx nd) {
+    if (nd.i >= g.nx || nd.j >= ids.j1 || h.n_valid == 0) return;
     const int qx = g.x0 + nd.i * g.cell + g.cell / 2;
     const int qy = g.y0 + nd.j * g.cell + g.cell / 2;
-    int32_t* o = ids + (node - node0) * k;
-    if (h.n_valid == 0) {
-        if (!kWide)
-            for (int i = 0; i < k; ++i) o[i] = -1;
-        return;
-    }
     const Bound b = knn_bound<K>(h, qx, qy);
-    const bool fits = packed_fits(h, b.tau0);
-    if constexpr (kWide) {
-        if (fits) return;
-        uint64_t d2[K];
-        int id[K];
-        const int keff = knn_scan<K, true>(h, qx, qy, b, d2, id);
+    if (packed_fits(h, b.tau0)) return;
+    uint64_t d2[K];
+    int id[K];
+    const int keff = knn_scan<K, true>(h, qx, qy, b, d2, id);
+    if (ids.stride == 0) {
+        int32_t* o = ids.p + ((int64_t)(nd.j - ids.j0) * g.nx + nd.i) * k;
 #pragma unroll
         for (int i = 0; i < K; ++i)
             if (i < k) o[i] = i < keff ? id[i] : -1;
     } else {
-        if (!fits) {
-            *flag = 1;
-            return;
-        }
-        const int keff = knn_scan_heap<K, 128>(h, qx, qy, b, hp);
-        const uint64_t mask = (1ull << h.idx_bits) - 1;
-        for (int i = 0; i < k; ++i) o[i] = i < keff ? (int)(hp[i * 128] & mask) : -1;
+        int32_t* o = ids.p + node_slot(ids, nd.i, nd.j);
+#pragma unroll
+        for (int i = 0; i < K; ++i)
+            if (i < k) {
+                o[i * ids.stride] = i < keff ? -2 - id[i] : -1;
+                if (nbr) nbr[((int64_t)nd.j * g.nx + nd.i) * k + i] = i < keff ? id[i] : -1;
+            }
     }
 }
 
@@ -289,194 +300,119 @@ __device__ __forceinline__ void knn_ids_point_wide(const HashView& h, int qx, in
 
 // ---------------------------------------------------------------- solve
 
-__host__ __device__ constexpr int tri(int r) { return r * (r + 1) / 2; }
+using u64 = unsigned long long;
 
-// d0 += a * b0, d1 += a * b1 in one packed two-lane FMA (each lane a correctly
-// rounded fused multiply-add, so the results equal two fmaf calls)
-__device__ __forceinline__ void ffma2(float& d0, float& d1, float a, float b0, float b1) {
-    asm("{\n\t.reg .b64 d, a, b;\n\t"
-        "mov.b64 d, {%0, %1};\n\t"
-        "mov.b64 a, {%2, %2};\n\t"
-        "mov.b64 b, {%3, %4};\n\t"
-        "fma.rn.f32x2 d, a, b, d;\n\t"
-        "mov.b64 {%0, %1}, d;\n\t}"
-        : "+f"(d0), "+f"(d1)
-        : "f"(a), "f"(b0), "f"(b1));
+__device__ __forceinline__ u64 dup2(float a) { return pk2(a, a); }
+__device__ __forceinline__ float lo2(u64 p) {
+    float a, b;
+    upk2(p, a, b);
+    return a;
+}
+__device__ __forceinline__ float hi2(u64 p) {
+    float a, b;
+    upk2(p, a, b);
+    return b;
+}
+__device__ __forceinline__ float lane2(u64 p, int i) { return i ? hi2(p) : lo2(p); }
+__device__ __forceinline__ u64 pk2u(uint32_t a, uint32_t b) {
+    u64 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(a), "r"(b));
+    return r;
+}
+__device__ __forceinline__ float rsqrt_approx(float x) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
 }
 
-// Cholesky column j of the register-held lower triangle: scale by the pivot
-// (one shuffle), then update the trailing rows with column j. Each thread
-// publishes its four entries of the column with one 16-byte store to a
-// column buffer and reads the group's entries back four rows per 16-byte
-// load (broadcast): fewer instructions than one shuffle per row. Two buffers
-// alternate by column, so one __syncwarp per column orders writes and reads.
-// A thread's columns c and c + G of one row take the same multiplier, and
-// the loaded rows c and c + G sit side by side in the 16-byte load: those two
-// updates go in one packed two-lane FMA (ffma2).
-// Expanded over j with an integer_sequence so every register index is a
-// compile-time constant (a nested #pragma unroll over the whole triangle is
-// beyond the unroller and would leave L in local memory).
-template <int K, int J>
-__device__ __forceinline__ void chol_column(float (&L)[Geo<K>::LEN], float (&dinv)[kR], int t,
-                                            int gbase, float* cb) {
-    using Gm = Geo<K>;
-    constexpr int G = Gm::G;
-    constexpr int SJ = J / G;
-    const float d = __shfl_sync(kFull, L[Gm::off(SJ) + J], gbase + J % G);
-    const float inv = rsqrtf(d);
-    float pub[kR];
-#pragma unroll
-    for (int s = 0; s < kR; ++s) {
-        pub[s] = 0.0f;
-        if (G * (s + 1) - 1 >= J) {
-            const int r = G * s + t;
-            if (r > J) L[Gm::off(s) + J] *= inv;
-            if (r == J) {
-                L[Gm::off(s) + J] = d * inv;
-                dinv[s] = inv;
-            }
-            pub[s] = L[Gm::off(s) + J];
-        }
-    }
-    if constexpr (G >= 4) {
-        // 16-byte aligned only when the per-system stride (= G mod 32) is a
-        // multiple of 4 floats
-        static_assert(kR == 4 && Gm::SYS_FLOATS % 4 == 0 && Gm::CB % 4 == 0, "float4 buffer");
-        float* col = cb + (J & 1) * K;
-        *reinterpret_cast<float4*>(col + 4 * t) = make_float4(pub[0], pub[1], pub[2], pub[3]);
-        __syncwarp();
-#pragma unroll
-        for (int tc = 0; tc < G; ++tc) {
-            if (G * (kR - 1) + tc <= J) continue;  // no row of this thread beyond J
-            const float4 q4 = *reinterpret_cast<const float4*>(col + 4 * tc);
-            const float q[4] = {q4.x, q4.y, q4.z, q4.w};
-#pragma unroll
-            for (int s = 0; s < kR; ++s) {
-                if (G * (s + 1) - 1 <= J) continue;  // slot s holds no column beyond J
-                const float a = -L[Gm::off(s) + J];
-#pragma unroll
-                for (int p = 0; p < kR / 2; ++p) {
-                    const int c1 = G * (2 * p) + tc, c2 = c1 + G;
-                    const bool in1 = 2 * p <= s && c1 > J, in2 = 2 * p + 1 <= s && c2 > J;
-                    if (in1 && in2) {
-                        ffma2(L[Gm::off(s) + c1], L[Gm::off(s) + c2], a, q[2 * p], q[2 * p + 1]);
-                    } else {
-                        if (in1) L[Gm::off(s) + c1] = fmaf(a, q[2 * p], L[Gm::off(s) + c1]);
-                        if (in2) L[Gm::off(s) + c2] = fmaf(a, q[2 * p + 1], L[Gm::off(s) + c2]);
-                    }
-                }
-            }
-        }
-    } else {
-        // small systems (G < 4): one shuffle per trailing row
-#pragma unroll
-        for (int c = J + 1; c < K; ++c) {
-            const float lcj = __shfl_sync(kFull, L[Gm::off(c / G) + J], gbase + c % G);
-#pragma unroll
-            for (int s = 0; s < kR; ++s)
-                if (G * (s + 1) - 1 >= c)
-                    L[Gm::off(s) + c] = fmaf(-L[Gm::off(s) + J], lcj, L[Gm::off(s) + c]);
-        }
-    }
+// ------------------------------------------------------------ tensor memory
+// Each warp of the 128-thread block reaches its own quarter of the 128 lanes;
+// a thread reads and writes its lane's columns (32x32b). Loads are collected
+// by tmem_wait_ld, which takes the loaded registers as operands so that no use
+// of them moves above it.
+
+__device__ __forceinline__ void tmem_ld16(uint32_t (&r)[16], uint32_t a) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+          "=r"(r[14]), "=r"(r[15])
+        : "r"(a));
+}
+__device__ __forceinline__ void tmem_st16(uint32_t a, const uint32_t (&r)[16]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15};" ::"r"(r[0]),
+        "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
+        "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(a));
+}
+__device__ __forceinline__ void tmem_wait_ld(uint32_t (&r)[16]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]),
+                   "+r"(r[6]), "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]),
+                   "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])::"memory");
+}
+__device__ __forceinline__ void tmem_wait_ld(uint32_t (&r)[16], uint32_t (&s)[16]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]),
+                   "+r"(r[6]), "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]),
+                   "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]), "+r"(s[0]), "+r"(s[1]),
+                   "+r"(s[2]), "+r"(s[3]), "+r"(s[4]), "+r"(s[5]), "+r"(s[6]), "+r"(s[7]),
+                   "+r"(s[8]), "+r"(s[9]), "+r"(s[10]), "+r"(s[11]), "+r"(s[12]), "+r"(s[13]),
+                   "+r"(s[14]), "+r"(s[15])::"memory");
+}
+// further registers of loads that a tmem_wait_ld before it has collected
+__device__ __forceinline__ void tmem_use(uint32_t (&r)[16]) {
+    asm volatile(""
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]),
+                   "+r"(r[6]), "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]),
+                   "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]));
+}
+__device__ __forceinline__ void tmem_wait_st() {
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
-// The factorization also runs the first solve's forward sweep: column J's
-// step of L y = v right after column J is final, the same operations in the
-// same order as the separate sweep, in the latency gaps of the factorization.
-template <int K, int J>
-__device__ __forceinline__ void fwd_step(const float (&L)[Geo<K>::LEN], const float (&dinv)[kR],
-                                         float (&v)[kR], int t, int gbase);
-
-template <int K, int... J>
-__device__ __forceinline__ void chol_factor(float (&L)[Geo<K>::LEN], float (&dinv)[kR], int t,
-                                            int gbase, float* cb, float (&v)[kR],
-                                            std::integer_sequence<int, J...>) {
-    ((chol_column<K, J>(L, dinv, t, gbase, cb), fwd_step<K, J>(L, dinv, v, t, gbase)), ...);
-}
-
-// forward sweep step j of L y = v (L rows in registers)
-template <int K, int J>
-__device__ __forceinline__ void fwd_step(const float (&L)[Geo<K>::LEN], const float (&dinv)[kR],
-                                         float (&v)[kR], int t, int gbase) {
-    using Gm = Geo<K>;
-    constexpr int G = Gm::G;
-    constexpr int SJ = J / G;
-    if (t == J % G) v[SJ] *= dinv[SJ];
-    const float yj = __shfl_sync(kFull, v[SJ], gbase + J % G);
-#pragma unroll
-    for (int s = 0; s < kR; ++s)
-        if (G * (s + 1) - 1 > J && G * s + t > J) v[s] = fmaf(-L[Gm::off(s) + J], yj, v[s]);
-}
-
-// back sweep for column J = K-1-I of L^T x = y in dot-product form, software
-// pipelined: each thread sums its register rows of L (no transposed copy of
-// the factor) and the group adds the partial sums by xor shuffles, but the
-// sum over the rows far below J is reduced kLook steps ahead, so that its
-// shuffles overlap the finishing of the columns in between; the terms of the
-// kLook rows just below J come from their owners by one shuffle each.
-//   kLook = 1: x_J = (y_J - P_J - L[J+1][J] x_{J+1}) / L[J][J], P_J over rows > J+1
-//   kLook = 2: x_J = (y_J - Q_J - E_J - L[J+1][J] x_{J+1}) / L[J][J], Q_J over
-//              rows > J+2, E_J = L[J+2][J] x_{J+2} (sent one step early)
-// p0 carries the far sum for column J into the step; p1 and e0 (kLook = 2)
-// carry Q_{J-1} and E_{J-1}. Every kernel takes the same depth (kBwdLook), so
-// the fused IDW + kriging pass stays bitwise equal to the kriging call.
-template <int K, int kLook, int I>
-__device__ __forceinline__ void bwd_step(const float (&L)[Geo<K>::LEN], const float (&dinv)[kR],
-                                         float (&v)[kR], int t, int gbase, float& p0, float& p1,
-                                         float& e0) {
-    static_assert(kLook == 1 || kLook == 2, "pipeline depth");
-    using Gm = Geo<K>;
-    constexpr int G = Gm::G;
-    constexpr int J = K - 1 - I;
-    constexpr int SJ = J / G;
-    float dj = 0.0f, en = 0.0f;
-    if constexpr (J + 1 < K) {
-        constexpr int S1 = (J + 1) / G;
-        dj = __shfl_sync(kFull, L[Gm::off(S1) + J] * v[S1], gbase + (J + 1) % G);
-        if constexpr (kLook == 2 && J > 0)
-            en = __shfl_sync(kFull, L[Gm::off(S1) + J - 1] * v[S1], gbase + (J + 1) % G);
+// A block's tensor memory (Geo<K>::COLS columns, a power of two), taken by warp
+// 0 at the start and given back by it at the end; `slot` is a shared word.
+// Returns the thread's base address (its warp's lanes).
+template <int COLS>
+__device__ __forceinline__ uint32_t tmem_take(uint32_t* slot) {
+    if constexpr (COLS == 0) return 0;
+    static_assert(COLS == 0 || COLS == 256 || COLS == 512, "an allocation size");
+    if (threadIdx.x < 32) {
+        const uint32_t sa = (uint32_t)__cvta_generic_to_shared(slot);
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(sa),
+                     "r"(COLS)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    // far sum for column J - kLook over the rows > J (all solved)
-    float pn = 0.0f;
-    if constexpr (J >= kLook) {
-#pragma unroll
-        for (int s = 0; s < kR; ++s)
-            if (G * (s + 1) - 1 > J)
-                pn = (G * s + t > J) ? fmaf(L[Gm::off(s) + J - kLook], v[s], pn) : pn;
-#pragma unroll
-        for (int o = 1; o < G; o <<= 1) pn += __shfl_xor_sync(kFull, pn, o);
-    }
-    if (t == J % G) v[SJ] = (((v[SJ] - p0) - e0) - dj) * dinv[SJ];
-    if constexpr (kLook == 1) {
-        p0 = pn;
-    } else {
-        p0 = p1;
-        p1 = pn;
-        e0 = en;
+    __syncthreads();
+    return *(volatile uint32_t*)slot + ((uint32_t)(threadIdx.x >> 5 & 3) << 21);
+}
+template <int COLS>
+__device__ __forceinline__ void tmem_give(const uint32_t* slot) {
+    if constexpr (COLS != 0) {
+        __syncthreads();
+        if (threadIdx.x < 32)
+            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(*slot),
+                         "r"(COLS)
+                         : "memory");
     }
 }
 
-template <int K, int kLook, int... J>
-__device__ __forceinline__ void chol_solve_seq(const float (&L)[Geo<K>::LEN],
-                                               const float (&dinv)[kR], float (&v)[kR], int t,
-                                               int gbase, bool fwd, std::integer_sequence<int, J...>) {
-    if (fwd) (fwd_step<K, J>(L, dinv, v, t, gbase), ...);  // else done in the factorization
-    float p0 = 0.0f, p1 = 0.0f, e0 = 0.0f;
-    (bwd_step<K, kLook, J>(L, dinv, v, t, gbase, p0, p1, e0), ...);
-}
-
-// L2 prefetch of the neighbour ids of solve block pb (sys systems of k ids
-// each, from ids[pb * sys * k]): warp 0, one 128-byte line per lane, within
-// the `nodes` systems of the launch. A hint that nothing waits on.
-__device__ __forceinline__ void prefetch_ids_l2(const int32_t* ids, int64_t nodes, int k,
-                                                int64_t pb, int sys) {
-    if (threadIdx.x >= 32) return;
-    const int64_t s0 = pb * sys;
-    if (s0 >= nodes) return;
-    const int64_t bytes = min((int64_t)sys, nodes - s0) * k * (int64_t)sizeof(int32_t);
-    const char* base = reinterpret_cast<const char*>(ids + s0 * k);
-    for (int64_t off = (int64_t)threadIdx.x * 128; off < bytes; off += 32 * 128)
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(base + off));
+// L2 prefetch of the neighbour ids of solve block pb of a range of `nsys`
+// systems. A hint that nothing waits on.
+__device__ __forceinline__ void prefetch_ids_l2(const IdsView& v, int64_t nsys, int k, int64_t pb) {
+    const int t = threadIdx.x;
+    const int64_t sys = pb * kSolveSystems;
+    if (v.stride == 0) {
+        if (t < kSolveSystems && sys + t < nsys)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(v.p + (sys + t) * k));
+    } else if (sys < nsys) {
+        for (int q = t; q < 4 * k; q += blockDim.x)  // 128 systems: four lines per neighbour
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(v.p + (q >> 2) * v.stride + sys + (q & 3) * 32));
+    }
 }
 
 // 2^e as a float (|e| <= 126)
@@ -485,405 +421,543 @@ __device__ __forceinline__ float pow2f(int e) { return __int_as_float((127 + e) 
 // exponent e with 2^(e-1) <= v < 2^e for finite v > 0
 __device__ __forceinline__ int exp_above(float v) { return ((__float_as_int(v) >> 23) & 0xff) - 126; }
 
-// The kriging systems of solve block `blk` (kWarps warps x SYS systems x
-// kRounds rounds) of a range of `nodes` grid nodes starting at node0, with the
-// neighbour ids of node node0 + i at ids[i * k]. smem: kWarps * WARP_FLOATS.
-// With kPts the "nodes" are query points whose coordinates are px[], py[]
-// (g unused).
+// round to nearest as int64 of |f| < 2^62, through two 32-bit conversions (a
+// 64-bit one runs at the FP64 rate)
+__device__ __forceinline__ long long float_to_ll(float f) {
+    const int hi = __float2int_rn(f * 2.3283064365386963e-10f);     // 2^-32
+    const int lo = __float2int_rn(fmaf((float)hi, -4294967296.0f, f));  // exact remainder
+    return ((long long)hi << 32) + lo;
+}
+// the float nearest to v up to one rounding of its upper half
+__device__ __forceinline__ float ll_to_float(long long v) {
+    const int lo = (int)v;
+    const int hi = (int)((v - lo) >> 32);
+    return fmaf((float)hi, 4294967296.0f, (float)lo);
+}
+
+// The tile function of the assembly: -A for two rows at once, in the
+// fixed-point scale. -A[r][c] = gamma(r, c) - Gamma_r0 - Gamma_c0; the records
+// hold zr = -Gamma_r0, and zc comes in as c0 - Gamma_c0 (all scaled).
+template <bool kSph>
+struct TileVgm {
+    u64 kinv2, k2, k3;
+    float c0s, cs;
+    __device__ __forceinline__ explicit TileVgm(const ScaledVgm& v)
+        : kinv2(dup2(v.kinv2)), k2(dup2(v.k2)), k3(dup2(v.k3)), c0s(v.c0s), cs(v.cs) {}
+    __device__ __forceinline__ u64 entry(u64 xr, u64 yr, u64 zr, float xc, float yc, float zc) const {
+        const u64 dx = sub2(xr, dup2(xc)), dy = sub2(yr, dup2(yc));
+        const u64 t2 = mul2(fma2(dx, dx, mul2(dy, dy)), kinv2);  // (h / a)^2
+        float ta, tb;
+        upk2(t2, ta, tb);
+        if constexpr (kSph) {
+            // the polynomial is the sill at t = 1
+            ta = fminf(ta, 1.0f);
+            tb = fminf(tb, 1.0f);
+            const u64 in = fma2(k2, pk2(ta, tb), k3);
+            return fma2(pk2(sqrt_approx(ta), sqrt_approx(tb)), in, add2(zr, dup2(zc)));
+        } else {
+            const u64 e = pk2(-expm1f(-sqrt_approx(ta)), -expm1f(-sqrt_approx(tb)));
+            return fma2(dup2(cs), e, add2(zr, dup2(zc)));
+        }
+    }
+};
+
+// Vectors of four rows of a system (see Geo): load / store the TB rows of tile
+// row b of array `at`.
+template <int K>
+struct Lane {
+    using Gm = Geo<K>;
+    static constexpr int TB = Gm::TB, P = Gm::P;
+    float4* s;  // the system's vectors, kSolveSystems apart
+    __device__ __forceinline__ float4& vec(int i) const { return s[i * kSolveSystems]; }
+    // rows 2 p, 2 p + 1 of tile row b
+    __device__ __forceinline__ float2& pair(int at, int b, int p) const {
+        return reinterpret_cast<float2*>(&vec(at + b * (TB / 4) + (p >> 1)))[p & 1];
+    }
+    __device__ __forceinline__ longlong2& long2(int at) const {
+        return *reinterpret_cast<longlong2*>(&vec(at));
+    }
+    __device__ __forceinline__ void pairs(int at, int b, u64 (&p)[P]) const {
+#pragma unroll
+        for (int i = 0; i < TB / 4; ++i) {
+            const float4 f = vec(at + b * (TB / 4) + i);
+            p[2 * i] = pk2(f.x, f.y);
+            p[2 * i + 1] = pk2(f.z, f.w);
+        }
+    }
+    __device__ __forceinline__ void floats(int at, int b, float (&p)[TB]) const {
+#pragma unroll
+        for (int i = 0; i < TB / 4; ++i) {
+            const float4 f = vec(at + b * (TB / 4) + i);
+            p[4 * i] = f.x;
+            p[4 * i + 1] = f.y;
+            p[4 * i + 2] = f.z;
+            p[4 * i + 3] = f.w;
+        }
+    }
+    __device__ __forceinline__ void put(int at, int b, const float (&p)[TB]) const {
+#pragma unroll
+        for (int i = 0; i < TB / 4; ++i)
+            vec(at + b * (TB / 4) + i) =
+                make_float4(p[4 * i], p[4 * i + 1], p[4 * i + 2], p[4 * i + 3]);
+    }
+    __device__ __forceinline__ void ints(int at, int b, int (&p)[TB]) const {
+        float f[TB];
+        floats(at, b, f);
+#pragma unroll
+        for (int i = 0; i < TB; ++i) p[i] = __float_as_int(f[i]);
+    }
+    __device__ __forceinline__ void put_ints(int at, int b, const int (&p)[TB]) const {
+        float f[TB];
+#pragma unroll
+        for (int i = 0; i < TB; ++i) f[i] = __int_as_float(p[i]);
+        put(at, b, f);
+    }
+};
+
+// With two threads per system, thread h of a system owns row pairs p = h and
+// 3 - h of every tile (rows 0, 1, 6, 7 or 2, 3, 4, 5: equal shares of the
+// diagonal tiles too), so the multiplies of a tile split without exchange; an
+// off-diagonal tile of the factor is stored as two halves of 32 words, the
+// four owned rows of column c at 4 c. The two threads of a system sit in
+// warps w and w + 4 (the same lanes of tensor memory) and meet at a named
+// barrier of the two warps.
+__device__ __forceinline__ void pair_sync() {
+    asm volatile("bar.sync %0, 64;" ::"r"(1 + (int)(threadIdx.x >> 5 & 3)) : "memory");
+}
+// tensor memory written by one warp of the pair is read by the other
+__device__ __forceinline__ void pair_sync_tmem() {
+    tmem_wait_st();
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    pair_sync();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+}
+// row r of a tile as (half, place): the half that owns it and its place there
+constexpr __host__ __device__ int half_of(int r) { return r >= 2 && r < 6; }
+constexpr __host__ __device__ int place_of(int r) { return r < 2 ? r : r < 6 ? r - 2 : r - 4; }
+
+// Row pairs p[0], p[1] (tile row I) of -A's tile columns: t[u][c] is pair
+// p[u] of column c of tile (I, J). Rows past the last neighbour have no
+// coupling (off-diagonal zero).
+template <int K, bool kSph>
+__device__ __forceinline__ void assemble_off(const Lane<K>& ln, const TileVgm<kSph>& vg, int I,
+                                             int J, const int (&pr)[2], int ke, bool full,
+                                             u64 (&t)[2][8]) {
+    using Gm = Geo<K>;
+    u64 xr[2], yr[2], zr[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        const float2 a = ln.pair(Gm::X, I, pr[u]), b = ln.pair(Gm::Y, I, pr[u]),
+                     c = ln.pair(Gm::Z, I, pr[u]);
+        xr[u] = pk2(a.x, a.y);
+        yr[u] = pk2(b.x, b.y);
+        zr[u] = pk2(c.x, c.y);
+    }
+    float xc[8], yc[8], zc[8];
+    ln.floats(Gm::X, J, xc);
+    ln.floats(Gm::Y, J, yc);
+    ln.floats(Gm::Z, J, zc);
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        const float z = zc[c] + vg.c0s;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) t[u][c] = vg.entry(xr[u], yr[u], zr[u], xc[c], yc[c], z);
+    }
+    if (!full) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                float a, b;
+                upk2(t[u][c], a, b);
+                const int r = I * 8 + 2 * pr[u];
+                t[u][c] = pk2(r + 1 < ke ? a : 0.0f, r + 2 < ke ? b : 0.0f);
+            }
+    }
+}
+
+// Row pair p of -A's diagonal tile J, columns 0 .. 2 p + 1 (the entry above the
+// diagonal is not used); on the diagonal of rows past the last neighbour the
+// identity in the fixed-point scale.
+template <int K, bool kSph, int p>
+__device__ __forceinline__ void assemble_diag(const Lane<K>& ln, const TileVgm<kSph>& vg, int J, int ke, float sa,
+                                              bool full, const float (&xc)[8], const float (&yc)[8],
+                                              const float (&zc)[8], u64 (&t)[2 * p + 2]) {
+    const u64 xr = pk2(xc[2 * p], xc[2 * p + 1]), yr = pk2(yc[2 * p], yc[2 * p + 1]),
+              zr = pk2(zc[2 * p], zc[2 * p + 1]);
+#pragma unroll
+    for (int c = 0; c < 2 * p + 2; ++c) t[c] = vg.entry(xr, yr, zr, xc[c], yc[c], zc[c] + vg.c0s);
+    // -A[c][c] = -2 Gamma_c0
+    float d0 = 2.0f * zc[2 * p], d1 = 2.0f * zc[2 * p + 1];
+    if (!full) {
+        const int r = J * 8 + 2 * p;
+        const bool real0 = r + 1 < ke, real1 = r + 2 < ke;
+        d0 = real0 ? d0 : -sa;
+        d1 = real1 ? d1 : -sa;
+#pragma unroll
+        for (int c = 0; c < 2 * p + 2; ++c) t[c] = pk2(real0 ? lo2(t[c]) : 0.0f, real1 ? hi2(t[c]) : 0.0f);
+    }
+    t[2 * p] = pk2(d0, hi2(t[2 * p]));
+    t[2 * p + 1] = pk2(lo2(t[2 * p + 1]), d1);
+}
+
+// The whole -A of a one-tile system: t[c][p], the pairs that hold a row >= c
+template <int K, bool kSph>
+__device__ __forceinline__ void assemble_one(const Lane<K>& ln, const TileVgm<kSph>& vg, int ke,
+                                             float sa, u64 (&t)[Geo<K>::TB][Geo<K>::P]) {
+    using Gm = Geo<K>;
+    u64 xr[Gm::P], yr[Gm::P], zr[Gm::P];
+    ln.pairs(Gm::X, 0, xr);
+    ln.pairs(Gm::Y, 0, yr);
+    ln.pairs(Gm::Z, 0, zr);
+#pragma unroll
+    for (int c = 0; c < Gm::TB; ++c) {
+        const float z0 = lane2(zr[c / 2], c & 1);
+        const float z = z0 + vg.c0s;
+#pragma unroll
+        for (int p = c / 2; p < Gm::P; ++p) {
+            float a, b;
+            upk2(vg.entry(xr[p], yr[p], zr[p], lane2(xr[c / 2], c & 1), lane2(yr[c / 2], c & 1), z),
+                 a, b);
+            t[c][p] = pk2(2 * p + 1 < ke ? a : 0.0f, 2 * p + 2 < ke ? b : 0.0f);
+        }
+        const float d = c + 1 < ke ? 2.0f * z0 : -sa;  // -A[c][c] = -2 Gamma_c0
+        t[c][c / 2] = (c & 1) ? pk2(lo2(t[c][c / 2]), d) : pk2(d, hi2(t[c][c / 2]));
+    }
+}
+
+// Factor a diagonal tile t[c][p] of -A (less the earlier columns) in
+// registers: the strictly lower entries column after column, ni = -1 /
+// diagonal, and one step of L y = v on the tile's rows (nvp = -v in, y out).
+template <int TB>
+__device__ __forceinline__ void factor_tile(u64 (&t)[TB][TB / 2], u64 (&nvp)[TB / 2],
+                                            float (&Ld)[TB * (TB - 1) / 2], float (&ni)[TB],
+                                            float (&y)[TB]) {
+    constexpr int P = TB / 2;
+    int at = 0;
+#pragma unroll
+    for (int c = 0; c < TB; ++c) {
+        ni[c] = -rsqrt_approx(-lane2(t[c][c / 2], c & 1));
+        const u64 m = dup2(ni[c]);
+        u64 L[P];
+#pragma unroll
+        for (int q = 0; q < P; ++q)
+            if (2 * q + 1 > c) L[q] = mul2(t[c][q], m);
+        y[c] = lane2(nvp[c / 2], c & 1) * ni[c];
+#pragma unroll
+        for (int r = c + 1; r < TB; ++r) {
+            const float l = lane2(L[r / 2], r & 1);
+            Ld[at++] = l;
+#pragma unroll
+            for (int q = r / 2; q < P; ++q) t[r][q] = fma2(L[q], dup2(l), t[r][q]);
+        }
+#pragma unroll
+        for (int q = 0; q < P; ++q)
+            if (2 * q + 1 > c) nvp[q] = fma2(L[q], dup2(y[c]), nvp[q]);
+    }
+}
+
+// forward substitution with a diagonal tile: nv = -v in, y out (L y = v)
+template <int TB>
+__device__ __forceinline__ void diag_forward(const float (&Ld)[TB * (TB - 1) / 2],
+                                             const float (&ni)[TB], float (&nv)[TB]) {
+    int at = 0;
+#pragma unroll
+    for (int c = 0; c < TB; ++c) {
+        nv[c] *= ni[c];
+#pragma unroll
+        for (int r = c + 1; r < TB; ++r) nv[r] = fmaf(Ld[at++], nv[c], nv[r]);
+    }
+}
+// back substitution: nv = -v in, x out (L^T x = v)
+template <int TB>
+__device__ __forceinline__ void diag_backward(const float (&Ld)[TB * (TB - 1) / 2],
+                                              const float (&ni)[TB], float (&nv)[TB]) {
+#pragma unroll
+    for (int c = TB - 1; c >= 0; --c) {
+        nv[c] *= ni[c];
+#pragma unroll
+        for (int j = 0; j < c; ++j)  // L[c][j] in column-major order below the diagonal
+            nv[j] = fmaf(Ld[j * TB - j * (j + 1) / 2 + (c - j - 1)], nv[c], nv[j]);
+    }
+}
+
+// The kriging systems of batches b0 .. b1 - 1 (128 systems each) of a range of
+// nsys, with the neighbour ids of `ids`; node0: the range's first node (rows
+// layout). smem: Geo<K>::SMEM bytes; tm: the thread's tensor memory. With kPts
+// the systems are query points whose coordinates are px[], py[] (g unused).
 // With kIdw the block also writes the IDW depth over the first fz.k of the
 // node's sorted neighbours (fz.k <= k): the same value bg_interp_idw gives, as
-// its operations are those of idw_from in the same order.
-template <int K, bool kPts, bool kIdw, int kWarps>
-__device__ __forceinline__ void okrige_solve_block(const HashView& h, const GridView& g, int k,
-                                                   const OkParams& p, int64_t node0, int64_t nodes,
-                                                   const int32_t* __restrict__ ids,
+// its operations are those of idw_sum in the same order. Every warp reaches
+// every barrier and tensor-memory instruction (idle lanes run the tile loops
+// too).
+template <int K, bool kSph, bool kPts, bool kIdw>
+__device__ __forceinline__ void okrige_solve_range(const HashView& h, const GridView& g, int k,
+                                                   const OkParams& p, int64_t node0, int64_t nsys,
+                                                   const IdsView& ids,
                                                    float* __restrict__ depth,
-                                                   float* __restrict__ var, int64_t blk,
-                                                   float* smem,
+                                                   float* __restrict__ var, int64_t b0, int64_t b1,
+                                                   float4* smem, uint32_t tm,
                                                    const int32_t* __restrict__ px = nullptr,
                                                    const int32_t* __restrict__ py = nullptr,
                                                    IdwFuse fz = IdwFuse{}) {
     using Gm = Geo<K>;
-    constexpr int G = Gm::G;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int grp = lane / G, t = lane % G, gbase = grp * G;
-    float* sysmem = smem + warp * Gm::WARP_FLOATS + grp * Gm::SYS_FLOATS;
-    int* Aq = reinterpret_cast<int*>(sysmem);      // packed lower triangle: fixed-point A
-    // per row r (neighbour r + 1), three arrays of K: x and y minus those of
-    // neighbour 0 (cm) at T[r] and T[K + r], Gamma(neighbour r + 1,
-    // neighbour 0) in the fixed-point scale at T[2K + r]; four consecutive
-    // rows load as one 16-byte vector. After assembly T[r] and T[K + r] hold
-    // the row's output terms.
-    float* T = sysmem + Gm::TRIP;
-    auto rec = [&](int r) { return make_float4(T[r], T[K + r], T[2 * K + r], 0.0f); };
-    const unsigned gmask = (G == 32) ? 0xffffffffu : (((1u << G) - 1u) << gbase);
-
-    for (int round = 0; round < kRounds; ++round) {
-        const int64_t sys = (blk * kWarps + warp) * (Gm::SYS * kRounds) +
-                            (int64_t)round * Gm::SYS + grp;
-        const bool live = sys < nodes;  // uniform within a group
-        const int64_t node = node0 + (live ? sys : 0);
-        const int32_t* my = ids + (live ? sys : 0) * k;
-
-        // neighbour ids of my rows (reduced row r <-> neighbour r + 1) and k_eff;
-        // ids are -1 exactly past k_eff
-        int nid[kR];
-        unsigned cnt = 0;
-#pragma unroll
-        for (int s = 0; s < kR; ++s) {
-            const int n = 1 + G * s + t;
-            nid[s] = (live && n < k) ? __ldg(my + n) : -1;
-            cnt += __popc(__ballot_sync(kFull, nid[s] >= 0) & gmask);
-        }
-        const int id0 = live ? __ldg(my) : -1;
-        const int ke = (id0 >= 0) ? 1 + (int)cnt : 0;  // 0: no output (no data, or past the end)
-        int qx, qy;
-        if constexpr (kPts) {
-            qx = __ldg(px + node);
-            qy = __ldg(py + node);
-        } else {
-            qx = g.x0 + (int)(node % g.nx) * g.cell + g.cell / 2;
-            qy = g.y0 + (int)(node / g.nx) * g.cell + g.cell / 2;
-        }
-
-        // gather the neighbours' records; offsets from neighbour 0 as exact floats
-        int4 r0 = make_int4(0, 0, 0, 0);
-        if (id0 >= 0) r0 = __ldg(h.orig + id0);
-        const float z0 = __int_as_float(r0.z);
-        const float g00 = gamma_cm(p, r0.x - qx, r0.y - qy, 0.0f);
-        float zr[kR], gr0[kR], g0r[kR];  // depth; Gamma(row's neighbour, nbr 0); gamma(node, row's nbr)
-        float pox[kR], poy[kR];  // row's offsets from neighbour 0 (cm)
-        int pdx[kR], pdy[kR];    // and from the node
-        bool preal[kR];
-        float gmax = 0.0f;
-        // fused IDW: squared distance to the nearest, and each row's weight and anomaly
-        uint64_t idw_d0 = 0;
-        float idw_d1 = 0.0f, idw_l1 = 0.0f, idw_w[kR], idw_a[kR];
-        if constexpr (kIdw) {
-            const long long dx = (long long)r0.x - qx, dy = (long long)r0.y - qy;
-            idw_d0 = (uint64_t)(dx * dx + dy * dy);
-            idw_d1 = idw_d2f(idw_d0);
-            if (fz.power != 2.0f) idw_l1 = log2f(idw_d1);
-        }
-#pragma unroll
-        for (int s = 0; s < kR; ++s) {
-            int4 rr = make_int4(0, 0, 0, 0);
-            const bool real = nid[s] >= 0;
-            if (real) rr = __ldg(h.orig + nid[s]);
-            const int r = G * s + t;
-            if constexpr (kIdw) {
-                idw_w[s] = idw_a[s] = 0.0f;
-                if (G * s + 1 < fz.k) {  // uniform: this slot holds IDW neighbours
-                    const long long dx = (long long)rr.x - qx, dy = (long long)rr.y - qy;
-                    idw_w[s] = idw_weight(idw_d1, idw_l1, 0.5f * fz.power, fz.power,
-                                          idw_d2f((uint64_t)(dx * dx + dy * dy)));
-                    idw_a[s] = __int_as_float(rr.z) - z0;
-                }
-            }
-            const float ox = (float)(rr.x - r0.x), oy = (float)(rr.y - r0.y);
-            T[r] = ox;
-            T[K + r] = oy;
-            zr[s] = __int_as_float(rr.z);
-            pox[s] = ox;
-            poy[s] = oy;
-            pdx[s] = rr.x - qx;
-            pdy[s] = rr.y - qy;
-            preal[s] = real;
-        }
-        if (p.model == BG_VARIOGRAM_SPHERICAL && kR % 2 == 0) {
-            // two rows per packed instruction: the same operations as
-            // gamma_pair_f and gamma_cm, lane by lane
-#pragma unroll
-            for (int s = 0; s < kR; s += 2) {
-                float ga, gb, ha, hb;
-                gamma_pair_sph2(p, pox[s], poy[s], pox[s + 1], poy[s + 1], ga, gb);
-                gamma_cm_sph2(p, pdx[s], pdy[s], pdx[s + 1], pdy[s + 1], ha, hb);
-                gr0[s] = preal[s] ? ga : 0.0f;
-                gr0[s + 1] = preal[s + 1] ? gb : 0.0f;
-                g0r[s] = preal[s] ? ha : 0.0f;
-                g0r[s + 1] = preal[s + 1] ? hb : 0.0f;
-            }
-        } else {
-#pragma unroll
-            for (int s = 0; s < kR; ++s) {
-                gr0[s] = preal[s] ? gamma_pair_f(p, pox[s], poy[s]) : 0.0f;
-                g0r[s] = preal[s] ? gamma_cm(p, pdx[s], pdy[s], 0.0f) : 0.0f;
-            }
-        }
-#pragma unroll
-        for (int s = 0; s < kR; ++s) gmax = fmaxf(gmax, gr0[s]);
-#pragma unroll
-        for (int o = 1; o < G; o <<= 1) gmax = fmaxf(gmax, __shfl_xor_sync(kFull, gmax, o));
-        if constexpr (kIdw) {
-            // thread t's partial holds neighbours 1 + t + G s in ascending s,
-            // and the xor shuffles combine the partials as idw_tree8 does
-            static_assert(G == kIdwLanes, "the fused IDW runs with 8 threads per system");
-            const int ki = min(fz.k, ke);
-            float num = 0.0f, den = 0.0f;
-#pragma unroll
-            for (int s = 0; s < kR; ++s)
-                if (1 + G * s + t < ki) {
-                    num = fmaf(idw_w[s], idw_a[s], num);
-                    den += idw_w[s];
-                }
-#pragma unroll
-            for (int o = 1; o < G; o <<= 1) {
-                num += __shfl_xor_sync(kFull, num, o);
-                den += __shfl_xor_sync(kFull, den, o);
-            }
-            if (live && t == 0)
-                fz.out[node] = ke == 0 ? __int_as_float(0x7fc00000)
-                                       : (idw_d0 == 0 ? z0 : z0 + num / (1.0f + den));
-        }
-        // A is SPD, so |A[r][c]| <= its largest diagonal entry max(1, 2 max Gamma_r0);
-        // fixed point with 30 bits below that bound
-        const int ea = 30 - exp_above(fmaxf(1.0f, 2.0f * gmax));
-        const float sa = pow2f(ea);
-#pragma unroll
-        for (int s = 0; s < kR; ++s) T[2 * K + G * s + t] = gr0[s] * sa;  // Gamma_r0, fixed-point scale
-        const ScaledVgm sv = scaled_vgm(p, sa);
-        __syncwarp();
-
-        // assemble the lower triangle once per entry, straight into fixed
-        // point. Every term is in the fixed-point scale already (the records'
-        // Gamma_r0 and the scaled variogram), so an entry is one rounding to
-        // integer. The triangle splits into G x G blocks: below the diagonal
-        // blocks, thread t owns the columns c = t + G q and the group walks
-        // the rows in step (a row's entries land in consecutive banks), four
-        // rows per batch, two per packed instruction. With G >= 4 a diagonal
-        // block is taken by a circulant assignment in each thread's own
-        // column (below); smaller groups deal its G (G + 1) / 2 entries out to
-        // the group's threads in turn.
-        auto entry_value = [&](auto spherical, int r, int c) {
-            constexpr bool kSph = decltype(spherical)::value;
-            const float4 a = rec(r), b = rec(c);
-            // a real row r (r + 1 < ke) implies a real column c < r
-            return (r == c) ? ((c + 1 < ke) ? 2.0f * b.z : sa)
-                   : (r + 1 < ke) ? (a.z + b.z) - gamma_pair_scaled<kSph>(sv, a.x - b.x, a.y - b.y)
-                                  : 0.0f;
-        };
-        constexpr int kDiag = G * (G + 1) / 2, kDiagSlots = (kDiag + G - 1) / G;
-        int dij[kDiagSlots];  // (row, column) in a diagonal block of this thread's slots
-#pragma unroll
-        for (int m = 0; m < kDiagSlots; ++m) {
-            const int e = t + G * m;
-            int i = 0;
-            while (tri(i + 1) <= e) ++i;
-            dij[m] = (i << 8) | (e - tri(i));
-        }
-        // loads and arithmetic of a batch ahead of its stores: the stores to
-        // the triangle then never sit between one entry's loads and the next
-        auto assemble = [&](auto spherical) {
-            constexpr bool kSph = decltype(spherical)::value;
-#pragma unroll
-            for (int q = 0; q < kR; ++q) {
-                const int c = t + G * q;
-                const float4 cc = rec(c);
-                const float xc = cc.x, yc = cc.y, gcc = cc.z;
-                if constexpr (G >= 4) {
-                    // the diagonal block: entry (t + d mod G, t) of this thread's
-                    // column for d = 1 .. G/2 (d = G/2 only for t < G/2, so each
-                    // pair of the block is taken once), evaluated with the
-                    // other row's record and stored at its lower-triangle place;
-                    // the value is symmetric, bit for bit, in the two records
-                    constexpr int kH = G / 2;
-                    float dv[kH];
-                    int ri[kH];
-#pragma unroll
-                    for (int d = 1; d <= kH; ++d) ri[d - 1] = G * q + (t + d) % G;
-                    if constexpr (kSph) {
-#pragma unroll
-                        for (int d = 0; d < kH; d += 2)
-                            gamma_rows2_sph(sv, T[ri[d]], T[ri[d + 1]], T[K + ri[d]], T[K + ri[d + 1]],
-                                            T[2 * K + ri[d]], T[2 * K + ri[d + 1]], xc, yc, gcc,
-                                            dv[d], dv[d + 1]);
-                    } else {
-#pragma unroll
-                        for (int d = 0; d < kH; ++d)
-                            dv[d] = (T[2 * K + ri[d]] + gcc) -
-                                    gamma_pair_scaled<false>(sv, T[ri[d]] - xc, T[K + ri[d]] - yc);
-                    }
-                    Aq[tri(c) + c] = __float2int_rn((c + 1 < ke) ? 2.0f * gcc : sa);
-#pragma unroll
-                    for (int d = 0; d < kH; ++d) {
-                        if (d + 1 == kH && t >= kH) break;  // the other half takes these
-                        const int hi = max(ri[d], c), lo = min(ri[d], c);
-                        Aq[tri(hi) + lo] = __float2int_rn((hi + 1 < ke) ? dv[d] : 0.0f);
-                    }
-                } else {
-                float dv[kDiagSlots];
-#pragma unroll
-                for (int m = 0; m < kDiagSlots; ++m)
-                    dv[m] = (kDiag % G == 0 || m + 1 < kDiagSlots || t + G * m < kDiag)
-                                ? entry_value(spherical, G * q + (dij[m] >> 8), G * q + (dij[m] & 0xff))
-                                : 0.0f;
-#pragma unroll
-                for (int m = 0; m < kDiagSlots; ++m)
-                    if (kDiag % G == 0 || m + 1 < kDiagSlots || t + G * m < kDiag)
-                        Aq[tri(G * q + (dij[m] >> 8)) + G * q + (dij[m] & 0xff)] = __float2int_rn(dv[m]);
-                }
-                constexpr int kB = 4;
-#pragma unroll
-                for (int r0 = G * (q + 1); r0 < K; r0 += kB) {
-                    // (K - G (q + 1) need not be a multiple of kB: rows from K on
-                    // are skipped at compile time)
-                    float vb[kB];
-                    if constexpr (G >= 4 && kSph) {
-                        // r0 is a multiple of 4: rows r0 .. r0 + 3 in one vector per
-                        // array, two rows per packed operation
-                        const float4 X = *reinterpret_cast<const float4*>(T + r0);
-                        const float4 Y = *reinterpret_cast<const float4*>(T + K + r0);
-                        const float4 Z = *reinterpret_cast<const float4*>(T + 2 * K + r0);
-                        gamma_rows2_sph(sv, X.x, X.y, Y.x, Y.y, Z.x, Z.y, xc, yc, gcc, vb[0], vb[1]);
-                        gamma_rows2_sph(sv, X.z, X.w, Y.z, Y.w, Z.z, Z.w, xc, yc, gcc, vb[2], vb[3]);
-#pragma unroll
-                        for (int u = 0; u < kB; ++u)
-                            if (!(r0 + u + 1 < ke)) vb[u] = 0.0f;
-                    } else {
-#pragma unroll
-                    for (int u = 0; u < kB; ++u) {
-                        const int r = r0 + u;
-                        vb[u] = 0.0f;
-                        if (r < K) {
-                            const float4 a = rec(r);
-                            if (r + 1 < ke)
-                                vb[u] = (a.z + gcc) - gamma_pair_scaled<kSph>(sv, a.x - xc, a.y - yc);
-                        }
-                    }
-                    }
-#pragma unroll
-                    for (int u = 0; u < kB; ++u)
-                        if (r0 + u < K) Aq[tri(r0 + u) + c] = __float2int_rn(vb[u]);
-                }
-            }
-        };
-        if (p.model == BG_VARIOGRAM_SPHERICAL)
-            assemble(std::true_type{});
-        else
-            assemble(std::false_type{});
-        __syncwarp();
-
-        // my rows into registers (zero above the diagonal), in the fixed-point
-        // scale: the factor is that of sa A, and the solves scale their
-        // right-hand sides by sa to match, so x comes out in A's units
-        float L[Gm::LEN];
-        float b[kR];
-#pragma unroll
-        for (int s = 0; s < kR; ++s) {
-            const int r = G * s + t;
-            b[s] = (r + 1 < ke) ? (gr0[s] + g00) - g0r[s] : 0.0f;
-            // the tables are free after assembly: keep the row's output terms
-            // there rather than in registers through the solve
-            T[r] = zr[s] - z0;
-            T[K + r] = g0r[s] - gr0[s];
-#pragma unroll
-            for (int c = 0; c < G * (s + 1); ++c) {
-                const int q = Aq[c <= r ? tri(r) + c : 0];
-                L[Gm::off(s) + c] = c <= r ? (float)q : 0.0f;
-            }
-        }
-
-        // factor in registers
-        float dinv[kR];
-#pragma unroll
-        for (int s = 0; s < kR; ++s) dinv[s] = 1.0f;
-        float v[kR], x[kR];
-#pragma unroll
-        for (int s = 0; s < kR; ++s) v[s] = b[s] * sa;
-        chol_factor<K>(L, dinv, t, gbase, sysmem + Gm::CB, v, std::make_integer_sequence<int, K>{});
-
-        // solve, one refinement step, solve again. The residual b - A' x' is
-        // exact: x' is x rounded to 24-bit fixed point (representable in FP32),
-        // A' the 30-bit copy, and the sum of the 2^54-bounded products is
-        // accumulated in 64-bit integers without rounding.
+    constexpr int TB = Gm::TB, NB = Gm::NB, P = Gm::P, TPS = Gm::TPS;
+    const int lane = threadIdx.x % kSolveSystems;
+    const int hh = TPS == 2 ? (int)threadIdx.x / kSolveSystems : 0;  // which thread of the system
+    const Lane<K> ln{smem + lane};
 #pragma unroll 1
-        for (int pass = 0; pass < 2; ++pass) {
-            chol_solve_seq<K, kBwdLook>(L, dinv, v, t, gbase, pass != 0,
-                                        std::make_integer_sequence<int, K>{});
-            if (pass == 1) {
-#pragma unroll
-                for (int s = 0; s < kR; ++s) x[s] += v[s];
-                break;
-            }
-            float xmax = 0.0f;
-#pragma unroll
-            for (int s = 0; s < kR; ++s) xmax = fmaxf(xmax, fabsf(v[s]));
-#pragma unroll
-            for (int o = 1; o < G; o <<= 1) xmax = fmaxf(xmax, __shfl_xor_sync(kFull, xmax, o));
-            const int ex = xmax > 0.0f ? 24 - exp_above(xmax) : 0;
-            const float sx = pow2f(ex), isx = pow2f(-ex);
-            int xq[kR];
-            long long acc[kR];
-#pragma unroll
-            for (int s = 0; s < kR; ++s) {
-                xq[s] = __float2int_rn(v[s] * sx);
-                x[s] = (float)xq[s] * isx;
-                acc[s] = __float2ll_rn((b[s] * sa) * sx);
-            }
-            if constexpr (G >= 4) {
-                // x' of the group through the column buffer: one 16-byte store
-                // per thread, four columns per 16-byte load
-                int* xb = reinterpret_cast<int*>(sysmem + Gm::CB);
-                *reinterpret_cast<int4*>(xb + 4 * t) = make_int4(xq[0], xq[1], xq[2], xq[3]);
-                __syncwarp();
-#pragma unroll 2
-                for (int tc = 0; tc < G; ++tc) {
-                    const int4 q4 = *reinterpret_cast<const int4*>(xb + 4 * tc);
-                    const int q[4] = {q4.x, q4.y, q4.z, q4.w};
-#pragma unroll
-                    for (int sc = 0; sc < kR; ++sc) {
-                        const int c = G * sc + tc;
-#pragma unroll
-                        for (int s = 0; s < kR; ++s) {
-                            // slots below / above mine hold columns below / above my row
-                            const int r = G * s + t;
-                            const int a = sc < s   ? Aq[tri(r) + c]
-                                          : sc > s ? Aq[tri(c) + r]
-                                                   : Aq[tri(max(r, c)) + min(r, c)];
-                            acc[s] -= (long long)a * (long long)q[sc];
-                        }
-                    }
-                }
-                __syncwarp();  // the buffer serves the next system's factor
-            } else {
-#pragma unroll
-                for (int sc = 0; sc < kR; ++sc) {
-#pragma unroll 4
-                    for (int tc = 0; tc < G; ++tc) {
-                        const int c = G * sc + tc;
-                        const int xc = __shfl_sync(kFull, xq[sc], gbase + tc);
-#pragma unroll
-                        for (int s = 0; s < kR; ++s) {
-                            const int r = G * s + t;
-                            const int a = Aq[tri(max(r, c)) + min(r, c)];
-                            acc[s] -= (long long)a * (long long)xc;
-                        }
-                    }
-                }
-            }
-#pragma unroll
-            for (int s = 0; s < kR; ++s) v[s] = (float)acc[s] * isx;  // sa (b - A' x')
+    for (int64_t blk = b0; blk < b1; ++blk) {
+    const int64_t sys = blk * kSolveSystems + lane;
+    bool live = sys < nsys;
+    int64_t node = node0 + (live ? sys : 0);
+    int qx, qy;
+    if constexpr (kPts) {
+        qx = __ldg(px + node);
+        qy = __ldg(py + node);
+    } else {
+        int i, j;
+        if (ids.stride > 0) {
+            live = slot_node(ids, g, live ? sys : 0, i, j) && live;
+            node = (int64_t)j * g.nx + i;
+        } else if (node < ((int64_t)1 << 31)) {
+            j = (int)((unsigned)node / (unsigned)g.nx);
+            i = (int)((unsigned)node - (unsigned)j * (unsigned)g.nx);
+        } else {
+            j = (int)(node / g.nx);
+            i = (int)(node % g.nx);
         }
+        qx = g.x0 + i * g.cell + g.cell / 2;
+        qy = g.y0 + j * g.cell + g.cell / 2;
+    }
 
-        // weights and outputs; the weight sum closes in FP64
-        float ps = 0.0f, pz = 0.0f, pv = 0.0f;
+    // ---- the neighbours: ids (-1 exactly past k_eff), records, variograms.
+    // Thread hh takes the groups of four neighbours 4 q + 1 .. 4 q + 4 (reduced
+    // rows 4 q .. 4 q + 3) with q = hh mod TPS; every load is issued before the
+    // first use.
+    constexpr int NQ = K / 4 / TPS;
+    int nid[4 * NQ], id0;
+    {
+        const int32_t* my = ids.p + (live ? sys : 0) * (ids.stride > 0 ? 1 : k);
+        const int64_t step = ids.stride > 0 ? ids.stride : 1;
+        id0 = live ? __ldg(my) : -1;
 #pragma unroll
-        for (int s = 0; s < kR; ++s) {
-            const bool row = G * s + t + 1 < ke;
-            const float lam = row ? x[s] : 0.0f;
-            ps += lam;
-            pz = fmaf(lam, T[G * s + t], pz);      // z_a - z_0
-            pv = fmaf(lam, T[K + G * s + t], pv);  // gamma_0a - Gamma_a0
+        for (int i = 0; i < 4 * NQ; ++i) {
+            const int n = 4 * (TPS * (i / 4) + hh) + i % 4 + 1;
+            nid[i] = (live && n < k) ? __ldg(my + n * step) : -1;
         }
-        double wsum = (double)ps;
+    }
+    // positions come from the records, upload indices from the upload order
+    const int4* const pos_base = ids.stride > 0 ? h.rec : h.orig;
+    auto record = [&](int id) {
+        return id >= 0 ? __ldg(pos_base + id) : id < -1 ? __ldg(h.orig + (-2 - id)) : make_int4(0, 0, 0, 0);
+    };
+    const int4 r0 = record(id0);
+    int4 rr[4 * NQ];
+    int ke = 0;
 #pragma unroll
-        for (int o = 1; o < G; o <<= 1) {
-            wsum += __shfl_xor_sync(kFull, wsum, o);
-            pz += __shfl_xor_sync(kFull, pz, o);
-            pv += __shfl_xor_sync(kFull, pv, o);
+    for (int i = 0; i < 4 * NQ; ++i) {
+        rr[i] = record(nid[i]);
+        ke += nid[i] != -1 ? 1 : 0;
+    }
+    const float z0 = __int_as_float(r0.z);
+    const float g00 = gamma_cm(p, r0.x - qx, r0.y - qy, 0.0f);
+    float gr0[4 * NQ];  // Gamma(row's neighbour, neighbour 0)
+    float gmax = 0.0f;
+    bool idw_on = false;  // the node lies on a sounding
+    float idw_num = 0.0f, idw_den = 0.0f;
+    if constexpr (kIdw) {
+        // idw_from's terms, in its order and partials: thread hh holds the partials
+        // 4 hh .. 4 hh + 3 of neighbours n >= 1 (n - 1 = 4 q + u, q = hh mod 2)
+        static_assert(TPS == 2 && kIdwLanes == 8, "the fused IDW runs with 2 threads per system");
+        // (32-bit distances where they fit in the whole warp: the same floats)
+        constexpr int kNear = 32000;
+        bool near = id0 == -1 || (abs(r0.x - qx) < kNear && abs(r0.y - qy) < kNear);
+        int ax[4 * NQ], ay[4 * NQ];
+#pragma unroll
+        for (int i = 0; i < 4 * NQ; ++i) {
+            ax[i] = rr[i].x - qx;
+            ay[i] = rr[i].y - qy;
+            near &= nid[i] == -1 || (abs(ax[i]) < kNear && abs(ay[i]) < kNear);
         }
-        const float lam0 = (float)(1.0 - wsum);
-        if (live && t == 0) {
+        float d[4 * NQ], d1;
+        if (__all_sync(kFull, near)) {
+            d1 = __int2float_rn((r0.x - qx) * (r0.x - qx) + (r0.y - qy) * (r0.y - qy));
+#pragma unroll
+            for (int i = 0; i < 4 * NQ; ++i) d[i] = __int2float_rn(ax[i] * ax[i] + ay[i] * ay[i]);
+        } else {
+            auto far = [&](int x, int y) {
+                const long long dx = (long long)x - qx, dy = (long long)y - qy;
+                return idw_d2f((uint64_t)(dx * dx + dy * dy));
+            };
+            d1 = far(r0.x, r0.y);
+#pragma unroll 1
+            for (int i = 0; i < 4 * NQ; ++i) {
+                int x = 0, y = 0;
+#pragma unroll
+                for (int e = 0; e < 4 * NQ; ++e) {
+                    x = e == i ? rr[e].x : x;
+                    y = e == i ? rr[e].y : y;
+                }
+                const float v = far(x, y);
+#pragma unroll
+                for (int e = 0; e < 4 * NQ; ++e) d[e] = e == i ? v : d[e];
+            }
+        }
+        idw_on = d1 == 0.0f;
+        float num[4], den[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) num[u] = den[u] = 0.0f;
+        auto terms = [&](float l1, float power) {
+#pragma unroll
+            for (int i = 0; i < 4 * NQ; ++i) {
+                const int n = 4 * (2 * (i / 4) + hh) + i % 4 + 1;
+                if (n >= fz.k) break;  // uniform over the warp
+                const float w = idw_weight(d1, l1, 0.5f * power, power, d[i]);
+                if (nid[i] != -1) {
+                    num[i % 4] = fmaf(w, __int_as_float(rr[i].z) - z0, num[i % 4]);
+                    den[i % 4] += w;
+                }
+            }
+        };
+        if (fz.power == 2.0f)
+            terms(0.0f, 2.0f);
+        else
+            terms(log2f(d1), fz.power);
+        idw_num = (num[0] + num[1]) + (num[2] + num[3]);
+        idw_den = (den[0] + den[1]) + (den[2] + den[3]);
+    }
+#pragma unroll
+    for (int j = 0; j < NQ; ++j) {
+        const int q = TPS * j + hh;
+        float ox[4], oy[4], dz[4], g0[4];
+        int pdx[4], pdy[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int4 v = rr[4 * j + u];
+            const bool real = nid[4 * j + u] != -1;
+            ox[u] = real ? (float)(v.x - r0.x) : 0.0f;
+            oy[u] = real ? (float)(v.y - r0.y) : 0.0f;
+            dz[u] = real ? __int_as_float(v.z) - z0 : 0.0f;
+            pdx[u] = v.x - qx;
+            pdy[u] = v.y - qy;
+        }
+        if constexpr (kSph) {
+#pragma unroll
+            for (int u = 0; u < 4; u += 2) {
+                gamma_pair_sph2(p, ox[u], oy[u], ox[u + 1], oy[u + 1], gr0[4 * j + u],
+                                gr0[4 * j + u + 1]);
+                gamma_cm_sph2(p, pdx[u], pdy[u], pdx[u + 1], pdy[u + 1], g0[u], g0[u + 1]);
+            }
+        } else {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                gr0[4 * j + u] = gamma_pair_f(p, ox[u], oy[u]);
+                g0[u] = gamma_cm(p, pdx[u], pdy[u], 0.0f);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (nid[4 * j + u] == -1) gr0[4 * j + u] = g0[u] = 0.0f;
+            gmax = fmaxf(gmax, gr0[4 * j + u]);
+        }
+        ln.vec(Gm::X + q) = make_float4(ox[0], ox[1], ox[2], ox[3]);
+        ln.vec(Gm::Y + q) = make_float4(oy[0], oy[1], oy[2], oy[3]);
+        ln.vec(Gm::DZ + q) = make_float4(dz[0], dz[1], dz[2], dz[3]);
+        ln.vec(Gm::G0 + q) = make_float4(g0[0], g0[1], g0[2], g0[3]);
+    }
+    if constexpr (TPS == 2) {
+        ln.vec(Gm::EX + hh) = make_float4(gmax, __int_as_float(ke), idw_num, idw_den);
+        pair_sync();
+        const float4 o = ln.vec(Gm::EX + 1 - hh);
+        gmax = fmaxf(gmax, o.x);
+        ke += __float_as_int(o.y);
+        idw_num += o.z;
+        idw_den += o.w;
+    }
+    ke = id0 != -1 ? ke + 1 : 0;  // neighbours; 0: no output (no data, or past the end)
+    if constexpr (kIdw) {
+        if (live && hh == 0)
+            fz.out[node] = ke == 0 ? __int_as_float(0x7fc00000)
+                                   : (idw_on ? z0 : z0 + idw_num / (1.0f + idw_den));
+    }
+    // A is SPD, so |A[r][c]| <= its largest diagonal entry max(1, 2 max Gamma_r0);
+    // fixed point with 30 bits below that bound
+    const int ea = 30 - exp_above(fmaxf(1.0f, 2.0f * gmax));
+    const float sa = pow2f(ea), isa = pow2f(-ea);
+#pragma unroll
+    for (int j = 0; j < NQ; ++j)
+        ln.vec(Gm::Z + TPS * j + hh) = make_float4(-gr0[4 * j] * sa, -gr0[4 * j + 1] * sa,
+                                                   -gr0[4 * j + 2] * sa, -gr0[4 * j + 3] * sa);
+    const TileVgm<kSph> vg(scaled_vgm(p, sa));
+    // -b in the scale, of row r with records z = -sa Gamma_r0 and g0 = gamma_0r
+    auto minus_b = [&](int r, float z, float g0) {
+        return r + 1 < ke ? -(__fadd_rn(__fadd_rn(-z * isa, g00), -g0) * sa) : 0.0f;
+    };
+
+    if constexpr (NB == 1) {
+        // ---- one tile: everything of the solve in registers
+        float nv[TB], ni[TB], Ld[Gm::TRI], b[TB];
+        {
+            float z[TB], g0[TB];
+            ln.floats(Gm::Z, 0, z);
+            ln.floats(Gm::G0, 0, g0);
+#pragma unroll
+            for (int r = 0; r < TB; ++r) b[r] = minus_b(r, z[r], g0[r]);
+        }
+        u64 t[TB][P];
+        {
+            u64 nvp[P];
+#pragma unroll
+            for (int q = 0; q < P; ++q) nvp[q] = pk2(b[2 * q], b[2 * q + 1]);
+            assemble_one<K, kSph>(ln, vg, ke, sa, t);
+            factor_tile<TB>(t, nvp, Ld, ni, nv);
+        }
+#pragma unroll
+        for (int r = 0; r < TB; ++r) nv[r] = -nv[r];
+        diag_backward<TB>(Ld, ni, nv);
+        float xmax = 0.0f;
+#pragma unroll
+        for (int r = 0; r < TB; ++r) xmax = fmaxf(xmax, fabsf(nv[r]));
+        const int ex = xmax > 0.0f ? 24 - exp_above(xmax) : 0;
+        const float sx = pow2f(ex), isx = pow2f(-ex);
+        int xq[TB];
+        long long acc[TB];
+#pragma unroll
+        for (int r = 0; r < TB; ++r) {
+            xq[r] = __float2int_rn(nv[r] * sx);
+            acc[r] = float_to_ll(-b[r] * sx);
+        }
+        assemble_one<K, kSph>(ln, vg, ke, sa, t);
+#pragma unroll
+        for (int c = 0; c < TB; ++c)
+#pragma unroll
+            for (int r = c; r < TB; ++r) {
+                const int a = __float2int_rn(lane2(t[c][r / 2], r & 1));
+                acc[r] += (long long)a * xq[c];
+                if (r != c) acc[c] += (long long)a * xq[r];
+            }
+#pragma unroll
+        for (int r = 0; r < TB; ++r) nv[r] = -(ll_to_float(acc[r]) * isx);  // -sa (b - A' x')
+        diag_forward<TB>(Ld, ni, nv);
+#pragma unroll
+        for (int r = 0; r < TB; ++r) nv[r] = -nv[r];
+        diag_backward<TB>(Ld, ni, nv);
+        int sq = 0;
+        float ps = 0.0f, pz = 0.0f, pv = 0.0f, dz[TB], g0[TB], z[TB];
+        ln.floats(Gm::DZ, 0, dz);
+        ln.floats(Gm::G0, 0, g0);
+        ln.floats(Gm::Z, 0, z);
+#pragma unroll
+        for (int r = 0; r < TB; ++r) {
+            const float lam = __fadd_rn(__fmul_rn((float)xq[r], isx), nv[r]);
+            sq += xq[r];
+            ps = __fadd_rn(ps, nv[r]);
+            pz = fmaf(lam, dz[r], pz);                            // z_a - z_0
+            pv = fmaf(lam, __fadd_rn(g0[r], z[r] * isa), pv);     // gamma_0a - Gamma_a0
+        }
+        const float lam0 = (float)(1.0 - ((double)sq * (double)isx + (double)ps));
+        if (live) {
             if (ke == 0) {
                 depth[node] = __int_as_float(0x7fc00000);  // no valid sounding
                 if (var) var[node] = __int_as_float(0x7fc00000);
@@ -892,7 +966,501 @@ __device__ __forceinline__ void okrige_solve_block(const HashView& h, const Grid
                 if (var) var[node] = fmaf(lam0, g00, g00 + pv);
             }
         }
-        __syncwarp();
+    } else {
+        pair_sync();  // every record is there
+        // every row but the last (row K - 1 has no neighbour) real, in the whole warp
+        const bool full = __all_sync(kFull, ke == K);
+        auto row_full = [&](int I) { return full && I + 1 < NB; };
+        const int pr[2] = {hh, 3 - hh};  // owned row pairs
+        const auto tcol = [&](int I, int J) {  // off-diagonal tile (I, J)
+            return tm + (uint32_t)((I * (I - 1) / 2 + J) * Gm::TILE);
+        };
+        const auto dcol = [&](int J) { return tm + (uint32_t)(Gm::OFF * Gm::TILE + J * Gm::DTILE); };
+        float Ld[Gm::TRI], ni[TB];  // the diagonal tile at hand and -1 / its diagonal
+
+        // ---- factor -A tile column by tile column; L y = b along the way
+#pragma unroll 1
+        for (int J = 0; J < NB; ++J) {
+            // (each thread of the pair its own code: pairs 0 and 3 or 1 and 2)
+            auto diag_part = [&](auto which) {
+                constexpr int p0 = decltype(which)::value, p1 = 3 - p0, N0 = 2 * p0 + 2, N1 = 2 * p1 + 2;
+                u64 t0[N0], t1[N1], nv[2];
+                {
+                    float xc[8], yc[8], zc[8], g0[8];
+                    ln.floats(Gm::X, J, xc);
+                    ln.floats(Gm::Y, J, yc);
+                    ln.floats(Gm::Z, J, zc);
+                    ln.floats(Gm::G0, J, g0);
+                    assemble_diag<K, kSph, p0>(ln, vg, J, ke, sa, row_full(J), xc, yc, zc, t0);
+                    assemble_diag<K, kSph, p1>(ln, vg, J, ke, sa, row_full(J), xc, yc, zc, t1);
+                    nv[0] = pk2(minus_b(8 * J + 2 * p0, zc[2 * p0], g0[2 * p0]),
+                                minus_b(8 * J + 2 * p0 + 1, zc[2 * p0 + 1], g0[2 * p0 + 1]));
+                    nv[1] = pk2(minus_b(8 * J + 2 * p1, zc[2 * p1], g0[2 * p1]),
+                                minus_b(8 * J + 2 * p1 + 1, zc[2 * p1 + 1], g0[2 * p1 + 1]));
+                }
+                if (K == 16 && J == 0) {  // kept for the residual: a = -A' of the first diagonal tile
+                    uint32_t w[32];
+#pragma unroll
+                    for (int c = 0; c < N0; ++c) {
+                        w[2 * c] = (uint32_t)__float2int_rn(lo2(t0[c]));
+                        w[2 * c + 1] = (uint32_t)__float2int_rn(hi2(t0[c]));
+                    }
+#pragma unroll
+                    for (int c = 0; c < N1; ++c) {
+                        w[2 * (N0 + c)] = (uint32_t)__float2int_rn(lo2(t1[c]));
+                        w[2 * (N0 + c) + 1] = (uint32_t)__float2int_rn(hi2(t1[c]));
+                    }
+                    uint32_t wa[16], wb[16];
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) {
+                        wa[e] = w[e];
+                        wb[e] = w[e < 4 ? 16 + e : 0];  // 20 words
+                    }
+                    tmem_st16(tm + Gm::KEEP + 64 + 32 * hh, wa);
+                    tmem_st16(tm + Gm::KEEP + 64 + 32 * hh + 16, wb);
+                }
+                if (J > 0) {  // less the earlier columns: four per step, loaded one step ahead
+                    uint32_t a[2][16], b[2][16];
+                    tmem_ld16(a[0], tcol(J, 0));
+                    tmem_ld16(b[0], tcol(J, 0) + 32);
+#pragma unroll 1
+                    for (int kb = 0; kb < J; ++kb) {
+                        float y[TB];
+                        ln.floats(Gm::V, kb, y);
+#pragma unroll
+                        for (int s = 0; s < 2; ++s) {
+                            tmem_wait_ld(a[s], b[s]);
+                            if (s == 0) {
+                                tmem_ld16(a[1], tcol(J, kb) + 16);
+                                tmem_ld16(b[1], tcol(J, kb) + 48);
+                            } else if (kb + 1 < J) {
+                                tmem_ld16(a[0], tcol(J, kb + 1));
+                                tmem_ld16(b[0], tcol(J, kb + 1) + 32);
+                            }
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                const uint32_t* o = (p0 == 0 ? a[s] : b[s]) + 4 * e;  // the owned rows
+                                const u64 L0 = pk2u(o[0], o[1]), L1 = pk2u(o[2], o[3]);
+#pragma unroll
+                                for (int c = 0; c < N1; ++c) {
+                                    const u64 m = dup2(__uint_as_float(
+                                        half_of(c) ? b[s][4 * e + place_of(c)]
+                                                   : a[s][4 * e + place_of(c)]));
+                                    if (c < N0) t0[c] = fma2(L0, m, t0[c]);
+                                    t1[c] = fma2(L1, m, t1[c]);
+                                }
+                                const u64 m = dup2(y[4 * s + e]);
+                                nv[0] = fma2(L0, m, nv[0]);
+                                nv[1] = fma2(L1, m, nv[1]);
+                            }
+                        }
+                    }
+                }
+                // the tile to both threads: pair p, columns 2 i and 2 i + 1 in
+                // vector 4 p + i
+#pragma unroll
+                for (int i = 0; i <= p0; ++i)
+                    ln.vec(Gm::DG + 4 * p0 + i) =
+                        make_float4(lo2(t0[2 * i]), hi2(t0[2 * i]), lo2(t0[2 * i + 1]), hi2(t0[2 * i + 1]));
+#pragma unroll
+                for (int i = 0; i <= p1; ++i)
+                    ln.vec(Gm::DG + 4 * p1 + i) =
+                        make_float4(lo2(t1[2 * i]), hi2(t1[2 * i]), lo2(t1[2 * i + 1]), hi2(t1[2 * i + 1]));
+                ln.pair(Gm::XB + 2 * (J & 1), 0, p0) = make_float2(lo2(nv[0]), hi2(nv[0]));
+                ln.pair(Gm::XB + 2 * (J & 1), 0, p1) = make_float2(lo2(nv[1]), hi2(nv[1]));
+            };
+            if (hh == 0)
+                diag_part(std::integral_constant<int, 0>{});
+            else
+                diag_part(std::integral_constant<int, 1>{});
+            pair_sync();
+            {
+                u64 t[TB][P], nvp[P];
+#pragma unroll
+                for (int q = 0; q < P; ++q)
+#pragma unroll
+                    for (int i = 0; i <= q; ++i) {
+                        const float4 f = ln.vec(Gm::DG + 4 * q + i);
+                        t[2 * i][q] = pk2(f.x, f.y);
+                        t[2 * i + 1][q] = pk2(f.z, f.w);
+                    }
+                ln.pairs(Gm::XB + 2 * (J & 1), 0, nvp);
+                float y[TB];
+                factor_tile<TB>(t, nvp, Ld, ni, y);
+                if (hh == 0) {
+                    ln.put(Gm::V, J, y);
+                    ln.put(Gm::DI, J, ni);
+                } else {
+                    uint32_t a[16], b[16];
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        a[i] = __float_as_uint(Ld[i]);
+                        b[i] = __float_as_uint(Ld[16 + i < Gm::TRI ? 16 + i : 0]);
+                    }
+                    tmem_st16(dcol(J), a);
+                    tmem_st16(dcol(J) + 16, b);
+                }
+            }
+#pragma unroll 1
+            for (int I = J + 1; I < NB; ++I) {
+                u64 t[2][8];
+                assemble_off<K, kSph>(ln, vg, I, J, pr, ke, row_full(I), t);
+                if constexpr (K == 16) {  // kept for the residual: a = -A' of the off-diagonal tile
+#pragma unroll
+                    for (int s = 0; s < 2; ++s) {
+                        uint32_t w[16];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e)
+#pragma unroll
+                            for (int u = 0; u < 2; ++u) {
+                                w[4 * e + 2 * u] = (uint32_t)__float2int_rn(lo2(t[u][4 * s + e]));
+                                w[4 * e + 2 * u + 1] = (uint32_t)__float2int_rn(hi2(t[u][4 * s + e]));
+                            }
+                        tmem_st16(tm + Gm::KEEP + 32 * hh + 16 * s, w);
+                    }
+                }
+                if (J > 0) {
+                    uint32_t a[2][16], b[2][16], o[2][16];
+                    tmem_ld16(a[0], tcol(J, 0));
+                    tmem_ld16(b[0], tcol(J, 0) + 32);
+                    tmem_ld16(o[0], tcol(I, 0) + 32 * hh);
+#pragma unroll 1
+                    for (int kb = 0; kb < J; ++kb) {
+#pragma unroll
+                        for (int s = 0; s < 2; ++s) {
+                            tmem_wait_ld(a[s], b[s]);
+                            tmem_use(o[s]);
+                            if (s == 0) {
+                                tmem_ld16(a[1], tcol(J, kb) + 16);
+                                tmem_ld16(b[1], tcol(J, kb) + 48);
+                                tmem_ld16(o[1], tcol(I, kb) + 32 * hh + 16);
+                            } else if (kb + 1 < J) {
+                                tmem_ld16(a[0], tcol(J, kb + 1));
+                                tmem_ld16(b[0], tcol(J, kb + 1) + 32);
+                                tmem_ld16(o[0], tcol(I, kb + 1) + 32 * hh);
+                            }
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                const u64 L0 = pk2u(o[s][4 * e], o[s][4 * e + 1]);
+                                const u64 L1 = pk2u(o[s][4 * e + 2], o[s][4 * e + 3]);
+#pragma unroll
+                                for (int c = 0; c < 8; ++c) {
+                                    const u64 m = dup2(__uint_as_float(
+                                        half_of(c) ? b[s][4 * e + place_of(c)]
+                                                   : a[s][4 * e + place_of(c)]));
+                                    t[0][c] = fma2(L0, m, t[0][c]);
+                                    t[1][c] = fma2(L1, m, t[1][c]);
+                                }
+                            }
+                        }
+                    }
+                }
+                // solve against the diagonal tile: X Ljj^T = A - ..., row by row
+                int at = 0;
+#pragma unroll
+                for (int c = 0; c < TB; ++c) {
+                    const u64 m = dup2(ni[c]);
+                    t[0][c] = mul2(t[0][c], m);
+                    t[1][c] = mul2(t[1][c], m);
+#pragma unroll
+                    for (int r = c + 1; r < TB; ++r) {
+                        const u64 l = dup2(Ld[at++]);
+                        t[0][r] = fma2(t[0][c], l, t[0][r]);
+                        t[1][r] = fma2(t[1][c], l, t[1][r]);
+                    }
+                }
+#pragma unroll
+                for (int s = 0; s < 2; ++s) {
+                    uint32_t a[16];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+#pragma unroll
+                        for (int u = 0; u < 2; ++u) {
+                            a[4 * e + 2 * u] = __float_as_uint(lo2(t[u][4 * s + e]));
+                            a[4 * e + 2 * u + 1] = __float_as_uint(hi2(t[u][4 * s + e]));
+                        }
+                    tmem_st16(tcol(I, J) + 32 * hh + 16 * s, a);
+                }
+            }
+            pair_sync_tmem();
+        }
+
+        // ---- solve, one refinement step, solve again: the unknowns in registers
+        // (the same in both threads); a tile row's sums are shared out and
+        // exchanged through the two buffers XB in turn
+        auto load_diag = [&](int J) {
+            uint32_t a[16], b[16];
+            tmem_ld16(a, dcol(J));
+            tmem_ld16(b, dcol(J) + 16);
+            ln.floats(Gm::DI, J, ni);
+            tmem_wait_ld(a, b);
+#pragma unroll
+            for (int i = 0; i < Gm::TRI; ++i) Ld[i] = __uint_as_float(i < 16 ? a[i] : b[i - 16]);
+        };
+        float x[NB][TB];
+        auto forward = [&]() {  // L y = v: thread hh brings -v of its row pairs in x's place
+#pragma unroll
+            for (int I = 0; I < NB; ++I) {
+                u64 nv[2] = {pk2(x[I][0], x[I][1]), pk2(x[I][2], x[I][3])};
+#pragma unroll
+                for (int J = 0; J < I; ++J) {
+                    uint32_t a[16], b[16];
+                    tmem_ld16(a, tcol(I, J) + 32 * hh);
+                    tmem_ld16(b, tcol(I, J) + 32 * hh + 16);
+                    tmem_wait_ld(a, b);
+#pragma unroll
+                    for (int c = 0; c < TB; ++c) {
+                        const uint32_t* w = c < 4 ? a + 4 * c : b + 4 * (c - 4);
+                        const u64 m = dup2(x[J][c]);
+                        nv[0] = fma2(pk2u(w[0], w[1]), m, nv[0]);
+                        nv[1] = fma2(pk2u(w[2], w[3]), m, nv[1]);
+                    }
+                }
+                load_diag(I);
+#pragma unroll
+                for (int u = 0; u < 2; ++u)
+                    ln.pair(Gm::XB + 2 * (I & 1), 0, pr[u]) = make_float2(lo2(nv[u]), hi2(nv[u]));
+                pair_sync();
+                ln.floats(Gm::XB + 2 * (I & 1), 0, x[I]);
+                diag_forward<TB>(Ld, ni, x[I]);
+            }
+        };
+        auto backward = [&]() {  // L^T x = y: thread hh brings y of columns 4 hh .. 4 hh + 3
+#pragma unroll
+            for (int J = NB - 1; J >= 0; --J) {
+                u64 sum[4];  // owned columns; partial sums of the even and the odd rows
+#pragma unroll
+                for (int c = 0; c < 4; ++c) sum[c] = 0;
+#pragma unroll
+                for (int I = NB - 1; I > J; --I) {
+                    uint32_t a[16], b[16];
+                    tmem_ld16(a, tcol(I, J) + 16 * hh);
+                    tmem_ld16(b, tcol(I, J) + 16 * hh + 32);
+                    tmem_wait_ld(a, b);
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        sum[c] = fma2(pk2u(a[4 * c], a[4 * c + 1]), pk2(x[I][0], x[I][1]), sum[c]);
+                        sum[c] = fma2(pk2u(b[4 * c], b[4 * c + 1]), pk2(x[I][2], x[I][3]), sum[c]);
+                        sum[c] = fma2(pk2u(b[4 * c + 2], b[4 * c + 3]), pk2(x[I][4], x[I][5]), sum[c]);
+                        sum[c] = fma2(pk2u(a[4 * c + 2], a[4 * c + 3]), pk2(x[I][6], x[I][7]), sum[c]);
+                    }
+                }
+                load_diag(J);
+                const int buf = Gm::XB + 2 * ((NB - 1 - J) & 1);
+                ln.vec(buf + hh) = make_float4(__fadd_rn(__fadd_rn(lo2(sum[0]), hi2(sum[0])), -x[J][0]),
+                                               __fadd_rn(__fadd_rn(lo2(sum[1]), hi2(sum[1])), -x[J][1]),
+                                               __fadd_rn(__fadd_rn(lo2(sum[2]), hi2(sum[2])), -x[J][2]),
+                                               __fadd_rn(__fadd_rn(lo2(sum[3]), hi2(sum[3])), -x[J][3]));
+                pair_sync();
+                ln.floats(buf, 0, x[J]);
+                diag_backward<TB>(Ld, ni, x[J]);
+            }
+        };
+#pragma unroll
+        for (int J = 0; J < NB; ++J) {
+            const float4 y = ln.vec(Gm::V + 2 * J + hh);
+            x[J][0] = y.x;
+            x[J][1] = y.y;
+            x[J][2] = y.z;
+            x[J][3] = y.w;
+        }
+        backward();
+        // The residual b - A' x' is exact: x' is x rounded to 24-bit fixed point
+        // (representable in FP32), A' the 30-bit copy, and the sum of the
+        // 2^54-bounded products is accumulated in 64-bit integers without rounding.
+        float xmax = 0.0f;
+#pragma unroll
+        for (int I = 0; I < NB; ++I)
+#pragma unroll
+            for (int r = 0; r < TB; ++r) xmax = fmaxf(xmax, fabsf(x[I][r]));
+        const int ex = xmax > 0.0f ? 24 - exp_above(xmax) : 0;
+        const float sx = pow2f(ex), isx = pow2f(-ex);
+        // (the solution of L y = b in V has been read by both threads: each passed
+        // a barrier of the back substitution after it)
+        if (hh == 0) {
+#pragma unroll
+            for (int I = 0; I < NB; ++I) {
+                int xq[TB];
+#pragma unroll
+                for (int r = 0; r < TB; ++r) xq[r] = __float2int_rn(x[I][r] * sx);
+                ln.put_ints(Gm::V, I, xq);
+            }
+        }
+        pair_sync();
+        const int acc0 = Gm::ACC + hh * 2 * Gm::Q;  // this thread's sums: pair p of row I at 4 I + p
+#pragma unroll 1
+        for (int I = 0; I < NB; ++I) {
+            long long accr[4];
+            int xi[TB], xr[4];
+            ln.ints(Gm::V, I, xi);
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const float2 z = ln.pair(Gm::Z, I, pr[u]), g0 = ln.pair(Gm::G0, I, pr[u]),
+                             xx = ln.pair(Gm::V, I, pr[u]);
+                accr[2 * u] = float_to_ll(-minus_b(8 * I + 2 * pr[u], z.x, g0.x) * sx);
+                accr[2 * u + 1] = float_to_ll(-minus_b(8 * I + 2 * pr[u] + 1, z.y, g0.y) * sx);
+                xr[2 * u] = __float_as_int(xx.x);
+                xr[2 * u + 1] = __float_as_int(xx.y);
+            }
+            // (the sums take + a x' with a = -A')
+#pragma unroll 1
+            for (int J = 0; J < I; ++J) {
+                u64 t[2][8];
+                uint32_t qa[16], qb[16];
+                if constexpr (K == 16) {
+                    tmem_ld16(qa, tm + Gm::KEEP + 32 * hh);
+                    tmem_ld16(qb, tm + Gm::KEEP + 32 * hh + 16);
+                    tmem_wait_ld(qa, qb);
+                } else {
+                    assemble_off<K, kSph>(ln, vg, I, J, pr, ke, row_full(I), t);
+                }
+                int xj[TB];
+                ln.ints(Gm::V, J, xj);
+#pragma unroll
+                for (int c2 = 0; c2 < 4; ++c2) {
+                    longlong2 aj = ln.long2(acc0 + 4 * J + c2);
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const int c = 2 * c2 + e;
+                        long long s = e ? aj.y : aj.x;
+#pragma unroll
+                        for (int u = 0; u < 2; ++u) {
+                            int a0, a1;
+                            if constexpr (K == 16) {
+                                a0 = (int)(c < 4 ? qa[4 * c + 2 * u] : qb[4 * (c - 4) + 2 * u]);
+                                a1 = (int)(c < 4 ? qa[4 * c + 2 * u + 1] : qb[4 * (c - 4) + 2 * u + 1]);
+                            } else {
+                                a0 = __float2int_rn(lo2(t[u][c]));
+                                a1 = __float2int_rn(hi2(t[u][c]));
+                            }
+                            accr[2 * u] += (long long)a0 * xj[c];
+                            accr[2 * u + 1] += (long long)a1 * xj[c];
+                            s += (long long)a0 * xr[2 * u];
+                            s += (long long)a1 * xr[2 * u + 1];
+                        }
+                        if (e)
+                            aj.y = s;
+                        else
+                            aj.x = s;
+                    }
+                    ln.long2(acc0 + 4 * J + c2) = aj;
+                }
+            }
+            auto diag_part = [&](auto which) {
+                constexpr int p0 = decltype(which)::value, p1 = 3 - p0, N0 = 2 * p0 + 2, N1 = 2 * p1 + 2;
+                long long acc[TB];
+#pragma unroll
+                for (int r = 0; r < TB; ++r) acc[r] = 0;
+                acc[2 * p0] = accr[0];
+                acc[2 * p0 + 1] = accr[1];
+                acc[2 * p1] = accr[2];
+                acc[2 * p1 + 1] = accr[3];
+                // entries below the diagonal also stand for their mirror image
+                auto add = [&](int r, int c, int a) {
+                    acc[r] += (long long)a * xi[c];
+                    if (r != c) acc[c] += (long long)a * xi[r];
+                };
+                auto add_tile = [&](auto at0, auto at1) {  // the entries of pair p0 and of pair p1
+#pragma unroll
+                    for (int c = 0; c < N0; ++c) {
+                        if (c <= 2 * p0) add(2 * p0, c, at0(2 * c));
+                        add(2 * p0 + 1, c, at0(2 * c + 1));
+                    }
+#pragma unroll
+                    for (int c = 0; c < N1; ++c) {
+                        if (c <= 2 * p1) add(2 * p1, c, at1(2 * c));
+                        add(2 * p1 + 1, c, at1(2 * c + 1));
+                    }
+                };
+                if (K == 16 && I == 0) {
+                    uint32_t a[16], b[16];
+                    tmem_ld16(a, tm + Gm::KEEP + 64 + 32 * hh);
+                    tmem_ld16(b, tm + Gm::KEEP + 64 + 32 * hh + 16);
+                    tmem_wait_ld(a, b);
+                    add_tile([&](int e) { return (int)a[e]; },
+                             [&](int e) { return (int)(2 * N0 + e < 16 ? a[2 * N0 + e] : b[2 * N0 + e - 16]); });
+                } else {
+                    float xc[8], yc[8], zc[8];
+                    ln.floats(Gm::X, I, xc);
+                    ln.floats(Gm::Y, I, yc);
+                    ln.floats(Gm::Z, I, zc);
+                    u64 t0[N0], t1[N1];
+                    assemble_diag<K, kSph, p0>(ln, vg, I, ke, sa, row_full(I), xc, yc, zc, t0);
+                    assemble_diag<K, kSph, p1>(ln, vg, I, ke, sa, row_full(I), xc, yc, zc, t1);
+                    add_tile([&](int e) { return __float2int_rn(lane2(t0[e / 2], e & 1)); },
+                             [&](int e) { return __float2int_rn(lane2(t1[e / 2], e & 1)); });
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    ln.long2(acc0 + 4 * I + q) = make_longlong2(acc[2 * q], acc[2 * q + 1]);
+            };
+            if (hh == 0)
+                diag_part(std::integral_constant<int, 0>{});
+            else
+                diag_part(std::integral_constant<int, 1>{});
+        }
+        pair_sync();
+#pragma unroll
+        for (int I = 0; I < NB; ++I)
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {  // -sa (b - A' x') of the owned rows
+                const longlong2 a = ln.long2(Gm::ACC + 4 * I + pr[u]);
+                const longlong2 b = ln.long2(Gm::ACC + 2 * Gm::Q + 4 * I + pr[u]);
+                x[I][2 * u] = -(ll_to_float(a.x + b.x) * isx);
+                x[I][2 * u + 1] = -(ll_to_float(a.y + b.y) * isx);
+            }
+        forward();
+        // y of the owned columns to the front, as backward() takes it
+#pragma unroll
+        for (int I = 0; I < NB; ++I)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) x[I][c] = hh ? x[I][c + 4] : x[I][c];
+        backward();
+
+        // ---- weights and outputs: thread 0 the depth, thread 1 the variance. The
+        // weight sum closes in FP64: x' sums exactly as integers (32 x 2^24), the
+        // correction in FP32. Sums run in eight partials, combined pairwise.
+        if (hh == 0) {
+            float pz[TB];
+#pragma unroll
+            for (int r = 0; r < TB; ++r) pz[r] = 0.0f;
+#pragma unroll
+            for (int I = 0; I < NB; ++I) {
+                float dz[TB];
+                int xq[TB];
+                ln.floats(Gm::DZ, I, dz);
+                ln.ints(Gm::V, I, xq);
+#pragma unroll
+                for (int r = 0; r < TB; ++r)  // lambda (z_a - z_0)
+                    pz[r] = fmaf(__fadd_rn(__fmul_rn((float)xq[r], isx), x[I][r]), dz[r], pz[r]);
+            }
+            if (live) depth[node] = ke == 0 ? __int_as_float(0x7fc00000) : z0 + idw_tree8(pz);  // no valid sounding: NaN
+        } else if (var) {
+            int sq = 0;
+            float ps[TB], pv[TB];
+#pragma unroll
+            for (int r = 0; r < TB; ++r) ps[r] = pv[r] = 0.0f;
+#pragma unroll
+            for (int I = 0; I < NB; ++I) {
+                float g0[TB], z[TB];
+                int xq[TB];
+                ln.floats(Gm::G0, I, g0);
+                ln.floats(Gm::Z, I, z);
+                ln.ints(Gm::V, I, xq);
+#pragma unroll
+                for (int r = 0; r < TB; ++r) {
+                    const float lam = __fadd_rn(__fmul_rn((float)xq[r], isx), x[I][r]);
+                    sq += xq[r];
+                    ps[r] = __fadd_rn(ps[r], x[I][r]);
+                    pv[r] = fmaf(lam, __fadd_rn(g0[r], z[r] * isa), pv[r]);  // gamma_0a - Gamma_a0
+                }
+            }
+            const float lam0 = (float)(1.0 - ((double)sq * (double)isx + (double)idw_tree8(ps)));
+            if (live)
+                var[node] = ke == 0 ? __int_as_float(0x7fc00000) : fmaf(lam0, g00, g00 + idw_tree8(pv));
+        }
+        pair_sync();  // the next batch overwrites the records
+    }
     }
 }
 

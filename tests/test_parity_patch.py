@@ -72,3 +72,26 @@ def test_idw_neighbours_and_depths(name, k):
     ref, ridx = oracle.idw(x, y, z, qx, qy, k, 2.0, want_idx=True)
     assert np.array_equal(nb, ridx)
     assert_idw(d, ref)
+
+
+@pytest.mark.parametrize("model,nugget,k", [(0, 0.25, 32), (0, 0.25, 15), (0, 0.25, 7), (1, 0.25, 32), (1, 0.25, 13),
+                                            (0, 0.25, 3)])
+@pytest.mark.parametrize("name", ["one_node", "whole_patch", "remainders", "past_the_edge", "many_per_node", "gap",
+                                  "sparse", "few"])
+def test_kriging_systems_of_every_size(name, model, nugget, k):
+    """Systems of k unknowns in tiles of 8 (whole and padded), by patches and by
+    rows, with the neighbour lists and without (the two layouts of the ids)."""
+    from gpu_util import assert_okrige
+    make, g = CASES[name]
+    x, y, z = make()
+    lib = Lib(x, y, z, g)
+    try:
+        d, v, nb = lib.okrige(k, model, nugget, 100.0, 50.0)
+        d2, v2, _ = lib.okrige(k, model, nugget, 100.0, 50.0, want_nbr=False)
+    finally:
+        lib.close()
+    qx, qy = oracle.grid_nodes(g.x0_cm, g.y0_cm, g.cell_cm, g.nx, g.ny)
+    rd, rv, ridx = oracle.okrige(x, y, z, qx, qy, k, model, nugget, 100.0, 50.0, want_idx=True)
+    assert np.array_equal(nb, ridx)
+    assert_okrige(d, v, rd, rv, nugget)
+    assert np.array_equal(d, d2) and np.array_equal(v, v2)
