@@ -35,20 +35,23 @@
 // instruction). The factor works on -A (the tile sums then need no negations).
 // What bounds it: issue and latency at two warps per scheduler (half of the
 // issue slots; FP32 pipe half busy in the factor, the square roots and
-// conversions half busy in the residual), K = 32 with the fused IDW: 52,000
-// cycles per 128 systems, of them factor 21,000, residual 16,000, gathers 3,500.
-// Measured on one survey line (3,001 x 692 nodes, k = 32, fused IDW): 2.76 ms
-// against 3.84 ms for 8 threads per system with the factor in registers (1,500
+// conversions half busy in the residual), K = 32 with the fused IDW: 48,000
+// cycles per 128 systems, of them factor 22,500, residual 11,300 (16,400 with the
+// tiles evaluated again, 9,900 with them rounded to integers before they are
+// kept, but then the factor takes 24,900), gathers 3,500.
+// Measured on one survey line (3,001 x 692 nodes, k = 32, fused IDW): 2.59 ms
+// (2.77 with the tiles evaluated again) against 3.84 ms for 8 threads per system with the factor in registers (1,500
 // warp instructions per system there, 780 here; one thread per system: 630, but
 // one warp per scheduler and 3.5 ms); 256 x 256 tile, k = 16: 29 against 37 us.
-// Loading the next batch's ids and records during the last solve, and keeping
-// one tile of A' in the shared memory that is left at K = 32, changed nothing.
+// Loading the next batch's ids and records during the last solve changed nothing.
 //
 // One step of iterative refinement follows the solve: A' is A rounded to a
 // 30-bit fixed point, x is rounded to 24-bit fixed point x' (exact in FP32),
-// and the residual b - A' x' is accumulated exactly in 64-bit integers; at K =
-// 32 the tiles of A are evaluated again rather than kept (on-chip memory holds
-// one of the two triangles), at K = 16 most are kept in tensor memory. The correction reuses the factor. The weight sum
+// and the residual b - A' x' is accumulated exactly in 64-bit integers. The
+// tiles of A are kept for it: at K = 16 most of them in tensor memory beside
+// the factor, at K = 32, where on-chip memory holds only one of the two
+// triangles, in the threads' local memory (1.1 KB a thread, 36 MB over the
+// device's resident systems: it stays in L2), read one tile ahead. The correction reuses the factor. The weight sum
 // closes in FP64: lambda_0 = 1 - sum(lambda'). Outputs:
 //     zhat    = z_0 + sum_a lambda_a (z_a - z_0)          (= sum lambda_i z_i)
 //     sigma^2 = lambda_0 gamma_00 + sum_a lambda_a gamma_a0 + mu.
@@ -977,6 +980,7 @@ __device__ __forceinline__ void okrige_solve_range(const HashView& h, const Grid
         };
         const auto dcol = [&](int J) { return tm + (uint32_t)(Gm::OFF * Gm::TILE + J * Gm::DTILE); };
         float Ld[Gm::TRI], ni[TB];  // the diagonal tile at hand and -1 / its diagonal
+        float4 kept[K == 32 ? 8 * (NB * (NB + 1) / 2) : 1];  // K = 32: -A of this thread's rows, tile (I, J) at 8 (I (I + 1) / 2 + J)
 
         // ---- factor -A tile column by tile column; L y = b along the way
 #pragma unroll 1
@@ -1018,6 +1022,16 @@ __device__ __forceinline__ void okrige_solve_range(const HashView& h, const Grid
                     }
                     tmem_st16(tm + Gm::KEEP + 64 + 32 * hh, wa);
                     tmem_st16(tm + Gm::KEEP + 64 + 32 * hh + 16, wb);
+                }
+                if constexpr (K == 32) {
+                    auto val = [&](int e) {
+                        return e < 2 * N0 ? lane2(t0[e < 2 * N0 ? e / 2 : 0], e & 1)
+                                          : lane2(t1[e < 2 * N0 ? 0 : (e - 2 * N0) / 2], e & 1);
+                    };
+#pragma unroll
+                    for (int v = 0; v < 5; ++v)
+                        kept[8 * (J * (J + 1) / 2 + J) + v] =
+                            make_float4(val(4 * v), val(4 * v + 1), val(4 * v + 2), val(4 * v + 3));
                 }
                 if (J > 0) {  // less the earlier columns: four per step, loaded one step ahead
                     uint32_t a[2][16], b[2][16];
@@ -1118,6 +1132,11 @@ __device__ __forceinline__ void okrige_solve_range(const HashView& h, const Grid
                             }
                         tmem_st16(tm + Gm::KEEP + 32 * hh + 16 * s, w);
                     }
+                } else {
+#pragma unroll
+                    for (int c = 0; c < TB; ++c)
+                        kept[8 * (I * (I + 1) / 2 + J) + c] =
+                            make_float4(lo2(t[0][c]), hi2(t[0][c]), lo2(t[1][c]), hi2(t[1][c]));
                 }
                 if (J > 0) {
                     uint32_t a[2][16], b[2][16], o[2][16];
@@ -1288,6 +1307,11 @@ __device__ __forceinline__ void okrige_solve_range(const HashView& h, const Grid
         }
         pair_sync();
         const int acc0 = Gm::ACC + hh * 2 * Gm::Q;  // this thread's sums: pair p of row I at 4 I + p
+        float4 nxt[8];  // the tile ahead
+        int tile = 0;
+        if constexpr (K == 32)
+#pragma unroll
+            for (int c = 0; c < 8; ++c) nxt[c] = kept[c];
 #pragma unroll 1
         for (int I = 0; I < NB; ++I) {
             long long accr[4];
@@ -1305,14 +1329,19 @@ __device__ __forceinline__ void okrige_solve_range(const HashView& h, const Grid
             // (the sums take + a x' with a = -A')
 #pragma unroll 1
             for (int J = 0; J < I; ++J) {
-                u64 t[2][8];
                 uint32_t qa[16], qb[16];
+                float4 cur[8];
+#pragma unroll
+                for (int c = 0; c < 8; ++c) cur[c] = nxt[c];
+                if constexpr (K == 32) {
+                    ++tile;
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) nxt[c] = kept[8 * tile + c];
+                }
                 if constexpr (K == 16) {
                     tmem_ld16(qa, tm + Gm::KEEP + 32 * hh);
                     tmem_ld16(qb, tm + Gm::KEEP + 32 * hh + 16);
                     tmem_wait_ld(qa, qb);
-                } else {
-                    assemble_off<K, kSph>(ln, vg, I, J, pr, ke, row_full(I), t);
                 }
                 int xj[TB];
                 ln.ints(Gm::V, J, xj);
@@ -1330,8 +1359,8 @@ __device__ __forceinline__ void okrige_solve_range(const HashView& h, const Grid
                                 a0 = (int)(c < 4 ? qa[4 * c + 2 * u] : qb[4 * (c - 4) + 2 * u]);
                                 a1 = (int)(c < 4 ? qa[4 * c + 2 * u + 1] : qb[4 * (c - 4) + 2 * u + 1]);
                             } else {
-                                a0 = __float2int_rn(lo2(t[u][c]));
-                                a1 = __float2int_rn(hi2(t[u][c]));
+                                a0 = __float2int_rn(u ? cur[c].z : cur[c].x);
+                                a1 = __float2int_rn(u ? cur[c].w : cur[c].y);
                             }
                             accr[2 * u] += (long long)a0 * xj[c];
                             accr[2 * u + 1] += (long long)a1 * xj[c];
@@ -1345,6 +1374,15 @@ __device__ __forceinline__ void okrige_solve_range(const HashView& h, const Grid
                     }
                     ln.long2(acc0 + 4 * J + c2) = aj;
                 }
+            }
+            float4 cur[8];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) cur[c] = nxt[c];
+            if constexpr (K == 32) {
+                ++tile;
+                if (I + 1 < NB)
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) nxt[c] = kept[8 * tile + c];
             }
             auto diag_part = [&](auto which) {
                 constexpr int p0 = decltype(which)::value, p1 = 3 - p0, N0 = 2 * p0 + 2, N1 = 2 * p1 + 2;
@@ -1379,6 +1417,12 @@ __device__ __forceinline__ void okrige_solve_range(const HashView& h, const Grid
                     tmem_wait_ld(a, b);
                     add_tile([&](int e) { return (int)a[e]; },
                              [&](int e) { return (int)(2 * N0 + e < 16 ? a[2 * N0 + e] : b[2 * N0 + e - 16]); });
+                } else if constexpr (K == 32) {
+                    auto val = [&](int e) {
+                        const float4 v = cur[e / 4];
+                        return __float2int_rn(e % 4 == 0 ? v.x : e % 4 == 1 ? v.y : e % 4 == 2 ? v.z : v.w);
+                    };
+                    add_tile([&](int e) { return val(e); }, [&](int e) { return val(2 * N0 + e); });
                 } else {
                     float xc[8], yc[8], zc[8];
                     ln.floats(Gm::X, I, xc);
