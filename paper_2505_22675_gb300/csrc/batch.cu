@@ -12,11 +12,11 @@
 //      exclusive scan, scatter (cell_start holds positions in the shared
 //      record array, so each tile's hash is a window of it);
 //   4. per-tile summed-area tables (one block per tile);
-//   5. a persistent kernel drains (tile, 16 S x 8 node patch) items, a thread
-//      gridding S consecutive nodes along x (S = 1, 2 or 4: the strip
-//      length; from the second node on, the previous node's K-th distance
-//      plus the step bounds the search): IDW tiles are gridded in place,
-//      kriging tiles get their neighbour ids;
+//   5. persistent kernels, one per search size, drain (tile, 16 S x 8 node patch)
+//      items (S = 1, 2 or 4: the strip length): a warp walks the item by
+//      patches of 8 x 4 nodes (knn_warp.cuh). Tiles with more soundings per node
+//      than that search holds go by threads, S consecutive nodes each along x.
+//      IDW tiles are gridded in place, kriging tiles get their neighbour ids;
 //   6. a persistent kernel per kriging system size and variogram model drains
 //      (tile, batches of 128 systems) items (okrige_solve_range);
 //   7. a wide-key pass, which returns at once unless a node's bound needed
@@ -45,11 +45,13 @@ struct TileDesc {
     const float* z;
     float* depth;        // outputs (device)
     float* var;
-    int32_t* ids;        // kriging: nx*ny*k neighbour ids
+    int32_t* ids;        // kriging: neighbour ids (IdsView)
+    int64_t stride;      // of the patches layout; 0: the batch keeps rows
+    int32_t patch;       // this run's k-NN goes by patches (written on the device)
     OkParams p;
     float power;
     int32_t method, k, K;  // K: kriging system size (4/8/16/32)
-    int32_t gx;          // node patches along x
+    int32_t gx;          // 16 x 8 node patches along x
     int64_t soff, n;     // soundings in the concatenation
     int64_t coff, cap;   // cells
     int64_t satoff, satcap;
@@ -161,8 +163,24 @@ __global__ void __launch_bounds__(kBT) k_batch_validate(const TileDesc* __restri
 }
 
 // 2. per-tile hash geometry (one thread per tile)
+__device__ __forceinline__ bool tile_patch_fits(const HashView& h, const GridView& g, int kq) {
+    auto fits = [&](auto K) {
+        return knn_patch_fits<decltype(K)::value>(h.n_valid, h.ncx, h.ncy, h.cs, g.cell, g.nx, g.ny);
+    };
+    return kq <= 4    ? fits(std::integral_constant<int, 4>{})
+           : kq <= 8  ? fits(std::integral_constant<int, 8>{})
+           : kq <= 16 ? fits(std::integral_constant<int, 16>{})
+                      : fits(std::integral_constant<int, 32>{});
+}
+
+// the ids of a tile as this run's k-NN writes them
+__device__ __forceinline__ IdsView tile_ids(const TileDesc& d) {
+    return IdsView{d.ids, d.patch ? d.stride : 0, (d.g.nx + 7) / 8, 0, d.g.ny};
+}
+
+// rest: set when some tile's k-NN goes by threads instead of patches
 __global__ void k_batch_geom(TileDesc* td, int T, const int* __restrict__ acc, float ppc,
-                             int* __restrict__ status) {
+                             int* __restrict__ status, int* __restrict__ rest) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= T) return;
     TileDesc& d = td[t];
@@ -175,6 +193,8 @@ __global__ void k_batch_geom(TileDesc* td, int T, const int* __restrict__ acc, f
     }
     if (h.n_valid == 0) {
         h.ncx = h.ncy = 0;
+        d.patch = 0;
+        *rest = 1;
         return;
     }
     const int64_t W = (int64_t)a[2] - a[0] + 1, H = (int64_t)a[3] - a[1] + 1;
@@ -197,6 +217,8 @@ __global__ void k_batch_geom(TileDesc* td, int T, const int* __restrict__ acc, f
     const double per_cell = (double)h.n_valid / ((double)h.ncx * h.ncy);
     int r = (int)ceil((sqrt((double)kq / per_cell) - 1.0) * 0.5);
     h.r0 = max(0, min(r, max(h.ncx, h.ncy)));
+    d.patch = tile_patch_fits(h, d.g, d.K);
+    if (!d.patch) *rest = 1;
 }
 
 // 3a/3c. histogram and scatter over the concatenated soundings
@@ -262,7 +284,53 @@ __device__ __forceinline__ HashView tile_view(const TileDesc& d, const int4* ori
     return h;
 }
 
-// 5. persistent k-NN items: IDW in place, kriging ids. An item is a
+// 5. persistent k-NN items of the tiles that go by patches (knn_warp.cuh), one
+// kernel per search size K: a warp claims a (16 kS) x 8 node item of one tile and
+// walks its two rows of patches. IDW in place, kriging ids.
+template <int K>
+__global__ void __launch_bounds__(64, KnnWarp<K>::kBlocksPerSM) k_batch_knn_patch(
+    const TileDesc* __restrict__ td, const int* __restrict__ tiles, int nt, const int64_t* __restrict__ off,
+    int64_t items, unsigned long long* __restrict__ ctr, const int4* __restrict__ orig, const int4* __restrict__ rec,
+    const int* __restrict__ cell_start, const int* __restrict__ sat, int* __restrict__ wide, int strip) {
+    __shared__ typename KnnWarp<K>::Smem smem[2];
+    typename KnnWarp<K>::Smem& sm = smem[threadIdx.x >> 5];
+    for (;;) {
+        long long item = 0;
+        if ((threadIdx.x & 31) == 0) item = (long long)atomicAdd(ctr, 1ull);
+        item = __shfl_sync(kFull, item, 0);
+        if (item >= items) break;
+        const int q = upper_tile(off, nt + 1, item);
+        const TileDesc& d = td[__ldg(tiles + q)];
+        if (!d.patch) continue;
+        const HashView h = tile_view(d, orig, rec, cell_start, sat);
+        const GridView g = d.g;
+        const int gx = (g.nx + 16 * strip - 1) / (16 * strip);
+        const int64_t at = item - __ldg(off + q);
+        const int p0 = (int)(at % gx) * 2 * strip, jb = (int)(at / gx) * 8;
+        const int k = d.k;
+        const IdsView ids = tile_ids(d);
+        auto out = [&](int i, int j) { return (int64_t)j * g.nx + i; };
+        auto slot = [&](int i, int j) {
+            return ids.p + (ids.stride > 0 ? node_slot(ids, i, j) : out(i, j) * k);
+        };
+        for (int row = jb; row < jb + 8 && row < g.ny; row += 4)
+            knn_patch_row<K>(
+                h, g, sm, row, g.ny, p0, p0 + 2 * strip, wide,
+                [&](int i, int j, int ux, int uy) {
+                    if (d.method == 0)
+                        idw_served<K>(h, sm, ux, uy, k, d.power, d.depth + out(i, j), nullptr);
+                    else
+                        ids_served<K>(h, sm, k, slot(i, j), ids.stride, nullptr);
+                },
+                [&](int i, int j, int qx, int qy, uint64_t* hp) {
+                    if (d.method == 0)
+                        return idw_lone<K>(h, qx, qy, hp, k, d.power, d.depth + out(i, j), nullptr);
+                    return ids_lone<K>(h, qx, qy, hp, k, slot(i, j), ids.stride, nullptr);
+                });
+    }
+}
+
+// The other tiles' items, by threads: IDW in place, kriging ids. An item is a
 // (16 kS) x 8 node patch of one tile; warp w covers its (8 kS) x 4 quarter,
 // each thread a strip of kS nodes along x.
 template <int kS>
@@ -270,7 +338,8 @@ __global__ void __launch_bounds__(kKnnThreads) k_batch_knn(
     const TileDesc* __restrict__ td, int T, const int64_t* __restrict__ item_off, int64_t items,
     unsigned long long* __restrict__ ctr, const int4* __restrict__ orig,
     const int4* __restrict__ rec, const int* __restrict__ cell_start, const int* __restrict__ sat,
-    int* __restrict__ wide) {
+    int* __restrict__ wide, const int* __restrict__ rest) {
+    if (*(volatile const int*)rest == 0) return;
     __shared__ uint64_t heap[32 * kKnnThreads];
     __shared__ long long s_item;
     __shared__ int s_tile;
@@ -287,6 +356,7 @@ __global__ void __launch_bounds__(kKnnThreads) k_batch_knn(
         __syncthreads();
         if (item >= items) break;
         const TileDesc& d = td[t];
+        if (d.patch) continue;
         const HashView h = tile_view(d, orig, rec, cell_start, sat);
         const GridView g = d.g;
         const int gx = (g.nx + 16 * kS - 1) / (16 * kS);
@@ -359,15 +429,16 @@ __global__ void __launch_bounds__(Geo<K>::THREADS, Geo<K>::BLOCKS) k_batch_solve
                 s_k = d.k;
                 s_depth = d.depth;
                 s_var = d.var;
-                s_ids = IdsView{d.ids, 0, 0, 0, 0};
+                s_ids = tile_ids(d);
             }
         }
         __syncthreads();
         const long long item = s_item;
         if (item >= items) break;
-        const int64_t b0 = (item - __ldg(off + s_j)) * nb, nodes = (int64_t)s_g.nx * s_g.ny;
-        const int64_t b1 = min(b0 + nb, (nodes + kSolveSystems - 1) / kSolveSystems);
-        okrige_solve_range<K, kSph, false, false>(s_h, s_g, s_k, s_p, 0, nodes, s_ids, s_depth, s_var, b0, b1,
+        const int64_t nsys = s_ids.stride > 0 ? s_ids.stride : (int64_t)s_g.nx * s_g.ny;
+        const int64_t b0 = (item - __ldg(off + s_j)) * nb;
+        const int64_t b1 = min(b0 + nb, (nsys + kSolveSystems - 1) / kSolveSystems);
+        okrige_solve_range<K, kSph, false, false>(s_h, s_g, s_k, s_p, 0, nsys, s_ids, s_depth, s_var, b0, b1,
                                                   smem, tm);
         __syncthreads();  // the next item overwrites the staged descriptor
     }
@@ -395,8 +466,14 @@ __device__ __forceinline__ void wide_node(const TileDesc& d, const HashView& h, 
             ii = id[i];
         });
     } else {
-        int32_t* o = d.ids + node * d.k;
-        for (int i = 0; i < d.k; ++i) o[i] = i < keff ? id[i] : -1;
+        const IdsView v = tile_ids(d);
+        int32_t* o = v.p + (v.stride > 0 ? node_slot(v, nd.i, nd.j) : node * d.k);
+        for (int i = 0; i < d.k; ++i) {
+            if (v.stride > 0)
+                o[i * v.stride] = i < keff ? -2 - id[i] : -1;
+            else
+                o[i] = i < keff ? id[i] : -1;
+        }
     }
 }
 
@@ -445,9 +522,17 @@ struct bg_batch_s {
         int64_t items;
         int* tiles;       // device: tile indices
         int64_t* off;     // device: item prefix (nt + 1)
-        std::vector<int64_t> nodes;  // host: nodes of each tile of the group
+        std::vector<int64_t> nodes;  // host: systems of each tile of the group
     };
     std::vector<Group> groups;
+    struct KnnGroup {   // tiles of one search size K, with their k-NN items per strip length
+        int K;
+        int nt;
+        int64_t items[3];
+        int* tiles;       // device: tile indices
+        int64_t* off[3];  // device: item prefix (nt + 1)
+    };
+    std::vector<KnnGroup> knn;
     // device buffers (one allocation, carved)
     void* mem = nullptr;
     size_t mem_bytes = 0;
@@ -462,8 +547,9 @@ struct bg_batch_s {
     int* d_sat = nullptr;
     int* d_bsum = nullptr;
     int* d_acc = nullptr;
-    int* d_flags = nullptr;                // [0] wide, [1] status
-    unsigned long long* d_ctr = nullptr;   // item counters: [0] k-NN, [1 + g] solve groups
+    int* d_flags = nullptr;                // [0] wide, [1] status, [2] k-NN by threads
+    unsigned long long* d_ctr = nullptr;   // item counters: [0] k-NN by threads, [1 + g] solve
+                                           // groups, [9 + g] k-NN groups by patches
     int32_t* d_ids = nullptr;
     cudaStream_t stream = nullptr;
     cudaEvent_t ev_in = nullptr, ev_out = nullptr;
@@ -480,13 +566,14 @@ void enqueue_batch(bg_batch_s* b, cudaStream_t st) {
     const int64_t n = b->total_n;
     const int ng = (int)b->groups.size();
     cudaMemsetAsync(b->d_count, 0, (size_t)b->total_cells * 4, st);
-    cudaMemsetAsync(b->d_flags, 0, 2 * sizeof(int), st);
-    cudaMemsetAsync(b->d_ctr, 0, (size_t)(1 + ng) * sizeof(unsigned long long), st);
+    cudaMemsetAsync(b->d_flags, 0, 3 * sizeof(int), st);
+    cudaMemsetAsync(b->d_ctr, 0, 16 * sizeof(unsigned long long), st);
     k_batch_init<<<grid_items(T, 128), 128, 0, st>>>(b->d_acc, T);
     const int cb = grid_items(n, kChunk);
     if (n > 0)
         k_batch_validate<<<cb, kBT, 0, st>>>(b->d_desc, T, b->d_soff, n, b->d_orig, b->d_acc);
-    k_batch_geom<<<grid_items(T, 64), 64, 0, st>>>(b->d_desc, T, b->d_acc, b->ppc, b->d_flags + 1);
+    k_batch_geom<<<grid_items(T, 64), 64, 0, st>>>(b->d_desc, T, b->d_acc, b->ppc, b->d_flags + 1,
+                                                   b->d_flags + 2);
     if (n > 0)
         k_batch_cells<false><<<cb, kBT, 0, st>>>(b->d_desc, T, b->d_soff, n, b->d_orig, b->d_count,
                                                  nullptr);
@@ -500,11 +587,26 @@ void enqueue_batch(bg_batch_s* b, cudaStream_t st) {
     if (b->knn_items > 0) {
         const int si = b->strip == 4 ? 2 : b->strip == 2 ? 1 : 0;
         const int64_t ki = b->knn_items_s[si];
+        for (size_t q = 0; q < b->knn.size(); ++q) {
+            const auto& G = b->knn[q];
+#define BG_KNN_PATCH(KK)                                                                                   \
+    k_batch_knn_patch<KK><<<(unsigned)std::min<int64_t>((G.items[si] + 1) / 2, 152 * KnnWarp<KK>::kBlocksPerSM), \
+                            64, 0, st>>>(b->d_desc, G.tiles, G.nt, G.off[si], G.items[si], b->d_ctr + 9 + q,  \
+                                         b->d_orig, b->d_rec, b->d_cell_start, b->d_sat, b->d_flags, b->strip)
+            switch (G.K) {
+                case 4: BG_KNN_PATCH(4); break;
+                case 8: BG_KNN_PATCH(8); break;
+                case 16: BG_KNN_PATCH(16); break;
+                default: BG_KNN_PATCH(32); break;
+            }
+#undef BG_KNN_PATCH
+            note_launches(1);
+        }
         const unsigned kg = (unsigned)std::min<int64_t>(ki, 152 * 13);
 #define BG_KNN(SS)                                                                               \
     k_batch_knn<SS><<<kg, kKnnThreads, 0, st>>>(b->d_desc, T, b->d_item_off_s[si], ki, b->d_ctr, \
                                                 b->d_orig, b->d_rec, b->d_cell_start, b->d_sat,  \
-                                                b->d_flags)
+                                                b->d_flags, b->d_flags + 2)
         if (b->strip == 4)
             BG_KNN(4);
         else if (b->strip == 2)
@@ -632,6 +734,8 @@ bg_status bg_batch_create(bg_ctx_t ctx, const bg_tile* tiles, int n_tiles, bg_ba
     std::vector<int64_t> soff(n_tiles + 1, 0), item_off(n_tiles + 1, 0);
     std::vector<std::vector<int64_t>> item_off_s(3, std::vector<int64_t>(n_tiles + 1, 0));
     const int Ks[4] = {4, 8, 16, 32};
+    std::vector<std::vector<int>> knn_tiles(4);  // by search size
+    int64_t slot_ids = 0, row_ids = 0;           // ids in the patches and in the rows layout
     std::vector<std::vector<int>> gt(8);  // by system size and variogram model: 2 q + model
     for (int t = 0; t < n_tiles; ++t) {
         const bg_tile& r = tiles[t];
@@ -670,15 +774,20 @@ bg_status bg_batch_create(bg_ctx_t ctx, const bg_tile* tiles, int n_tiles, bg_ba
             item_off_s[si][t + 1] = item_off_s[si][t] + (int64_t)((r.nx + 16 * kStrips[si] - 1) /
                                                                   (16 * kStrips[si])) *
                                                         ((r.ny + 7) / 8);
+        knn_tiles[d.K == 4 ? 0 : d.K == 8 ? 1 : d.K == 16 ? 2 : 3].push_back(t);
         if (r.method == 1) {
-            b->total_ids += m * r.k;
+            d.stride = (int64_t)((r.nx + 7) / 8) * ((r.ny + 3) / 4) * 32;
+            slot_ids += d.stride * r.k;
+            row_ids += m * r.k;
             for (int q = 0; q < 4; ++q)
                 if (Ks[q] == d.K) gt[2 * q + (r.variogram.model != 0)].push_back(t);
         }
     }
     b->knn_items = item_off[n_tiles];
     for (int si = 0; si < 3; ++si) b->knn_items_s[si] = item_off_s[si][n_tiles];
-    // carve one allocation
+    b->total_ids = slot_ids;
+    // carve one allocation (the ids last: the patches layout, rounded up to whole
+    // patches, gives way to the rows layout where the budget has no room for it)
     size_t off = 0;
     auto take = [&](size_t bytes) {
         const size_t o = off;
@@ -699,13 +808,18 @@ bg_status bg_batch_create(bg_ctx_t ctx, const bg_tile* tiles, int n_tiles, bg_ba
     const size_t o_acc = take(32 * (size_t)std::max(1, n_tiles));
     const size_t o_flags = take(16);
     const size_t o_ctr = take(8 * 16);  // [0] k-NN items, [1 + g] solve groups
-    const size_t o_ids = take(4 * (size_t)b->total_ids);
     std::vector<size_t> o_gt, o_go;
     for (int q = 0; q < 8; ++q) {
         o_gt.push_back(take(4 * (gt[q].size() + 1)));
         o_go.push_back(take(8 * (gt[q].size() + 1)));
     }
-    b->mem_bytes = off;
+    size_t o_kt[4], o_ko[4][3];
+    for (int q = 0; q < 4; ++q) {
+        o_kt[q] = take(4 * (knn_tiles[q].size() + 1));
+        for (int si = 0; si < 3; ++si) o_ko[q][si] = take(8 * (knn_tiles[q].size() + 1));
+    }
+    const size_t o_ids = off;
+    b->mem_bytes = o_ids + 4 * (size_t)b->total_ids;
     cudaStream_t st = nullptr;
     int prev = 0;
     cudaGetDevice(&prev);
@@ -717,6 +831,12 @@ bg_status bg_batch_create(bg_ctx_t ctx, const bg_tile* tiles, int n_tiles, bg_ba
     st = b->stream;
     bg_status rc = e == cudaSuccess ? BG_OK : cuda_fail(e, "batch stream");
     if (rc == BG_OK) rc = dalloc(ctx, &b->mem, b->mem_bytes, st);
+    if (rc == BG_ERR_OOM_BUDGET && row_ids < slot_ids) {
+        b->total_ids = row_ids;
+        b->mem_bytes = o_ids + 4 * (size_t)row_ids;
+        for (TileDesc& d : b->host_desc) d.stride = 0;
+        rc = dalloc(ctx, &b->mem, b->mem_bytes, st);
+    }
     if (rc != BG_OK) {
         cudaSetDevice(prev);
         bg_batch_destroy(b);
@@ -742,15 +862,17 @@ bg_status bg_batch_create(bg_ctx_t ctx, const bg_tile* tiles, int n_tiles, bg_ba
         TileDesc& d = b->host_desc[t];
         if (d.method == 1) {
             d.ids = b->d_ids + ids_at;
-            ids_at += (int64_t)d.g.nx * d.g.ny * d.k;
+            ids_at += (d.stride > 0 ? d.stride : (int64_t)d.g.nx * d.g.ny) * d.k;
         }
     }
     for (int q = 0; q < 8; ++q) {
         if (gt[q].empty()) continue;
         bg_batch_s::Group G{Ks[q / 2], q & 1, (int)gt[q].size(), 0, (int*)(base + o_gt[q]),
                             (int64_t*)(base + o_go[q]), {}};
-        for (int t : gt[q])
-            G.nodes.push_back((int64_t)b->host_desc[t].g.nx * b->host_desc[t].g.ny);
+        for (int t : gt[q]) {
+            const TileDesc& d = b->host_desc[t];
+            G.nodes.push_back(d.stride > 0 ? d.stride : (int64_t)d.g.nx * d.g.ny);
+        }
         e = cudaMemcpyAsync(G.tiles, gt[q].data(), 4 * gt[q].size(), cudaMemcpyHostToDevice, st);
         if (e != cudaSuccess) break;
         b->groups.push_back(std::move(G));
@@ -758,6 +880,22 @@ bg_status bg_batch_create(bg_ctx_t ctx, const bg_tile* tiles, int n_tiles, bg_ba
         if (e != cudaSuccess) break;
     }
     if (e == cudaSuccess && set_solve_offsets(b) != BG_OK) e = cudaErrorUnknown;
+    for (int q = 0; q < 4 && e == cudaSuccess; ++q) {
+        const std::vector<int>& kt = knn_tiles[q];
+        if (kt.empty()) continue;
+        bg_batch_s::KnnGroup G{Ks[q], (int)kt.size(), {}, (int*)(base + o_kt[q]), {}};
+        e = cudaMemcpyAsync(G.tiles, kt.data(), 4 * kt.size(), cudaMemcpyHostToDevice, st);
+        for (int si = 0; si < 3 && e == cudaSuccess; ++si) {
+            std::vector<int64_t> ko(kt.size() + 1, 0);
+            for (size_t j = 0; j < kt.size(); ++j)
+                ko[j + 1] = ko[j] + item_off_s[si][kt[j] + 1] - item_off_s[si][kt[j]];
+            G.items[si] = ko.back();
+            G.off[si] = (int64_t*)(base + o_ko[q][si]);
+            e = cudaMemcpyAsync(G.off[si], ko.data(), 8 * ko.size(), cudaMemcpyHostToDevice, st);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // ko goes out of scope
+        }
+        b->knn.push_back(G);
+    }
     for (int si = 0; si < 3 && e == cudaSuccess; ++si)
         e = cudaMemcpyAsync(b->d_item_off_s[si], item_off_s[si].data(), 8 * (n_tiles + 1),
                             cudaMemcpyHostToDevice, st);

@@ -43,28 +43,6 @@ __global__ void __launch_bounds__(128) k_idw(HashView h, GridView g, int k, floa
     knn_strip<128, decltype(emit), true, kLen>(h, g, K, o.i, o.j, hp, flag, emit);
 }
 
-struct KnnFar {
-    int cnt;
-    float d1, dk;
-};
-
-// Per-thread search and IDW of a node that the patch search did not serve
-template <int K>
-__device__ __noinline__ KnnFar knn_lane_idw(const HashView& h, int qx, int qy, uint64_t* hp, int k, float power,
-                                            float* depth, int32_t* nbr) {
-    const int cnt = knn_lane<K>(h, qx, qy, hp);
-    if (cnt < 0) return KnnFar{cnt, 0.0f, 0.0f};
-    const int bits = h.idx_bits, keff = min(cnt, k);
-    const uint64_t mask = (1ull << bits) - 1;
-    *depth = idw_from(h, keff, power, [&](int n, uint64_t& dd, int& ii) {
-        const uint64_t v = hp[n * 32];
-        dd = v >> bits;
-        ii = (int)(v & mask);
-    });
-    if (nbr) emit_ids<32>(nbr, hp, k, keff, mask);
-    return KnnFar{cnt, sqrtf((float)(hp[0] >> bits)), cnt == K ? sqrtf((float)(hp[(K - 1) * 32] >> bits)) : 0.0f};
-}
-
 // The same by patches of 8 x 4 nodes per warp (knn_warp.cuh), a strip of `len`
 // patches along x each; spr strips per patch row.
 template <int K>
@@ -74,48 +52,18 @@ __global__ void __launch_bounds__(64, KnnWarp<K>::kBlocksPerSM) k_idw_patch(Hash
                                                   int len, int spr) {
     __shared__ typename KnnWarp<K>::Smem smem[2];
     typename KnnWarp<K>::Smem& sm = smem[threadIdx.x >> 5];
-    const int lane = threadIdx.x & 31;
     const unsigned w = blockIdx.x * 2 + (threadIdx.x >> 5);
     const int py = (int)(w / (unsigned)spr), p0 = (int)(w % (unsigned)spr) * len;
     if (py * 4 >= g.ny) return;
-    const int j = py * 4 + (lane >> 3), qy = g.y0 + j * g.cell + g.cell / 2;
-    KnnChain ch;
-    for (int p = p0; p < p0 + len && p * 8 < g.nx; ++p) {
-        const int i = p * 8 + (lane & 7), qx = g.x0 + i * g.cell + g.cell / 2;
-        const bool on = i < g.nx && j < g.ny;
-        const int ox = g.x0 + p * 8 * g.cell + g.cell / 2, oy = g.y0 + py * 4 * g.cell + g.cell / 2;
-        uint32_t base;
-        const float r = knn_first_radius<K>(h, ch, on, qx, qy, 8.0f * (float)g.cell, base);
-        const unsigned served = knn_patch<K>(h, sm, on, qx, qy, ox, oy, r, base, ch);
-        const int64_t node = (int64_t)j * g.nx + i;
-        int32_t* o = nbr ? nbr + node * k : nullptr;
-        if (served >> lane & 1) {
-            const int ux = qx - ox, uy = qy - oy;
-            depth[node] = idw_sum(k, power, [&](int n, float& d, float& z) {
-                const uint32_t q = sm.buf[n * 32 + lane] & kPlaceMask;
-                const int4 c = sm.st[q];
-                const int dx = c.x - ux, dy = c.y - uy;
-                d = __int2float_rn(dx * dx + dy * dy);
-                z = __int_as_float(__ldg(&h.rec[sm.pos[q]].z));
-            });
-            if (o)
-                for (int n = 0; n < k; ++n) o[n] = __ldg(&h.rec[sm.pos[sm.buf[n * 32 + lane] & kPlaceMask]].w);
-        }
-        if (served != kFull) {
-            __syncwarp();
-            if (on && !(served >> lane & 1)) {
-                ch.dk = -1.0f;
-                const KnnFar f = knn_lane_idw<K>(h, qx, qy, reinterpret_cast<uint64_t*>(sm.buf) + lane, k, power,
-                                                 depth + node, o);
-                if (f.cnt < 0) *flag = 1;  // the wide pass picks this node up
-                if (f.cnt == K) {
-                    ch.d1 = f.d1;
-                    ch.dk = f.dk;
-                }
-            }
-        }
-        __syncwarp();
-    }
+    auto out = [&](int i, int j) { return (int64_t)j * g.nx + i; };
+    knn_patch_row<K>(
+        h, g, sm, py * 4, g.ny, p0, p0 + len, flag,
+        [&](int i, int j, int ux, int uy) {
+            idw_served<K>(h, sm, ux, uy, k, power, depth + out(i, j), nbr ? nbr + out(i, j) * k : nullptr);
+        },
+        [&](int i, int j, int qx, int qy, uint64_t* hp) {
+            return idw_lone<K>(h, qx, qy, hp, k, power, depth + out(i, j), nbr ? nbr + out(i, j) * k : nullptr);
+        });
 }
 
 // Wide-key pass over the nodes the packed pass could not take; it returns at

@@ -19,6 +19,7 @@
 
 #include "bg_internal.h"
 #include "knn.cuh"
+#include "knn_warp.cuh"
 
 namespace bg {
 
@@ -97,6 +98,40 @@ __device__ __forceinline__ float idw_from(const HashView& h, int keff, float pow
         d = idw_d2f(d2);
         z = __int_as_float(__ldg(zb + 4 * (int64_t)i));
     });
+}
+
+// IDW of a node that the patch search served (knn_patch_row), and its k
+// neighbours' upload indices to nbr, if any.
+template <int K>
+__device__ __forceinline__ void idw_served(const HashView& h, const typename KnnWarp<K>::Smem& sm, int ux, int uy,
+                                           int k, float power, float* depth, int32_t* nbr) {
+    const uint32_t* col = sm.buf + (threadIdx.x & 31);
+    *depth = idw_sum(k, power, [&](int n, float& d, float& z) {
+        const uint32_t q = col[n * 32] & kPlaceMask;
+        const int4 c = sm.st[q];
+        const int dx = c.x - ux, dy = c.y - uy;
+        d = __int2float_rn(dx * dx + dy * dy);
+        z = __int_as_float(__ldg(&h.rec[sm.pos[q]].z));
+    });
+    if (nbr)
+        for (int n = 0; n < k; ++n) nbr[n] = __ldg(&h.rec[sm.pos[col[n * 32] & kPlaceMask]].w);
+}
+// The same of a node that it did not serve: a per-thread search, out of the way
+// of the patch search's code.
+template <int K>
+__device__ __noinline__ KnnFar idw_lone(const HashView& h, int qx, int qy, uint64_t* hp, int k, float power,
+                                        float* depth, int32_t* nbr) {
+    const int cnt = knn_lane<K>(h, qx, qy, hp);
+    if (cnt < 0) return KnnFar{cnt, 0.0f, 0.0f};
+    const int bits = h.idx_bits, keff = min(cnt, k);
+    const uint64_t mask = (1ull << bits) - 1;
+    *depth = idw_from(h, keff, power, [&](int n, uint64_t& dd, int& ii) {
+        const uint64_t v = hp[n * 32];
+        dd = v >> bits;
+        ii = (int)(v & mask);
+    });
+    if (nbr) emit_ids<32>(nbr, hp, k, keff, mask);
+    return knn_far<K>(h, hp, cnt);
 }
 
 template <int K, bool kWide>

@@ -476,18 +476,70 @@ __device__ __noinline__ int knn_lane(const HashView& h, int qx, int qy, uint64_t
     }
 }
 
+// What a lane's own search (a node that knn_patch did not serve) found.
+struct KnnFar {
+    int cnt;       // neighbours; -1: left to the wide pass
+    float d1, dk;  // distances to the nearest and the K-th (cnt == K)
+};
+template <int K>
+__device__ __forceinline__ KnnFar knn_far(const HashView& h, const uint64_t* hp, int cnt) {
+    return KnnFar{cnt, cnt > 0 ? sqrtf((float)(hp[0] >> h.idx_bits)) : 0.0f,
+                  cnt == K ? sqrtf((float)(hp[(K - 1) * 32] >> h.idx_bits)) : 0.0f};
+}
+
+// Patches p0 .. p1 - 1 of the patch row whose first grid row is jb (rows below
+// j1), one after another by one warp. served(i, j, ux, uy) runs for the nodes
+// that the patch search served (knn_patch: the lane's buffer column and the
+// staged list hold the neighbours), lone(i, j, qx, qy, heap) for the others:
+// it searches by itself (knn_lane) and returns a KnnFar.
+template <int K, class Served, class Lone>
+__device__ __forceinline__ void knn_patch_row(const HashView& h, const GridView& g, typename KnnWarp<K>::Smem& sm,
+                                              int jb, int j1, int p0, int p1, int* flag, Served served, Lone lone) {
+    const int lane = threadIdx.x & 31;
+    const int j = jb + (lane >> 3), qy = g.y0 + j * g.cell + g.cell / 2;
+    KnnChain ch;
+#pragma unroll 1
+    for (int p = p0; p < p1 && p * 8 < g.nx; ++p) {
+        const int i = p * 8 + (lane & 7), qx = g.x0 + i * g.cell + g.cell / 2;
+        const bool on = i < g.nx && j < j1;
+        const int ox = g.x0 + p * 8 * g.cell + g.cell / 2, oy = g.y0 + jb * g.cell + g.cell / 2;
+        uint32_t base;
+        const float r = knn_first_radius<K>(h, ch, on, qx, qy, 8.0f * (float)g.cell, base);
+        const unsigned m = knn_patch<K>(h, sm, on, qx, qy, ox, oy, r, base, ch);
+        if (m >> lane & 1) served(i, j, qx - ox, qy - oy);
+        if (m != kFull) {
+            __syncwarp();
+            if (on && !(m >> lane & 1)) {
+                ch.dk = -1.0f;
+                const KnnFar f = lone(i, j, qx, qy, reinterpret_cast<uint64_t*>(sm.buf) + lane);
+                if (f.cnt < 0) *flag = 1;  // the wide pass picks this node up
+                if (f.cnt == K) {
+                    ch.d1 = f.d1;
+                    ch.dk = f.dk;
+                }
+            }
+        }
+        __syncwarp();
+    }
+}
+
 // Is the patch search the better one for a grid of this cell over this hash?
 // Its staged list must hold the soundings of a patch and the radius around it
 // (0.8 of it at the mean density; a patch of more costs a try and then its
 // lanes' own searches), and the bounds of its 32-bit arithmetic must hold.
 template <int K>
+__host__ __device__ inline bool knn_patch_fits(int64_t n_valid, int32_t ncx, int32_t ncy, int32_t hash_cell,
+                                               int32_t cell, int nx, int ny) {
+    if (n_valid <= 2 * K || cell >= 1400 || hash_cell > 6000) return false;
+    const double rho = (double)n_valid / ((double)ncx * (double)ncy * (double)hash_cell * (double)hash_cell);
+    const double r = sqrt(KnnWarp<K>::kArea * K / (3.14159265 * rho)), c = hash_cell;
+    const double w = (nx < 8 ? nx - 1 : 7) * (double)cell + 2 * r + c;
+    const double t = (ny < 4 ? ny - 1 : 3) * (double)cell + 2 * r + c;
+    return w * t * rho < 0.8 * KnnWarp<K>::CAP;
+}
+template <int K>
 inline bool knn_patch_fits(const bg_soundings_info& info, int32_t cell, int nx, int ny) {
-    const double cells = (double)info.ncx * (double)info.ncy;
-    if (info.n_valid <= 2 * K || cells <= 0) return false;
-    const double rho = (double)info.n_valid / (cells * (double)info.cell_cm * (double)info.cell_cm);
-    const double r = std::sqrt(KnnWarp<K>::kArea * K / (3.14159265 * rho)), c = info.cell_cm;
-    const double w = std::min(7, nx - 1) * (double)cell + 2 * r + c, hgt = std::min(3, ny - 1) * (double)cell + 2 * r + c;
-    return w * hgt * rho < 0.8 * KnnWarp<K>::CAP && cell < 1400 && info.cell_cm <= 6000;
+    return knn_patch_fits<K>(info.n_valid, info.ncx, info.ncy, info.cell_cm, cell, nx, ny);
 }
 
 // Patches a warp takes along x: strips carry the radius from patch to patch,

@@ -3,7 +3,6 @@
 // is in okrige_dev.cuh; see there for the formulation.
 #include <algorithm>
 
-#include "knn_warp.cuh"
 #include "okrige_dev.cuh"
 
 namespace bg {
@@ -61,50 +60,18 @@ __global__ void __launch_bounds__(64, KnnWarp<K>::kBlocksPerSM) k_knn_ids_patch(
                                                                                 int len, int spr) {
     __shared__ typename KnnWarp<K>::Smem smem[2];
     typename KnnWarp<K>::Smem& sm = smem[threadIdx.x >> 5];
-    const int lane = threadIdx.x & 31;
     const unsigned w = blockIdx.x * 2 + (threadIdx.x >> 5);
     const int py = (int)(w / (unsigned)spr), p0 = (int)(w % (unsigned)spr) * len;
-    const int jb = ids.j0 + py * 4, j = jb + (lane >> 3), qy = g.y0 + j * g.cell + g.cell / 2;
+    const int jb = ids.j0 + py * 4;
     if (jb >= ids.j1) return;
-    KnnChain ch;
-    for (int p = p0; p < p0 + len && p < ids.pnx; ++p) {
-        const int i = p * 8 + (lane & 7), qx = g.x0 + i * g.cell + g.cell / 2;
-        const bool on = i < g.nx && j < ids.j1;
-        const int ox = g.x0 + p * 8 * g.cell + g.cell / 2, oy = g.y0 + jb * g.cell + g.cell / 2;
-        uint32_t base;
-        const float r = knn_first_radius<K>(h, ch, on, qx, qy, 8.0f * (float)g.cell, base);
-        const unsigned served = knn_patch<K>(h, sm, on, qx, qy, ox, oy, r, base, ch);
-        int32_t* o = ids.p + ((int64_t)py * ids.pnx + p) * 32 + lane;
-        if (served >> lane & 1) {
-#pragma unroll 8
-            for (int n = 0; n < k; ++n) o[n * ids.stride] = sm.pos[sm.buf[n * 32 + lane] & kPlaceMask];
-            if (nbr)
-                for (int n = 0; n < k; ++n)
-                    nbr[((int64_t)j * g.nx + i) * k + n] =
-                        __ldg(&h.rec[sm.pos[sm.buf[n * 32 + lane] & kPlaceMask]].w);
-        }
-        if (served != kFull) {
-            __syncwarp();
-            if (on && !(served >> lane & 1)) {
-                ch.dk = -1.0f;
-                uint64_t* hp = reinterpret_cast<uint64_t*>(sm.buf) + lane;
-                const int cnt = knn_lane<K>(h, qx, qy, hp);
-                if (cnt < 0) *flag = 1;  // the wide pass picks this node up
-                const uint64_t mask = (1ull << h.idx_bits) - 1;
-#pragma unroll 1
-                for (int n = 0; n < k; ++n) {
-                    const int u = n < cnt ? (int)(hp[n * 32] & mask) : -1;
-                    o[n * ids.stride] = u < 0 ? -1 : -2 - u;
-                    if (nbr) nbr[((int64_t)j * g.nx + i) * k + n] = u;
-                }
-                if (cnt == K) {
-                    ch.d1 = sqrtf((float)(hp[0] >> h.idx_bits));
-                    ch.dk = sqrtf((float)(hp[(K - 1) * 32] >> h.idx_bits));
-                }
-            }
-        }
-        __syncwarp();
-    }
+    auto slot = [&](int i, int j) { return ids.p + node_slot(ids, i, j); };
+    auto list = [&](int i, int j) { return nbr ? nbr + ((int64_t)j * g.nx + i) * k : nullptr; };
+    knn_patch_row<K>(
+        h, g, sm, jb, ids.j1, p0, p0 + len, flag,
+        [&](int i, int j, int, int) { ids_served<K>(h, sm, k, slot(i, j), ids.stride, list(i, j)); },
+        [&](int i, int j, int qx, int qy, uint64_t* hp) {
+            return ids_lone<K>(h, qx, qy, hp, k, slot(i, j), ids.stride, list(i, j));
+        });
 }
 
 template <int K>

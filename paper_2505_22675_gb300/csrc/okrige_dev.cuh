@@ -66,6 +66,7 @@
 #include "bg_internal.h"
 #include "idw_dev.cuh"
 #include "knn.cuh"
+#include "knn_warp.cuh"
 
 namespace bg {
 
@@ -254,6 +255,38 @@ __device__ __forceinline__ bool slot_node(const IdsView& v, const GridView& g, i
 }
 __device__ __forceinline__ int64_t node_slot(const IdsView& v, int i, int j) {
     return ((int64_t)((j - v.j0) >> 2) * v.pnx + (i >> 3)) * 32 + ((j - v.j0) & 3) * 8 + (i & 7);
+}
+
+// The k ids of a node that the patch search served, to slot `o` of the patches
+// layout (or, with stride 0, to o[0 .. k) as upload indices), and as upload
+// indices to nbr, if any.
+template <int K>
+__device__ __forceinline__ void ids_served(const HashView& h, const typename KnnWarp<K>::Smem& sm, int k, int32_t* o,
+                                           int64_t stride, int32_t* nbr) {
+    const uint32_t* col = sm.buf + (threadIdx.x & 31);
+    if (stride > 0) {
+#pragma unroll 8
+        for (int n = 0; n < k; ++n) o[n * stride] = sm.pos[col[n * 32] & kPlaceMask];
+    } else {
+        nbr = o;
+    }
+    if (nbr)
+        for (int n = 0; n < k; ++n) nbr[n] = __ldg(&h.rec[sm.pos[col[n * 32] & kPlaceMask]].w);
+}
+// The same of a node that it did not serve, by a per-thread search.
+template <int K>
+__device__ __noinline__ KnnFar ids_lone(const HashView& h, int qx, int qy, uint64_t* hp, int k, int32_t* o,
+                                        int64_t stride, int32_t* nbr) {
+    const int cnt = knn_lane<K>(h, qx, qy, hp);
+    if (cnt < 0) return KnnFar{cnt, 0.0f, 0.0f};
+    const uint64_t mask = (1ull << h.idx_bits) - 1;
+    if (stride == 0) nbr = o;
+    for (int n = 0; n < k; ++n) {
+        const int u = n < cnt ? (int)(hp[n * 32] & mask) : -1;
+        if (stride > 0) o[n * stride] = u < 0 ? -1 : -2 - u;
+        if (nbr) nbr[n] = u;
+    }
+    return knn_far<K>(h, hp, cnt);
 }
 
 // Wide-key neighbour ids of one grid node whose table bound does not fit the
