@@ -178,9 +178,8 @@ __device__ __forceinline__ IdsView tile_ids(const TileDesc& d) {
     return IdsView{d.ids, d.patch ? d.stride : 0, (d.g.nx + 7) / 8, 0, d.g.ny};
 }
 
-// rest: set when some tile's k-NN goes by threads instead of patches
 __global__ void k_batch_geom(TileDesc* td, int T, const int* __restrict__ acc, float ppc,
-                             int* __restrict__ status, int* __restrict__ rest) {
+                             int* __restrict__ status) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= T) return;
     TileDesc& d = td[t];
@@ -194,7 +193,6 @@ __global__ void k_batch_geom(TileDesc* td, int T, const int* __restrict__ acc, f
     if (h.n_valid == 0) {
         h.ncx = h.ncy = 0;
         d.patch = 0;
-        *rest = 1;
         return;
     }
     const int64_t W = (int64_t)a[2] - a[0] + 1, H = (int64_t)a[3] - a[1] + 1;
@@ -218,7 +216,31 @@ __global__ void k_batch_geom(TileDesc* td, int T, const int* __restrict__ acc, f
     int r = (int)ceil((sqrt((double)kq / per_cell) - 1.0) * 0.5);
     h.r0 = max(0, min(r, max(h.ncx, h.ncy)));
     d.patch = tile_patch_fits(h, d.g, d.K);
-    if (!d.patch) *rest = 1;
+}
+
+// Item prefix of the tiles whose k-NN goes by threads (the others have none
+// there): rest[t] from the prefix of all tiles. One block. Draining all items
+// and passing over the others' took 2.5 ms for 233,000 items.
+__global__ void __launch_bounds__(kBT) k_batch_rest(const TileDesc* __restrict__ td, int T,
+                                                    const int64_t* __restrict__ off, int64_t* __restrict__ rest) {
+    __shared__ long long sm[kBT];
+    long long carry = 0;
+    for (int base = 0; base < T; base += kBT) {
+        const int t = base + threadIdx.x;
+        const long long v = t < T && !td[t].patch ? off[t + 1] - off[t] : 0;
+        sm[threadIdx.x] = v;
+        __syncthreads();
+        for (int o = 1; o < kBT; o <<= 1) {
+            const long long u = (int)threadIdx.x >= o ? sm[threadIdx.x - o] : 0;
+            __syncthreads();
+            sm[threadIdx.x] += u;
+            __syncthreads();
+        }
+        if (t < T) rest[t] = carry + sm[threadIdx.x] - v;
+        carry += sm[kBT - 1];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) rest[T] = carry;
 }
 
 // 3a/3c. histogram and scatter over the concatenated soundings
@@ -335,11 +357,12 @@ __global__ void __launch_bounds__(64, KnnWarp<K>::kBlocksPerSM) k_batch_knn_patc
 // each thread a strip of kS nodes along x.
 template <int kS>
 __global__ void __launch_bounds__(kKnnThreads) k_batch_knn(
-    const TileDesc* __restrict__ td, int T, const int64_t* __restrict__ item_off, int64_t items,
+    const TileDesc* __restrict__ td, int T, const int64_t* __restrict__ item_off,
     unsigned long long* __restrict__ ctr, const int4* __restrict__ orig,
     const int4* __restrict__ rec, const int* __restrict__ cell_start, const int* __restrict__ sat,
-    int* __restrict__ wide, const int* __restrict__ rest) {
-    if (*(volatile const int*)rest == 0) return;
+    int* __restrict__ wide) {
+    const int64_t items = item_off[T];
+    if (items == 0) return;
     __shared__ uint64_t heap[32 * kKnnThreads];
     __shared__ long long s_item;
     __shared__ int s_tile;
@@ -356,7 +379,6 @@ __global__ void __launch_bounds__(kKnnThreads) k_batch_knn(
         __syncthreads();
         if (item >= items) break;
         const TileDesc& d = td[t];
-        if (d.patch) continue;
         const HashView h = tile_view(d, orig, rec, cell_start, sat);
         const GridView g = d.g;
         const int gx = (g.nx + 16 * kS - 1) / (16 * kS);
@@ -540,6 +562,7 @@ struct bg_batch_s {
     int64_t* d_soff = nullptr;
     int64_t* d_item_off = nullptr;         // 16 x 8 patch prefix (wide pass)
     int64_t* d_item_off_s[3] = {nullptr, nullptr, nullptr};  // k-NN item prefix per strip
+    int64_t* d_rest_off = nullptr;         // k-NN item prefix of the tiles that go by threads
     int4* d_orig = nullptr;
     int4* d_rec = nullptr;
     int* d_cell_start = nullptr;
@@ -547,7 +570,7 @@ struct bg_batch_s {
     int* d_sat = nullptr;
     int* d_bsum = nullptr;
     int* d_acc = nullptr;
-    int* d_flags = nullptr;                // [0] wide, [1] status, [2] k-NN by threads
+    int* d_flags = nullptr;                // [0] wide, [1] status
     unsigned long long* d_ctr = nullptr;   // item counters: [0] k-NN by threads, [1 + g] solve
                                            // groups, [9 + g] k-NN groups by patches
     int32_t* d_ids = nullptr;
@@ -566,14 +589,13 @@ void enqueue_batch(bg_batch_s* b, cudaStream_t st) {
     const int64_t n = b->total_n;
     const int ng = (int)b->groups.size();
     cudaMemsetAsync(b->d_count, 0, (size_t)b->total_cells * 4, st);
-    cudaMemsetAsync(b->d_flags, 0, 3 * sizeof(int), st);
+    cudaMemsetAsync(b->d_flags, 0, 2 * sizeof(int), st);
     cudaMemsetAsync(b->d_ctr, 0, 16 * sizeof(unsigned long long), st);
     k_batch_init<<<grid_items(T, 128), 128, 0, st>>>(b->d_acc, T);
     const int cb = grid_items(n, kChunk);
     if (n > 0)
         k_batch_validate<<<cb, kBT, 0, st>>>(b->d_desc, T, b->d_soff, n, b->d_orig, b->d_acc);
-    k_batch_geom<<<grid_items(T, 64), 64, 0, st>>>(b->d_desc, T, b->d_acc, b->ppc, b->d_flags + 1,
-                                                   b->d_flags + 2);
+    k_batch_geom<<<grid_items(T, 64), 64, 0, st>>>(b->d_desc, T, b->d_acc, b->ppc, b->d_flags + 1);
     if (n > 0)
         k_batch_cells<false><<<cb, kBT, 0, st>>>(b->d_desc, T, b->d_soff, n, b->d_orig, b->d_count,
                                                  nullptr);
@@ -603,10 +625,10 @@ void enqueue_batch(bg_batch_s* b, cudaStream_t st) {
             note_launches(1);
         }
         const unsigned kg = (unsigned)std::min<int64_t>(ki, 152 * 13);
+        k_batch_rest<<<1, kBT, 0, st>>>(b->d_desc, T, b->d_item_off_s[si], b->d_rest_off);
 #define BG_KNN(SS)                                                                               \
-    k_batch_knn<SS><<<kg, kKnnThreads, 0, st>>>(b->d_desc, T, b->d_item_off_s[si], ki, b->d_ctr, \
-                                                b->d_orig, b->d_rec, b->d_cell_start, b->d_sat,  \
-                                                b->d_flags, b->d_flags + 2)
+    k_batch_knn<SS><<<kg, kKnnThreads, 0, st>>>(b->d_desc, T, b->d_rest_off, b->d_ctr, b->d_orig, \
+                                                b->d_rec, b->d_cell_start, b->d_sat, b->d_flags)
         if (b->strip == 4)
             BG_KNN(4);
         else if (b->strip == 2)
@@ -617,7 +639,7 @@ void enqueue_batch(bg_batch_s* b, cudaStream_t st) {
         k_batch_wide<<<(unsigned)std::min<int64_t>(b->knn_items, 152 * 4), kItemThreads, 0, st>>>(
             b->d_desc, T, b->d_item_off, b->knn_items, b->d_orig, b->d_rec, b->d_cell_start,
             b->d_sat, b->d_flags);
-        note_launches(2);
+        note_launches(3);
     }
     for (int gi = 0; gi < ng; ++gi) {
         const auto& G = b->groups[gi];
@@ -799,6 +821,7 @@ bg_status bg_batch_create(bg_ctx_t ctx, const bg_tile* tiles, int n_tiles, bg_ba
     const size_t o_item = take(8 * (n_tiles + 1));
     size_t o_item_s[3];
     for (int si = 0; si < 3; ++si) o_item_s[si] = take(8 * (n_tiles + 1));
+    const size_t o_rest = take(8 * (n_tiles + 1));
     const size_t o_orig = take(16 * (size_t)b->total_n);
     const size_t o_rec = take(16 * (size_t)b->total_n);
     const size_t o_cs = take(4 * (size_t)(b->total_cells + 1));
@@ -847,6 +870,7 @@ bg_status bg_batch_create(bg_ctx_t ctx, const bg_tile* tiles, int n_tiles, bg_ba
     b->d_soff = (int64_t*)(base + o_soff);
     b->d_item_off = (int64_t*)(base + o_item);
     for (int si = 0; si < 3; ++si) b->d_item_off_s[si] = (int64_t*)(base + o_item_s[si]);
+    b->d_rest_off = (int64_t*)(base + o_rest);
     b->d_orig = (int4*)(base + o_orig);
     b->d_rec = (int4*)(base + o_rec);
     b->d_cell_start = (int*)(base + o_cs);

@@ -114,6 +114,16 @@ __device__ __forceinline__ void append_if(int d, int lim, uint32_t key, uint32_t
         : "r"(d), "r"(lim), "r"(key)
         : "memory");
 }
+__device__ __forceinline__ void append_if(uint32_t d, uint32_t lim, uint32_t key, uint32_t& a) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.le.u32 p, %1, %2;\n\t"
+        "@p st.shared.b32 [%0], %3;\n\t"
+        "@p add.u32 %0, %0, 128;\n\t}"
+        : "+r"(a)
+        : "r"(d), "r"(lim), "r"(key)
+        : "memory");
+}
 
 // What a lane carries from one patch of its strip to the next.
 struct KnnChain {
@@ -178,8 +188,14 @@ __device__ __forceinline__ float knn_first_radius(const HashView& h, const KnnCh
 }
 
 __device__ __forceinline__ int4 staged(int x, int y, int place) {
-    return make_int4(x, y, x * x + y * y, place);
+    return make_int4(x, y, (int)((uint32_t)(x * x) + (uint32_t)(y * y)), place);
 }
+
+// Bounds of the 32-bit squared distances, in cm: radius, patch and hash cell. The
+// far scan takes only records within a lane's radius along each axis (d < 2^32);
+// the near scan, in signed sums of the staged squares, needs every staged record
+// within kNearMax of every node along each axis.
+constexpr int kRadiusMax = 46000, kPatchMax = 10000, kCellMax = 30000, kNearMax = 26000;
 
 // Stage every record within the radii of the patch (r of the lanes with `on`,
 // at (ux, uy) relative to the corner (ox, oy)); returns their number, or -1 when
@@ -263,7 +279,7 @@ __device__ __forceinline__ int knn_stage(const HashView& h, typename KnnWarp<K>:
         T += total;
     }
     // to a whole step, beyond any radius
-    if (lane < W::kStep && T + lane < W::CAP) sm.st[T + lane] = staged(28000, 0, 0);
+    if (lane < W::kStep && T + lane < W::CAP) sm.st[T + lane] = make_int4(60000, 0, 0x7fff0000, 0);
     __syncwarp();
     return T;
 }
@@ -277,21 +293,21 @@ __device__ __forceinline__ bool key_less(const Smem& sm, const int4* rec, int ux
     return da != db ? da < db : __ldg(&rec[sm.pos[ca.w]].w) < __ldg(&rec[sm.pos[cb.w]].w);
 }
 
-// An appended word as the key it sorts by. Without shifted distances (sh = 0)
-// the scan appends 512 (d - u^2) + place, modulo 2^32, and the bias 512 (u^2 -
-// base) makes it 512 (d - base) + place; with them it appends the key itself.
-__device__ __forceinline__ uint32_t sort_key(uint32_t v, uint32_t bias, int sh) { return sh == 0 ? v + bias : v; }
+// An appended word as the key it sorts by. The near scan appends 512 (d - u^2) +
+// place, modulo 2^32, and the bias 512 (u^2 - base) makes it 512 (d - base) +
+// place; the far scan appends the key itself (bias 0).
+__device__ __forceinline__ uint32_t sort_key(uint32_t v, uint32_t bias) { return v + bias; }
 
 // The K nearest of a lane's cnt appended keys in exact order to the front of its
 // buffer column, where keys alone cannot tell (dk: the K-th key). Out of the
 // way of the search's straight path.
 template <class Smem>
 __device__ __noinline__ void knn_order_exact(Smem& sm, const int4* rec, int ux, int uy, int cnt, uint32_t dk,
-                                             uint32_t bias, int sh) {
+                                             uint32_t bias) {
     uint32_t* buf = sm.buf + (threadIdx.x & 31);
     int m = 0;
     for (int i = 0; i < cnt; ++i) {
-        const uint32_t v = sort_key(buf[i * 32], bias, sh);
+        const uint32_t v = sort_key(buf[i * 32], bias);
         if ((v >> kPlaceBits) > (dk >> kPlaceBits)) continue;
         int j = m++;
         for (; j > 0; --j) {
@@ -318,11 +334,8 @@ __device__ __forceinline__ unsigned knn_patch(const HashView& h, typename KnnWar
     constexpr int B = W::B, S = W::kStep;
     const int lane = threadIdx.x & 31;
     const int ux = qx - ox, uy = qy - oy;
-    // signed 32-bit squared distances: radius, patch and cell side are bounded
-    // (knn_patch_fits), so that a staged record lies within 26,000 cm of a node
-    // along each axis
-    constexpr float kMaxR = 10000.0f;
-    on = on && r >= 0.0f && r < kMaxR && (unsigned)ux < 10000u && (unsigned)uy < 10000u;
+    constexpr float kMaxR = (float)kRadiusMax;
+    on = on && r >= 0.0f && r < kMaxR && (unsigned)ux < (unsigned)kPatchMax && (unsigned)uy < (unsigned)kPatchMax;
     if (!__any_sync(kFull, on)) return 0;
     uint32_t* buf = sm.buf + lane;
     const uint32_t buf0 = (uint32_t)__cvta_generic_to_shared(buf);
@@ -330,7 +343,7 @@ __device__ __forceinline__ unsigned knn_patch(const HashView& h, typename KnnWar
     const float d0 = sqrtf((float)base);
     const int u2 = on ? ux * ux + uy * uy : 0;
     const uint32_t mx2 = on ? -2 * ux : 0, my2 = on ? -2 * uy : 0;  // (sums wrap, results fit)
-    const uint32_t bias = ((uint32_t)u2 - base) << kPlaceBits;
+    uint32_t bias = 0;
     int T = 0, cnt = 0, sh = 0;
     bool stage = true, grew = false, shrunk = false;
 #pragma unroll 1
@@ -338,30 +351,42 @@ __device__ __forceinline__ unsigned knn_patch(const HashView& h, typename KnnWar
         if (stage) T = knn_stage<K>(h, sm, on, ux, uy, ox, oy, r);
         bool few = false, over = false;
         if (T >= 0) {
-            // d = |c|^2 - 2 c u + |u|^2, compared less |u|^2
-            const int tau = (int)(r * r), lim = on ? tau - u2 : INT_MIN;
+            // d = |c|^2 - 2 c u + |u|^2
+            const int tau = (int)(r * r);
             // low bits of a distance that the key does not hold (none up to 28.9 m)
             sh = max(0, kPlaceBits - __clz(__reduce_max_sync(kFull, on ? (uint32_t)tau - base : 0u)));
             uint32_t at = buf0;
-            auto scan = [&](auto key_of) {
+            auto scan = [&](auto append) {
 #pragma unroll 1
                 for (int i = 0; i < T; i += S) {  // the buffer has S rows of slack
 #pragma unroll
                     for (int u = 0; u < S; ++u) {
                         const int4 c = sm.st[i + u];
-                        const int d = (int)((uint32_t)c.x * mx2 + ((uint32_t)c.y * my2 + (uint32_t)c.z));
-                        append_if(d, lim, key_of(d, c.w), at);
+                        append((uint32_t)c.x * mx2 + ((uint32_t)c.y * my2 + (uint32_t)c.z), (uint32_t)c.w, c);
                     }
                     over |= at > buf0 + B * 128;
                     at = min(at, buf0 + B * 128);
                 }
             };
-            if (sh == 0)
-                scan([&](int d, int place) { return (uint32_t)d * (1u << kPlaceBits) + (uint32_t)place; });
-            else
-                scan([&](int d, int place) {
-                    return (((uint32_t)(d + u2) - base) >> sh) * (1u << kPlaceBits) + (uint32_t)place;
+            // (near: every staged record within kNearMax)
+            if (__all_sync(kFull, !on || r + (float)(kPatchMax + h.cs) < (float)kNearMax) && sh == 0) {
+                // compared less |u|^2, in signed arithmetic
+                const int lim = on ? tau - u2 : INT_MIN;
+                bias = ((uint32_t)u2 - base) << kPlaceBits;
+                scan([&](uint32_t d, uint32_t place, const int4&) {
+                    append_if((int)d, lim, d * (1u << kPlaceBits) + place, at);
                 });
+            } else {
+                const uint32_t lim = on ? (uint32_t)tau - base : 0u;
+                const int R = on ? __float2int_ru(r) : 0;
+                bias = 0;
+                scan([&](uint32_t, uint32_t place, const int4& c) {
+                    const int dx = c.x - ux, dy = c.y - uy;
+                    const bool box = (unsigned)(dx + R) <= 2u * R && (unsigned)(dy + R) <= 2u * R;
+                    const uint32_t e = (uint32_t)dx * dx + (uint32_t)dy * dy - base;
+                    append_if(box ? e : kNoKey, lim, (e >> sh) * (1u << kPlaceBits) + place, at);
+                });
+            }
             cnt = (int)(at - buf0) / 128;
             over = on && over;
             few = on && !over && cnt < K;
@@ -399,7 +424,7 @@ __device__ __forceinline__ unsigned knn_patch(const HashView& h, typename KnnWar
 #pragma unroll
         for (int i = 0; i < K; ++i) {
             const uint32_t w = buf[(b * K + i) * 32];
-            v[i] = b * K + i < cnt ? sort_key(w, bias, sh) : kNoKey;
+            v[i] = b * K + i < cnt ? sort_key(w, bias) : kNoKey;
         }
         net_sort<0, K>(v);
         if (b == 0) {
@@ -439,7 +464,7 @@ __device__ __forceinline__ unsigned knn_patch(const HashView& h, typename KnnWar
         pair |= eq;
     }
     if (on && lng) {
-        knn_order_exact(sm, h.rec, ux, uy, cnt, key[K - 1], bias, sh);
+        knn_order_exact(sm, h.rec, ux, uy, cnt, key[K - 1], bias);
     } else {
 #pragma unroll
         for (int i = 0; i < K; ++i) buf[i * 32] = key[i];
@@ -530,12 +555,12 @@ __device__ __forceinline__ void knn_patch_row(const HashView& h, const GridView&
 template <int K>
 __host__ __device__ inline bool knn_patch_fits(int64_t n_valid, int32_t ncx, int32_t ncy, int32_t hash_cell,
                                                int32_t cell, int nx, int ny) {
-    if (n_valid <= 2 * K || cell >= 1400 || hash_cell > 6000) return false;
+    if (n_valid <= 2 * K || cell >= kPatchMax / 7 || hash_cell > kCellMax) return false;
     const double rho = (double)n_valid / ((double)ncx * (double)ncy * (double)hash_cell * (double)hash_cell);
     const double r = sqrt(KnnWarp<K>::kArea * K / (3.14159265 * rho)), c = hash_cell;
     const double w = (nx < 8 ? nx - 1 : 7) * (double)cell + 2 * r + c;
     const double t = (ny < 4 ? ny - 1 : 3) * (double)cell + 2 * r + c;
-    return w * t * rho < 0.8 * KnnWarp<K>::CAP;
+    return w * t * rho < 0.8 * KnnWarp<K>::CAP && 1.3 * r < kRadiusMax;
 }
 template <int K>
 inline bool knn_patch_fits(const bg_soundings_info& info, int32_t cell, int nx, int ny) {

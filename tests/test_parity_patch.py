@@ -53,6 +53,7 @@ CASES = {
     "near_capacity": (lambda: _uniform(6, 12_000, 4_000, 4_000), GridSpec(0, 0, 100, 40, 39)),
     "gap": (lambda: _gap(7), GridSpec(0, 0, 200, 150, 105)),
     "sparse": (lambda: _uniform(8, 3_000, 200_000, 200_000), GridSpec(50_000, 50_000, 600, 45, 33)),
+    "very_sparse": (lambda: _uniform(11, 2_000, 400_000, 400_000), GridSpec(100_000, 150_000, 1_300, 31, 27)),
     "cluster": (lambda: _cluster(9), GridSpec(0, 0, 150, 40, 40)),
     "few": (lambda: _uniform(10, 40, 6_000, 6_000), GridSpec(0, 0, 300, 20, 20)),
 }
