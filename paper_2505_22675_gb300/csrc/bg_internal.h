@@ -214,12 +214,13 @@ bg_status build_hash_in_arena(const int32_t* x, const int32_t* y, const float* z
 int scan_blocks(int64_t n);
 void launch_excl_scan(const int* in, int64_t n, int* out, int* out2, int* bsum, cudaStream_t st);
 
-// IDW launch with a caller-provided device flag (one int) instead of an allocated one.
+// IDW launch with a caller-provided device flag (one int; NULL: allocated when
+// the per-thread search needs one).
 bg_status launch_idw_with_flag(const bg_soundings_s* s, const GridView& g, int k, float power,
                                float* depth, int32_t* nbr, int* d_flag, cudaStream_t st);
 
-// Each call allocates (stream-ordered) a one-int flag that tells the wide-key
-// pass whether the packed pass left nodes for it.
+// The per-thread search allocates (stream-ordered) a one-int flag that tells the
+// wide-key pass whether the packed pass left nodes for it.
 bg_status launch_idw(const bg_soundings_s* s, const GridView& g, int k, float power,
                      float* depth, int32_t* nbr, cudaStream_t st);
 // fz: NULL, or an IDW to write in the same pass (fz->k <= k)

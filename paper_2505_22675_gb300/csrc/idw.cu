@@ -81,20 +81,29 @@ __global__ void __launch_bounds__(128) k_idw_wide(HashView h, GridView g, int k,
                           patch_node((int)(b % gx), (int)(b / gx), warp, lane), nullptr);
 }
 
+// d_flag: one int, or NULL to allocate one where it is needed
 template <int K>
 bg_status launch_k(const bg_soundings_s* s, const HashView& h, const GridView& g, int k, float power,
                    float* depth, int32_t* nbr, int* d_flag, cudaStream_t st, bg_ctx_s* prof_ctx) {
     const int64_t nb = (int64_t)((g.nx + 15) / 16) * ((g.ny + 7) / 8);
     const int len = strip_len_for((int64_t)g.nx * g.ny);
     const int64_t nbs = (int64_t)((g.nx + 16 * len - 1) / (16 * len)) * ((g.ny + 7) / 8);
-    BG_CUDA(cudaMemsetAsync(d_flag, 0, sizeof(int), st));
-    {
+    const int pnx = (g.nx + 7) / 8, pny = (g.ny + 3) / 4;
+    const int plen = patch_strip_len((int64_t)pnx * pny), spr = (pnx + plen - 1) / plen;
+    const bool wide = !packed_always(h, g);  // (an empty hash too: its nodes need no search)
+    int* own = nullptr;
+    if (!wide) d_flag = nullptr;
+    if (wide && !d_flag) {
+        const bg_status rc = dalloc(s->ctx, (void**)&own, sizeof(int), st);
+        if (rc != BG_OK) return rc;
+        d_flag = own;
+    }
+    cudaError_t e = wide ? cudaMemsetAsync(d_flag, 0, sizeof(int), st) : cudaSuccess;
+    if (e == cudaSuccess) {
         ProfScope ps(prof_ctx, kProfIdw, (int64_t)g.nx * g.ny, st);
-        const int pnx = (g.nx + 7) / 8, pny = (g.ny + 3) / 4;
-        const int plen = patch_strip_len((int64_t)pnx * pny), spr = (pnx + plen - 1) / plen;
         if (knn_patch_fits<K>(s->info, g.cell, g.nx, g.ny) && (int64_t)spr * pny < ((int64_t)1 << 31))
-            k_idw_patch<K><<<(unsigned)(((int64_t)spr * pny + 1) / 2), 64, 0, st>>>(
-                h, g, k, power, depth, nbr, d_flag, plen, spr);
+            k_idw_patch<K><<<(unsigned)(((int64_t)spr * pny + 1) / 2), 64, 0, st>>>(h, g, k, power, depth, nbr, d_flag,
+                                                                                   plen, spr);
         else if (len == 1)
             k_idw<K, 1><<<(unsigned)nbs, 128, 0, st>>>(h, g, k, power, depth, nbr, d_flag);
         else if (len == 2)
@@ -102,11 +111,12 @@ bg_status launch_k(const bg_soundings_s* s, const HashView& h, const GridView& g
         else
             k_idw<K, 4><<<(unsigned)nbs, 128, 0, st>>>(h, g, k, power, depth, nbr, d_flag);
     }
-    k_idw_wide<K><<<(unsigned)std::min<int64_t>(nb, 152 * 4), 128, 0, st>>>(h, g, k, power, depth,
-                                                                        nbr, d_flag);
-    note_launches(2);
-    BG_CUDA(cudaGetLastError());
-    return BG_OK;
+    if (wide && e == cudaSuccess)
+        k_idw_wide<K><<<(unsigned)std::min<int64_t>(nb, 152 * 4), 128, 0, st>>>(h, g, k, power, depth, nbr, d_flag);
+    note_launches(wide ? 2 : 1);
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (own) dfree(s->ctx, own, sizeof(int), st);
+    return e == cudaSuccess ? BG_OK : cuda_fail(e, "IDW launch");
 }
 
 // Query points: kLen consecutive points per thread (knn_chain).
@@ -203,20 +213,7 @@ bg_status launch_idw_points(const bg_soundings_s* s, const PointsView& q, int k,
 
 bg_status launch_idw(const bg_soundings_s* s, const GridView& g, int k, float power,
                      float* depth, int32_t* nbr, cudaStream_t st) {
-    HashView h = s->h;
-    const int K = k <= 4 ? 4 : k <= 8 ? 8 : k <= 16 ? 16 : 32;
-    h.r0 = start_halfwidth(s, K);
-    int* flag = nullptr;
-    bg_status rc = dalloc(s->ctx, (void**)&flag, sizeof(int), st);
-    if (rc != BG_OK) return rc;
-    switch (K) {
-        case 4: rc = launch_k<4>(s, h, g, k, power, depth, nbr, flag, st, s->ctx); break;
-        case 8: rc = launch_k<8>(s, h, g, k, power, depth, nbr, flag, st, s->ctx); break;
-        case 16: rc = launch_k<16>(s, h, g, k, power, depth, nbr, flag, st, s->ctx); break;
-        default: rc = launch_k<32>(s, h, g, k, power, depth, nbr, flag, st, s->ctx); break;
-    }
-    dfree(s->ctx, flag, sizeof(int), st);
-    return rc;
+    return launch_idw_with_flag(s, g, k, power, depth, nbr, nullptr, st);
 }
 
 bg_status launch_idw_with_flag(const bg_soundings_s* s, const GridView& g, int k, float power,

@@ -485,8 +485,7 @@ __device__ __forceinline__ unsigned knn_patch(const HashView& h, typename KnnWar
 
 // The per-thread search of one node for a lane that knn_patch did not serve:
 // its packed keys sorted ascending in hp (stride 32); returns their number, or
-// -1 when the bound does not fit a packed key (left to the wide pass). Lanes
-// run it on their own. Out of the way of the patch search's code.
+// -1 when the bound does not fit a packed key. Lanes run it on their own. Out of the way of the patch search's code.
 template <int K>
 __device__ __noinline__ int knn_lane(const HashView& h, int qx, int qy, uint64_t* hp) {
     const Bound b = knn_bound_rt(h, qx, qy, K);
@@ -516,7 +515,8 @@ __device__ __forceinline__ KnnFar knn_far(const HashView& h, const uint64_t* hp,
 // j1), one after another by one warp. served(i, j, ux, uy) runs for the nodes
 // that the patch search served (knn_patch: the lane's buffer column and the
 // staged list hold the neighbours), lone(i, j, qx, qy, heap) for the others:
-// it searches by itself (knn_lane) and returns a KnnFar.
+// it searches by itself (knn_lane) and returns a KnnFar. flag is set when a node
+// is left to the wide pass (NULL: packed_always holds).
 template <int K, class Served, class Lone>
 __device__ __forceinline__ void knn_patch_row(const HashView& h, const GridView& g, typename KnnWarp<K>::Smem& sm,
                                               int jb, int j1, int p0, int p1, int* flag, Served served, Lone lone) {
@@ -537,7 +537,7 @@ __device__ __forceinline__ void knn_patch_row(const HashView& h, const GridView&
             if (on && !(m >> lane & 1)) {
                 ch.dk = -1.0f;
                 const KnnFar f = lone(i, j, qx, qy, reinterpret_cast<uint64_t*>(sm.buf) + lane);
-                if (f.cnt < 0) *flag = 1;  // the wide pass picks this node up
+                if (f.cnt < 0 && flag) *flag = 1;
                 if (f.cnt == K) {
                     ch.d1 = f.d1;
                     ch.dk = f.dk;
@@ -565,6 +565,17 @@ __host__ __device__ inline bool knn_patch_fits(int64_t n_valid, int32_t ncx, int
 template <int K>
 inline bool knn_patch_fits(const bg_soundings_info& info, int32_t cell, int nx, int ny) {
     return knn_patch_fits<K>(info.n_valid, info.ncx, info.ncy, info.cell_cm, cell, nx, ny);
+}
+
+// Does every bound over this grid fit a packed key? The farthest corner of the
+// hash from any node bounds them all. Then no node is left to a wide pass, which
+// saves a small call its flag and a launch (5 of 60 us).
+inline bool packed_always(const HashView& h, const GridView& g) {
+    const double x0 = (double)g.x0 + g.cell / 2, x1 = x0 + (double)(g.nx - 1) * g.cell;
+    const double y0 = (double)g.y0 + g.cell / 2, y1 = y0 + (double)(g.ny - 1) * g.cell;
+    const double hx1 = (double)h.hx0 + (double)h.ncx * h.cs, hy1 = (double)h.hy0 + (double)h.ncy * h.cs;
+    const double dx = std::max(hx1 - x0, x1 - h.hx0), dy = std::max(hy1 - y0, y1 - h.hy0);
+    return 1.001 * (dx * dx + dy * dy) + 2.0 < std::ldexp(1.0, 64 - h.idx_bits);
 }
 
 // Patches a warp takes along x: strips carry the radius from patch to patch,

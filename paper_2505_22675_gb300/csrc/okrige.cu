@@ -51,20 +51,22 @@ __global__ void __launch_bounds__(64) k_knn_ids(HashView h, GridView g, int k, i
 }
 
 // The same by patches of 8 x 4 nodes per warp (knn_warp.cuh), a strip of `len`
-// patches along x each, spr strips per patch row, into the patch layout (and,
-// as upload indices, to nbr [node][k], if any).
+// patches along x each, spr strips per patch row, into either layout (and, as
+// upload indices, to nbr [node][k], if any).
 template <int K>
 __global__ void __launch_bounds__(64, KnnWarp<K>::kBlocksPerSM) k_knn_ids_patch(HashView h, GridView g, int k,
                                                                                 IdsView ids, int32_t* __restrict__ nbr,
-                                                                                int* __restrict__ flag,
-                                                                                int len, int spr) {
+                                                                                int* __restrict__ flag, int len,
+                                                                                int spr) {
     __shared__ typename KnnWarp<K>::Smem smem[2];
     typename KnnWarp<K>::Smem& sm = smem[threadIdx.x >> 5];
     const unsigned w = blockIdx.x * 2 + (threadIdx.x >> 5);
     const int py = (int)(w / (unsigned)spr), p0 = (int)(w % (unsigned)spr) * len;
     const int jb = ids.j0 + py * 4;
     if (jb >= ids.j1) return;
-    auto slot = [&](int i, int j) { return ids.p + node_slot(ids, i, j); };
+    auto slot = [&](int i, int j) {
+        return ids.p + (ids.stride > 0 ? node_slot(ids, i, j) : ((int64_t)(j - ids.j0) * g.nx + i) * k);
+    };
     auto list = [&](int i, int j) { return nbr ? nbr + ((int64_t)j * g.nx + i) * k : nullptr; };
     knn_patch_row<K>(
         h, g, sm, jb, ids.j1, p0, p0 + len, flag,
@@ -142,29 +144,25 @@ bg_status launch_k(const bg_soundings_s* snd, const HashView& h, const GridView&
                    float* var, int32_t* nbr, bg_ctx_s* ctx, cudaStream_t st, const IdwFuse* fz,
                    const HostOut* ho) {
     using Gm = Geo<K>;
-    // grid rows per chunk: the id buffer stays near 1 GiB. The patch layout rounds
-    // the rows up to whole patches; where the search by patches does not serve, or
-    // the budget has no room for that, the rows layout does, in nbr_out itself
-    // when the caller passed it (then whole).
+    // grid rows per chunk: the id buffer stays near 1 GiB. Without a budget the
+    // patch search writes the patches layout (rounded up to whole patches). Under
+    // a budget it does so only where that needs no more memory, else the rows
+    // layout, in nbr_out itself when the caller passed it (then whole), as the
+    // per-thread search always does.
     const int64_t most = std::max<int64_t>(8, ((((int64_t)1 << 28) / ((int64_t)k * g.nx)) / 8) * 8);
     int64_t rows = std::min<int64_t>(g.ny, most);
     const size_t flag_bytes = 256;
     const int pnx = (g.nx + 7) / 8;
-    bool patches = knn_patch_fits<K>(snd->info, g.cell, g.nx, g.ny);
     const int64_t slots = (int64_t)pnx * ((rows + 3) / 4) * 32;
-    size_t id_bytes = patches ? (size_t)slots * k * sizeof(int32_t) : 0;
+    const bool patches = knn_patch_fits<K>(snd->info, g.cell, g.nx, g.ny);
+    const bool slot_ids = patches && (ctx->budget == 0 || (!nbr && slots <= rows * g.nx));
+    if (!slot_ids && nbr) rows = g.ny;
+    const size_t id_bytes =
+        slot_ids ? (size_t)slots * k * sizeof(int32_t) : nbr ? 0 : (size_t)rows * g.nx * k * sizeof(int32_t);
     void* scratch = nullptr;
-    bg_status rc = BG_OK;
-    if (patches) {
-        rc = dalloc(ctx, &scratch, flag_bytes + id_bytes, st);
-        patches = rc == BG_OK;
-    }
-    if (!patches) {
-        if (nbr) rows = g.ny;
-        id_bytes = nbr ? 0 : (size_t)rows * g.nx * k * sizeof(int32_t);
-        rc = dalloc(ctx, &scratch, flag_bytes + id_bytes, st);
-        if (rc != BG_OK) return rc;
-    }
+    bg_status rc = dalloc(ctx, &scratch, flag_bytes + id_bytes, st);
+    if (rc != BG_OK) return rc;
+    const bool wide = !packed_always(h, g);
     int* flag = (int*)scratch;
     const int gx = (g.nx + 15) / 16;
     cudaError_t ea = cudaFuncSetAttribute(k_okrige_solve<K, kSph, false>,
@@ -183,22 +181,22 @@ bg_status launch_k(const bg_soundings_s* snd, const HashView& h, const GridView&
         const int len = strip_len_for((j1 - j0) * (int64_t)g.nx);
         const int64_t nbs = (int64_t)((g.nx + 16 * len - 1) / (16 * len)) * ((j1 - j0 + 3) / 4);
         int32_t* chunk_ids =
-            nbr && !patches ? nbr + j0 * g.nx * k : (int32_t*)((char*)scratch + flag_bytes);
-        cudaError_t e = cudaMemsetAsync(flag, 0, sizeof(int), st);
+            nbr && !slot_ids ? nbr + j0 * g.nx * k : (int32_t*)((char*)scratch + flag_bytes);
+        cudaError_t e = wide ? cudaMemsetAsync(flag, 0, sizeof(int), st) : cudaSuccess;
         if (e != cudaSuccess) {
             rc = cuda_fail(e, "memset");
             break;
         }
         const int64_t nodes = (j1 - j0) * g.nx;
         const int pny = (int)((j1 - j0 + 3) / 4);
-        const IdsView ids{chunk_ids, patches ? slots : 0, pnx, (int)j0, (int)j1};
-        const int64_t nsys = patches ? (int64_t)pnx * pny * 32 : nodes;
+        const IdsView ids{chunk_ids, slot_ids ? slots : 0, pnx, (int)j0, (int)j1};
+        const int64_t nsys = slot_ids ? (int64_t)pnx * pny * 32 : nodes;
         {
             ProfScope ps(ctx, kProfKnnIds, nodes, st);
             const int plen = patch_strip_len((int64_t)pnx * pny), spr = (pnx + plen - 1) / plen;
             if (patches)
-                k_knn_ids_patch<K><<<(unsigned)(((int64_t)spr * pny + 1) / 2), 64, 0, st>>>(h, g, k, ids, nbr, flag,
-                                                                                           plen, spr);
+                k_knn_ids_patch<K><<<(unsigned)(((int64_t)spr * pny + 1) / 2), 64, 0, st>>>(
+                    h, g, k, ids, slot_ids ? nbr : nullptr, flag, plen, spr);
             else if (len == 1)
                 k_knn_ids<K, 1><<<(unsigned)nbs, 64, 0, st>>>(h, g, k, (int)j0, (int)j1, chunk_ids, flag);
             else if (len == 2)
@@ -206,8 +204,10 @@ bg_status launch_k(const bg_soundings_s* snd, const HashView& h, const GridView&
             else
                 k_knn_ids<K, 4><<<(unsigned)nbs, 64, 0, st>>>(h, g, k, (int)j0, (int)j1, chunk_ids, flag);
         }
-        k_knn_ids_wide<K><<<(unsigned)std::min<int64_t>(nb, 152 * 4), 128, 0, st>>>(
-            h, g, k, ids, patches ? nbr : nullptr, flag);
+        if (wide)
+            k_knn_ids_wide<K><<<(unsigned)std::min<int64_t>(nb, 152 * 4), 128, 0, st>>>(
+                h, g, k, ids, slot_ids ? nbr : nullptr, flag);
+        note_launches(wide ? 3 : 2);
         const int64_t batches = (nsys + kSolveSystems - 1) / kSolveSystems;
         const int per = solve_batches_per_block<K>(batches);
         const unsigned sb = (unsigned)((batches + per - 1) / per);
@@ -225,7 +225,6 @@ bg_status launch_k(const bg_soundings_s* snd, const HashView& h, const GridView&
                 k_okrige_solve<K, kSph, false><<<sb, Gm::THREADS, Gm::SMEM, st>>>(
                     h, g, k, p, j0 * g.nx, nsys, ids, depth, var, IdwFuse{}, per);
         }
-        note_launches(3);
         e = cudaGetLastError();
         if (e != cudaSuccess) {
             rc = cuda_fail(e, "kriging launch");

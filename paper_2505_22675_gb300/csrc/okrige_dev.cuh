@@ -278,9 +278,9 @@ template <int K>
 __device__ __noinline__ KnnFar ids_lone(const HashView& h, int qx, int qy, uint64_t* hp, int k, int32_t* o,
                                         int64_t stride, int32_t* nbr) {
     const int cnt = knn_lane<K>(h, qx, qy, hp);
-    if (cnt < 0) return KnnFar{cnt, 0.0f, 0.0f};
     const uint64_t mask = (1ull << h.idx_bits) - 1;
     if (stride == 0) nbr = o;
+    if (cnt < 0) return KnnFar{cnt, 0.0f, 0.0f};
     for (int n = 0; n < k; ++n) {
         const int u = n < cnt ? (int)(hp[n * 32] & mask) : -1;
         if (stride > 0) o[n * stride] = u < 0 ? -1 : -2 - u;
@@ -480,9 +480,14 @@ struct TileVgm {
     float c0s, cs;
     __device__ __forceinline__ explicit TileVgm(const ScaledVgm& v)
         : kinv2(dup2(v.kinv2)), k2(dup2(v.k2)), k3(dup2(v.k3)), c0s(v.c0s), cs(v.cs) {}
-    __device__ __forceinline__ u64 entry(u64 xr, u64 yr, u64 zr, float xc, float yc, float zc) const {
+    // (h / a)^2; an entry from it. A tile takes these one after the other for all
+    // its entries: the chain of one entry (a square root in it) is far longer
+    // than its issue slots.
+    __device__ __forceinline__ u64 dist(u64 xr, u64 yr, float xc, float yc) const {
         const u64 dx = sub2(xr, dup2(xc)), dy = sub2(yr, dup2(yc));
-        const u64 t2 = mul2(fma2(dx, dx, mul2(dy, dy)), kinv2);  // (h / a)^2
+        return mul2(fma2(dx, dx, mul2(dy, dy)), kinv2);
+    }
+    __device__ __forceinline__ u64 entry(u64 t2, u64 zr, float zc) const {
         float ta, tb;
         upk2(t2, ta, tb);
         if constexpr (kSph) {
@@ -594,11 +599,13 @@ __device__ __forceinline__ void assemble_off(const Lane<K>& ln, const TileVgm<kS
     ln.floats(Gm::Y, J, yc);
     ln.floats(Gm::Z, J, zc);
 #pragma unroll
-    for (int c = 0; c < 8; ++c) {
-        const float z = zc[c] + vg.c0s;
+    for (int c = 0; c < 8; ++c)
 #pragma unroll
-        for (int u = 0; u < 2; ++u) t[u][c] = vg.entry(xr[u], yr[u], zr[u], xc[c], yc[c], z);
-    }
+        for (int u = 0; u < 2; ++u) t[u][c] = vg.dist(xr[u], yr[u], xc[c], yc[c]);
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+#pragma unroll
+        for (int u = 0; u < 2; ++u) t[u][c] = vg.entry(t[u][c], zr[u], zc[c] + vg.c0s);
     if (!full) {
 #pragma unroll
         for (int u = 0; u < 2; ++u)
@@ -622,7 +629,9 @@ __device__ __forceinline__ void assemble_diag(const Lane<K>& ln, const TileVgm<k
     const u64 xr = pk2(xc[2 * p], xc[2 * p + 1]), yr = pk2(yc[2 * p], yc[2 * p + 1]),
               zr = pk2(zc[2 * p], zc[2 * p + 1]);
 #pragma unroll
-    for (int c = 0; c < 2 * p + 2; ++c) t[c] = vg.entry(xr, yr, zr, xc[c], yc[c], zc[c] + vg.c0s);
+    for (int c = 0; c < 2 * p + 2; ++c) t[c] = vg.dist(xr, yr, xc[c], yc[c]);
+#pragma unroll
+    for (int c = 0; c < 2 * p + 2; ++c) t[c] = vg.entry(t[c], zr, zc[c] + vg.c0s);
     // -A[c][c] = -2 Gamma_c0
     float d0 = 2.0f * zc[2 * p], d1 = 2.0f * zc[2 * p + 1];
     if (!full) {
@@ -653,8 +662,7 @@ __device__ __forceinline__ void assemble_one(const Lane<K>& ln, const TileVgm<kS
 #pragma unroll
         for (int p = c / 2; p < Gm::P; ++p) {
             float a, b;
-            upk2(vg.entry(xr[p], yr[p], zr[p], lane2(xr[c / 2], c & 1), lane2(yr[c / 2], c & 1), z),
-                 a, b);
+            upk2(vg.entry(vg.dist(xr[p], yr[p], lane2(xr[c / 2], c & 1), lane2(yr[c / 2], c & 1)), zr[p], z), a, b);
             t[c][p] = pk2(2 * p + 1 < ke ? a : 0.0f, 2 * p + 2 < ke ? b : 0.0f);
         }
         const float d = c + 1 < ke ? 2.0f * z0 : -sa;  // -A[c][c] = -2 Gamma_c0

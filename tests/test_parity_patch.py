@@ -96,3 +96,24 @@ def test_kriging_systems_of_every_size(name, model, nugget, k):
     assert np.array_equal(nb, ridx)
     assert_okrige(d, v, rd, rv, nugget)
     assert np.array_equal(d, d2) and np.array_equal(v, v2)
+
+
+@pytest.mark.parametrize("n,w,h,hint", [(4_096, 8_000, 8_000, 0), (4_097, 8_000, 8_000, 0), (9_000, 900_000, 40, 0),
+                                        (9_000, 40, 900_000, 0), (30_000, 20_000, 20_000, 87), (30_000, 20_000, 20_000, 80),
+                                        (262_144, 60_000, 60_000, 400), (262_145, 60_000, 60_000, 400),
+                                        (5_000, 3, 3, 0)])
+def test_hash_builds_of_every_size(n, w, h, hint):
+    """One block, one cluster and the multi-kernel build: sizes on both sides of
+    their limits (soundings, cells), one row or column of cells, a single cell."""
+    x, y, z = _uniform(n, n, w, h)
+    z[::97] = np.nan
+    g = GridSpec(w // 3, h // 3, 2 * max(1, max(w, h) // 400), 9, 5)
+    lib = Lib(x, y, z, g, cell_hint=hint)
+    try:
+        d, nb = lib.idw(8, 2.0)
+    finally:
+        lib.close()
+    qx, qy = oracle.grid_nodes(g.x0_cm, g.y0_cm, g.cell_cm, g.nx, g.ny)
+    ref, ridx = oracle.idw(x, y, z, qx, qy, 8, 2.0, want_idx=True)
+    assert np.array_equal(nb, ridx)
+    assert_idw(d, ref)
