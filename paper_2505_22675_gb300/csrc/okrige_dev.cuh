@@ -425,6 +425,36 @@ __device__ __forceinline__ float ll_to_float(long long v) {
     return fmaf((float)hi, 4294967296.0f, (float)lo);
 }
 
+// 1 - exp(-sqrt(ta)), 1 - exp(-sqrt(tb)), for the tiles of the exponential
+// model: an FMA-bound assembly, so two entries share each instruction, which a
+// library call for each cannot (k = 12, 170,163 systems: solve 104 -> 79 us).
+// Argument reduction of Cody and Waite: sqrt(ta) = n ln 2 + r, |r| <= ln 2 / 2;
+// 1 - exp(-r) = r - r^2 q(r), q of degree 4 by interpolation at the Chebyshev
+// nodes of that interval (off by 6e-8 at most); then (1 - s) + s (1 - exp(-r)),
+// s = 2^-n, which does not cancel at short range. Within 1.01 ulp (2e6 draws in
+// each of six intervals); past 25 the result is 1 in any case.
+__device__ __forceinline__ u64 one_minus_exp2(float ta, float tb) {
+    const u64 magic = dup2(12582912.0f);  // 1.5 * 2^23: the low bits of a sum hold the integer
+    const auto root = [](float t2) {
+        float c;
+        asm("min.NaN.f32 %0, %1, 0f441C4000;" : "=f"(c) : "f"(t2));  // 625
+        return sqrt_approx(c);
+    };
+    const u64 t = pk2(root(ta), root(tb));
+    const u64 y = fma2(t, dup2(1.44269504f), magic);
+    const u64 r = fma2(sub2(y, magic), dup2(-0.693147181f), t);
+    u64 q = fma2(dup2(-0.00139261840f), r, dup2(0.00836317893f));
+    q = fma2(q, r, dup2(-0.0416665561f));
+    q = fma2(q, r, dup2(0.166665763f));
+    q = fma2(q, r, dup2(-0.5f));
+    const u64 m = fma2(mul2(r, r), q, r);
+    const auto pow2 = [](float v) {  // 2^-n
+        return __uint_as_float(0x3f800000u - (__float_as_uint(v) << 23));
+    };
+    const u64 s = pk2(pow2(lo2(y)), pow2(hi2(y)));
+    return fma2(s, m, sub2(dup2(1.0f), s));
+}
+
 // The tile function of the assembly: -A for two rows at once, in the
 // fixed-point scale. -A[r][c] = gamma(r, c) - Gamma_r0 - Gamma_c0; the records
 // hold zr = -Gamma_r0, and zc comes in as c0 - Gamma_c0 (all scaled).
@@ -451,8 +481,7 @@ struct TileVgm {
             const u64 in = fma2(k2, pk2(ta, tb), k3);
             return fma2(pk2(sqrt_approx(ta), sqrt_approx(tb)), in, add2(zr, dup2(zc)));
         } else {
-            const u64 e = pk2(-expm1f(-sqrt_approx(ta)), -expm1f(-sqrt_approx(tb)));
-            return fma2(dup2(cs), e, add2(zr, dup2(zc)));
+            return fma2(dup2(cs), one_minus_exp2(ta, tb), add2(zr, dup2(zc)));
         }
     }
 };
@@ -533,7 +562,7 @@ constexpr __host__ __device__ int place_of(int r) { return r < 2 ? r : r < 6 ? r
 
 // Row pairs p[0], p[1] (tile row I) of -A's tile columns: t[u][c] is pair
 // p[u] of column c of tile (I, J). Rows past the last neighbour have no
-// coupling (off-diagonal zero).
+// coupling (off-diagonal zero); full: every neighbour of the warp's systems real.
 template <int K, bool kSph>
 __device__ __forceinline__ void assemble_off(const Lane<K>& ln, const TileVgm<kSph>& vg, int I,
                                              int J, const int (&pr)[2], int ke, bool full,
@@ -570,6 +599,9 @@ __device__ __forceinline__ void assemble_off(const Lane<K>& ln, const TileVgm<kS
                 const int r = I * 8 + 2 * pr[u];
                 t[u][c] = pk2(r + 1 < ke ? a : 0.0f, r + 2 < ke ? b : 0.0f);
             }
+    } else if (I + 1 == Gm::NB && pr[1] == 3) {  // a whole system lacks only its last row
+#pragma unroll
+        for (int c = 0; c < 8; ++c) t[1][c] = pk2(lo2(t[1][c]), 0.0f);
     }
 }
 
@@ -595,6 +627,10 @@ __device__ __forceinline__ void assemble_diag(const Lane<K>& ln, const TileVgm<k
         d1 = real1 ? d1 : -sa;
 #pragma unroll
         for (int c = 0; c < 2 * p + 2; ++c) t[c] = pk2(real0 ? lo2(t[c]) : 0.0f, real1 ? hi2(t[c]) : 0.0f);
+    } else if (p == 3 && J + 1 == Geo<K>::NB) {  // a whole system lacks only its last row
+        d1 = -sa;
+#pragma unroll
+        for (int c = 0; c < 2 * p + 2; ++c) t[c] = pk2(lo2(t[c]), 0.0f);
     }
     t[2 * p] = pk2(d0, hi2(t[2 * p]));
     t[2 * p + 1] = pk2(lo2(t[2 * p + 1]), d1);
@@ -968,7 +1004,6 @@ __device__ __forceinline__ void okrige_solve_range(const HashView& h, const Grid
         pair_sync();  // every record is there
         // every row but the last (row K - 1 has no neighbour) real, in the whole warp
         const bool full = __all_sync(kFull, ke == K);
-        auto row_full = [&](int I) { return full && I + 1 < NB; };
         const int pr[2] = {hh, 3 - hh};  // owned row pairs
         const auto tcol = [&](int I, int J) {  // off-diagonal tile (I, J)
             return tm + (uint32_t)((I * (I - 1) / 2 + J) * Gm::TILE);
@@ -990,8 +1025,8 @@ __device__ __forceinline__ void okrige_solve_range(const HashView& h, const Grid
                     ln.floats(Gm::Y, J, yc);
                     ln.floats(Gm::Z, J, zc);
                     ln.floats(Gm::G0, J, g0);
-                    assemble_diag<K, kSph, p0>(ln, vg, J, ke, sa, row_full(J), xc, yc, zc, t0);
-                    assemble_diag<K, kSph, p1>(ln, vg, J, ke, sa, row_full(J), xc, yc, zc, t1);
+                    assemble_diag<K, kSph, p0>(ln, vg, J, ke, sa, full, xc, yc, zc, t0);
+                    assemble_diag<K, kSph, p1>(ln, vg, J, ke, sa, full, xc, yc, zc, t1);
                     nv[0] = pk2(minus_b(8 * J + 2 * p0, zc[2 * p0], g0[2 * p0]),
                                 minus_b(8 * J + 2 * p0 + 1, zc[2 * p0 + 1], g0[2 * p0 + 1]));
                     nv[1] = pk2(minus_b(8 * J + 2 * p1, zc[2 * p1], g0[2 * p1]),
@@ -1113,7 +1148,7 @@ __device__ __forceinline__ void okrige_solve_range(const HashView& h, const Grid
 #pragma unroll 1
             for (int I = J + 1; I < NB; ++I) {
                 u64 t[2][8];
-                assemble_off<K, kSph>(ln, vg, I, J, pr, ke, row_full(I), t);
+                assemble_off<K, kSph>(ln, vg, I, J, pr, ke, full, t);
                 if constexpr (K == 16) {  // kept for the residual: a = -A' of the off-diagonal tile
 #pragma unroll
                     for (int s = 0; s < 2; ++s) {
@@ -1424,8 +1459,8 @@ __device__ __forceinline__ void okrige_solve_range(const HashView& h, const Grid
                     ln.floats(Gm::Y, I, yc);
                     ln.floats(Gm::Z, I, zc);
                     u64 t0[N0], t1[N1];
-                    assemble_diag<K, kSph, p0>(ln, vg, I, ke, sa, row_full(I), xc, yc, zc, t0);
-                    assemble_diag<K, kSph, p1>(ln, vg, I, ke, sa, row_full(I), xc, yc, zc, t1);
+                    assemble_diag<K, kSph, p0>(ln, vg, I, ke, sa, full, xc, yc, zc, t0);
+                    assemble_diag<K, kSph, p1>(ln, vg, I, ke, sa, full, xc, yc, zc, t1);
                     add_tile([&](int e) { return __float2int_rn(lane2(t0[e / 2], e & 1)); },
                              [&](int e) { return __float2int_rn(lane2(t1[e / 2], e & 1)); });
                 }

@@ -98,6 +98,24 @@ def test_kriging_systems_of_every_size(name, model, nugget, k):
     assert np.array_equal(d, d2) and np.array_equal(v, v2)
 
 
+@pytest.mark.parametrize("k", [12, 32])
+@pytest.mark.parametrize("range_m", [0.05, 2.0, 30.0, 400.0])
+def test_exponential_model_at_every_range(range_m, k):
+    """Entries from h / a << 1 (where 1 - exp(-h / a) cancels) to h / a > 25
+    (where it is 1)."""
+    from gpu_util import assert_okrige
+    x, y, z = _uniform(3, 3_000, 8_000, 8_000)
+    g = GridSpec(0, 0, 200, 41, 37)
+    lib = Lib(x, y, z, g)
+    try:
+        d, v, _ = lib.okrige(k, 1, 0.25, 100.0, range_m, want_nbr=False)
+    finally:
+        lib.close()
+    qx, qy = oracle.grid_nodes(g.x0_cm, g.y0_cm, g.cell_cm, g.nx, g.ny)
+    rd, rv = oracle.okrige(x, y, z, qx, qy, k, 1, 0.25, 100.0, range_m)[:2]
+    assert_okrige(d, v, rd, rv, 0.25)
+
+
 @pytest.mark.parametrize("n,w,h,hint", [(4_096, 8_000, 8_000, 0), (4_097, 8_000, 8_000, 0), (9_000, 900_000, 40, 0),
                                         (9_000, 40, 900_000, 0), (30_000, 20_000, 20_000, 87), (30_000, 20_000, 20_000, 80),
                                         (262_144, 60_000, 60_000, 400), (262_145, 60_000, 60_000, 400),
