@@ -68,6 +68,19 @@ __global__ void __launch_bounds__(64, KnnWarp<K>::kBlocksPerSM) k_idw_patch(Hash
 
 // Wide-key pass over the nodes the packed pass could not take; it returns at
 // once when the packed pass flagged none.
+// G lanes per query: points of a list or nodes of a grid.
+template <int G, class Queries>
+__global__ void __launch_bounds__(32 * kQueryWarps) k_idw_query(HashView h, Queries q, int64_t m, int k, float power,
+                                                               float* __restrict__ depth,
+                                                               int32_t* __restrict__ nbr, int* __restrict__ flag) {
+    __shared__ uint64_t buf[32 * kQueryWarps * 2];
+    const int n = threadIdx.x / G;
+    const int64_t i = (int64_t)blockIdx.x * (32 * kQueryWarps / G) + n;
+    int qx = h.hx0, qy = h.hy0;
+    const bool ok = i < m && query_xy(q, i, qx, qy);
+    idw_query<G>(h, i < m, ok, qx, qy, k, power, buf + n * 2 * G, depth + i, nbr ? nbr + i * k : nullptr, flag);
+}
+
 template <int K>
 __global__ void __launch_bounds__(128) k_idw_wide(HashView h, GridView g, int k, float power,
                                                   float* __restrict__ depth,
@@ -104,6 +117,9 @@ bg_status launch_k(const bg_soundings_s* s, const HashView& h, const GridView& g
         if (knn_patch_fits<K>(s->info, g.cell, g.nx, g.ny) && (int64_t)spr * pny < ((int64_t)1 << 31))
             k_idw_patch<K><<<(unsigned)(((int64_t)spr * pny + 1) / 2), 64, 0, st>>>(h, g, k, power, depth, nbr, d_flag,
                                                                                    plen, spr);
+        else if (query_by_warp((int64_t)g.nx * g.ny))
+            k_idw_query<query_lanes(K)><<<query_blocks<K>((int64_t)g.nx * g.ny), 32 * kQueryWarps, 0, st>>>(
+                h, g, (int64_t)g.nx * g.ny, k, power, depth, nbr, d_flag);
         else if (len == 1)
             k_idw<K, 1><<<(unsigned)nbs, 128, 0, st>>>(h, g, k, power, depth, nbr, d_flag);
         else if (len == 2)
@@ -176,7 +192,10 @@ bg_status launch_pts_k(const HashView& h, const PointsView& q, int k, float powe
     BG_CUDA(cudaMemsetAsync(d_flag, 0, sizeof(int), st));
     {
         ProfScope ps(prof_ctx, kProfIdw, q.m, st);
-        if (len == 1)
+        if (query_by_warp(q.m))
+            k_idw_query<query_lanes(K)><<<query_blocks<K>(q.m), 32 * kQueryWarps, 0, st>>>(
+                h, q, q.m, k, power, depth, nbr, d_flag);
+        else if (len == 1)
             k_idw_pts<K, 1><<<(unsigned)nb, 128, 0, st>>>(h, q, k, power, depth, nbr, d_flag);
         else if (len == 2)
             k_idw_pts<K, 2><<<(unsigned)nb, 128, 0, st>>>(h, q, k, power, depth, nbr, d_flag);

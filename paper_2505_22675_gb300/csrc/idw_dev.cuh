@@ -19,6 +19,7 @@
 
 #include "bg_internal.h"
 #include "knn.cuh"
+#include "knn_query.cuh"
 #include "knn_warp.cuh"
 
 namespace bg {
@@ -152,6 +153,47 @@ __device__ __noinline__ KnnFar idw_lone(const HashView& h, int qx, int qy, uint6
     });
     if (nbr) emit_ids<32>(nbr, hp, k, keff, mask);
     return knn_far<K>(h, hp, cnt);
+}
+
+// IDW of the queries of a warp (knn_query): lane n of a query's G holds neighbour
+// n, lanes 0 .. 7 the eight partial sums. valid: there is a query; ok: in range.
+template <int G>
+__device__ __forceinline__ void idw_query(const HashView& h, bool valid, bool ok, int qx, int qy, int k, float power,
+                                          uint64_t* buf, float* depth, int32_t* nbr, int* flag) {
+    const int lane = threadIdx.x & (G - 1);
+    uint64_t key = 0;
+    const int found = h.n_valid > 0 ? knn_query<G>(h, ok, qx, qy, k, buf, key) : 0, cnt = max(found, 0);
+    const int u = lane < cnt ? (int)(key & ((1ull << h.idx_bits) - 1)) : -1;
+    float d = 1.0f, z = 0.0f;
+    if (u >= 0) {
+        d = idw_d2f(key >> h.idx_bits);
+        z = __int_as_float(__ldg(&h.orig[u].z));
+    }
+    const float d1 = __shfl_sync(kFull, d, 0, G), z1 = __shfl_sync(kFull, z, 0, G);
+    float l1 = 0.0f;
+    if (power != 2.0f) l1 = log2f(d1);
+    const float w = idw_weight(d1, l1, 0.5f * power, power, d), dz = z - z1;
+    float num = 0.0f, den = 0.0f;
+    for (int n0 = 1; n0 < k; n0 += kIdwLanes) {
+        const int n = n0 + (lane & 7);
+        const float wn = __shfl_sync(kFull, w, n, G), dn = __shfl_sync(kFull, dz, n, G);
+        if (n < cnt) {
+            num = fmaf(wn, dn, num);
+            den += wn;
+        }
+    }
+#pragma unroll
+    for (int s = 1; s < kIdwLanes; s *= 2) {
+        num += __shfl_xor_sync(kFull, num, s);
+        den += __shfl_xor_sync(kFull, den, s);
+    }
+    if (!valid) return;
+    if (found < 0) {
+        if (lane == 0) *flag = 1;
+        return;
+    }
+    if (nbr && lane < k) nbr[lane] = u;
+    if (lane == 0) *depth = cnt == 0 ? __int_as_float(0x7fc00000) : d1 == 0.0f ? z1 : z1 + num / (1.0f + den);
 }
 
 template <int K, bool kWide>

@@ -76,6 +76,25 @@ __global__ void __launch_bounds__(64, KnnWarp<K>::kBlocksPerSM) k_knn_ids_patch(
         });
 }
 
+// The ids of queries i0 .. i0 + m - 1, G lanes each, as upload indices.
+template <int G, class Queries>
+__global__ void __launch_bounds__(32 * kQueryWarps) k_knn_ids_query(HashView h, Queries q, int64_t i0, int64_t m, int k,
+                                                                   int32_t* __restrict__ ids, int* __restrict__ flag) {
+    __shared__ uint64_t buf[32 * kQueryWarps * 2];
+    const int n = threadIdx.x / G, lane = threadIdx.x & (G - 1);
+    const int64_t i = (int64_t)blockIdx.x * (32 * kQueryWarps / G) + n;
+    int qx = h.hx0, qy = h.hy0;
+    const bool ok = i < m && query_xy(q, i0 + i, qx, qy);
+    uint64_t key = 0;
+    const int cnt = h.n_valid > 0 ? knn_query<G>(h, ok, qx, qy, k, buf + n * 2 * G, key) : 0;
+    if (i >= m) return;
+    if (cnt < 0) {
+        if (lane == 0) *flag = 1;
+    } else if (lane < k) {
+        ids[i * k + lane] = lane < cnt ? (int)(key & ((1ull << h.idx_bits) - 1)) : -1;
+    }
+}
+
 template <int K>
 __global__ void __launch_bounds__(128) k_knn_ids_wide(HashView h, GridView g, int k, IdsView ids,
                                                       int32_t* __restrict__ nbr, int* __restrict__ flag) {
@@ -197,6 +216,9 @@ bg_status launch_k(const bg_soundings_s* snd, const HashView& h, const GridView&
             if (patches)
                 k_knn_ids_patch<K><<<(unsigned)(((int64_t)spr * pny + 1) / 2), 64, 0, st>>>(
                     h, g, k, ids, slot_ids ? nbr : nullptr, flag, plen, spr);
+            else if (query_by_warp(nodes))
+                k_knn_ids_query<query_lanes(K)><<<query_blocks<K>(nodes), 32 * kQueryWarps, 0, st>>>(
+                    h, g, j0 * g.nx, nodes, k, chunk_ids, flag);
             else if (len == 1)
                 k_knn_ids<K, 1><<<(unsigned)nbs, 64, 0, st>>>(h, g, k, (int)j0, (int)j1, chunk_ids, flag);
             else if (len == 2)
@@ -321,7 +343,10 @@ bg_status launch_pts_k(const HashView& h, const PointsView& q, int k, const OkPa
         const int64_t nb = ((n + len - 1) / len + 127) / 128;
         {
             ProfScope ps(ctx, kProfKnnIds, n, st);
-            if (len == 1)
+            if (query_by_warp(n))
+                k_knn_ids_query<query_lanes(K)><<<query_blocks<K>(n), 32 * kQueryWarps, 0, st>>>(
+                    h, q, p0, n, k, chunk_ids, flag);
+            else if (len == 1)
                 k_knn_ids_pts<K, 1><<<(unsigned)nb, 128, 0, st>>>(h, q, k, p0, p1, chunk_ids, flag);
             else if (len == 2)
                 k_knn_ids_pts<K, 2><<<(unsigned)nb, 128, 0, st>>>(h, q, k, p0, p1, chunk_ids, flag);

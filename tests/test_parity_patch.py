@@ -98,6 +98,38 @@ def test_kriging_systems_of_every_size(name, model, nugget, k):
     assert np.array_equal(d, d2) and np.array_equal(v, v2)
 
 
+@pytest.mark.parametrize("k", [3, 8, 13, 32])
+@pytest.mark.parametrize("rows", [291, 292])
+@pytest.mark.parametrize("name", ["uniform", "lattice", "gap"])
+def test_queries_by_warps_and_by_threads(name, rows, k):
+    """200 x 291 nodes (lanes of a warp each where patches do not serve) and 200 x
+    292 (a thread each), as a grid of many soundings per node and as a list of points."""
+    import torch
+    make, cell = {"uniform": (lambda: _uniform(21, 400_000, 20_000, 29_200), 100),
+                  "lattice": (lambda: _lattice(400, 600, 50), 100),
+                  "gap": (lambda: _gap(22), 150)}[name]
+    x, y, z = make()
+    g = GridSpec(0, 0, cell, 200, rows)
+    qx, qy = oracle.grid_nodes(g.x0_cm, g.y0_cm, g.cell_cm, g.nx, g.ny)
+    lib = Lib(x, y, z, g)
+    try:
+        d, nb = lib.idw(k, 2.0)
+        pd = torch.empty(qx.size, device="cuda")
+        pn = torch.empty(qx.size * k, dtype=torch.int32, device="cuda")
+        lib.bg.interp_idw_points(lib.s, torch.from_numpy(qx.astype(np.int32)).cuda(),
+                                 torch.from_numpy(qy.astype(np.int32)).cuda(), k, 2.0, pd, pn)
+        _, _, kn = lib.okrige(k, 0, 0.25, 100.0, 50.0)
+        torch.cuda.synchronize()
+    finally:
+        lib.close()
+    assert np.array_equal(d.view(np.uint32), pd.cpu().numpy().view(np.uint32))
+    assert np.array_equal(nb, pn.cpu().numpy().reshape(-1, k)) and np.array_equal(nb, kn)
+    sel = np.random.default_rng(k).choice(qx.size, 1_500, replace=False)
+    ref, ridx = oracle.idw(x, y, z, qx[sel].astype(np.int32), qy[sel].astype(np.int32), k, 2.0, want_idx=True)
+    assert np.array_equal(nb[sel], ridx)
+    assert_idw(d[sel], ref)
+
+
 @pytest.mark.parametrize("k", [12, 32])
 @pytest.mark.parametrize("range_m", [0.05, 2.0, 30.0, 400.0])
 def test_exponential_model_at_every_range(range_m, k):
