@@ -117,7 +117,7 @@ bg_status launch_k(const bg_soundings_s* s, const HashView& h, const GridView& g
         if (knn_patch_fits<K>(s->info, g.cell, g.nx, g.ny) && (int64_t)spr * pny < ((int64_t)1 << 31))
             k_idw_patch<K><<<(unsigned)(((int64_t)spr * pny + 1) / 2), 64, 0, st>>>(h, g, k, power, depth, nbr, d_flag,
                                                                                    plen, spr);
-        else if (query_by_warp((int64_t)g.nx * g.ny))
+        else if (query_by_lanes<K>((int64_t)g.nx * g.ny))
             k_idw_query<query_lanes(K)><<<query_blocks<K>((int64_t)g.nx * g.ny), 32 * kQueryWarps, 0, st>>>(
                 h, g, (int64_t)g.nx * g.ny, k, power, depth, nbr, d_flag);
         else if (len == 1)
@@ -192,7 +192,7 @@ bg_status launch_pts_k(const HashView& h, const PointsView& q, int k, float powe
     BG_CUDA(cudaMemsetAsync(d_flag, 0, sizeof(int), st));
     {
         ProfScope ps(prof_ctx, kProfIdw, q.m, st);
-        if (query_by_warp(q.m))
+        if (query_by_lanes<K>(q.m))
             k_idw_query<query_lanes(K)><<<query_blocks<K>(q.m), 32 * kQueryWarps, 0, st>>>(
                 h, q, q.m, k, power, depth, nbr, d_flag);
         else if (len == 1)

@@ -33,14 +33,19 @@ inline unsigned query_blocks(int64_t m) {
     return (unsigned)((m + n - 1) / n);
 }
 
-// Lanes per query, or a thread each? By threads 50 (k = 8) to 75 us (k = 32) go by
-// whatever the number, up to some 60,000 queries. us, threads / lanes: 1,600
-// points k = 32 76 / 14, 6,000 points k = 16 54 / 16, 6,000 nodes k = 32 130 / 20,
-// 10,000 nodes k = 8 55 / 18, 81,000 points k = 8 53 / 69, 81,000 points k = 16 87
-// / 74, 90,000 nodes k = 8 50 / 62, k = 16 81 / 72, k = 32 125 / 121, 210,000
-// points k = 16 135 / 158, k = 32 206 / 284. The line is below where the smallest
-// k breaks even.
-inline bool query_by_warp(int64_t m) { return m <= 152 * 384; }
+// Lanes per query, or a thread each? By threads 33 (k = 8), 52 (16), 80 us (32) go
+// by whatever the number; by lanes 0.8 or 1.3 us a 1000. us, threads / lanes, IDW:
+// 1,600 points k = 32 76 / 14, 6,000 nodes k = 32 130 / 20; holes of 5 % of a grid:
+//   points      k = 8      k = 16      k = 32
+//   30,000    34 / 31     52 / 31     82 / 51
+//   45,000    35 / 41     55 / 41     90 / 74
+//   60,000    35 / 49     55 / 52     99 / 95
+//   80,000    36 / 60     56 / 64    117 / 124
+// (1 % and 10 %: the same signs at k = 8; at the others the lines hold too).
+template <int K>
+inline bool query_by_lanes(int64_t m) {
+    return m <= (K <= 8 ? 152 * 224 : 152 * 384);
+}
 
 // G lanes (16 or 32) work on a query; both halves of a warp take every step
 // together, so a half that has finished repeats or idles until the other has.

@@ -216,7 +216,7 @@ bg_status launch_k(const bg_soundings_s* snd, const HashView& h, const GridView&
             if (patches)
                 k_knn_ids_patch<K><<<(unsigned)(((int64_t)spr * pny + 1) / 2), 64, 0, st>>>(
                     h, g, k, ids, slot_ids ? nbr : nullptr, flag, plen, spr);
-            else if (query_by_warp(nodes))
+            else if (query_by_lanes<K>(nodes))
                 k_knn_ids_query<query_lanes(K)><<<query_blocks<K>(nodes), 32 * kQueryWarps, 0, st>>>(
                     h, g, j0 * g.nx, nodes, k, chunk_ids, flag);
             else if (len == 1)
@@ -343,7 +343,7 @@ bg_status launch_pts_k(const HashView& h, const PointsView& q, int k, const OkPa
         const int64_t nb = ((n + len - 1) / len + 127) / 128;
         {
             ProfScope ps(ctx, kProfKnnIds, n, st);
-            if (query_by_warp(n))
+            if (query_by_lanes<K>(n))
                 k_knn_ids_query<query_lanes(K)><<<query_blocks<K>(n), 32 * kQueryWarps, 0, st>>>(
                     h, q, p0, n, k, chunk_ids, flag);
             else if (len == 1)
