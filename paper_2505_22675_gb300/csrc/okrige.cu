@@ -107,12 +107,26 @@ __global__ void __launch_bounds__(128) k_knn_ids_wide(HashView h, GridView g, in
 }
 
 // Solve blocks take `per` consecutive batches of 128 systems: one take of the
-// tensor memory and one block start for several batches (about 10 us each),
-// but at least four waves of blocks, so that the last wave stays short and
-// small grids spread over the SMs.
+// tensor memory and one block start (a twentieth of a batch) for several, in at
+// least four rounds of blocks, so that small grids spread over the SMs. Of those
+// the count whose rounds add up to the fewest batches: a last round of which
+// most blocks are missing takes as long as a whole one (16,262 batches over 152
+// places: 14 rounds of 8 2575 us, 27 of 4 2511, 107 of 1 2589; 1,639: 6 rounds of
+// 2 305 us, 11 of 1 289).
 template <int K>
 int solve_batches_per_block(int64_t batches) {
-    return (int)std::min<int64_t>(8, std::max<int64_t>(1, batches / (4 * 152 * Geo<K>::BLOCKS)));
+    const int64_t places = 152 * Geo<K>::BLOCKS;
+    int best = 1;
+    double least = 1e300;
+    for (int per = 1; per <= 8 && (per == 1 || batches >= 4 * places * per); ++per) {
+        const int64_t blocks = (batches + per - 1) / per, rounds = (blocks + places - 1) / places;
+        const double t = (double)rounds * (per + 0.05);
+        if (t < least) {
+            least = t;
+            best = per;
+        }
+    }
+    return best;
 }
 
 template <int K, class Fn>
