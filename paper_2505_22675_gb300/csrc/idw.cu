@@ -139,7 +139,7 @@ bg_status launch_k(const bg_soundings_s* s, const HashView& h, const GridView& g
 template <int K, int kLen>
 __global__ void __launch_bounds__(128) k_idw_pts(HashView h, PointsView q, int k, float power,
                                                  float* __restrict__ depth,
-                                                 int32_t* __restrict__ nbr, int* __restrict__ flag) {
+                                                 int32_t* __restrict__ nbr) {
     __shared__ uint64_t heap[K * 128];
     const int64_t p0 = ((int64_t)blockIdx.x * 128 + threadIdx.x) * kLen;
     if (p0 >= q.m) return;
@@ -168,15 +168,13 @@ __global__ void __launch_bounds__(128) k_idw_pts(HashView h, PointsView q, int k
         });
         if (nbr) emit_ids<128>(nbr + p * k, hp, k, keff, mask);
     };
-    knn_chain<128, decltype(emit), kLen>(h, q.x, q.y, p0, q.m, K, hp, flag, emit);
+    knn_chain<128, decltype(emit), kLen>(h, q.x, q.y, p0, q.m, K, hp, emit);
 }
 
 template <int K>
 __global__ void __launch_bounds__(128) k_idw_pts_wide(HashView h, PointsView q, int k, float power,
                                                       float* __restrict__ depth,
-                                                      int32_t* __restrict__ nbr,
-                                                      int* __restrict__ flag) {
-    if (*(volatile int*)flag == 0) return;
+                                                      int32_t* __restrict__ nbr) {
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < q.m;
          p += (int64_t)gridDim.x * blockDim.x)
         idw_point_wide<K>(h, __ldg(q.x + p), __ldg(q.y + p), k, power, depth + p,
@@ -185,25 +183,24 @@ __global__ void __launch_bounds__(128) k_idw_pts_wide(HashView h, PointsView q, 
 
 template <int K>
 bg_status launch_pts_k(const HashView& h, const PointsView& q, int k, float power, float* depth,
-                       int32_t* nbr, int* d_flag, cudaStream_t st, bg_ctx_s* prof_ctx) {
+                       int32_t* nbr, cudaStream_t st, bg_ctx_s* prof_ctx) {
     const int len = strip_len_for(q.m);
     const int64_t threads = (q.m + len - 1) / len;
     const int64_t nb = (threads + 127) / 128;
-    BG_CUDA(cudaMemsetAsync(d_flag, 0, sizeof(int), st));
     {
         ProfScope ps(prof_ctx, kProfIdw, q.m, st);
         if (query_by_lanes<K>(q.m))
             k_idw_query<query_lanes(K)><<<query_blocks<K>(q.m), 32 * kQueryWarps, 0, st>>>(
-                h, q, q.m, k, power, depth, nbr, d_flag);
+                h, q, q.m, k, power, depth, nbr, nullptr);
         else if (len == 1)
-            k_idw_pts<K, 1><<<(unsigned)nb, 128, 0, st>>>(h, q, k, power, depth, nbr, d_flag);
+            k_idw_pts<K, 1><<<(unsigned)nb, 128, 0, st>>>(h, q, k, power, depth, nbr);
         else if (len == 2)
-            k_idw_pts<K, 2><<<(unsigned)nb, 128, 0, st>>>(h, q, k, power, depth, nbr, d_flag);
+            k_idw_pts<K, 2><<<(unsigned)nb, 128, 0, st>>>(h, q, k, power, depth, nbr);
         else
-            k_idw_pts<K, 4><<<(unsigned)nb, 128, 0, st>>>(h, q, k, power, depth, nbr, d_flag);
+            k_idw_pts<K, 4><<<(unsigned)nb, 128, 0, st>>>(h, q, k, power, depth, nbr);
     }
     k_idw_pts_wide<K><<<(unsigned)std::min<int64_t>((q.m + 127) / 128, 152 * 4), 128, 0, st>>>(
-        h, q, k, power, depth, nbr, d_flag);
+        h, q, k, power, depth, nbr);
     note_launches(2);
     BG_CUDA(cudaGetLastError());
     return BG_OK;
@@ -217,17 +214,12 @@ bg_status launch_idw_points(const bg_soundings_s* s, const PointsView& q, int k,
     HashView h = s->h;
     const int K = k <= 4 ? 4 : k <= 8 ? 8 : k <= 16 ? 16 : 32;
     h.r0 = start_halfwidth(s, K);
-    int* flag = nullptr;
-    bg_status rc = dalloc(s->ctx, (void**)&flag, sizeof(int), st);
-    if (rc != BG_OK) return rc;
     switch (K) {
-        case 4: rc = launch_pts_k<4>(h, q, k, power, depth, nbr, flag, st, s->ctx); break;
-        case 8: rc = launch_pts_k<8>(h, q, k, power, depth, nbr, flag, st, s->ctx); break;
-        case 16: rc = launch_pts_k<16>(h, q, k, power, depth, nbr, flag, st, s->ctx); break;
-        default: rc = launch_pts_k<32>(h, q, k, power, depth, nbr, flag, st, s->ctx); break;
+        case 4: return launch_pts_k<4>(h, q, k, power, depth, nbr, st, s->ctx);
+        case 8: return launch_pts_k<8>(h, q, k, power, depth, nbr, st, s->ctx);
+        case 16: return launch_pts_k<16>(h, q, k, power, depth, nbr, st, s->ctx);
+        default: return launch_pts_k<32>(h, q, k, power, depth, nbr, st, s->ctx);
     }
-    dfree(s->ctx, flag, sizeof(int), st);
-    return rc;
 }
 
 bg_status launch_idw(const bg_soundings_s* s, const GridView& g, int k, float power,

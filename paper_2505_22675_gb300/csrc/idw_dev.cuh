@@ -123,7 +123,7 @@ template <int K>
 __device__ __forceinline__ void idw_point_wide(const HashView& h, int qx, int qy, int k,
                                                float power, float* __restrict__ dout,
                                                int32_t* __restrict__ o) {
-    if (h.n_valid == 0 || !query_in_range(qx, qy)) return;
+    if (!point_may_be_wide(h, qx, qy)) return;
     const Bound b = knn_bound<K>(h, qx, qy);
     if (packed_fits(h, b.tau0)) return;
     uint64_t d2[K];
@@ -189,7 +189,7 @@ __device__ __forceinline__ void idw_query(const HashView& h, bool valid, bool ok
     }
     if (!valid) return;
     if (found < 0) {
-        if (lane == 0) *flag = 1;
+        if (lane == 0 && flag) *flag = 1;
         return;
     }
     if (nbr && lane < k) nbr[lane] = u;

@@ -291,7 +291,7 @@ __device__ __forceinline__ void knn_ids_node_wide(const HashView& h, const GridV
 template <int K>
 __device__ __forceinline__ void knn_ids_point_wide(const HashView& h, int qx, int qy, int k,
                                                    int32_t* __restrict__ o) {
-    if (h.n_valid == 0 || !query_in_range(qx, qy)) return;
+    if (!point_may_be_wide(h, qx, qy)) return;
     const Bound b = knn_bound<K>(h, qx, qy);
     if (packed_fits(h, b.tau0)) return;
     uint64_t d2[K];
