@@ -125,25 +125,41 @@ __device__ __forceinline__ float gamma_cm(const OkParams& p, int dx, int dy, flo
     return variogram(p, d2 * rsqrtf(d2) * 0.01f);
 }
 
-// gamma between two distinct soundings from float offsets in cm (exact
-// integers below 2^24); zero separation gives the nugget c0 (the h -> 0+
-// limit) without a branch: t = min(h/a, 1) makes the spherical model's
-// polynomial equal the sill beyond the range
-__device__ __forceinline__ float gamma_pair_f(const OkParams& p, float dx, float dy) {
-    const float d2 = fmaf(dx, dx, dy * dy);
-    const float h_cm = d2 * rsqrtf(d2 + 1e-30f);
-    if (p.model == BG_VARIOGRAM_SPHERICAL) {
-        const float t = fminf(h_cm * p.inv_a * 0.01f, 1.0f);
-        return fmaf(p.c * t, fmaf(-0.5f * t, t, 1.5f), p.c0);
-    }
-    return fmaf(p.c, -expm1f(-h_cm * p.inv_a * 0.01f), p.c0);
-}
-
 // one hardware square-root approximation (a few ulp, 0 at 0 and below 2^-126)
 __device__ __forceinline__ float sqrt_approx(float x) {
     float y;
     asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
+}
+
+// 1 - exp(-t) for two t in [0, 25] at once (past 25 it is 1 in any case), for the
+// exponential model: a solve is bound by its instructions, and two entries share
+// each here, which a library call for each cannot (k = 12, 170,163 systems: solve
+// 104 -> 74 us). Argument reduction of Cody and Waite: t = n ln 2 + r, |r| <=
+// ln 2 / 2; 1 - exp(-r) = r - r^2 q(r), q of degree 4 by interpolation at the
+// Chebyshev nodes of that interval (off by 6e-8 at most); then (1 - s) + s (1 -
+// exp(-r)), s = 2^-n, which does not cancel at short range. Errors, 2e6 draws in
+// each of nine intervals: 1.01 ulp at most, 0.22 to 0.35 rms (-expm1f: 1.13, 0.22
+// to 0.50).
+__device__ __forceinline__ u64 one_minus_exp2(u64 t) {
+    const u64 magic = dup2(12582912.0f);  // 1.5 * 2^23: the low bits of a sum hold the integer
+    const u64 y = fma2(t, dup2(1.44269504f), magic);
+    const u64 r = fma2(sub2(y, magic), dup2(-0.693147181f), t);
+    u64 q = fma2(dup2(-0.00139261840f), r, dup2(0.00836317893f));
+    q = fma2(q, r, dup2(-0.0416665561f));
+    q = fma2(q, r, dup2(0.166665763f));
+    q = fma2(q, r, dup2(-0.5f));
+    const u64 m = fma2(mul2(r, r), q, r);
+    const auto pow2 = [](float v) {  // 2^-n
+        return __uint_as_float(0x3f800000u - (__float_as_uint(v) << 23));
+    };
+    const u64 s = pk2(pow2(lo2(y)), pow2(hi2(y)));
+    return fma2(s, m, sub2(dup2(1.0f), s));
+}
+__device__ __forceinline__ float exp_clamp(float x, float most) {  // min that keeps a NaN
+    float c;
+    asm("min.NaN.f32 %0, %1, %2;" : "=f"(c) : "f"(x), "f"(most));
+    return c;
 }
 
 // The variogram of the assembly in the fixed-point scale of the system: with
@@ -162,8 +178,10 @@ __device__ __forceinline__ ScaledVgm scaled_vgm(const OkParams& p, float sa) {
     return ScaledVgm{kinv * kinv, p.c0 * sa, cs, -0.5f * cs, 1.5f * cs};
 }
 
-// gamma_pair_f, spherical model, for two rows at once (packed FP32, each lane
-// the scalar operations in the same order)
+// gamma between two distinct soundings from float offsets in cm (exact integers
+// below 2^24), spherical model, for two rows at once (packed FP32); zero
+// separation gives the nugget c0 (the h -> 0+ limit) without a branch: t =
+// min(h / a, 1) makes the polynomial equal the sill beyond the range
 __device__ __forceinline__ void gamma_pair_sph2(const OkParams& p, float dxa, float dya, float dxb,
                                                 float dyb, float& ga, float& gb) {
     const unsigned long long dx = pk2(dxa, dxb), dy = pk2(dya, dyb);
@@ -194,6 +212,30 @@ __device__ __forceinline__ void gamma_cm_sph2(const OkParams& p, int dxa, int dy
     upk2(fma2(mul2(pk2(p.c, p.c), t), in, pk2(p.c0, p.c0)), va, vb);
     ga = ((dxa | dya) == 0) ? 0.0f : (ta >= 1.0f ? p.sill : va);
     gb = ((dxb | dyb) == 0) ? 0.0f : (tb >= 1.0f ? p.sill : vb);
+}
+
+// The two above, exponential model
+__device__ __forceinline__ void gamma_pair_exp2(const OkParams& p, float dxa, float dya, float dxb, float dyb,
+                                                float& ga, float& gb) {
+    const u64 dx = pk2(dxa, dxb), dy = pk2(dya, dyb);
+    const u64 d2 = fma2(dx, dx, mul2(dy, dy));
+    const u64 e = add2(d2, dup2(1e-30f));
+    float ta, tb;
+    upk2(mul2(mul2(mul2(d2, pk2(rsqrtf(lo2(e)), rsqrtf(hi2(e)))), dup2(p.inv_a)), dup2(0.01f)), ta, tb);
+    const u64 t = pk2(exp_clamp(ta, 25.0f), exp_clamp(tb, 25.0f));
+    upk2(fma2(dup2(p.c), one_minus_exp2(t), dup2(p.c0)), ga, gb);
+}
+__device__ __forceinline__ void gamma_cm_exp2(const OkParams& p, int dxa, int dya, int dxb, int dyb,
+                                              float& ga, float& gb) {
+    const u64 fx = pk2((float)dxa, (float)dxb), fy = pk2((float)dya, (float)dyb);
+    const u64 d2 = fma2(fx, fx, mul2(fy, fy));
+    float ta, tb;
+    upk2(mul2(mul2(mul2(d2, pk2(rsqrtf(lo2(d2)), rsqrtf(hi2(d2)))), dup2(0.01f)), dup2(p.inv_a)), ta, tb);
+    const u64 t = pk2(exp_clamp(ta, 25.0f), exp_clamp(tb, 25.0f));
+    float va, vb;
+    upk2(fma2(dup2(p.c), one_minus_exp2(t), dup2(p.c0)), va, vb);
+    ga = (dxa | dya) == 0 ? 0.0f : va;
+    gb = (dxb | dyb) == 0 ? 0.0f : vb;
 }
 
 // ------------------------------------------------------------ k-NN -> ids
@@ -425,36 +467,6 @@ __device__ __forceinline__ float ll_to_float(long long v) {
     return fmaf((float)hi, 4294967296.0f, (float)lo);
 }
 
-// 1 - exp(-sqrt(ta)), 1 - exp(-sqrt(tb)), for the tiles of the exponential
-// model: an FMA-bound assembly, so two entries share each instruction, which a
-// library call for each cannot (k = 12, 170,163 systems: solve 104 -> 79 us).
-// Argument reduction of Cody and Waite: sqrt(ta) = n ln 2 + r, |r| <= ln 2 / 2;
-// 1 - exp(-r) = r - r^2 q(r), q of degree 4 by interpolation at the Chebyshev
-// nodes of that interval (off by 6e-8 at most); then (1 - s) + s (1 - exp(-r)),
-// s = 2^-n, which does not cancel at short range. Within 1.01 ulp (2e6 draws in
-// each of six intervals); past 25 the result is 1 in any case.
-__device__ __forceinline__ u64 one_minus_exp2(float ta, float tb) {
-    const u64 magic = dup2(12582912.0f);  // 1.5 * 2^23: the low bits of a sum hold the integer
-    const auto root = [](float t2) {
-        float c;
-        asm("min.NaN.f32 %0, %1, 0f441C4000;" : "=f"(c) : "f"(t2));  // 625
-        return sqrt_approx(c);
-    };
-    const u64 t = pk2(root(ta), root(tb));
-    const u64 y = fma2(t, dup2(1.44269504f), magic);
-    const u64 r = fma2(sub2(y, magic), dup2(-0.693147181f), t);
-    u64 q = fma2(dup2(-0.00139261840f), r, dup2(0.00836317893f));
-    q = fma2(q, r, dup2(-0.0416665561f));
-    q = fma2(q, r, dup2(0.166665763f));
-    q = fma2(q, r, dup2(-0.5f));
-    const u64 m = fma2(mul2(r, r), q, r);
-    const auto pow2 = [](float v) {  // 2^-n
-        return __uint_as_float(0x3f800000u - (__float_as_uint(v) << 23));
-    };
-    const u64 s = pk2(pow2(lo2(y)), pow2(hi2(y)));
-    return fma2(s, m, sub2(dup2(1.0f), s));
-}
-
 // The tile function of the assembly: -A for two rows at once, in the
 // fixed-point scale. -A[r][c] = gamma(r, c) - Gamma_r0 - Gamma_c0; the records
 // hold zr = -Gamma_r0, and zc comes in as c0 - Gamma_c0 (all scaled).
@@ -481,7 +493,8 @@ struct TileVgm {
             const u64 in = fma2(k2, pk2(ta, tb), k3);
             return fma2(pk2(sqrt_approx(ta), sqrt_approx(tb)), in, add2(zr, dup2(zc)));
         } else {
-            return fma2(dup2(cs), one_minus_exp2(ta, tb), add2(zr, dup2(zc)));
+            const u64 t = pk2(sqrt_approx(exp_clamp(ta, 625.0f)), sqrt_approx(exp_clamp(tb, 625.0f)));
+            return fma2(dup2(cs), one_minus_exp2(t), add2(zr, dup2(zc)));
         }
     }
 };
@@ -885,9 +898,9 @@ __device__ __forceinline__ void okrige_solve_range(const HashView& h, const Grid
             }
         } else {
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                gr0[4 * j + u] = gamma_pair_f(p, ox[u], oy[u]);
-                g0[u] = gamma_cm(p, pdx[u], pdy[u], 0.0f);
+            for (int u = 0; u < 4; u += 2) {
+                gamma_pair_exp2(p, ox[u], oy[u], ox[u + 1], oy[u + 1], gr0[4 * j + u], gr0[4 * j + u + 1]);
+                gamma_cm_exp2(p, pdx[u], pdy[u], pdx[u + 1], pdy[u + 1], g0[u], g0[u + 1]);
             }
         }
 #pragma unroll
