@@ -481,7 +481,7 @@ __device__ __forceinline__ void wide_node(const TileDesc& d, const HashView& h, 
     uint64_t d2[K];
     int id[K];
     // the bound above used kq <= K soundings; the K-slot scan keeps the kq nearest in front
-    const int keff = min(knn_scan<K, true>(h, qx, qy, b, d2, id), d.k);
+    const int keff = min(knn_scan_wide<K>(h, qx, qy, b, d2, id), d.k);
     if (d.method == 0) {
         d.depth[node] = idw_from(h, keff, d.power, [&](int i, uint64_t& dd, int& ii) {
             dd = d2[i];

@@ -90,8 +90,7 @@ __global__ void __launch_bounds__(128) k_idw_wide(HashView h, GridView g, int k,
     const int gx = (g.nx + 15) / 16;
     const int64_t nb = (int64_t)gx * ((g.ny + 7) / 8);
     for (int64_t b = blockIdx.x; b < nb; b += gridDim.x)
-        idw_node<K, true>(h, g, k, power, depth, nbr, flag,
-                          patch_node((int)(b % gx), (int)(b / gx), warp, lane), nullptr);
+        idw_node_wide<K>(h, g, k, power, depth, nbr, patch_node((int)(b % gx), (int)(b / gx), warp, lane));
 }
 
 // d_flag: one int, or NULL to allocate one where it is needed

@@ -41,9 +41,9 @@ __device__ __forceinline__ float idw_weight(float d1, float l1, float hp, float 
 // them gets bitwise the same depth: neighbour n >= 1 goes to partial n_t =
 // (n - 1) mod 8, each partial adds its neighbours in ascending n, and the 8
 // partials combine pairwise as ((p0 + p1) + (p2 + p3)) + ((p4 + p5) + (p6 +
-// p7)). The kriging solve (8 threads per system, thread t holding neighbours
-// 1 + t + 8 s) forms the same partials in registers and combines them with
-// xor shuffles in that pattern.
+// p7)). The kriging solve (2 threads per system, thread h holding the partials
+// 4 h .. 4 h + 3) and the search by lanes (a lane per partial) form the same
+// partials and combine them in that pattern.
 constexpr int kIdwLanes = 8;
 
 __device__ __forceinline__ float idw_tree8(const float (&p)[kIdwLanes]) {
@@ -128,7 +128,7 @@ __device__ __forceinline__ void idw_point_wide(const HashView& h, int qx, int qy
     if (packed_fits(h, b.tau0)) return;
     uint64_t d2[K];
     int id[K];
-    const int keff = min(knn_scan<K, true>(h, qx, qy, b, d2, id), k);
+    const int keff = min(knn_scan_wide<K>(h, qx, qy, b, d2, id), k);
     *dout = idw_from(h, keff, power, [&](int i, uint64_t& dd, int& ii) {
         dd = d2[i];
         ii = id[i];
@@ -196,52 +196,26 @@ __device__ __forceinline__ void idw_query(const HashView& h, bool valid, bool ok
     if (lane == 0) *depth = cnt == 0 ? __int_as_float(0x7fc00000) : d1 == 0.0f ? z1 : z1 + num / (1.0f + den);
 }
 
-template <int K, bool kWide>
-__device__ __forceinline__ void idw_node(const HashView& h, const GridView& g, int k, float power,
-                                         float* __restrict__ depth, int32_t* __restrict__ nbr,
-                                         int* __restrict__ flag, NodeIdx nd, uint64_t* hp) {
-    if (nd.i >= g.nx || nd.j >= g.ny) return;
+// Wide-key IDW of one grid node whose table bound does not fit the packed key
+// (rare); others return.
+template <int K>
+__device__ __forceinline__ void idw_node_wide(const HashView& h, const GridView& g, int k, float power,
+                                              float* __restrict__ depth, int32_t* __restrict__ nbr, NodeIdx nd) {
+    if (nd.i >= g.nx || nd.j >= g.ny || h.n_valid == 0) return;
     const int64_t node = (int64_t)nd.j * g.nx + nd.i;
     const int qx = g.x0 + nd.i * g.cell + g.cell / 2;
     const int qy = g.y0 + nd.j * g.cell + g.cell / 2;
-    int32_t* o = nbr ? nbr + node * k : nullptr;
-    if (h.n_valid == 0) {
-        if (kWide) return;
-        depth[node] = __int_as_float(0x7fc00000);
-        if (o)
-            for (int i = 0; i < k; ++i) o[i] = -1;
-        return;
-    }
     const Bound b = knn_bound<K>(h, qx, qy);
-    const bool fits = packed_fits(h, b.tau0);
-    if constexpr (kWide) {
-        if (fits) return;  // done by the packed pass
-        uint64_t d2[K];
-        int id[K];
-        const int keff = min(knn_scan<K, true>(h, qx, qy, b, d2, id), k);
-        depth[node] = idw_from(h, keff, power, [&](int i, uint64_t& dd, int& ii) {
-            // the register arrays are read with a runtime index only here, in the rare wide pass
-            dd = d2[i];
-            ii = id[i];
-        });
-        if (o)
-            for (int i = 0; i < k; ++i) o[i] = i < keff ? id[i] : -1;
-    } else {
-        if (!fits) {
-            *flag = 1;  // the wide pass picks this node up
-            return;
-        }
-        const int keff = min(knn_scan_heap<K, 128>(h, qx, qy, b, hp), k);
-        const int bits = h.idx_bits;
-        const uint64_t mask = (1ull << bits) - 1;
-        depth[node] = idw_from(h, keff, power, [&](int i, uint64_t& dd, int& ii) {
-            const uint64_t key = hp[i * 128];
-            dd = key >> bits;
-            ii = (int)(key & mask);
-        });
-        if (o)
-            for (int i = 0; i < k; ++i) o[i] = i < keff ? (int)(hp[i * 128] & mask) : -1;
-    }
+    if (packed_fits(h, b.tau0)) return;
+    uint64_t d2[K];
+    int id[K];
+    const int keff = min(knn_scan_wide<K>(h, qx, qy, b, d2, id), k);
+    depth[node] = idw_from(h, keff, power, [&](int i, uint64_t& dd, int& ii) {
+        dd = d2[i];
+        ii = id[i];
+    });
+    if (nbr)
+        for (int i = 0; i < k; ++i) nbr[node * k + i] = i < keff ? id[i] : -1;
 }
 
 }  // namespace bg

@@ -148,14 +148,6 @@ __device__ __forceinline__ bool packed_fits(const HashView& h, int64_t tau0) {
     return ((uint64_t)(tau0 + 1) >> (64 - h.idx_bits)) == 0;
 }
 
-template <int K>
-__device__ __forceinline__ void insert_packed(uint64_t (&key)[K], uint64_t c) {
-    // precondition: c < key[K-1]; keeps key[] ascending
-#pragma unroll
-    for (int j = K - 1; j > 0; --j) key[j] = (c < key[j - 1]) ? key[j - 1] : ((c < key[j]) ? c : key[j]);
-    key[0] = (c < key[0]) ? c : key[0];
-}
-
 __device__ __forceinline__ bool wide_less(uint64_t ad, int ai, uint64_t bd, int bi) {
     return ad < bd || (ad == bd && ai < bi);
 }
@@ -178,20 +170,20 @@ __device__ __forceinline__ void insert_wide(uint64_t (&kd)[K], int (&ki)[K], uin
     }
 }
 
-// Phase 2. On return d2o[0..keff) / ido[0..keff) hold the neighbours in
+// Phase 2 with wide keys, sorted in registers. On return d2o[0..keff) / ido[0..keff) hold the neighbours in
 // ascending (d2, index) order; returns keff (<= K).
-template <int K, bool kWide>
-__device__ __forceinline__ int knn_scan(const HashView& h, int qx, int qy, const Bound& b,
-                                        uint64_t (&d2o)[K], int (&ido)[K]) {
-    const int bits = h.idx_bits;
+template <int K>
+__device__ __forceinline__ int knn_scan_wide(const HashView& h, int qx, int qy, const Bound& b,
+                                             uint64_t (&d2o)[K], int (&ido)[K]) {
     const int64_t tau0 = b.tau0;
-    uint64_t key[K];   // packed form (or the d2 half of the wide form)
-    int kid[kWide ? K : 1];
-    const uint64_t sentinel = kWide ? (uint64_t)(tau0 + 1) : ((uint64_t)(tau0 + 1) << bits);
+    uint64_t key[K];
+    int kid[K];
+    const uint64_t sentinel = (uint64_t)(tau0 + 1);
 #pragma unroll
-    for (int i = 0; i < K; ++i) key[i] = sentinel;
-#pragma unroll
-    for (int i = 0; i < (kWide ? K : 1); ++i) kid[i] = INT_MAX;
+    for (int i = 0; i < K; ++i) {
+        key[i] = sentinel;
+        kid[i] = INT_MAX;
+    }
     int64_t tau = tau0;
     int up = b.cy, dn = b.cy - 1;
     const int64_t xmin = h.hx0;
@@ -223,32 +215,16 @@ __device__ __forceinline__ int knn_scan(const HashView& h, int qx, int qy, const
             const int ddx = v.x - qx, ddy = v.y - qy;
             const uint64_t d2 = (uint64_t)((long long)ddx * ddx + (long long)ddy * ddy);
             if (d2 > utau) continue;
-            if constexpr (kWide) {
-                if (wide_less(d2, v.w, key[K - 1], kid[K - 1])) insert_wide<K>(key, kid, d2, v.w);
-            } else {
-                const uint64_t c = (d2 << bits) | (uint32_t)v.w;
-                if (c < key[K - 1]) insert_packed<K>(key, c);
-            }
+            if (wide_less(d2, v.w, key[K - 1], kid[K - 1])) insert_wide<K>(key, kid, d2, v.w);
         }
-        int64_t kth;
-        if constexpr (kWide)
-            kth = (int64_t)key[K - 1];
-        else
-            kth = (int64_t)(key[K - 1] >> bits);
-        tau = min(tau, kth);
+        tau = min(tau, (int64_t)key[K - 1]);
     }
     int keff = 0;
-    const uint64_t mask = (bits >= 64) ? ~0ull : ((1ull << bits) - 1);
 #pragma unroll
     for (int i = 0; i < K; ++i) {
         const bool ok = key[i] < sentinel;  // every real key has d2 <= tau0
-        if constexpr (kWide) {
-            d2o[i] = key[i];
-            ido[i] = ok ? kid[i] : -1;
-        } else {
-            d2o[i] = key[i] >> bits;
-            ido[i] = ok ? (int)(key[i] & mask) : -1;
-        }
+        d2o[i] = key[i];
+        ido[i] = ok ? kid[i] : -1;
         keff += ok ? 1 : 0;
     }
     return keff;
@@ -382,12 +358,6 @@ __device__ __forceinline__ int knn_scan_heap_rt(const HashView& h, int qx, int q
         }
     }
     return cnt;
-}
-
-template <int K, int S>
-__device__ __forceinline__ int knn_scan_heap(const HashView& h, int qx, int qy, const Bound& b,
-                                             uint64_t* hp) {
-    return knn_scan_heap_rt<S>(h, qx, qy, b, hp, K);
 }
 
 // The first k ids of a thread's sorted heap (stride S) to out, -1 from cnt

@@ -39,20 +39,23 @@
 // cycles per 128 systems, of them factor 22,500, residual 11,300 (16,400 with the
 // tiles evaluated again, 9,900 with them rounded to integers before they are
 // kept, but then the factor takes 24,900), gathers 3,500.
-// Measured on one survey line (3,001 x 692 nodes, k = 32, fused IDW): 2.59 ms
-// (2.77 with the tiles evaluated again) against 3.84 ms for 8 threads per system with the factor in registers (1,500
-// warp instructions per system there, 780 here; one thread per system: 630, but
-// one warp per scheduler and 3.5 ms); 256 x 256 tile, k = 16: 29 against 37 us.
-// Loading the next batch's ids and records during the last solve changed nothing.
+// Measured on one survey line (3,001 x 692 nodes, k = 32, fused IDW): 2.52 ms
+// (2.77 with the tiles evaluated again) against 3.84 ms for 8 threads per system
+// with the factor in registers (1,500 warp instructions per system there, 664
+// here; one thread per system: 630, but one warp per scheduler and 3.5 ms); 256 x
+// 256 tile, k = 16: 28 against 37 us. Loading the next batch's ids and records
+// during the last solve changed nothing.
 //
 // One step of iterative refinement follows the solve: A' is A rounded to a
 // 30-bit fixed point, x is rounded to 24-bit fixed point x' (exact in FP32),
 // and the residual b - A' x' is accumulated exactly in 64-bit integers. The
 // tiles of A are kept for it: at K = 16 most of them in tensor memory beside
 // the factor, at K = 32, where on-chip memory holds only one of the two
-// triangles, in the threads' local memory (1.1 KB a thread, 36 MB over the
-// device's resident systems: it stays in L2), read one tile ahead. The correction reuses the factor. The weight sum
-// closes in FP64: lambda_0 = 1 - sum(lambda'). Outputs:
+// triangles, in the threads' local memory (1.3 KB a thread, 50 MB over the
+// device's resident systems: L2 holds them but for 0.4 KB a system that is
+// written back, 6 % of the DRAM's bandwidth with the ids), read one tile ahead.
+// The correction reuses the factor. The weight sum closes in FP64: lambda_0 = 1 -
+// sum(lambda'). Outputs:
 //     zhat    = z_0 + sum_a lambda_a (z_a - z_0)          (= sum lambda_i z_i)
 //     sigma^2 = lambda_0 gamma_00 + sum_a lambda_a gamma_a0 + mu.
 // Rows beyond k_eff - 1 are identity rows with zero right-hand side, so every
@@ -311,7 +314,7 @@ __device__ __forceinline__ void knn_ids_node_wide(const HashView& h, const GridV
     if (packed_fits(h, b.tau0)) return;
     uint64_t d2[K];
     int id[K];
-    const int keff = knn_scan<K, true>(h, qx, qy, b, d2, id);
+    const int keff = knn_scan_wide<K>(h, qx, qy, b, d2, id);
     if (ids.stride == 0) {
         int32_t* o = ids.p + ((int64_t)(nd.j - ids.j0) * g.nx + nd.i) * k;
 #pragma unroll
@@ -338,7 +341,7 @@ __device__ __forceinline__ void knn_ids_point_wide(const HashView& h, int qx, in
     if (packed_fits(h, b.tau0)) return;
     uint64_t d2[K];
     int id[K];
-    const int keff = knn_scan<K, true>(h, qx, qy, b, d2, id);
+    const int keff = knn_scan_wide<K>(h, qx, qy, b, d2, id);
 #pragma unroll
     for (int i = 0; i < K; ++i)
         if (i < k) o[i] = i < keff ? id[i] : -1;
