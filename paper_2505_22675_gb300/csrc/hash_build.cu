@@ -12,7 +12,7 @@
 // All four passes stream through HBM; none has a data-dependent loop. An input
 // of at most 262,144 soundings whose counts fit in shared memory (a tile: some
 // 48,000 cells) takes them in one cluster of eight 1024-thread blocks instead
-// (k_hash_cluster): one launch instead of eight.
+// (k_hash_cluster): one launch instead of seven.
 #include <algorithm>
 #include <climits>
 #include <cmath>
@@ -113,19 +113,6 @@ __global__ void __launch_bounds__(kThreads) k_cell_hist(const int4* __restrict__
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
         const int4 r = orig[i];
         if (r.w) atomicAdd(&count[cell_index(g, r.x, r.y)], 1);
-    }
-}
-
-__global__ void __launch_bounds__(kThreads) k_scatter(const int4* __restrict__ orig, int64_t n,
-                                                      CellGeom g, int* __restrict__ cursor,
-                                                      int4* __restrict__ rec) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        const int4 r = orig[i];
-        if (r.w) {
-            const int pos = atomicAdd(&cursor[cell_index(g, r.x, r.y)], 1);
-            rec[pos] = make_int4(r.x, r.y, r.z, (int)i);
-        }
     }
 }
 
@@ -237,25 +224,51 @@ __global__ void __launch_bounds__(kThreads) k_scan_apply(const int* in, int64_t 
 // sat[(y)*(ncx+1) + x] = number of soundings in cells [0, x) x [0, y).
 // The row prefix of row r at column x is cell_start[r*ncx + x] - cell_start[r*ncx].
 
-__global__ void k_sat_chunk(const int* __restrict__ cs, int ncx, int ncy, int rows,
-                            int* __restrict__ csum) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int ch = blockIdx.y;
-    if (x > ncx) return;
-    const int y0 = ch * rows, y1 = min(ncy, y0 + rows);
-    int s = 0;
-    for (int y = y0; y < y1; ++y) s += cs[(int64_t)y * ncx + x] - cs[(int64_t)y * ncx];
-    csum[(int64_t)ch * (ncx + 1) + x] = s;
+// Column sums of each chunk of `rows` rows, 256 columns a block; beside them the
+// scatter of the records, which waits for the same scan and for memory where the
+// chunks wait for their loads (4.0M soundings, 1M cells: 33 us in two launches, 28 in
+// one). The first sat_blocks blocks take chunks.
+__global__ void __launch_bounds__(kThreads) k_scatter_and_chunks(const int4* __restrict__ orig, int64_t n, CellGeom g,
+                                                                 int* __restrict__ cursor, int4* __restrict__ rec,
+                                                                 const int* __restrict__ cs, int rows,
+                                                                 int* __restrict__ csum, int64_t sat_blocks) {
+    if (blockIdx.x < sat_blocks) {
+        const int gx = (g.ncx + kThreads) / kThreads;
+        const int x = (int)(blockIdx.x % (unsigned)gx) * kThreads + threadIdx.x, ch = (int)(blockIdx.x / (unsigned)gx);
+        if (x > g.ncx) return;
+        const int y0 = ch * rows, y1 = min(g.ncy, y0 + rows);
+        int s = 0;
+#pragma unroll 8
+        for (int y = y0; y < y1; ++y) s += cs[(int64_t)y * g.ncx + x] - cs[(int64_t)y * g.ncx];
+        csum[(int64_t)ch * (g.ncx + 1) + x] = s;
+        return;
+    }
+    const int64_t stride = (int64_t)(gridDim.x - sat_blocks) * kThreads;
+    for (int64_t i = (int64_t)(blockIdx.x - sat_blocks) * kThreads + threadIdx.x; i < n; i += stride) {
+        const int4 r = orig[i];
+        if (r.w) {
+            const int pos = atomicAdd(&cursor[cell_index(g, r.x, r.y)], 1);
+            rec[pos] = make_int4(r.x, r.y, r.z, (int)i);
+        }
+    }
 }
 
+// Exclusive scan of the chunks' sums in place, eight loads ahead of their sums (one at
+// a time 11.6 us there, so 6.2).
 __global__ void k_sat_chunkscan(int* __restrict__ csum, int ncx, int nch) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x > ncx) return;
     int run = 0;
-    for (int ch = 0; ch < nch; ++ch) {
-        const int t = csum[(int64_t)ch * (ncx + 1) + x];
-        csum[(int64_t)ch * (ncx + 1) + x] = run;
-        run += t;
+    for (int c0 = 0; c0 < nch; c0 += 8) {
+        int* p = csum + (int64_t)c0 * (ncx + 1) + x;
+        int v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = c0 + u < nch ? p[(int64_t)u * (ncx + 1)] : 0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            if (c0 + u < nch) p[(int64_t)u * (ncx + 1)] = run;
+            run += v[u];
+        }
     }
 }
 
@@ -268,10 +281,29 @@ __global__ void k_sat_apply(const int* __restrict__ cs, const int* __restrict__ 
     const int y0 = ch * rows, y1 = min(ncy, y0 + rows);
     int run = csum[(int64_t)ch * W + x];
     if (ch == 0) sat[x] = 0;
+#pragma unroll 8
     for (int y = y0; y < y1; ++y) {
         run += cs[(int64_t)y * ncx + x] - cs[(int64_t)y * ncx];
         sat[(int64_t)(y + 1) * W + x] = run;
     }
+}
+
+int grid_for(int64_t n, int per_block, int cap) {
+    int64_t b = (n + per_block - 1) / per_block;
+    if (b < 1) b = 1;
+    if (b > cap) b = cap;
+    return (int)b;
+}
+
+// The last three passes: scatter, chunk sums, summed-area table.
+void launch_scatter_sat(const int4* orig, int64_t n, const CellGeom& g, int* cursor, int4* rec, const int* cell_start,
+                        int sat_rows, int nch, int* csum, int* sat, cudaStream_t st) {
+    const int gx = (g.ncx + kThreads) / kThreads;
+    const int64_t chunks = (int64_t)gx * nch;
+    k_scatter_and_chunks<<<(unsigned)(chunks + grid_for(n, kThreads * 4, 152 * 16)), kThreads, 0, st>>>(
+        orig, n, g, cursor, rec, cell_start, sat_rows, csum, chunks);
+    k_sat_chunkscan<<<gx, kThreads, 0, st>>>(csum, g.ncx, nch);
+    k_sat_apply<<<dim3(gx, nch), kThreads, 0, st>>>(cell_start, csum, g.ncx, g.ncy, sat_rows, sat);
 }
 
 // ---------------------------------------------------- small inputs, one cluster
@@ -286,7 +318,7 @@ __global__ void k_sat_apply(const int* __restrict__ cs, const int* __restrict__ 
 // within a cell differs (every search result is keyed by (d2, index), so no
 // result depends on it). Bound by latency: 20,000 soundings 14.6 us against 41.8
 // for one block with its counts in its own shared memory; 50,000 soundings 24 us
-// against 43 for the eight launches (each from a cold start). For 1,000 a
+// against 43 for eight launches (each from a cold start). For 1,000 a
 // single block takes 7.8 us, the cluster 8.5.
 constexpr int kClusterBlocks = 8;       // 1 for at most 4,096 soundings (a cluster starts slower)
 constexpr int64_t kOneBlockN = 1 << 12;
@@ -487,12 +519,6 @@ __global__ void __cluster_dims__(kBlocks, 1, 1) __launch_bounds__(kSmallThreads)
     cl.sync();
 }
 
-int grid_for(int64_t n, int per_block, int cap) {
-    int64_t b = (n + per_block - 1) / per_block;
-    if (b < 1) b = 1;
-    if (b > cap) b = cap;
-    return (int)b;
-}
 
 }  // namespace
 
@@ -681,13 +707,9 @@ bg_status build_soundings(bg_ctx_s* ctx, const int32_t* x, const int32_t* y, con
         k_scan_reduce<<<nb, kThreads, 0, st>>>(count, ncells, bsum);
         k_scan_blocksums<<<1, kThreads, 0, st>>>(bsum, nb, cell_start + ncells);
         k_scan_apply<<<nb, kThreads, 0, st>>>(count, ncells, bsum, cell_start, count);
-        k_scatter<<<grid_for(n, kThreads * 4, 152 * 16), kThreads, 0, st>>>(
-            (const int4*)s->d_orig, n, g, count, (int4*)s->d_rec);
-        const dim3 sg((ncx + 1 + 255) / 256, nch);
-        k_sat_chunk<<<sg, 256, 0, st>>>(cell_start, ncx, ncy, sat_rows, csum);
-        k_sat_chunkscan<<<(ncx + 1 + 255) / 256, 256, 0, st>>>(csum, ncx, nch);
-        k_sat_apply<<<sg, 256, 0, st>>>(cell_start, csum, ncx, ncy, sat_rows, (int*)s->d_sat);
-        note_launches(8);
+        launch_scatter_sat((const int4*)s->d_orig, n, g, count, (int4*)s->d_rec, cell_start, sat_rows, nch, csum,
+                           (int*)s->d_sat, st);
+        note_launches(7);
         BG_CUDA(cudaGetLastError());
     }
 
@@ -782,14 +804,8 @@ bg_status build_hash_in_arena(const int32_t* x, const int32_t* y, const float* z
     k_scan_blocksums<<<1, kThreads, 0, st>>>(ar.bsum, (int)nb, ar.cell_start + ncells);
     k_scan_apply<<<(unsigned)nb, kThreads, 0, st>>>(ar.count, ncells, ar.bsum, ar.cell_start,
                                                     ar.count);
-    k_scatter<<<grid_for(n, kThreads * 4, 152 * 16), kThreads, 0, st>>>(ar.orig, n, g, ar.count,
-                                                                        ar.rec);
-    const dim3 sg((unsigned)((ncx + 1 + 255) / 256), (unsigned)nch);
-    k_sat_chunk<<<sg, 256, 0, st>>>(ar.cell_start, (int)ncx, (int)ncy, (int)sat_rows, ar.csum);
-    k_sat_chunkscan<<<(unsigned)((ncx + 1 + 255) / 256), 256, 0, st>>>(ar.csum, (int)ncx, (int)nch);
-    k_sat_apply<<<sg, 256, 0, st>>>(ar.cell_start, ar.csum, (int)ncx, (int)ncy, (int)sat_rows,
-                                    ar.sat);
-    note_launches(8);
+    launch_scatter_sat(ar.orig, n, g, ar.count, ar.rec, ar.cell_start, (int)sat_rows, (int)nch, ar.csum, ar.sat, st);
+    note_launches(7);
     BG_CUDA(cudaGetLastError());
 
     s->h.rec = ar.rec;
