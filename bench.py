@@ -76,13 +76,13 @@ def knn_int_ops_per_node(k):
 HASH_BYTES_PER_SOUNDING = 36.0
 
 # DRAM bytes (read + write) per node, from one ncu capture of each kernel on
-# the 2-line swath (3.384M nodes, one launch); traffic grows with the nodes of
+# one survey line (2.077M nodes, one launch); traffic grows with the nodes of
 # a launch:
-#  - k_okrige_solve<32> with the fused IDW: 451.6 MB read + 38.5 MB written,
-#    mostly the 128 B of neighbour ids per node;
-#  - k_knn_ids<32>: 20.1 MB read + 379.2 MB written (the ids).
-SOLVE_DRAM_BYTES_PER_NODE = (451.642368e6 + 38.503936e6) / 3.384e6
-KNN_DRAM_BYTES_PER_NODE = (20.107264e6 + 379.174144e6) / 3.384e6
+#  - k_okrige_solve<32> with the fused IDW: 456.5 MB read + 809.7 MB written
+#    (128 B of neighbour ids per node, and the kept tiles that leave L2);
+#  - k_knn_ids_patch<32>: 14.5 MB read + 216.3 MB written (the ids).
+SOLVE_DRAM_BYTES_PER_NODE = (456.527616e6 + 809.679104e6) / 2.076692e6
+KNN_DRAM_BYTES_PER_NODE = (14.480384e6 + 216.262656e6) / 2.076692e6
 
 
 def load_peaks():
@@ -673,7 +673,7 @@ def rooflines(prof, sep_prof, peaks, mpeaks, step_mhz, sms, w, steps, sep_mhz):
         "avg_launch_ms": avg, "nodes_per_launch": npl, "launches_per_step": s_launch / steps,
         "peak_source": f"measured FP32 FMA rate per SM cycle x {sms} SMs x {step_mhz:.0f} MHz "
                        "(median SM clock of the timed steps)",
-        "traffic_source": "ncu dram bytes of the same kernel on a 3.384M-node swath, scaled "
+        "traffic_source": "ncu dram bytes of the same kernel on a 2.077M-node line, scaled "
                           "per node",
         "hbm_frac": SOLVE_DRAM_BYTES_PER_NODE * npl / (avg / 1e3) / 1e9 / hbm}
     # k-NN ids (k = 32) of the kriging pass
@@ -683,7 +683,7 @@ def rooflines(prof, sep_prof, peaks, mpeaks, step_mhz, sms, w, steps, sep_mhz):
     ach = knn_int_ops_per_node(OK_K) * npl / (avg / 1e3) / 1e12
     byt = 4.0 * OK_K * npl
     out["knn_ids_k32"] = {
-        "bound": "alu", "kernel": "k_knn_ids<32>", "achieved": ach, "peak": int32,
+        "bound": "alu", "kernel": "k_knn_ids_patch<32>", "achieved": ach, "peak": int32,
         "unit": "Tops/s (INT32)", "frac": ach / int32,
         "int_ops_per_node": knn_int_ops_per_node(OK_K), "avg_launch_ms": avg,
         "nodes_per_launch": npl, "hbm_gbs": byt / (avg / 1e3) / 1e9,
@@ -701,7 +701,7 @@ def rooflines(prof, sep_prof, peaks, mpeaks, step_mhz, sms, w, steps, sep_mhz):
         byt = (16.0 * nval) / i_launch + 4.0 * npl
         ach = knn_int_ops_per_node(IDW_K) * npl / (avg / 1e3) / 1e12
         out["idw_k16"] = {
-            "bound": "alu", "kernel": "k_idw<16>", "achieved": ach, "peak": int32s,
+            "bound": "alu", "kernel": "k_idw_patch<16>", "achieved": ach, "peak": int32s,
             "unit": "Tops/s (INT32)", "frac": ach / int32s,
             "int_ops_per_node": knn_int_ops_per_node(IDW_K),
             "hbm": {"bytes_per_launch": byt, "achieved_gbs": byt / (avg / 1e3) / 1e9,

@@ -138,7 +138,7 @@ bg_status launch_k(const bg_soundings_s* s, const HashView& h, const GridView& g
 template <int K, int kLen>
 __global__ void __launch_bounds__(128) k_idw_pts(HashView h, PointsView q, int k, float power,
                                                  float* __restrict__ depth,
-                                                 int32_t* __restrict__ nbr) {
+                                                 int32_t* __restrict__ nbr, int* __restrict__ flag) {
     __shared__ uint64_t heap[K * 128];
     const int64_t p0 = ((int64_t)blockIdx.x * 128 + threadIdx.x) * kLen;
     if (p0 >= q.m) return;
@@ -167,13 +167,15 @@ __global__ void __launch_bounds__(128) k_idw_pts(HashView h, PointsView q, int k
         });
         if (nbr) emit_ids<128>(nbr + p * k, hp, k, keff, mask);
     };
-    knn_chain<128, decltype(emit), kLen>(h, q.x, q.y, p0, q.m, K, hp, emit);
+    knn_chain<128, decltype(emit), kLen>(h, q.x, q.y, p0, q.m, K, hp, flag, emit);
 }
 
 template <int K>
 __global__ void __launch_bounds__(128) k_idw_pts_wide(HashView h, PointsView q, int k, float power,
                                                       float* __restrict__ depth,
-                                                      int32_t* __restrict__ nbr) {
+                                                      int32_t* __restrict__ nbr,
+                                                      const int* __restrict__ flag) {
+    if (flag && *(const volatile int*)flag == 0) return;
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < q.m;
          p += (int64_t)gridDim.x * blockDim.x)
         idw_point_wide<K>(h, __ldg(q.x + p), __ldg(q.y + p), k, power, depth + p,
@@ -186,23 +188,30 @@ bg_status launch_pts_k(const HashView& h, const PointsView& q, int k, float powe
     const int len = strip_len_for(q.m);
     const int64_t threads = (q.m + len - 1) / len;
     const int64_t nb = (threads + 127) / 128;
+    int* flag = nullptr;
+    if (!query_by_lanes<K>(q.m)) {
+        const bg_status rc = dalloc(prof_ctx, (void**)&flag, sizeof(int), st);
+        if (rc != BG_OK) return rc;
+    }
+    cudaError_t e = flag ? cudaMemsetAsync(flag, 0, sizeof(int), st) : cudaSuccess;
     {
         ProfScope ps(prof_ctx, kProfIdw, q.m, st);
         if (query_by_lanes<K>(q.m))
             k_idw_query<query_lanes(K)><<<query_blocks<K>(q.m), 32 * kQueryWarps, 0, st>>>(
                 h, q, q.m, k, power, depth, nbr, nullptr);
         else if (len == 1)
-            k_idw_pts<K, 1><<<(unsigned)nb, 128, 0, st>>>(h, q, k, power, depth, nbr);
+            k_idw_pts<K, 1><<<(unsigned)nb, 128, 0, st>>>(h, q, k, power, depth, nbr, flag);
         else if (len == 2)
-            k_idw_pts<K, 2><<<(unsigned)nb, 128, 0, st>>>(h, q, k, power, depth, nbr);
+            k_idw_pts<K, 2><<<(unsigned)nb, 128, 0, st>>>(h, q, k, power, depth, nbr, flag);
         else
-            k_idw_pts<K, 4><<<(unsigned)nb, 128, 0, st>>>(h, q, k, power, depth, nbr);
+            k_idw_pts<K, 4><<<(unsigned)nb, 128, 0, st>>>(h, q, k, power, depth, nbr, flag);
     }
     k_idw_pts_wide<K><<<(unsigned)std::min<int64_t>((q.m + 127) / 128, 152 * 4), 128, 0, st>>>(
-        h, q, k, power, depth, nbr);
+        h, q, k, power, depth, nbr, flag);
     note_launches(2);
-    BG_CUDA(cudaGetLastError());
-    return BG_OK;
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (flag) dfree(prof_ctx, flag, sizeof(int), st);
+    return e == cudaSuccess ? BG_OK : cuda_fail(e, "IDW launch");
 }
 
 }  // namespace

@@ -496,9 +496,10 @@ __device__ __forceinline__ bool query_in_range(int qx, int qy) {
 }
 
 // May this point have been left to the wide pass? Not where the hash's farthest
-// corner fits a packed key: the usual case, so that the wide pass of a list of
-// points reads the points and nothing else, and needs no flag (whose allocation
-// and clearing cost a call 4 us).
+// corner fits a packed key, the usual case: then the wide pass of a short list needs
+// no flag, whose allocation and clearing cost a call 4 us. For a long list (over
+// the line of query_by_lanes) the flag is cheaper than a pass over the points (3.4M
+// points: 0.08 of 2.1 ms).
 __device__ __forceinline__ bool point_may_be_wide(const HashView& h, int qx, int qy) {
     if (h.n_valid == 0 || !query_in_range(qx, qy)) return false;
     const int64_t x = (int64_t)qx - h.hx0, y = (int64_t)qy - h.hy0;
@@ -510,11 +511,11 @@ __device__ __forceinline__ bool point_may_be_wide(const HashView& h, int qx, int
 // Packed-key k-NN of points p0 .. p0 + kLen - 1 (those below m). emit(p, cnt)
 // runs after each point with its keys sorted ascending in hp[0 .. cnt), or
 // with cnt = -1 for a point outside the coordinate range; a point whose table
-// bound does not fit the packed key is left to the wide pass.
+// bound does not fit the packed key is left to the wide pass (*flag = 1).
 template <int S, class Emit, int kLen = kStrip>
 __device__ __forceinline__ void knn_chain(const HashView& h, const int32_t* __restrict__ px,
                                           const int32_t* __restrict__ py, int64_t p0, int64_t m,
-                                          int kc, uint64_t* hp, Emit emit) {
+                                          int kc, uint64_t* hp, int* flag, Emit emit) {
     int64_t prev = -1;  // K-th squared distance of the previous point, -1 if none
     int qxp = 0, qyp = 0;
     for (int s = 0; s < kLen; ++s) {
@@ -541,6 +542,7 @@ __device__ __forceinline__ void knn_chain(const HashView& h, const int32_t* __re
         if (!ok) {
             b = knn_bound_rt(h, qx, qy, kc);
             if (!packed_fits(h, b.tau0)) {
+                *flag = 1;
                 prev = -1;
                 continue;
             }

@@ -285,7 +285,8 @@ bg_status launch_k(const bg_soundings_s* snd, const HashView& h, const GridView&
 // points [p0, p1), kLen consecutive points per thread (strip_len_for)
 template <int K, int kLen>
 __global__ void __launch_bounds__(128) k_knn_ids_pts(HashView h, PointsView q, int k, int64_t p0,
-                                                     int64_t p1, int32_t* __restrict__ ids) {
+                                                     int64_t p1, int32_t* __restrict__ ids,
+                                                     int* __restrict__ flag) {
     __shared__ uint64_t heap[K * 128];
     const int64_t a = p0 + ((int64_t)blockIdx.x * 128 + threadIdx.x) * kLen;
     if (a >= p1) return;
@@ -297,13 +298,15 @@ __global__ void __launch_bounds__(128) k_knn_ids_pts(HashView h, PointsView q, i
     }
     const uint64_t mask = (1ull << h.idx_bits) - 1;
     auto emit = [&](int64_t p, int cnt) { emit_ids<128>(ids + (p - p0) * k, hp, k, cnt, mask); };
-    knn_chain<128, decltype(emit), kLen>(h, q.x, q.y, a, p1, K, hp, emit);
+    knn_chain<128, decltype(emit), kLen>(h, q.x, q.y, a, p1, K, hp, flag, emit);
 }
 
 template <int K>
 __global__ void __launch_bounds__(128) k_knn_ids_pts_wide(HashView h, PointsView q, int k,
                                                           int64_t p0, int64_t p1,
-                                                          int32_t* __restrict__ ids) {
+                                                          int32_t* __restrict__ ids,
+                                                          const int* __restrict__ flag) {
+    if (flag && *(const volatile int*)flag == 0) return;
     for (int64_t p = p0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < p1;
          p += (int64_t)gridDim.x * blockDim.x)
         knn_ids_point_wide<K>(h, __ldg(q.x + p), __ldg(q.y + p), k, ids + (p - p0) * k);
@@ -329,36 +332,45 @@ bg_status launch_pts_k(const HashView& h, const PointsView& q, int k, const OkPa
     // passed nbr_out, which then holds all ids
     int64_t per = q.m;
     if (!nbr) per = std::min<int64_t>(q.m, std::max<int64_t>(4096, ((int64_t)1 << 28) / k));
+    const size_t flag_bytes = 256;
     const size_t id_bytes = nbr ? 0 : (size_t)per * k * sizeof(int32_t);
     void* scratch = nullptr;
-    bg_status rc = nbr ? BG_OK : dalloc(ctx, &scratch, id_bytes, st);
+    const bool flagged = !query_by_lanes<K>(per);
+    const size_t bytes = id_bytes + (flagged ? flag_bytes : 0);
+    bg_status rc = bytes ? dalloc(ctx, &scratch, bytes, st) : BG_OK;
     if (rc != BG_OK) return rc;
+    int* flag = flagged ? (int*)((char*)scratch + id_bytes) : nullptr;
     const cudaError_t ea = cudaFuncSetAttribute(
         k_okrige_solve_pts<K, kSph>, cudaFuncAttributeMaxDynamicSharedMemorySize, Gm::SMEM);
     if (ea != cudaSuccess) {
-        if (scratch) dfree(ctx, scratch, id_bytes, st);
+        if (scratch) dfree(ctx, scratch, bytes, st);
         return cuda_fail(ea, "solve shared-memory size");
     }
     for (int64_t p0 = 0; p0 < q.m; p0 += per) {
         const int64_t p1 = std::min<int64_t>(q.m, p0 + per);
         const int64_t n = p1 - p0;
         int32_t* chunk_ids = nbr ? nbr + p0 * k : (int32_t*)scratch;
+        cudaError_t e = flag ? cudaMemsetAsync(flag, 0, sizeof(int), st) : cudaSuccess;
+        if (e != cudaSuccess) {
+            rc = cuda_fail(e, "memset");
+            break;
+        }
         const int len = strip_len_for(n);
         const int64_t nb = ((n + len - 1) / len + 127) / 128;
         {
             ProfScope ps(ctx, kProfKnnIds, n, st);
             if (query_by_lanes<K>(n))
                 k_knn_ids_query<query_lanes(K)><<<query_blocks<K>(n), 32 * kQueryWarps, 0, st>>>(
-                    h, q, p0, n, k, chunk_ids, nullptr);
+                    h, q, p0, n, k, chunk_ids, flag);
             else if (len == 1)
-                k_knn_ids_pts<K, 1><<<(unsigned)nb, 128, 0, st>>>(h, q, k, p0, p1, chunk_ids);
+                k_knn_ids_pts<K, 1><<<(unsigned)nb, 128, 0, st>>>(h, q, k, p0, p1, chunk_ids, flag);
             else if (len == 2)
-                k_knn_ids_pts<K, 2><<<(unsigned)nb, 128, 0, st>>>(h, q, k, p0, p1, chunk_ids);
+                k_knn_ids_pts<K, 2><<<(unsigned)nb, 128, 0, st>>>(h, q, k, p0, p1, chunk_ids, flag);
             else
-                k_knn_ids_pts<K, 4><<<(unsigned)nb, 128, 0, st>>>(h, q, k, p0, p1, chunk_ids);
+                k_knn_ids_pts<K, 4><<<(unsigned)nb, 128, 0, st>>>(h, q, k, p0, p1, chunk_ids, flag);
         }
         k_knn_ids_pts_wide<K><<<(unsigned)std::min<int64_t>((n + 127) / 128, 152 * 4), 128, 0, st>>>(
-            h, q, k, p0, p1, chunk_ids);
+            h, q, k, p0, p1, chunk_ids, flag);
         const int64_t batches = (n + kSolveSystems - 1) / kSolveSystems;
         const int bper = solve_batches_per_block<K>(batches);
         {
@@ -368,13 +380,13 @@ bg_status launch_pts_k(const HashView& h, const PointsView& q, int k, const OkPa
                     h, q, k, p, p0, n, IdsView{chunk_ids, 0, 0, 0, 0}, depth, var, bper);
         }
         note_launches(3);
-        const cudaError_t e = cudaGetLastError();
+        e = cudaGetLastError();
         if (e != cudaSuccess) {
             rc = cuda_fail(e, "kriging launch");
             break;
         }
     }
-    if (scratch) dfree(ctx, scratch, id_bytes, st);
+    if (scratch) dfree(ctx, scratch, bytes, st);
     return rc;
 }
 
