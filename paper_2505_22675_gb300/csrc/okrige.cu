@@ -76,10 +76,11 @@ __global__ void __launch_bounds__(64, KnnWarp<K>::kBlocksPerSM) k_knn_ids_patch(
         });
 }
 
-// The ids of queries i0 .. i0 + m - 1, G lanes each, as upload indices.
+// The ids of queries i0 .. i0 + m - 1, G lanes each (put_point_id).
 template <int G, class Queries>
 __global__ void __launch_bounds__(32 * kQueryWarps) k_knn_ids_query(HashView h, Queries q, int64_t i0, int64_t m, int k,
-                                                                   int32_t* __restrict__ ids, int* __restrict__ flag) {
+                                                                   int32_t* __restrict__ ids, int64_t stride,
+                                                                   int* __restrict__ flag) {
     __shared__ uint64_t buf[32 * kQueryWarps * 2];
     const int n = threadIdx.x / G, lane = threadIdx.x & (G - 1);
     const int64_t i = (int64_t)blockIdx.x * (32 * kQueryWarps / G) + n;
@@ -91,7 +92,8 @@ __global__ void __launch_bounds__(32 * kQueryWarps) k_knn_ids_query(HashView h, 
     if (cnt < 0) {
         if (lane == 0 && flag) *flag = 1;
     } else if (lane < k) {
-        ids[i * k + lane] = lane < cnt ? (int)(key & ((1ull << h.idx_bits) - 1)) : -1;
+        put_point_id(ids + i * (stride > 0 ? 1 : k), stride, lane,
+                     lane < cnt ? (int)(key & ((1ull << h.idx_bits) - 1)) : -1);
     }
 }
 
@@ -232,7 +234,7 @@ bg_status launch_k(const bg_soundings_s* snd, const HashView& h, const GridView&
                     h, g, k, ids, slot_ids ? nbr : nullptr, flag, plen, spr);
             else if (query_by_lanes<K>(nodes))
                 k_knn_ids_query<query_lanes(K)><<<query_blocks<K>(nodes), 32 * kQueryWarps, 0, st>>>(
-                    h, g, j0 * g.nx, nodes, k, chunk_ids, flag);
+                    h, g, j0 * g.nx, nodes, k, chunk_ids, 0, flag);
             else if (len == 1)
                 k_knn_ids<K, 1><<<(unsigned)nbs, 64, 0, st>>>(h, g, k, (int)j0, (int)j1, chunk_ids, flag);
             else if (len == 2)
@@ -285,7 +287,7 @@ bg_status launch_k(const bg_soundings_s* snd, const HashView& h, const GridView&
 // points [p0, p1), kLen consecutive points per thread (strip_len_for)
 template <int K, int kLen>
 __global__ void __launch_bounds__(128) k_knn_ids_pts(HashView h, PointsView q, int k, int64_t p0,
-                                                     int64_t p1, int32_t* __restrict__ ids,
+                                                     int64_t p1, int32_t* __restrict__ ids, int64_t stride,
                                                      int* __restrict__ flag) {
     __shared__ uint64_t heap[K * 128];
     const int64_t a = p0 + ((int64_t)blockIdx.x * 128 + threadIdx.x) * kLen;
@@ -293,23 +295,29 @@ __global__ void __launch_bounds__(128) k_knn_ids_pts(HashView h, PointsView q, i
     uint64_t* hp = heap + threadIdx.x;
     if (h.n_valid == 0) {
         for (int64_t p = a; p < min(a + kLen, p1); ++p)
-            for (int i = 0; i < k; ++i) ids[(p - p0) * k + i] = -1;
+            for (int i = 0; i < k; ++i) put_point_id(ids + (p - p0) * (stride > 0 ? 1 : k), stride, i, -1);
         return;
     }
     const uint64_t mask = (1ull << h.idx_bits) - 1;
-    auto emit = [&](int64_t p, int cnt) { emit_ids<128>(ids + (p - p0) * k, hp, k, cnt, mask); };
+    auto emit = [&](int64_t p, int cnt) {
+        if (stride > 0)
+            for (int i = 0; i < k; ++i)
+                put_point_id(ids + (p - p0), stride, i, i < cnt ? (int)(hp[i * 128] & mask) : -1);
+        else
+            emit_ids<128>(ids + (p - p0) * k, hp, k, cnt, mask);
+    };
     knn_chain<128, decltype(emit), kLen>(h, q.x, q.y, a, p1, K, hp, flag, emit);
 }
 
 template <int K>
 __global__ void __launch_bounds__(128) k_knn_ids_pts_wide(HashView h, PointsView q, int k,
                                                           int64_t p0, int64_t p1,
-                                                          int32_t* __restrict__ ids,
+                                                          int32_t* __restrict__ ids, int64_t stride,
                                                           const int* __restrict__ flag) {
     if (flag && *(const volatile int*)flag == 0) return;
     for (int64_t p = p0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < p1;
          p += (int64_t)gridDim.x * blockDim.x)
-        knn_ids_point_wide<K>(h, __ldg(q.x + p), __ldg(q.y + p), k, ids + (p - p0) * k);
+        knn_ids_point_wide<K>(h, __ldg(q.x + p), __ldg(q.y + p), k, ids + (p - p0) * (stride > 0 ? 1 : k), stride);
 }
 
 // dynamic shared memory: Geo<K>::SMEM bytes
@@ -350,6 +358,7 @@ bg_status launch_pts_k(const HashView& h, const PointsView& q, int k, const OkPa
         const int64_t p1 = std::min<int64_t>(q.m, p0 + per);
         const int64_t n = p1 - p0;
         int32_t* chunk_ids = nbr ? nbr + p0 * k : (int32_t*)scratch;
+        const int64_t stride = nbr ? 0 : n;
         cudaError_t e = flag ? cudaMemsetAsync(flag, 0, sizeof(int), st) : cudaSuccess;
         if (e != cudaSuccess) {
             rc = cuda_fail(e, "memset");
@@ -361,23 +370,23 @@ bg_status launch_pts_k(const HashView& h, const PointsView& q, int k, const OkPa
             ProfScope ps(ctx, kProfKnnIds, n, st);
             if (query_by_lanes<K>(n))
                 k_knn_ids_query<query_lanes(K)><<<query_blocks<K>(n), 32 * kQueryWarps, 0, st>>>(
-                    h, q, p0, n, k, chunk_ids, flag);
+                    h, q, p0, n, k, chunk_ids, stride, flag);
             else if (len == 1)
-                k_knn_ids_pts<K, 1><<<(unsigned)nb, 128, 0, st>>>(h, q, k, p0, p1, chunk_ids, flag);
+                k_knn_ids_pts<K, 1><<<(unsigned)nb, 128, 0, st>>>(h, q, k, p0, p1, chunk_ids, stride, flag);
             else if (len == 2)
-                k_knn_ids_pts<K, 2><<<(unsigned)nb, 128, 0, st>>>(h, q, k, p0, p1, chunk_ids, flag);
+                k_knn_ids_pts<K, 2><<<(unsigned)nb, 128, 0, st>>>(h, q, k, p0, p1, chunk_ids, stride, flag);
             else
-                k_knn_ids_pts<K, 4><<<(unsigned)nb, 128, 0, st>>>(h, q, k, p0, p1, chunk_ids, flag);
+                k_knn_ids_pts<K, 4><<<(unsigned)nb, 128, 0, st>>>(h, q, k, p0, p1, chunk_ids, stride, flag);
         }
         k_knn_ids_pts_wide<K><<<(unsigned)std::min<int64_t>((n + 127) / 128, 152 * 4), 128, 0, st>>>(
-            h, q, k, p0, p1, chunk_ids, flag);
+            h, q, k, p0, p1, chunk_ids, stride, flag);
         const int64_t batches = (n + kSolveSystems - 1) / kSolveSystems;
         const int bper = solve_batches_per_block<K>(batches);
         {
             ProfScope ps(ctx, kProfSolve, n, st);
             k_okrige_solve_pts<K, kSph>
                 <<<(unsigned)((batches + bper - 1) / bper), Gm::THREADS, Gm::SMEM, st>>>(
-                    h, q, k, p, p0, n, IdsView{chunk_ids, 0, 0, 0, 0}, depth, var, bper);
+                    h, q, k, p, p0, n, IdsView{chunk_ids, stride, 0, 0, 0}, depth, var, bper);
         }
         note_launches(3);
         e = cudaGetLastError();

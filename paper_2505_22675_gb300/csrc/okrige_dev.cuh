@@ -331,11 +331,22 @@ __device__ __forceinline__ void knn_ids_node_wide(const HashView& h, const GridV
     }
 }
 
+// Neighbour i of a query point, upload index u (-1: none), to o: the first slot of
+// its list with stride 0 (the caller's lists), else its slot of the patches layout,
+// which the solve reads in whole lines (a line per lane otherwise: 209,715 points k =
+// 32: solve 289 -> 282 us).
+__device__ __forceinline__ void put_point_id(int32_t* o, int64_t stride, int i, int u) {
+    if (stride > 0)
+        o[i * stride] = u < 0 ? -1 : -2 - u;
+    else
+        o[i] = u;
+}
+
 // Wide-key neighbour ids of one query point whose table bound does not fit
 // the packed key; other points return.
 template <int K>
 __device__ __forceinline__ void knn_ids_point_wide(const HashView& h, int qx, int qy, int k,
-                                                   int32_t* __restrict__ o) {
+                                                   int32_t* __restrict__ o, int64_t stride) {
     if (!point_may_be_wide(h, qx, qy)) return;
     const Bound b = knn_bound<K>(h, qx, qy);
     if (packed_fits(h, b.tau0)) return;
@@ -344,7 +355,7 @@ __device__ __forceinline__ void knn_ids_point_wide(const HashView& h, int qx, in
     const int keff = knn_scan_wide<K>(h, qx, qy, b, d2, id);
 #pragma unroll
     for (int i = 0; i < K; ++i)
-        if (i < k) o[i] = i < keff ? id[i] : -1;
+        if (i < k) put_point_id(o, stride, i, i < keff ? id[i] : -1);
 }
 
 // ---------------------------------------------------------------- solve
@@ -446,7 +457,7 @@ __device__ __forceinline__ void prefetch_ids_l2(const IdsView& v, int64_t nsys, 
             asm volatile("prefetch.global.L2 [%0];" ::"l"(v.p + (sys + t) * k));
     } else if (sys < nsys) {
         for (int q = t; q < 4 * k; q += blockDim.x)  // 128 systems: four lines per neighbour
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(v.p + (q >> 2) * v.stride + sys + (q & 3) * 32));
+            if (sys + (q & 3) * 32 < nsys) asm volatile("prefetch.global.L2 [%0];" ::"l"(v.p + (q >> 2) * v.stride + sys + (q & 3) * 32));
     }
 }
 
