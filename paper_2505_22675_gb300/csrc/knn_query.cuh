@@ -41,10 +41,13 @@ inline unsigned query_blocks(int64_t m) {
 //   45,000    35 / 41     55 / 41     90 / 74
 //   60,000    35 / 49     55 / 52     99 / 95
 //   80,000    36 / 60     56 / 64    117 / 124
-// (1 % and 10 %: the same signs at k = 8; at the others the lines hold too).
+// and of 1 %, where a thread's records are farther apart:
+//   60,000    35 / 51     67 / 61    158 / 107
+//   80,000    47 / 65     78 / 76    181 / 131    (k = 16, ids 92 / 72)
+// The line of k = 16 lies where the sparse lists gain what the dense ones lose.
 template <int K>
 inline bool query_by_lanes(int64_t m) {
-    return m <= (K <= 8 ? 152 * 224 : 152 * 384);
+    return m <= (K <= 8 ? 152 * 224 : K == 16 ? 152 * 576 : 152 * 384);
 }
 
 // G lanes (16 or 32) work on a query; both halves of a warp take every step

@@ -99,11 +99,11 @@ def test_kriging_systems_of_every_size(name, model, nugget, k):
 
 
 @pytest.mark.parametrize("k", [3, 8, 13, 32])
-@pytest.mark.parametrize("rows", [170, 291, 292])
+@pytest.mark.parametrize("rows", [170, 171, 291, 292, 437, 438])
 @pytest.mark.parametrize("name", ["uniform", "lattice", "gap"])
 def test_queries_by_warps_and_by_threads(name, rows, k):
     """The largest grids of lanes of a warp each where patches do not serve (200 x
-    170 nodes for k <= 8, x 291 beyond) and the next of a thread each, as a grid of many soundings per node and as a list of points."""
+    170 nodes for k <= 8, x 437 up to 16, x 291 beyond) and the next of a thread each, as a grid of many soundings per node and as a list of points."""
     import torch
     make, cell = {"uniform": (lambda: _uniform(21, 400_000, 20_000, 29_200), 100),
                   "lattice": (lambda: _lattice(400, 600, 50), 100),
