@@ -138,19 +138,21 @@ __device__ __forceinline__ float sqrt_approx(float x) {
 // 1 - exp(-t) for two t in [0, 25] at once (past 25 it is 1 in any case), for the
 // exponential model: a solve is bound by its instructions, and two entries share
 // each here, which a library call for each cannot (k = 12, 170,163 systems: solve
-// 104 -> 74 us). Argument reduction of Cody and Waite: t = n ln 2 + r, |r| <=
-// ln 2 / 2; 1 - exp(-r) = r - r^2 q(r), q of degree 4 by interpolation at the
-// Chebyshev nodes of that interval (off by 6e-8 at most); then (1 - s) + s (1 -
-// exp(-r)), s = 2^-n, which does not cancel at short range. Errors, 2e6 draws in
-// each of nine intervals: 1.01 ulp at most, 0.22 to 0.35 rms (-expm1f: 1.13, 0.22
-// to 0.50).
+// 104 -> 75 us). Argument reduction of Cody and Waite: t = n ln 2 + r, |r| <= ln 2
+// / 2; 1 - exp(-r) = r - r^2 q(r), q of degree 5 by interpolation at the Chebyshev
+// nodes of that interval (off by 1.3e-9 at most); then (1 - s) + s (1 - exp(-r)), s
+// = 2^-n, which does not cancel at short range. Errors, 2e6 draws in each of nine
+// intervals: 0.89 ulp at most, 0.22 to 0.34 rms (-expm1f: 1.13, 0.22 to 0.50; with
+// q of degree 4 1.01, 0.22 to 0.35 and 2 us less, but the variances of some ranges
+// 3 % further off than with the library call; so 1 to 6 % nearer).
 __device__ __forceinline__ u64 one_minus_exp2(u64 t) {
     const u64 magic = dup2(12582912.0f);  // 1.5 * 2^23: the low bits of a sum hold the integer
     const u64 y = fma2(t, dup2(1.44269504f), magic);
     const u64 r = fma2(sub2(y, magic), dup2(-0.693147181f), t);
-    u64 q = fma2(dup2(-0.00139261840f), r, dup2(0.00836317893f));
-    q = fma2(q, r, dup2(-0.0416665561f));
-    q = fma2(q, r, dup2(0.166665763f));
+    u64 q = fma2(dup2(0.000198909911f), r, dup2(-0.00139336498f));
+    q = fma2(q, r, dup2(0.00833331048f));
+    q = fma2(q, r, dup2(-0.0416664667f));
+    q = fma2(q, r, dup2(0.166666672f));
     q = fma2(q, r, dup2(-0.5f));
     const u64 m = fma2(mul2(r, r), q, r);
     const auto pow2 = [](float v) {  // 2^-n
