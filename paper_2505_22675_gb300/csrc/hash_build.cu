@@ -354,11 +354,13 @@ __device__ __forceinline__ int block_excl_scan_1024(int v, int* ws) {
     return ws[w] + inc - v;
 }
 
-// pack: also write the upload-order records (when no earlier pass did).
+// x, y, z: NULL where an earlier pass has written the upload-order records, else
+// arrays of the library's own (this build runs after the upload has returned, when
+// the caller's may have changed) that it packs first.
 template <int kBlocks>
 __global__ void __cluster_dims__(kBlocks, 1, 1) __launch_bounds__(kSmallThreads) k_hash_cluster(
     const int32_t* __restrict__ x, const int32_t* __restrict__ y, const float* __restrict__ z,
-    int n, int pack, int4* __restrict__ orig, CellGeom g, int* __restrict__ cell_start,
+    int n, int4* __restrict__ orig, CellGeom g, int* __restrict__ cell_start,
     int4* __restrict__ rec, int* __restrict__ sat) {
     namespace cg = cooperative_groups;
     extern __shared__ int cnt[];
@@ -373,11 +375,15 @@ __global__ void __cluster_dims__(kBlocks, 1, 1) __launch_bounds__(kSmallThreads)
     const int i0 = (int)((int64_t)n * rank / kBlocks), i1 = (int)((int64_t)n * (rank + 1) / kBlocks);
 #pragma unroll 2
     for (int i = i0 + tid; i < i1; i += kSmallThreads) {
-        const int xi = x[i], yi = y[i];
-        const float zi = z[i];
-        const int valid = isnan(zi) ? 0 : 1;
-        if (pack) orig[i] = make_int4(xi, yi, __float_as_int(zi), valid);
-        if (valid) atomicAdd(&cnt[cell_index(g, xi, yi)], 1);
+        int4 r;
+        if (x) {
+            const float zi = z[i];
+            r = make_int4(x[i], y[i], __float_as_int(zi), isnan(zi) ? 0 : 1);
+            orig[i] = r;
+        } else {
+            r = orig[i];
+        }
+        if (r.w) atomicAdd(&cnt[cell_index(g, r.x, r.y)], 1);
     }
     cl.sync();
     // this block's rows of cells: total of each cell, and the eight counts to
@@ -453,24 +459,24 @@ __global__ void __cluster_dims__(kBlocks, 1, 1) __launch_bounds__(kSmallThreads)
         }
     }
 #pragma unroll 2
-    for (int i = i0 + tid; i < i1; i += kSmallThreads) {
-        const float zi = z[i];
-        if (!isnan(zi)) {
-            const int xi = x[i], yi = y[i];
-            const int pos = atomicAdd(&cnt[cell_index(g, xi, yi)], 1);
-            rec[pos] = make_int4(xi, yi, __float_as_int(zi), i);
+    for (int i = i0 + tid; i < i1; i += kSmallThreads) {  // (the thread's own records)
+        const int4 r = orig[i];
+        if (r.w) {
+            const int pos = atomicAdd(&cnt[cell_index(g, r.x, r.y)], 1);
+            rec[pos] = make_int4(r.x, r.y, r.z, i);
         }
     }
     cl.sync();  // no block leaves while another reads its shared memory
 }
 
 // Bounding box of a small input by one cluster, straight to page-locked host
-// memory: no accumulator to set up and no copy. out: min x, min y, max x, max y,
-// valid count, out-of-range count.
+// memory: no accumulator to set up and no copy. It also packs the upload-order
+// records: nothing reads the caller's arrays after it. out: min x, min y, max x, max
+// y, valid count, out-of-range count.
 template <int kBlocks>
 __global__ void __cluster_dims__(kBlocks, 1, 1) __launch_bounds__(kSmallThreads) k_bbox_cluster(
     const int32_t* __restrict__ x, const int32_t* __restrict__ y, const float* __restrict__ z, int n,
-    int* __restrict__ out) {
+    int4* __restrict__ orig, int* __restrict__ out) {
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
     __shared__ int sm[32][6];
@@ -481,7 +487,10 @@ __global__ void __cluster_dims__(kBlocks, 1, 1) __launch_bounds__(kSmallThreads)
 #pragma unroll 4
     for (int i = i0 + threadIdx.x; i < i1; i += kSmallThreads) {
         const int xi = x[i], yi = y[i];
-        if (!isnan(z[i])) {
+        const float zi = z[i];
+        const int valid = isnan(zi) ? 0 : 1;
+        orig[i] = make_int4(xi, yi, __float_as_int(zi), valid);
+        if (valid) {
             v[0] = min(v[0], xi);
             v[1] = min(v[1], yi);
             v[2] = max(v[2], xi);
@@ -573,6 +582,10 @@ bool cluster_takes(const int32_t* a, int64_t n, int64_t cs) {
 bg_status build_soundings(bg_ctx_s* ctx, const int32_t* x, const int32_t* y, const float* z,
                           int64_t n, int on_device, int32_t cell_hint, cudaStream_t st,
                           bg_soundings_s* s, const HostBBox* known) {
+    if (known && on_device) {  // (the arrays are read after the return)
+        set_error("a known bounding box goes with host arrays");
+        return BG_ERR_INTERNAL;
+    }
     bg_status rc = BG_OK;
     const int32_t *dx = x, *dy = y;
     const float* dz = z;
@@ -602,9 +615,10 @@ bg_status build_soundings(bg_ctx_s* ctx, const int32_t* x, const int32_t* y, con
         s->bytes += (size_t)n * 16;
         s->h.orig = (const int4*)s->d_orig;
     }
-    // a small input is packed by the one-cluster build itself, where that takes it;
-    // its bounding box comes from the caller's scan or from a cluster that writes
-    // it to the host
+    // The records are packed before the one synchronization, by the pass that finds the
+    // bounding box, so that the caller may reuse its arrays on return. With the box
+    // known there is no such pass, and no array of the caller's: the one-cluster build
+    // packs by itself.
     bool packed = false;
     auto pack = [&](int* acc) {
         if (acc) k_bbox_init<<<1, 32, 0, st>>>(acc);
@@ -635,11 +649,12 @@ bg_status build_soundings(bg_ctx_s* ctx, const int32_t* x, const int32_t* y, con
             BG_CUDA(cudaMemcpyAsync(ctx->h_pinned, acc, 6 * sizeof(int), cudaMemcpyDeviceToHost, st));
         } else {
             if (cluster_blocks(n) == 1)
-                k_bbox_cluster<1><<<1, kSmallThreads, 0, st>>>(dx, dy, dz, (int)n, ctx->h_pinned);
+                k_bbox_cluster<1><<<1, kSmallThreads, 0, st>>>(dx, dy, dz, (int)n, (int4*)s->d_orig, ctx->h_pinned);
             else
-                k_bbox_cluster<kClusterBlocks><<<kClusterBlocks, kSmallThreads, 0, st>>>(dx, dy, dz, (int)n,
-                                                                                         ctx->h_pinned);
+                k_bbox_cluster<kClusterBlocks><<<kClusterBlocks, kSmallThreads, 0, st>>>(
+                    dx, dy, dz, (int)n, (int4*)s->d_orig, ctx->h_pinned);
             note_launches(1);
+            packed = true;
             BG_CUDA(cudaGetLastError());
         }
         BG_CUDA(cudaStreamSynchronize(st));
@@ -683,7 +698,8 @@ bg_status build_soundings(bg_ctx_s* ctx, const int32_t* x, const int32_t* y, con
         const auto kernel = cluster_blocks(n) == 1 ? k_hash_cluster<1> : k_hash_cluster<kClusterBlocks>;
         if (smem > (48 << 10))
             BG_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClusterSmem));
-        kernel<<<cluster_blocks(n), kSmallThreads, smem, st>>>(dx, dy, dz, (int)n, packed ? 0 : 1, (int4*)s->d_orig, g,
+        kernel<<<cluster_blocks(n), kSmallThreads, smem, st>>>(packed ? nullptr : dx, packed ? nullptr : dy,
+                                                               packed ? nullptr : dz, (int)n, (int4*)s->d_orig, g,
                                                                cell_start, (int4*)s->d_rec, (int*)s->d_sat);
         note_launches(1);
         BG_CUDA(cudaGetLastError());
