@@ -467,7 +467,10 @@ __global__ void __launch_bounds__(Geo<K>::THREADS, Geo<K>::BLOCKS) k_batch_solve
     tmem_give<Geo<K>::COLS>(&slot);
 }
 
-// 7. wide-key pass over every item of every tile; returns at once unless flagged
+// 7. wide-key pass over every item of every tile; returns at once unless flagged. It
+// takes the nodes whose bound for K soundings does not fit: what a search left to it,
+// by patches (bound for K) or by threads (for k <= K, so the bound for K is no
+// smaller), is among them, and what else is comes out the same.
 template <int K>
 __device__ __forceinline__ void wide_node(const TileDesc& d, const HashView& h, NodeIdx nd) {
     const GridView& g = d.g;
@@ -475,12 +478,11 @@ __device__ __forceinline__ void wide_node(const TileDesc& d, const HashView& h, 
     const int64_t node = (int64_t)nd.j * g.nx + nd.i;
     const int qx = g.x0 + nd.i * g.cell + g.cell / 2;
     const int qy = g.y0 + nd.j * g.cell + g.cell / 2;
-    const int kq = d.method == 0 ? d.k : d.K;
-    const Bound b = knn_bound_rt(h, qx, qy, kq);
+    const Bound b = knn_bound_rt(h, qx, qy, d.K);
     if (packed_fits(h, b.tau0)) return;
     uint64_t d2[K];
     int id[K];
-    // the bound above used kq <= K soundings; the K-slot scan keeps the kq nearest in front
+    // the bound above used d.K <= K soundings; the K-slot scan keeps the nearest in front
     const int keff = min(knn_scan_wide<K>(h, qx, qy, b, d2, id), d.k);
     if (d.method == 0) {
         d.depth[node] = idw_from(h, keff, d.power, [&](int i, uint64_t& dd, int& ii) {
@@ -511,10 +513,9 @@ __global__ void __launch_bounds__(kItemThreads) k_batch_wide(
         const HashView h = tile_view(d, orig, rec, cell_start, sat);
         const int64_t patch = item - __ldg(item_off + t);
         const NodeIdx nd = patch_node((int)(patch % d.gx), (int)(patch / d.gx), warp, lane);
-        const int kq = d.method == 0 ? d.k : d.K;
-        if (kq <= 8)
+        if (d.K <= 8)
             wide_node<8>(d, h, nd);
-        else if (kq <= 16)
+        else if (d.K <= 16)
             wide_node<16>(d, h, nd);
         else
             wide_node<32>(d, h, nd);
