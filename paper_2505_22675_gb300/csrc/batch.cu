@@ -342,12 +342,12 @@ __global__ void __launch_bounds__(64, KnnWarp<K>::kBlocksPerSM) k_batch_knn_patc
                     if (d.method == 0)
                         idw_served<K>(h, sm, ux, uy, k, d.power, d.depth + out(i, j), nullptr);
                     else
-                        ids_served<K>(h, sm, k, slot(i, j), ids.stride, nullptr);
+                        ids_served<K>(h, sm, k, slot(i, j), ids.stride);
                 },
                 [&](int i, int j, int qx, int qy, uint64_t* hp) {
                     if (d.method == 0)
                         return idw_lone<K>(h, qx, qy, hp, k, d.power, d.depth + out(i, j), nullptr);
-                    return ids_lone<K>(h, qx, qy, hp, k, slot(i, j), ids.stride, nullptr);
+                    return ids_lone<K>(h, qx, qy, hp, k, slot(i, j), ids.stride);
                 });
     }
 }

@@ -51,11 +51,10 @@ __global__ void __launch_bounds__(64) k_knn_ids(HashView h, GridView g, int k, i
 }
 
 // The same by patches of 8 x 4 nodes per warp (knn_warp.cuh), a strip of `len`
-// patches along x each, spr strips per patch row, into either layout (and, as
-// upload indices, to nbr [node][k], if any).
+// patches along x each, spr strips per patch row, into either layout.
 template <int K>
 __global__ void __launch_bounds__(64, KnnWarp<K>::kBlocksPerSM) k_knn_ids_patch(HashView h, GridView g, int k,
-                                                                                IdsView ids, int32_t* __restrict__ nbr,
+                                                                                IdsView ids,
                                                                                 int* __restrict__ flag, int len,
                                                                                 int spr) {
     __shared__ typename KnnWarp<K>::Smem smem[2];
@@ -67,12 +66,11 @@ __global__ void __launch_bounds__(64, KnnWarp<K>::kBlocksPerSM) k_knn_ids_patch(
     auto slot = [&](int i, int j) {
         return ids.p + (ids.stride > 0 ? node_slot(ids, i, j) : ((int64_t)(j - ids.j0) * g.nx + i) * k);
     };
-    auto list = [&](int i, int j) { return nbr ? nbr + ((int64_t)j * g.nx + i) * k : nullptr; };
     knn_patch_row<K>(
         h, g, sm, jb, ids.j1, p0, p0 + len, flag,
-        [&](int i, int j, int, int) { ids_served<K>(h, sm, k, slot(i, j), ids.stride, list(i, j)); },
+        [&](int i, int j, int, int) { ids_served<K>(h, sm, k, slot(i, j), ids.stride); },
         [&](int i, int j, int qx, int qy, uint64_t* hp) {
-            return ids_lone<K>(h, qx, qy, hp, k, slot(i, j), ids.stride, list(i, j));
+            return ids_lone<K>(h, qx, qy, hp, k, slot(i, j), ids.stride);
         });
 }
 
@@ -99,13 +97,13 @@ __global__ void __launch_bounds__(32 * kQueryWarps) k_knn_ids_query(HashView h, 
 
 template <int K>
 __global__ void __launch_bounds__(128) k_knn_ids_wide(HashView h, GridView g, int k, IdsView ids,
-                                                      int32_t* __restrict__ nbr, int* __restrict__ flag) {
+                                                      int* __restrict__ flag) {
     if (*(volatile int*)flag == 0) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int gx = (g.nx + 15) / 16;
     const int64_t nb = (int64_t)gx * ((ids.j1 - ids.j0 + 7) / 8);
     for (int64_t b = blockIdx.x; b < nb; b += gridDim.x)
-        knn_ids_node_wide<K>(h, g, k, ids, nbr, patch_node((int)(b % gx), ids.j0 / 8 + (int)(b / gx), warp, lane));
+        knn_ids_node_wide<K>(h, g, k, ids, patch_node((int)(b % gx), ids.j0 / 8 + (int)(b / gx), warp, lane));
 }
 
 // Solve blocks take `per` consecutive batches of 128 systems: one take of the
@@ -181,17 +179,17 @@ bg_status launch_k(const bg_soundings_s* snd, const HashView& h, const GridView&
     using Gm = Geo<K>;
     // grid rows per chunk: the id buffer stays near 1 GiB. Without a budget the
     // patch search writes the patches layout (rounded up to whole patches). Under
-    // a budget it does so only where that needs no more memory, else the rows
-    // layout, in nbr_out itself when the caller passed it (then whole), as the
-    // per-thread search always does.
+    // a budget it does so only where that needs no more memory, else the rows layout,
+    // as the per-thread search always does. With lists the caller's nbr_out is the
+    // (whole) buffer: a call that brings one takes no memory for another.
     const int64_t most = std::max<int64_t>(8, ((((int64_t)1 << 28) / ((int64_t)k * g.nx)) / 8) * 8);
     int64_t rows = std::min<int64_t>(g.ny, most);
     const size_t flag_bytes = 256;
     const int pnx = (g.nx + 7) / 8;
     const int64_t slots = (int64_t)pnx * ((rows + 3) / 4) * 32;
     const bool patches = knn_patch_fits<K>(snd->info, g.cell, g.nx, g.ny);
-    const bool slot_ids = patches && (ctx->budget == 0 || (!nbr && slots <= rows * g.nx));
-    if (!slot_ids && nbr) rows = g.ny;
+    const bool slot_ids = patches && !nbr && (ctx->budget == 0 || slots <= rows * g.nx);
+    if (nbr) rows = g.ny;
     const size_t id_bytes =
         slot_ids ? (size_t)slots * k * sizeof(int32_t) : nbr ? 0 : (size_t)rows * g.nx * k * sizeof(int32_t);
     void* scratch = nullptr;
@@ -215,8 +213,7 @@ bg_status launch_k(const bg_soundings_s* snd, const HashView& h, const GridView&
         const int64_t nb = (int64_t)gx * ((j1 - j0 + 7) / 8);
         const int len = strip_len_for((j1 - j0) * (int64_t)g.nx);
         const int64_t nbs = (int64_t)((g.nx + 16 * len - 1) / (16 * len)) * ((j1 - j0 + 3) / 4);
-        int32_t* chunk_ids =
-            nbr && !slot_ids ? nbr + j0 * g.nx * k : (int32_t*)((char*)scratch + flag_bytes);
+        int32_t* chunk_ids = nbr ? nbr + j0 * g.nx * k : (int32_t*)((char*)scratch + flag_bytes);
         cudaError_t e = wide ? cudaMemsetAsync(flag, 0, sizeof(int), st) : cudaSuccess;
         if (e != cudaSuccess) {
             rc = cuda_fail(e, "memset");
@@ -231,7 +228,7 @@ bg_status launch_k(const bg_soundings_s* snd, const HashView& h, const GridView&
             const int plen = patch_strip_len((int64_t)pnx * pny), spr = (pnx + plen - 1) / plen;
             if (patches)
                 k_knn_ids_patch<K><<<(unsigned)(((int64_t)spr * pny + 1) / 2), 64, 0, st>>>(
-                    h, g, k, ids, slot_ids ? nbr : nullptr, flag, plen, spr);
+                    h, g, k, ids, flag, plen, spr);
             else if (query_by_lanes<K>(nodes))
                 k_knn_ids_query<query_lanes(K)><<<query_blocks<K>(nodes), 32 * kQueryWarps, 0, st>>>(
                     h, g, j0 * g.nx, nodes, k, chunk_ids, 0, flag);
@@ -244,7 +241,7 @@ bg_status launch_k(const bg_soundings_s* snd, const HashView& h, const GridView&
         }
         if (wide)
             k_knn_ids_wide<K><<<(unsigned)std::min<int64_t>(nb, 152 * 4), 128, 0, st>>>(
-                h, g, k, ids, slot_ids ? nbr : nullptr, flag);
+                h, g, k, ids, flag);
         note_launches(wide ? 3 : 2);
         const int64_t batches = (nsys + kSolveSystems - 1) / kSolveSystems;
         const int per = solve_batches_per_block<K>(batches);

@@ -273,42 +273,40 @@ __device__ __forceinline__ int64_t node_slot(const IdsView& v, int i, int j) {
 }
 
 // The k ids of a node that the patch search served, to slot `o` of the patches
-// layout (or, with stride 0, to o[0 .. k) as upload indices), and as upload
-// indices to nbr, if any.
+// layout (or, with stride 0, to o[0 .. k) as upload indices).
 template <int K>
 __device__ __forceinline__ void ids_served(const HashView& h, const typename KnnWarp<K>::Smem& sm, int k, int32_t* o,
-                                           int64_t stride, int32_t* nbr) {
+                                           int64_t stride) {
     const uint32_t* col = sm.buf + (threadIdx.x & 31);
     if (stride > 0) {
 #pragma unroll 8
         for (int n = 0; n < k; ++n) o[n * stride] = sm.pos[col[n * 32] & kPlaceMask];
     } else {
-        nbr = o;
+        for (int n = 0; n < k; ++n) o[n] = __ldg(&h.rec[sm.pos[col[n * 32] & kPlaceMask]].w);
     }
-    if (nbr)
-        for (int n = 0; n < k; ++n) nbr[n] = __ldg(&h.rec[sm.pos[col[n * 32] & kPlaceMask]].w);
 }
 // The same of a node that it did not serve, by a per-thread search.
 template <int K>
 __device__ __noinline__ KnnFar ids_lone(const HashView& h, int qx, int qy, uint64_t* hp, int k, int32_t* o,
-                                        int64_t stride, int32_t* nbr) {
+                                        int64_t stride) {
     const int cnt = knn_lane<K>(h, qx, qy, hp);
     const uint64_t mask = (1ull << h.idx_bits) - 1;
-    if (stride == 0) nbr = o;
     if (cnt < 0) return KnnFar{cnt, 0.0f, 0.0f};
     for (int n = 0; n < k; ++n) {
         const int u = n < cnt ? (int)(hp[n * 32] & mask) : -1;
-        if (stride > 0) o[n * stride] = u < 0 ? -1 : -2 - u;
-        if (nbr) nbr[n] = u;
+        if (stride > 0)
+            o[n * stride] = u < 0 ? -1 : -2 - u;
+        else
+            o[n] = u;
     }
     return knn_far<K>(h, hp, cnt);
 }
 
 // Wide-key neighbour ids of one grid node whose table bound does not fit the
-// packed key (patches layout: also to nbr, if any); other nodes return.
+// packed key; other nodes return.
 template <int K>
 __device__ __forceinline__ void knn_ids_node_wide(const HashView& h, const GridView& g, int k, const IdsView& ids,
-                                                  int32_t* __restrict__ nbr, NodeIdx nd) {
+                                                  NodeIdx nd) {
     if (nd.i >= g.nx || nd.j >= ids.j1 || h.n_valid == 0) return;
     const int qx = g.x0 + nd.i * g.cell + g.cell / 2;
     const int qy = g.y0 + nd.j * g.cell + g.cell / 2;
@@ -326,10 +324,7 @@ __device__ __forceinline__ void knn_ids_node_wide(const HashView& h, const GridV
         int32_t* o = ids.p + node_slot(ids, nd.i, nd.j);
 #pragma unroll
         for (int i = 0; i < K; ++i)
-            if (i < k) {
-                o[i * ids.stride] = i < keff ? -2 - id[i] : -1;
-                if (nbr) nbr[((int64_t)nd.j * g.nx + nd.i) * k + i] = i < keff ? id[i] : -1;
-            }
+            if (i < k) o[i * ids.stride] = i < keff ? -2 - id[i] : -1;
     }
 }
 
