@@ -46,7 +46,7 @@ struct TileDesc {
     float* depth;        // outputs (device)
     float* var;
     int32_t* ids;        // kriging: neighbour ids (IdsView)
-    int64_t stride;      // of the patches layout; 0: the batch keeps rows
+    int64_t stride;      // of the patches layout; 0: the tile's ids keep rows
     int32_t patch;       // this run's k-NN goes by patches (written on the device)
     OkParams p;
     float power;
@@ -799,8 +799,9 @@ bg_status bg_batch_create(bg_ctx_t ctx, const bg_tile* tiles, int n_tiles, bg_ba
                                                         ((r.ny + 7) / 8);
         knn_tiles[d.K == 4 ? 0 : d.K == 8 ? 1 : d.K == 16 ? 2 : 3].push_back(t);
         if (r.method == 1) {
-            d.stride = (int64_t)((r.nx + 7) / 8) * ((r.ny + 3) / 4) * 32;
-            slot_ids += d.stride * r.k;
+            const int64_t slots = (int64_t)((r.nx + 7) / 8) * ((r.ny + 3) / 4) * 32;
+            d.stride = slots_pay(slots, m) ? slots : 0;
+            slot_ids += (d.stride > 0 ? slots : m) * r.k;
             row_ids += m * r.k;
             for (int q = 0; q < 4; ++q)
                 if (Ks[q] == d.K) gt[2 * q + (r.variogram.model != 0)].push_back(t);

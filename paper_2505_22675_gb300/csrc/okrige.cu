@@ -177,23 +177,35 @@ bg_status launch_k(const bg_soundings_s* snd, const HashView& h, const GridView&
                    float* var, int32_t* nbr, bg_ctx_s* ctx, cudaStream_t st, const IdwFuse* fz,
                    const HostOut* ho) {
     using Gm = Geo<K>;
-    // grid rows per chunk: the id buffer stays near 1 GiB. Without a budget the
-    // patch search writes the patches layout (rounded up to whole patches). Under
-    // a budget it does so only where that needs no more memory, else the rows layout,
-    // as the per-thread search always does. With lists the caller's nbr_out is the
-    // (whole) buffer: a call that brings one takes no memory for another.
-    const int64_t most = std::max<int64_t>(8, ((((int64_t)1 << 28) / ((int64_t)k * g.nx)) / 8) * 8);
-    int64_t rows = std::min<int64_t>(g.ny, most);
+    // grid rows per chunk: the id buffer stays near 1 GiB. The patch search writes the
+    // patches layout where its rounding up to whole patches costs little
+    // (slots_pay) and, under a budget, no memory; else the rows layout, as the
+    // per-thread search always does. With lists the caller's nbr_out is the (whole)
+    // buffer: a call that brings one takes no memory for another.
+    const auto chunk_rows = [&](int64_t width) {
+        const int64_t most = ((((int64_t)1 << 28) / (k * width)) / 8) * 8;
+        return std::min<int64_t>(g.ny, std::max<int64_t>(8, most));
+    };
     const size_t flag_bytes = 256;
     const int pnx = (g.nx + 7) / 8;
+    int64_t rows = chunk_rows((int64_t)pnx * 8);
     const int64_t slots = (int64_t)pnx * ((rows + 3) / 4) * 32;
     const bool patches = knn_patch_fits<K>(snd->info, g.cell, g.nx, g.ny);
-    const bool slot_ids = patches && !nbr && (ctx->budget == 0 || slots <= rows * g.nx);
-    if (nbr) rows = g.ny;
-    const size_t id_bytes =
-        slot_ids ? (size_t)slots * k * sizeof(int32_t) : nbr ? 0 : (size_t)rows * g.nx * k * sizeof(int32_t);
+    bool slot_ids = patches && !nbr && (ctx->budget ? slots <= rows * g.nx : slots_pay(slots, rows * g.nx));
+    size_t id_bytes = 0;
     void* scratch = nullptr;
-    bg_status rc = dalloc(ctx, &scratch, flag_bytes + id_bytes, st);
+    bg_status rc = BG_OK;
+    if (slot_ids) {
+        id_bytes = (size_t)slots * k * sizeof(int32_t);
+        rc = dalloc(ctx, &scratch, flag_bytes + id_bytes, st);
+        if (rc == BG_ERR_CUDA) cudaGetLastError();  // a full device: the rows layout needs less
+        slot_ids = rc == BG_OK;
+    }
+    if (!slot_ids) {
+        rows = nbr ? g.ny : chunk_rows(g.nx);
+        id_bytes = nbr ? 0 : (size_t)rows * g.nx * k * sizeof(int32_t);
+        rc = dalloc(ctx, &scratch, flag_bytes + id_bytes, st);
+    }
     if (rc != BG_OK) return rc;
     const bool wide = !packed_always(h, g);
     int* flag = (int*)scratch;

@@ -1,5 +1,6 @@
 """Device memory that a kriging call takes for its neighbour ids, 4 k bytes a node:
-none beside the caller's nbr_out.
+none beside the caller's nbr_out, and whole 8 x 4 patches of nodes only where a grid
+fills them.
 """
 import numpy as np
 import pytest
@@ -18,7 +19,7 @@ def _soundings(torch):
         (3500 + r.normal(0, 5, n)).astype(np.float32))]
 
 
-@pytest.mark.parametrize("lists", [True])
+@pytest.mark.parametrize("lists", [False, True])
 @pytest.mark.parametrize("nx,ny", SHAPES)
 def test_ids_of_a_grid(nx, ny, lists):
     """Device memory that one call makes the context's pool take."""
@@ -46,4 +47,24 @@ def test_ids_of_a_grid(nx, ny, lists):
         bg.soundings_destroy(s)
     finally:
         bg.ctx_destroy(ctx)
-    assert taken <= (0 if lists else 1.25 * 4 * K * m) + (96 << 20)  # the pool maps whole blocks
+    assert taken <= (0 if lists else 1.1 * 4 * K * m) + (96 << 20)  # the pool maps whole blocks
+
+
+@pytest.mark.parametrize("nx,ny", [(nx // 16 if nx > ny else nx, ny // 16 if ny >= nx else ny) for nx, ny in SHAPES])
+def test_ids_of_a_batch(nx, ny):
+    import torch
+
+    import paper_2505_22675_gb300 as bg
+    x, y, z = _soundings(torch)
+    d, v = torch.empty(nx * ny, device="cuda"), torch.empty(nx * ny, device="cuda")
+    ctx = bg.ctx_create(0)
+    try:
+        held = []
+        for method in (0, 1):
+            b = bg.batch_create(ctx, [dict(x_cm=x, y_cm=y, z_m=z, grid_spec=(0, 0, 2, nx, ny), method=method, k=K,
+                                           depth_out=d, var_out=v)])
+            held.append(bg.ctx_device_bytes(ctx))
+            bg.batch_destroy(b)
+    finally:
+        bg.ctx_destroy(ctx)
+    assert held[1] - held[0] <= 1.1 * 4 * K * nx * ny + 4096
