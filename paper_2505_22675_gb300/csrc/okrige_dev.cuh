@@ -375,10 +375,10 @@ __device__ __forceinline__ float rsqrt_approx(float x) {
 }
 
 // ------------------------------------------------------------ tensor memory
-// Each warp of the 128-thread block reaches its own quarter of the 128 lanes;
-// a thread reads and writes its lane's columns (32x32b). Loads are collected
-// by tmem_wait_ld, which takes the loaded registers as operands so that no use
-// of them moves above it.
+// A warp reaches the quarter of the 128 lanes that its index modulo 4 names, so the
+// two warps of a system (w and w + 4) share theirs; a thread reads and writes its
+// lane's columns (32x32b). Loads are collected by tmem_wait_ld, which takes the
+// loaded registers as operands so that no use of them moves above it.
 
 __device__ __forceinline__ void tmem_ld16(uint32_t (&r)[16], uint32_t a) {
     asm volatile(
@@ -422,6 +422,15 @@ __device__ __forceinline__ void tmem_wait_st() {
     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
+// Around a barrier that hands tensor memory from one warp to another: what the one has
+// read or written (and waited for) lies before what the other does with it.
+__device__ __forceinline__ void tmem_before_sync() {
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_after_sync() {
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+}
+
 // A block's tensor memory (Geo<K>::COLS columns, a power of two), taken by warp
 // 0 at the start and given back by it at the end; `slot` is a shared word.
 // Returns the thread's base address (its warp's lanes).
@@ -436,13 +445,17 @@ __device__ __forceinline__ uint32_t tmem_take(uint32_t* slot) {
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    tmem_before_sync();
     __syncthreads();
+    tmem_after_sync();
     return *(volatile uint32_t*)slot + ((uint32_t)(threadIdx.x >> 5 & 3) << 21);
 }
 template <int COLS>
 __device__ __forceinline__ void tmem_give(const uint32_t* slot) {
     if constexpr (COLS != 0) {
+        tmem_before_sync();
         __syncthreads();
+        tmem_after_sync();
         if (threadIdx.x < 32)
             asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(*slot),
                          "r"(COLS)
@@ -579,12 +592,13 @@ struct Lane {
 __device__ __forceinline__ void pair_sync() {
     asm volatile("bar.sync %0, 64;" ::"r"(1 + (int)(threadIdx.x >> 5 & 3)) : "memory");
 }
-// tensor memory written by one warp of the pair is read by the other
+// tensor memory that one warp of the pair has read (the loads waited for) or written
+// is the other's to write or read
 __device__ __forceinline__ void pair_sync_tmem() {
     tmem_wait_st();
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    tmem_before_sync();
     pair_sync();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    tmem_after_sync();
 }
 // row r of a tile as (half, place): the half that owns it and its place there
 constexpr __host__ __device__ int half_of(int r) { return r >= 2 && r < 6; }
@@ -1563,7 +1577,7 @@ __device__ __forceinline__ void okrige_solve_range(const HashView& h, const Grid
             if (live)
                 var[node] = ke == 0 ? __int_as_float(0x7fc00000) : fmaf(lam0, g00, g00 + idw_tree8(pv));
         }
-        pair_sync();  // the next batch overwrites the records
+        pair_sync_tmem();  // the next batch overwrites the records and the factor
     }
     }
 }
