@@ -811,7 +811,7 @@ bg_status bg_batch_create(bg_ctx_t ctx, const bg_tile* tiles, int n_tiles, bg_ba
     for (int si = 0; si < 3; ++si) b->knn_items_s[si] = item_off_s[si][n_tiles];
     b->total_ids = slot_ids;
     // carve one allocation (the ids last: the patches layout, rounded up to whole
-    // patches, gives way to the rows layout where the budget has no room for it)
+    // patches, gives way to the rows layout where the budget or the device has no room for it)
     size_t off = 0;
     auto take = [&](size_t bytes) {
         const size_t o = off;
@@ -856,7 +856,8 @@ bg_status bg_batch_create(bg_ctx_t ctx, const bg_tile* tiles, int n_tiles, bg_ba
     st = b->stream;
     bg_status rc = e == cudaSuccess ? BG_OK : cuda_fail(e, "batch stream");
     if (rc == BG_OK) rc = dalloc(ctx, &b->mem, b->mem_bytes, st);
-    if (rc == BG_ERR_OOM_BUDGET && row_ids < slot_ids) {
+    if ((rc == BG_ERR_OOM_BUDGET || (rc == BG_ERR_CUDA && e == cudaSuccess)) && row_ids < slot_ids) {
+        if (rc == BG_ERR_CUDA) cudaGetLastError();  // a full device
         b->total_ids = row_ids;
         b->mem_bytes = o_ids + 4 * (size_t)row_ids;
         for (TileDesc& d : b->host_desc) d.stride = 0;
