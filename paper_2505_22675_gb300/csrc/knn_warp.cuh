@@ -284,13 +284,21 @@ __device__ __forceinline__ int knn_stage(const HashView& h, typename KnnWarp<K>:
     return T;
 }
 
-// (distance, upload index) order of two keys, from the exact values
+// (distance, upload index) order of two keys, from the exact values (after
+// knn_stage_indices)
 template <class Smem>
-__device__ __forceinline__ bool key_less(const Smem& sm, const int4* rec, int ux, int uy, uint32_t a, uint32_t b) {
+__device__ __forceinline__ bool key_less(const Smem& sm, int ux, int uy, uint32_t a, uint32_t b) {
     const int4 ca = sm.st[a & kPlaceMask], cb = sm.st[b & kPlaceMask];
     const int ax = ca.x - ux, ay = ca.y - uy, bx = cb.x - ux, by = cb.y - uy;
     const int da = ax * ax + ay * ay, db = bx * bx + by * by;
-    return da != db ? da < db : __ldg(&rec[sm.pos[ca.w]].w) < __ldg(&rec[sm.pos[cb.w]].w);
+    return da != db ? da < db : ca.z < cb.z;
+}
+// The upload indices of the staged records in place of their squares; all lanes.
+template <class Smem>
+__device__ __forceinline__ void knn_stage_indices(Smem& sm, const int4* rec, int T) {
+#pragma unroll 2
+    for (int i = threadIdx.x & 31; i < T; i += 32) sm.st[i].z = __ldg(&rec[sm.pos[i]].w);
+    __syncwarp();
 }
 
 // An appended word as the key it sorts by. The near scan appends 512 (d - u^2) +
@@ -298,24 +306,27 @@ __device__ __forceinline__ bool key_less(const Smem& sm, const int4* rec, int ux
 // place; the far scan appends the key itself (bias 0).
 __device__ __forceinline__ uint32_t sort_key(uint32_t v, uint32_t bias) { return v + bias; }
 
-// The K nearest of a lane's cnt appended keys in exact order to the front of its
-// buffer column, where keys alone cannot tell (dk: the K-th key). Out of the
-// way of the search's straight path.
-template <class Smem>
-__device__ __noinline__ void knn_order_exact(Smem& sm, const int4* rec, int ux, int uy, int cnt, uint32_t dk,
-                                             uint32_t bias) {
+// Of a lane's cnt appended keys those at the distance (as far as keys hold it) of the
+// K-th, dk: the m nearest in exact order to the rows K - m .. K - 1 of its buffer
+// column. Out of the way of the search's straight path. On a lattice every node comes
+// here (511 x 511 nodes k = 32 over one of 2 m: 123 us; 469 with all keys sorted anew
+// and indices from global memory, 201 by threads).
+template <int K, class Smem>
+__device__ __noinline__ void knn_last_group(Smem& sm, int ux, int uy, int cnt, int m, uint32_t dk, uint32_t bias) {
     uint32_t* buf = sm.buf + (threadIdx.x & 31);
-    int m = 0;
+    int n = 0;
     for (int i = 0; i < cnt; ++i) {
         const uint32_t v = sort_key(buf[i * 32], bias);
-        if ((v >> kPlaceBits) > (dk >> kPlaceBits)) continue;
-        int j = m++;
-        for (; j > 0; --j) {
-            const uint32_t u = buf[(j - 1) * 32];
-            if ((u >> kPlaceBits) < (v >> kPlaceBits)) break;
-            if ((u >> kPlaceBits) == (v >> kPlaceBits) && !key_less(sm, rec, ux, uy, v, u)) break;
-            buf[j * 32] = u;
-        }
+        if ((v ^ dk) <= kPlaceMask) buf[n++ * 32] = v;
+    }
+    // (K - m + n <= cnt: no row past the appended ones)
+    for (int i = n - 1; i >= 0; --i) buf[(K - m + i) * 32] = buf[i * 32];
+    buf += (K - m) * 32;
+    for (int i = 1; i < n; ++i) {
+        const uint32_t v = buf[i * 32];
+        if (i >= m && !key_less(sm, ux, uy, v, buf[(m - 1) * 32])) continue;
+        int j = min(i, m - 1);
+        for (; j > 0 && key_less(sm, ux, uy, v, buf[(j - 1) * 32]); --j) buf[j * 32] = buf[(j - 1) * 32];
         buf[j * 32] = v;
     }
 }
@@ -454,29 +465,36 @@ __device__ __forceinline__ unsigned knn_patch(const HashView& h, typename KnnWar
         ch.beta = fmaxf(1.04f, ch.beta * (shrunk ? 0.96f : 0.99f));
 
     // equal distances (as far as the keys hold them): into (distance, index)
-    // order. A pair inside the list is put right in place; longer runs, and the
-    // K-th distance where a key left out shares it, go the long way.
-    bool pair = false, lng = (key[K - 1] ^ drop) <= kPlaceMask;
+    // order, in place; where a key left out shares the K-th distance, from all that do
+    const bool last = on && (key[K - 1] ^ drop) <= kPlaceMask;
+    bool pair = false;
 #pragma unroll
-    for (int i = 0; i + 1 < K; ++i) {
-        const bool eq = (key[i] ^ key[i + 1]) <= kPlaceMask;
-        lng |= pair && eq && (key[i > 0 ? i - 1 : 0] ^ key[i + 1]) <= kPlaceMask;
-        pair |= eq;
+    for (int i = 0; i + 1 < K; ++i) pair |= (key[i] ^ key[i + 1]) <= kPlaceMask;
+    int put = K;  // keys that are in place but for pairs
+    if (__any_sync(kFull, last || (on && pair))) {
+        knn_stage_indices(sm, h.rec, T);
+        if (last) {
+            put = 0;
+#pragma unroll
+            for (int i = 0; i < K; ++i) put += (key[i] ^ key[K - 1]) > kPlaceMask;
+            knn_last_group<K>(sm, ux, uy, cnt, K - put, key[K - 1], bias);
+        }
     }
-    if (on && lng) {
-        knn_order_exact(sm, h.rec, ux, uy, cnt, key[K - 1], bias);
-    } else {
 #pragma unroll
-        for (int i = 0; i < K; ++i) buf[i * 32] = key[i];
-        if (on && pair) {
+    for (int i = 0; i < K; ++i)
+        if (i < put) buf[i * 32] = key[i];
+    if (on && pair) {
 #pragma unroll 1
-            for (int i = 0; i + 1 < K; ++i) {
-                const uint32_t a = buf[i * 32], b = buf[(i + 1) * 32];
-                if ((a ^ b) <= kPlaceMask && key_less(sm, h.rec, ux, uy, b, a)) {
-                    buf[i * 32] = b;
-                    buf[(i + 1) * 32] = a;
-                }
+        for (int i = 1; i < put; ++i) {
+            const uint32_t v = buf[i * 32];
+            int j = i;
+#pragma unroll 1
+            for (; j > 0; --j) {
+                const uint32_t u = buf[(j - 1) * 32];
+                if ((u ^ v) > kPlaceMask || !key_less(sm, ux, uy, v, u)) break;
+                buf[j * 32] = u;
             }
+            if (j < i) buf[j * 32] = v;
         }
     }
     __syncwarp();
