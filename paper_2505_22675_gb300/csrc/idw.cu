@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(64, KnnWarp<K>::kBlocksPerSM) k_idw_patch(Hash
 // once when the packed pass flagged none.
 // G lanes per query: points of a list or nodes of a grid.
 template <int G, class Queries>
-__global__ void __launch_bounds__(32 * kQueryWarps) k_idw_query(HashView h, Queries q, int64_t m, int k, float power,
+__global__ void __launch_bounds__(32 * kQueryWarps, 9) k_idw_query(HashView h, Queries q, int64_t m, int k, float power,
                                                                float* __restrict__ depth,
                                                                int32_t* __restrict__ nbr, int* __restrict__ flag) {
     __shared__ uint64_t buf[32 * kQueryWarps * 2];

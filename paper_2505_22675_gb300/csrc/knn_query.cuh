@@ -13,8 +13,9 @@
 //      (and below the k-th key so far) are collected in shared memory, and each
 //      32 (16) of them are sorted across the lanes and merged into the best.
 // The first bound is the radius that holds k + 2.5 sqrt(k) soundings at the
-// square's density; with fewer than k inside, the scan runs again from the
-// square's farthest corner. Keys and order are those of knn.cuh.
+// square's density; with fewer than k inside, the scan runs again from the square's
+// farthest corner, or in steps towards it where the square is large (query_wider).
+// Keys and order are those of knn.cuh.
 //
 // Bound by instructions from about 10,000 queries on: 0.8 us for 1000 of them by
 // halves of a warp, 1.3 by whole ones, most in 64-bit keys (sorting 32 takes 15
@@ -83,6 +84,45 @@ __device__ __forceinline__ uint64_t query_merge(uint64_t a, uint64_t b, int lane
 #pragma unroll
     for (int s = G / 2; s > 0; s /= 2) x = query_pick(x, s, (lane & s) == 0);
     return x;
+}
+
+// How far (cm, rounded down) a query x, y from the hash's origin lies outside of the hash.
+__device__ __forceinline__ float query_outside(int64_t x, int64_t y, int cs, int ncx, int ncy) {
+    const float ox = (float)max(max(-x, x - ((int64_t)ncx * cs - 1)), (int64_t)0);
+    const float oy = (float)max(max(-y, y - ((int64_t)ncy * cs - 1)), (int64_t)0);
+    return 0.99999f * sqrtf(ox * ox + oy * oy);
+}
+
+// The squared bound to try after one of tau has held fewer than kc: the part of its radius
+// past the distance that the kc-th can have at least is doubled, up to tau0. The
+// square of half-width lo cells around the query's cell holds fewer than kc, the next one
+// count. Out of the way: a miss is rare where soundings lie all around. The farthest
+// corner at once costs a query off to one side most of what lies within its reach: 21,845
+// points k = 8, half of them up to 250 m from the soundings, 673 us; so 89, by threads
+// 185.
+static __device__ __noinline__ int64_t query_wider(int64_t x, int64_t y, int cs, int ncx, int ncy, int lo, int count, int kc,
+                                            int64_t tau, int64_t tau0) {
+    const int cx = (int)min(max(x / cs, (int64_t)0), (int64_t)ncx - 1), cy = (int)min(max(y / cs, (int64_t)0), (int64_t)ncy - 1);
+    int64_t d = LLONG_MAX;
+    if (cx - lo > 0) d = min(d, x - (int64_t)(cx - lo) * cs);
+    if (cx + lo < ncx - 1) d = min(d, (int64_t)(cx + lo + 1) * cs - x);
+    if (cy - lo > 0) d = min(d, y - (int64_t)(cy - lo) * cs);
+    if (cy + lo < ncy - 1) d = min(d, (int64_t)(cy + lo + 1) * cs - y);
+    const float in = lo < 0 || d == LLONG_MAX ? 0.0f : 0.99999f * (float)max(d, (int64_t)0);
+    const float near = fmaxf(in, query_outside(x, y, cs, ncx, ncy)), c = (float)cs;
+    float past = sqrtf((float)tau) - near;
+    if (past <= 0.0f) {
+        // soundings on one side only: they begin in the ring of cells between the two squares;
+        // past it by the height of the circle's segment that holds kc + 2.5 sqrt(kc) at
+        // the density of one side of the ring
+        const float want = (float)kc + 2.5f * sqrtf((float)kc), side = (float)(2 * lo + 3) * c * c;
+        past = c + __powf(0.75f * want * side / ((float)max(count, 1) * sqrtf(2.0f * near)), 0.6666667f);
+    } else {
+        past = 2.0f * past + 0.5f * c;
+    }
+    const float r = near + past;
+    // (a 64th more at least: the steps end whatever the rounding)
+    return min(tau0, r * r < 0.64f * (float)tau0 ? max((int64_t)(r * r), tau + tau / 64 + 1) : tau0);
 }
 
 // The kc (<= G) nearest of (qx, qy), the same in every lane of the query: lane n
@@ -205,7 +245,12 @@ __device__ __forceinline__ int knn_query(const HashView& h, bool ok, int qx, int
         const int cnt = min(kc, __popc(query_ballot<G>(best != ~0ull)));
         const bool more = cnt < kc && tau != tau0;
         if (!__any_sync(kFull, more)) return ok && !fits ? -1 : cnt;
-        if (more) tau = tau0;
+        if (more) {  // (a few cells hold enough: their corner)
+            if (lo <= 1)
+                tau = tau0;
+            else
+                tau = query_wider((int64_t)qx - h.hx0, (int64_t)qy - h.hy0, h.cs, h.ncx, h.ncy, lo, count, kc, tau, tau0);
+        }
     }
 }
 

@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(64, KnnWarp<K>::kBlocksPerSM) k_knn_ids_patch(
 
 // The ids of queries i0 .. i0 + m - 1, G lanes each (put_point_id).
 template <int G, class Queries>
-__global__ void __launch_bounds__(32 * kQueryWarps) k_knn_ids_query(HashView h, Queries q, int64_t i0, int64_t m, int k,
+__global__ void __launch_bounds__(32 * kQueryWarps, 9) k_knn_ids_query(HashView h, Queries q, int64_t i0, int64_t m, int k,
                                                                    int32_t* __restrict__ ids, int64_t stride,
                                                                    int* __restrict__ flag) {
     __shared__ uint64_t buf[32 * kQueryWarps * 2];
