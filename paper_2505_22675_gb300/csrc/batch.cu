@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(kBT) k_batch_validate(const TileDesc* __restri
 // 2. per-tile hash geometry (one thread per tile)
 __device__ __forceinline__ bool tile_patch_fits(const HashView& h, const GridView& g, int kq) {
     auto fits = [&](auto K) {
-        return knn_patch_fits<decltype(K)::value>(h.n_valid, h.ncx, h.ncy, h.cs, g.cell, g.nx, g.ny);
+        return knn_patch_fits<decltype(K)::value>(h.n_valid, h.hx0, h.hy0, h.ncx, h.ncy, h.cs, g);
     };
     return kq <= 4    ? fits(std::integral_constant<int, 4>{})
            : kq <= 8  ? fits(std::integral_constant<int, 8>{})
@@ -344,10 +344,10 @@ __global__ void __launch_bounds__(64, KnnWarp<K>::kBlocksPerSM) k_batch_knn_patc
                     else
                         ids_served<K>(h, sm, k, slot(i, j), ids.stride);
                 },
-                [&](int i, int j, int qx, int qy, uint64_t* hp) {
+                [&](int i, int j, int qx, int qy, uint64_t* hp, float ub) {
                     if (d.method == 0)
-                        return idw_lone<K>(h, qx, qy, hp, k, d.power, d.depth + out(i, j), nullptr);
-                    return ids_lone<K>(h, qx, qy, hp, k, slot(i, j), ids.stride);
+                        return idw_lone<K>(h, qx, qy, hp, ub, k, d.power, d.depth + out(i, j), nullptr);
+                    return ids_lone<K>(h, qx, qy, hp, ub, k, slot(i, j), ids.stride);
                 });
     }
 }

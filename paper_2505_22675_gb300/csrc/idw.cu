@@ -61,8 +61,8 @@ __global__ void __launch_bounds__(64, KnnWarp<K>::kBlocksPerSM) k_idw_patch(Hash
         [&](int i, int j, int ux, int uy) {
             idw_served<K>(h, sm, ux, uy, k, power, depth + out(i, j), nbr ? nbr + out(i, j) * k : nullptr);
         },
-        [&](int i, int j, int qx, int qy, uint64_t* hp) {
-            return idw_lone<K>(h, qx, qy, hp, k, power, depth + out(i, j), nbr ? nbr + out(i, j) * k : nullptr);
+        [&](int i, int j, int qx, int qy, uint64_t* hp, float ub) {
+            return idw_lone<K>(h, qx, qy, hp, ub, k, power, depth + out(i, j), nbr ? nbr + out(i, j) * k : nullptr);
         });
 }
 
@@ -113,10 +113,10 @@ bg_status launch_k(const bg_soundings_s* s, const HashView& h, const GridView& g
     cudaError_t e = wide ? cudaMemsetAsync(d_flag, 0, sizeof(int), st) : cudaSuccess;
     if (e == cudaSuccess) {
         ProfScope ps(prof_ctx, kProfIdw, (int64_t)g.nx * g.ny, st);
-        if (knn_patch_fits<K>(s->info, g.cell, g.nx, g.ny) && (int64_t)spr * pny < ((int64_t)1 << 31))
+        if (knn_patch_fits<K>(s->info, g) && (int64_t)spr * pny < ((int64_t)1 << 31))
             k_idw_patch<K><<<(unsigned)(((int64_t)spr * pny + 1) / 2), 64, 0, st>>>(h, g, k, power, depth, nbr, d_flag,
                                                                                    plen, spr);
-        else if (query_by_lanes<K>((int64_t)g.nx * g.ny))
+        else if (grid_by_lanes<K>(s->info, g, (int64_t)g.nx * g.ny))
             k_idw_query<query_lanes(K)><<<query_blocks<K>((int64_t)g.nx * g.ny), 32 * kQueryWarps, 0, st>>>(
                 h, g, (int64_t)g.nx * g.ny, k, power, depth, nbr, d_flag);
         else if (len == 1)

@@ -140,9 +140,9 @@ __device__ __forceinline__ void idw_point_wide(const HashView& h, int qx, int qy
 // The same of a node that it did not serve: a per-thread search, out of the way
 // of the patch search's code.
 template <int K>
-__device__ __noinline__ KnnFar idw_lone(const HashView& h, int qx, int qy, uint64_t* hp, int k, float power,
-                                        float* depth, int32_t* nbr) {
-    const int cnt = knn_lane<K>(h, qx, qy, hp);
+__device__ __noinline__ KnnFar idw_lone(const HashView& h, int qx, int qy, uint64_t* hp, float ub, int k,
+                                        float power, float* depth, int32_t* nbr) {
+    const int cnt = knn_lane<K>(h, qx, qy, hp, ub);
     if (cnt < 0) return KnnFar{cnt, 0.0f, 0.0f};
     const int bits = h.idx_bits, keff = min(cnt, k);
     const uint64_t mask = (1ull << bits) - 1;

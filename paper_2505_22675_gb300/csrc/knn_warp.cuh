@@ -6,6 +6,8 @@
 // every lane tests each of them, without divergence:
 //   1. a radius per lane: from the density around the patch (summed-area
 //      table), later from the lane's neighbour distances in the previous patch;
+//      where that misses by far (soundings to one side, clusters), from the exact
+//      neighbours of a node in the middle, found by the whole warp (knn_query.cuh);
 //   2. the records of every cell run that can hold a point within the largest
 //      radius of the patch go to shared memory (coalesced loads);
 //   3. each lane computes its squared distance to each staged record (a
@@ -21,8 +23,9 @@
 // put in (distance, upload index) order afterwards, from the exact values; so
 // are distances that a key holds only in part (large radii drop low bits).
 //
-// What bounds it: latency at 20 (K <= 16) or 14 (K = 32) resident warps per
-// SM, half of the issue slots used; a per-thread heap was bound by divergence.
+// What bounds it: latency at 16 (K <= 16) or 12 (K = 32) resident warps per
+// SM, half of the issue slots used (18 warps of 96 registers instead of 16 of 128 spill
+// and take 1.40 ms where these take 1.27); a per-thread heap was bound by divergence.
 // IDW k = 16 on a two-line swath (4,000 x 1,692 nodes, a 154 m gap): a heap per
 // thread 277 warp instructions per node with 16 of 32 lanes active, 2.04 ms;
 // this search 105 with 30, 1.20 ms. A candidate costs a warp 7 instructions for
@@ -30,6 +33,10 @@
 // patch. The straight path is kept short (rare courses in functions of their
 // own): with everything inlined the instruction cache missed on three of four
 // issues and the same search took 3.3 ms.
+// Uneven soundings, us by threads / with the density's radius alone / so: 256 x 256
+// nodes k = 8, half of the box empty 106 / 137 / 114, the other half denser 153 / 191 /
+// 105; 500 x 500 over clusters 224 / 286 / 204; single-beam lines 500 m apart, 400 x 350
+// nodes k = 16 467 / 690 / 386, 2,000 x 1,900 over denser ones 11,032 / 31,418 / 12,276.
 // Patches the staged list cannot hold (many soundings per node), nodes far
 // outside the data and the like are left to the caller's per-thread search.
 #pragma once
@@ -39,10 +46,11 @@
 #include <type_traits>
 
 #include "knn.cuh"
+#include "knn_query.cuh"
 
 namespace bg {
 
-// Staged records per patch, buffer rows per lane (before the slack of one
+// Staged records per patch, buffer rows per lane (with the slack of one
 // unrolled step), and the radius the first patch of a strip starts with, as a
 // multiple of the area that holds K soundings at the local density (about three
 // standard deviations of a random count above K).
@@ -50,10 +58,10 @@ template <int K>
 struct KnnWarp {
     static constexpr int kStep = 8;  // candidates per unrolled step
     static constexpr int CAP = K == 32 ? 320 : 256;
-    static constexpr int ROWS = K == 32 ? 80 : K == 16 ? 48 : K == 8 ? 40 : 24;
+    static constexpr int ROWS = K == 32 ? 80 : K == 16 ? 48 : 40;
     static constexpr int B = ROWS - kStep;
     static constexpr float kArea = K == 32 ? 1.6f : K == 16 ? 1.9f : K == 8 ? 2.2f : 3.0f;
-    static constexpr int kBlocksPerSM = K == 32 ? 7 : 10;  // of two warps: by shared memory
+    static constexpr int kBlocksPerSM = K == 32 ? 6 : 8;  // of two warps: by shared memory
     struct Smem {
         uint32_t buf[ROWS * 32];  // column per lane (the per-thread heap, 8 K bytes, fits too)
         int4 st[CAP];             // {x, y relative to the patch, x^2 + y^2, place}
@@ -331,32 +339,61 @@ __device__ __noinline__ void knn_last_group(Smem& sm, int ux, int uy, int cnt, i
     }
 }
 
+// For each lane's node a radius (cm) that holds K soundings, ub, and one that holds fewer,
+// lo, from the exact K nearest of lane src's node: ub reaches all of those, lo is short
+// of the K-th by the way between the nodes. r: the radius that failed. ub < 0: none.
+struct KnnBracket {
+    float lo, ub;
+};
+template <int K>
+__device__ __noinline__ KnnBracket knn_centre(const HashView& h, int qx, int qy, float r, int src, uint64_t* buf) {
+    const int sx = __shfl_sync(kFull, qx, src), sy = __shfl_sync(kFull, qy, src);
+    uint64_t key = 0;
+    // (off the data: its nodes share little)
+    if (query_outside((int64_t)sx - h.hx0, (int64_t)sy - h.hy0, h.cs, h.ncx, h.ncy) > 4.0f * r) return KnnBracket{0.0f, -1.0f};
+    if (knn_query<32>(h, true, sx, sy, K, buf, key) != K) return KnnBracket{0.0f, -1.0f};
+    int4 p = make_int4(0, 0, 0, 0);
+    if ((threadIdx.x & 31) < K) p = __ldg(h.orig + (key & ((1ull << h.idx_bits) - 1)));
+    float most = 0.0f;
+#pragma unroll 4
+    for (int i = 0; i < K; ++i) {
+        const float dx = (float)(__shfl_sync(kFull, p.x, i) - qx), dy = (float)(__shfl_sync(kFull, p.y, i) - qy);
+        most = fmaxf(most, fmaf(dx, dx, dy * dy));
+    }
+    const float wx = (float)(qx - sx), wy = (float)(qy - sy);
+    const float d = sqrtf((float)(__shfl_sync(kFull, key, K - 1) >> h.idx_bits));
+    return KnnBracket{fmaxf(0.0f, 0.999999f * (d - sqrtf(wx * wx + wy * wy)) - 1.0f), 1.000001f * sqrtf(most) + 1.0f};
+}
+
 // The K nearest of each lane's node (qx, qy), for lanes with `on`; (ox, oy)
 // is the patch's corner (the staged coordinates are relative to it; no node
 // lies before it). r: the lane's first radius (cm; < 0: none), base: a lower
-// bound of its squared distances. Returns the lanes that were served: the low
+// bound of its squared distances; lo: a radius known to hold fewer than K. probe: what
+// the caller can better with another radius, 0 nothing, 1 more records than the list
+// holds, 2 also a radius far too small. No lane is served then and probe stays as it
+// was; else it becomes 0. Returns the lanes that were served: the low
 // kPlaceBits of the first K rows of their buffer columns index the staged list
 // in ascending (distance, upload index) order.
 template <int K>
 __device__ __forceinline__ unsigned knn_patch(const HashView& h, typename KnnWarp<K>::Smem& sm, bool on,
                                               int qx, int qy, int ox, int oy, float r, uint32_t base,
-                                              KnnChain& ch) {
+                                              float lo, int& probe, KnnChain& ch) {
     using W = KnnWarp<K>;
     constexpr int B = W::B, S = W::kStep;
     const int lane = threadIdx.x & 31;
     const int ux = qx - ox, uy = qy - oy;
     constexpr float kMaxR = (float)kRadiusMax;
     on = on && r >= 0.0f && r < kMaxR && (unsigned)ux < (unsigned)kPatchMax && (unsigned)uy < (unsigned)kPatchMax;
-    if (!__any_sync(kFull, on)) return 0;
+    if (!__any_sync(kFull, on)) return 0;  // (a probe too: the caller finds another radius)
     uint32_t* buf = sm.buf + lane;
     const uint32_t buf0 = (uint32_t)__cvta_generic_to_shared(buf);
-    float lo = 0.0f, hi = 1e30f;  // radii known to hold fewer than K, and too many
+    float hi = 1e30f;  // a radius known to hold too many
     const float d0 = sqrtf((float)base);
     const int u2 = on ? ux * ux + uy * uy : 0;
     const uint32_t mx2 = on ? -2 * ux : 0, my2 = on ? -2 * uy : 0;  // (sums wrap, results fit)
     uint32_t bias = 0;
     int T = 0, cnt = 0, sh = 0;
-    bool stage = true, grew = false, shrunk = false;
+    bool stage = true, grew = false, shrunk = false, full = false;
 #pragma unroll 1
     for (int it = 0;; ++it) {
         if (stage) T = knn_stage<K>(h, sm, on, ux, uy, ox, oy, r);
@@ -403,8 +440,10 @@ __device__ __forceinline__ unsigned knn_patch(const HashView& h, typename KnnWar
             few = on && !over && cnt < K;
         } else {  // more than the list holds: smaller radii for lanes that have missed below
             over = on && lo > 0.0f;
-            if (!__any_sync(kFull, over)) return 0;
+            if (full || probe != 0 || !__any_sync(kFull, over)) return 0;
+            full = true;
         }
+        if (probe == 2 && __any_sync(kFull, few && (it == 0 ? cnt == 0 : 2 * cnt <= K))) return 0;
         if (!__any_sync(kFull, few || over)) break;
         if (it >= 7) {
             if (T < 0) return 0;
@@ -424,6 +463,7 @@ __device__ __forceinline__ unsigned knn_patch(const HashView& h, typename KnnWar
             r = lo > 0.0f ? 0.5f * (lo + hi) : d0 + (hi - d0) * 0.85f;
         }
     }
+    probe = 0;
     const unsigned served = __ballot_sync(kFull, on);
     if (served == 0) return 0;
 
@@ -503,9 +543,17 @@ __device__ __forceinline__ unsigned knn_patch(const HashView& h, typename KnnWar
 
 // The per-thread search of one node for a lane that knn_patch did not serve:
 // its packed keys sorted ascending in hp (stride 32); returns their number, or
-// -1 when the bound does not fit a packed key. Lanes run it on their own. Out of the way of the patch search's code.
+// -1 when the bound does not fit a packed key. ub: a radius known to hold K soundings,
+// < 0: none. Lanes run it on their own. Out of the way of the patch search's code.
 template <int K>
-__device__ __noinline__ int knn_lane(const HashView& h, int qx, int qy, uint64_t* hp) {
+__device__ __noinline__ int knn_lane(const HashView& h, int qx, int qy, uint64_t* hp, float ub) {
+    if (ub >= 0.0f && ub < 2e9f) {
+        const Bound t{(int64_t)(1.000001f * ub * ub) + 1, clamp_cell(h, (int64_t)qy - h.hy0, h.ncy), 0, 0};
+        if (packed_fits(h, t.tau0)) {
+            const int cnt = knn_scan_heap_rt<32, true>(h, qx, qy, t, hp, K);
+            if (cnt == K) return cnt;
+        }
+    }
     const Bound b = knn_bound_rt(h, qx, qy, K);
     if (!packed_fits(h, b.tau0)) return -1;
     Bound bt = b;
@@ -532,7 +580,7 @@ __device__ __forceinline__ KnnFar knn_far(const HashView& h, const uint64_t* hp,
 // Patches p0 .. p1 - 1 of the patch row whose first grid row is jb (rows below
 // j1), one after another by one warp. served(i, j, ux, uy) runs for the nodes
 // that the patch search served (knn_patch: the lane's buffer column and the
-// staged list hold the neighbours), lone(i, j, qx, qy, heap) for the others:
+// staged list hold the neighbours), lone(i, j, qx, qy, heap, ub) for the others:
 // it searches by itself (knn_lane) and returns a KnnFar. flag is set when a node
 // is left to the wide pass (NULL: packed_always holds).
 template <int K, class Served, class Lone>
@@ -547,14 +595,31 @@ __device__ __forceinline__ void knn_patch_row(const HashView& h, const GridView&
         const bool on = i < g.nx && j < j1;
         const int ox = g.x0 + p * 8 * g.cell + g.cell / 2, oy = g.y0 + jb * g.cell + g.cell / 2;
         uint32_t base;
-        const float r = knn_first_radius<K>(h, ch, on, qx, qy, 8.0f * (float)g.cell, base);
-        const unsigned m = knn_patch<K>(h, sm, on, qx, qy, ox, oy, r, base, ch);
+        const float step = 8.0f * (float)g.cell;
+        int probe = __all_sync(kFull, !on || ch.dk >= 0.0f) ? 1 : 2;
+        float ub = ch.dk >= 0.0f ? 1.000001f * (ch.dk + step) + 2.0f : -1.0f, lo = 0.0f;
+        float r = knn_first_radius<K>(h, ch, on, qx, qy, step, base);
+        unsigned m;
+        for (;;) {
+            m = knn_patch<K>(h, sm, on, qx, qy, ox, oy, r, base, lo, probe, ch);
+            if (probe == 0) break;
+            // the exact neighbours of a node in the middle bound every lane's
+            probe = 0;
+            __syncwarp();
+            const unsigned all = __ballot_sync(kFull, on);
+            const int src = all == kFull ? 12 : 31 - __clz(all);
+            const KnnBracket b = knn_centre<K>(h, qx, qy, fmaxf(0.0f, __shfl_sync(kFull, r, src)), src,
+                                               reinterpret_cast<uint64_t*>(sm.buf));
+            lo = b.lo;
+            r = ub = b.ub;
+            base = 0;
+        }
         if (m >> lane & 1) served(i, j, qx - ox, qy - oy);
         if (m != kFull) {
             __syncwarp();
             if (on && !(m >> lane & 1)) {
                 ch.dk = -1.0f;
-                const KnnFar f = lone(i, j, qx, qy, reinterpret_cast<uint64_t*>(sm.buf) + lane);
+                const KnnFar f = lone(i, j, qx, qy, reinterpret_cast<uint64_t*>(sm.buf) + lane, ub);
                 if (f.cnt < 0 && flag) *flag = 1;
                 if (f.cnt == K) {
                     ch.d1 = f.d1;
@@ -566,23 +631,40 @@ __device__ __forceinline__ void knn_patch_row(const HashView& h, const GridView&
     }
 }
 
-// Is the patch search the better one for a grid of this cell over this hash?
-// Its staged list must hold the soundings of a patch and the radius around it
-// (0.8 of it at the mean density; a patch of more costs a try and then its
-// lanes' own searches), and the bounds of its 32-bit arithmetic must hold.
+// Does a grid lie off the soundings (a hash of corner, cells and their side)?
+__host__ __device__ inline bool grid_off(int32_t hx0, int32_t hy0, int32_t ncx, int32_t ncy, int32_t hash_cell,
+                                         const GridView& g) {
+    const int64_t x0 = (int64_t)g.x0 + g.cell / 2, y0 = (int64_t)g.y0 + g.cell / 2;
+    const int64_t x1 = x0 + (int64_t)(g.nx - 1) * g.cell, y1 = y0 + (int64_t)(g.ny - 1) * g.cell;
+    return x1 < hx0 || y1 < hy0 || x0 > hx0 + (int64_t)ncx * hash_cell || y0 > hy0 + (int64_t)ncy * hash_cell;
+}
+// Is the patch search the better one for a grid over this hash? Its staged list must
+// hold the soundings of a patch and the radius around it (0.8 of it at the mean
+// density; a patch of more costs a try and then its lanes' own searches), the
+// bounds of its 32-bit arithmetic must hold, and the grid must not lie off the soundings
+// (256 x 256 nodes 0.6 to 0.1 km off, IDW k = 32: 166 us by patches, 114 by threads;
+// 6 km 216, 150).
 template <int K>
-__host__ __device__ inline bool knn_patch_fits(int64_t n_valid, int32_t ncx, int32_t ncy, int32_t hash_cell,
-                                               int32_t cell, int nx, int ny) {
-    if (n_valid <= 2 * K || cell >= kPatchMax / 7 || hash_cell > kCellMax) return false;
+__host__ __device__ inline bool knn_patch_fits(int64_t n_valid, int32_t hx0, int32_t hy0, int32_t ncx, int32_t ncy,
+                                               int32_t hash_cell, const GridView& g) {
+    if (n_valid <= 2 * K || g.cell >= kPatchMax / 7 || hash_cell > kCellMax) return false;
+    if (grid_off(hx0, hy0, ncx, ncy, hash_cell, g)) return false;
     const double rho = (double)n_valid / ((double)ncx * (double)ncy * (double)hash_cell * (double)hash_cell);
     const double r = sqrt(KnnWarp<K>::kArea * K / (3.14159265 * rho)), c = hash_cell;
-    const double w = (nx < 8 ? nx - 1 : 7) * (double)cell + 2 * r + c;
-    const double t = (ny < 4 ? ny - 1 : 3) * (double)cell + 2 * r + c;
+    const double w = (g.nx < 8 ? g.nx - 1 : 7) * (double)g.cell + 2 * r + c;
+    const double t = (g.ny < 4 ? g.ny - 1 : 3) * (double)g.cell + 2 * r + c;
     return w * t * rho < 0.8 * KnnWarp<K>::CAP && 1.3 * r < kRadiusMax;
 }
 template <int K>
-inline bool knn_patch_fits(const bg_soundings_info& info, int32_t cell, int nx, int ny) {
-    return knn_patch_fits<K>(info.n_valid, info.ncx, info.ncy, info.cell_cm, cell, nx, ny);
+inline bool knn_patch_fits(const bg_soundings_info& s, const GridView& g) {
+    return knn_patch_fits<K>(s.n_valid, s.bbox_x0_cm, s.bbox_y0_cm, s.ncx, s.ncy, s.cell_cm, g);
+}
+// Where patches do not serve: lanes of a warp for a node of the grid, or a thread? Off the
+// soundings a lane's share of the records pays half as long (65,536 nodes k = 16 6 km
+// off: 171 us by lanes, 100 by threads).
+template <int K>
+inline bool grid_by_lanes(const bg_soundings_info& s, const GridView& g, int64_t nodes) {
+    return query_by_lanes<K>(grid_off(s.bbox_x0_cm, s.bbox_y0_cm, s.ncx, s.ncy, s.cell_cm, g) ? 2 * nodes : nodes);
 }
 
 // Does every bound over this grid fit a packed key? The farthest corner of the

@@ -69,8 +69,8 @@ __global__ void __launch_bounds__(64, KnnWarp<K>::kBlocksPerSM) k_knn_ids_patch(
     knn_patch_row<K>(
         h, g, sm, jb, ids.j1, p0, p0 + len, flag,
         [&](int i, int j, int, int) { ids_served<K>(h, sm, k, slot(i, j), ids.stride); },
-        [&](int i, int j, int qx, int qy, uint64_t* hp) {
-            return ids_lone<K>(h, qx, qy, hp, k, slot(i, j), ids.stride);
+        [&](int i, int j, int qx, int qy, uint64_t* hp, float ub) {
+            return ids_lone<K>(h, qx, qy, hp, ub, k, slot(i, j), ids.stride);
         });
 }
 
@@ -190,7 +190,7 @@ bg_status launch_k(const bg_soundings_s* snd, const HashView& h, const GridView&
     const int pnx = (g.nx + 7) / 8;
     int64_t rows = chunk_rows((int64_t)pnx * 8);
     const int64_t slots = (int64_t)pnx * ((rows + 3) / 4) * 32;
-    const bool patches = knn_patch_fits<K>(snd->info, g.cell, g.nx, g.ny);
+    const bool patches = knn_patch_fits<K>(snd->info, g);
     bool slot_ids = patches && !nbr && (ctx->budget ? slots <= rows * g.nx : slots_pay(slots, rows * g.nx));
     size_t id_bytes = 0;
     void* scratch = nullptr;
@@ -241,7 +241,7 @@ bg_status launch_k(const bg_soundings_s* snd, const HashView& h, const GridView&
             if (patches)
                 k_knn_ids_patch<K><<<(unsigned)(((int64_t)spr * pny + 1) / 2), 64, 0, st>>>(
                     h, g, k, ids, flag, plen, spr);
-            else if (query_by_lanes<K>(nodes))
+            else if (grid_by_lanes<K>(snd->info, g, nodes))
                 k_knn_ids_query<query_lanes(K)><<<query_blocks<K>(nodes), 32 * kQueryWarps, 0, st>>>(
                     h, g, j0 * g.nx, nodes, k, chunk_ids, 0, flag);
             else if (len == 1)

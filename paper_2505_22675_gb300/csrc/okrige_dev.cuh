@@ -293,9 +293,9 @@ __device__ __forceinline__ void ids_served(const HashView& h, const typename Knn
 }
 // The same of a node that it did not serve, by a per-thread search.
 template <int K>
-__device__ __noinline__ KnnFar ids_lone(const HashView& h, int qx, int qy, uint64_t* hp, int k, int32_t* o,
-                                        int64_t stride) {
-    const int cnt = knn_lane<K>(h, qx, qy, hp);
+__device__ __noinline__ KnnFar ids_lone(const HashView& h, int qx, int qy, uint64_t* hp, float ub, int k,
+                                        int32_t* o, int64_t stride) {
+    const int cnt = knn_lane<K>(h, qx, qy, hp, ub);
     const uint64_t mask = (1ull << h.idx_bits) - 1;
     if (cnt < 0) return KnnFar{cnt, 0.0f, 0.0f};
     for (int n = 0; n < k; ++n) {
