@@ -10,7 +10,7 @@
 //                      rectangle of cells is counted with four loads
 //
 // All four passes stream through HBM; none has a data-dependent loop. An input
-// of at most 262,144 soundings whose counts fit in shared memory (a tile: some
+// of at most 131,072 soundings whose counts fit in shared memory (a tile: some
 // 48,000 cells) takes them in one cluster of eight 1024-thread blocks instead
 // (k_hash_cluster): one launch instead of seven.
 #include <algorithm>
@@ -319,11 +319,16 @@ void launch_scatter_sat(const int4* orig, int64_t n, const CellGeom& g, int* cur
 // result depends on it). Bound by latency: 20,000 soundings 14.6 us against 41.8
 // for one block with its counts in its own shared memory; 50,000 soundings 24 us
 // against 43 for eight launches (each from a cold start). For 1,000 a
-// single block takes 7.8 us, the cluster 8.5.
+// single block takes 7.8 us, the cluster 8.5. Eight SMs are too few for large inputs:
+// whole uploads, us, by the cluster / by seven kernels after the box: 50,000 soundings
+// 41 / 60, 80,000 52 / 60, 100,000 64 / 57, 130,000 74 / 61, 200,000 88 / 66. The line
+// lies above the crossing: beside a busy serving queue each launch waits for it (95,324
+// soundings: 302 us a pass by the cluster, 350 by seven kernels).
 constexpr int kClusterBlocks = 8;       // 1 for at most 4,096 soundings (a cluster starts slower)
 constexpr int64_t kOneBlockN = 1 << 12;
 constexpr int kSmallThreads = 1024;
-constexpr int64_t kSmallN = 1 << 18;
+constexpr int64_t kSmallN = 1 << 17;    // the whole build by one cluster
+constexpr int64_t kSmallBox = 1 << 18;  // its bounding box
 constexpr int64_t kClusterSmem = 224 << 10;
 
 // shared memory of a block, in ints: counts of all cells, then the starts of its
@@ -638,7 +643,7 @@ bg_status build_soundings(bg_ctx_s* ctx, const int32_t* x, const int32_t* y, con
         a[5] = known->out_of_range;
     } else if (n > 0) {
         int* acc = nullptr;
-        if (n > kSmallN) {
+        if (n > kSmallBox) {
             if ((rc = accbuf.alloc(8 * sizeof(int))) != BG_OK) return rc;
             acc = (int*)accbuf.p;  // min x, min y, max x, max y, valid count, out-of-range count
         }
