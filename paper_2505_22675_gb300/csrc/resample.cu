@@ -397,16 +397,16 @@ __global__ void __launch_bounds__(kThreads, kMethod == BG_RESAMPLE_CATMULL_ROM ?
                     }
                 }
             } else {
+                // on a source row: the nodes' own values, as resample_at rounds them (an
+                // infinite one gives NaN). 8192 x 8192 Catmull-Rom 108 us; by resample_at
+                // 255 (220 in bands of 8 rows, before the rolling rows above)
+                const bool in = vin && ay.in;
 #pragma unroll
                 for (int k = 0; k < kVec; ++k) {
-                    // the node column i0 + k as axis_of gives it: cell index clamped
-                    // to nx - 2, remainder 0, or cell on the last column
-                    Axis ax;
-                    ax.in = vin;
-                    ax.i = vin ? (int)min(i0 + k, (int64_t)s.nx - 2) : 0;
-                    ax.r = (vin && i0 + k == s.nx - 1) ? s.cell : 0;
-                    const auto fetch = [&](int b, int) { return lane_of(R[b], k); };
-                    f[k] = resample_at<kMethod, true>(s, ax, ay, fetch, h[k]);
+                    const float q = ay.r == 0 ? lane_of(R[1], k) : lane_of(R[2], k);
+                    const float v = q + (q - q);
+                    f[k] = in ? v : __int_as_float(0x7fc00000);
+                    h[k] = !in || isnan(kCr ? q : v) ? 2 : 0;
                 }
             }
             const int64_t p = (int64_t)row * o.nx + c;
