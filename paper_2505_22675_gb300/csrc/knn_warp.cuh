@@ -34,9 +34,10 @@
 // own): with everything inlined the instruction cache missed on three of four
 // issues and the same search took 3.3 ms.
 // Uneven soundings, us by threads / with the density's radius alone / so: 256 x 256
-// nodes k = 8, half of the box empty 106 / 137 / 114, the other half denser 153 / 191 /
-// 105; 500 x 500 over clusters 224 / 286 / 204; single-beam lines 500 m apart, 400 x 350
-// nodes k = 16 467 / 690 / 386, 2,000 x 1,900 over denser ones 11,032 / 31,418 / 12,276.
+// nodes k = 8, half of the box empty 106 / 137 / 95, the other half denser 153 / 191 /
+// 123, eight of the former in a batch 418 / 730 / 371; 500 x 500 over clusters 224 / 286 /
+// 199; single-beam lines 500 m apart, 400 x 350 nodes k = 16 467 / 690 / 385, 2,000 x
+// 1,900 over denser ones 11,032 / 31,418 / 12,342.
 // Patches the staged list cannot hold (many soundings per node), nodes far
 // outside the data and the like are left to the caller's per-thread search.
 #pragma once
@@ -213,15 +214,21 @@ __device__ __forceinline__ int knn_stage(const HashView& h, typename KnnWarp<K>:
                                          int uy, int ox, int oy, float r) {
     using W = KnnWarp<K>;
     const int lane = threadIdx.x & 31;
-    const int xmin = __reduce_min_sync(kFull, on ? ux : INT_MAX), xmax = __reduce_max_sync(kFull, on ? ux : INT_MIN);
     // largest radius of each 8-lane group (a row of a grid patch), and its y range
-    int rg = on ? __float2int_ru(r) : 0, yg = on ? uy : INT_MAX, yh = on ? uy : INT_MIN;
+    const int ri = on ? __float2int_ru(r) : 0;
+    int rg = ri, yg = on ? uy : INT_MAX, yh = on ? uy : INT_MIN;
 #pragma unroll
     for (int o = 1; o < 8; o <<= 1) {
         rg = max(rg, __shfl_xor_sync(kFull, rg, o));
         yg = min(yg, __shfl_xor_sync(kFull, yg, o));
         yh = max(yh, __shfl_xor_sync(kFull, yh, o));
     }
+    // Circles of the largest radius about [xmin, xmax] hold every lane's: of circles that
+    // reach as far along x, the largest falls back least above and below. (Where the
+    // soundings lie to one side the radii differ by as much as the nodes' places, and
+    // circles about those would reach in that much deeper.)
+    const int xmin = __reduce_min_sync(kFull, on ? ux - ri + rg : INT_MAX);
+    const int xmax = __reduce_max_sync(kFull, on ? ux + ri - rg : INT_MIN);
     const int ylo = __reduce_min_sync(kFull, yg <= yh ? yg - rg : INT_MAX);
     const int yhi = __reduce_max_sync(kFull, yg <= yh ? yh + rg : INT_MIN);
     // the corner relative to the hash (both lie in (-2^30, 2^30) cm)
