@@ -78,11 +78,11 @@ HASH_BYTES_PER_SOUNDING = 36.0
 # DRAM bytes (read + write) per node, from one ncu capture of each kernel on
 # one survey line (2.077M nodes, one launch); traffic grows with the nodes of
 # a launch:
-#  - k_okrige_solve<32> with the fused IDW: 456.5 MB read + 809.7 MB written
+#  - k_okrige_solve<32> with the fused IDW: 452.5 MB read + 813.7 MB written
 #    (128 B of neighbour ids per node, and the kept tiles that leave L2);
-#  - k_knn_ids_patch<32>: 14.5 MB read + 216.3 MB written (the ids).
-SOLVE_DRAM_BYTES_PER_NODE = (456.527616e6 + 809.679104e6) / 2.076692e6
-KNN_DRAM_BYTES_PER_NODE = (14.480384e6 + 216.262656e6) / 2.076692e6
+#  - k_knn_ids_patch<32>: 14.4 MB read + 213.4 MB written (the ids).
+SOLVE_DRAM_BYTES_PER_NODE = (452.503296e6 + 813.745408e6) / 2.076692e6
+KNN_DRAM_BYTES_PER_NODE = (14.395136e6 + 213.387008e6) / 2.076692e6
 
 
 def load_peaks():

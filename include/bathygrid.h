@@ -81,7 +81,9 @@ typedef struct bg_soundings_info {
 
 /* Create a context on CUDA device `device` that may hold at most
  * `hbm_budget_bytes` of device memory (0 = no limit). Allocations that would
- * exceed the budget fail with BG_ERR_OOM_BUDGET. */
+ * exceed the budget fail with BG_ERR_OOM_BUDGET. Not counted: what CUDA itself
+ * takes for the process's kernels (code; local memory, some 82 MB once kriging with k
+ * above 16 has run). */
 bg_status bg_ctx_create(int device, size_t hbm_budget_bytes, bg_ctx_t* out);
 
 /* Destroy a context. Every grid and soundings handle made from it must have
@@ -335,9 +337,9 @@ bg_status bg_batch_create(bg_ctx_t ctx, const bg_tile* tiles, int n_tiles, bg_ba
 
 /* Grid every tile of the batch, ordered after prior work on cuda_stream and
  * before later work on it. The first run records the launch sequence (hash
- * build for all tiles, one persistent k-NN/IDW kernel, one persistent solve
- * kernel per kriging system size and model) as a CUDA graph; later runs replay it, with
- * no host synchronization. */
+ * build for all tiles, a persistent k-NN/IDW kernel per search size and one for the
+ * tiles searched by threads, a persistent solve kernel per kriging system size and
+ * model) as a CUDA graph; later runs replay it, with no host synchronization. */
 bg_status bg_batch_run(bg_batch_t b, void* cuda_stream);
 
 /* Hash cell side as a target number of soundings per cell (default 2); the

@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(kBT) k_batch_validate(const TileDesc* __restri
     }
 }
 
-// 2. per-tile hash geometry (one thread per tile)
+// does the patch search serve this tile (knn_patch_fits for its search size)?
 __device__ __forceinline__ bool tile_patch_fits(const HashView& h, const GridView& g, int kq) {
     auto fits = [&](auto K) {
         return knn_patch_fits<decltype(K)::value>(h.n_valid, h.hx0, h.hy0, h.ncx, h.ncy, h.cs, g);
@@ -178,6 +178,7 @@ __device__ __forceinline__ IdsView tile_ids(const TileDesc& d) {
     return IdsView{d.ids, d.patch ? d.stride : 0, (d.g.nx + 7) / 8, 0, d.g.ny};
 }
 
+// 2. per-tile hash geometry (one thread per tile)
 __global__ void k_batch_geom(TileDesc* td, int T, const int* __restrict__ acc, float ppc,
                              int* __restrict__ status) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;

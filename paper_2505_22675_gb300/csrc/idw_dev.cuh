@@ -1,7 +1,9 @@
 // Device code of fused k-NN + IDW, shared by the per-grid kernels (idw.cu)
 // and the batched persistent kernels (batch.cu).
 //
-// Fused exact k-NN + inverse-distance weighting, one thread per grid node.
+// Fused exact k-NN + inverse-distance weighting: a node per lane of a patch search
+// (knn_warp.cuh), a query per half or whole warp (knn_query.cuh), or one per thread
+// (knn.cuh).
 //
 // zhat = sum w_i z_i / sum w_i with w_i = d_i^-p over the k nearest valid
 // soundings. It is evaluated as z_1 + sum w_i (z_i - z_1) / sum w_i with
@@ -117,26 +119,6 @@ __device__ __forceinline__ void idw_served(const HashView& h, const typename Knn
     if (nbr)
         for (int n = 0; n < k; ++n) nbr[n] = __ldg(&h.rec[sm.pos[col[n * 32] & kPlaceMask]].w);
 }
-// Wide-key IDW of one node or point whose table bound does not fit the packed
-// key (rare); others return.
-template <int K>
-__device__ __forceinline__ void idw_point_wide(const HashView& h, int qx, int qy, int k,
-                                               float power, float* __restrict__ dout,
-                                               int32_t* __restrict__ o) {
-    if (!point_may_be_wide(h, qx, qy)) return;
-    const Bound b = knn_bound<K>(h, qx, qy);
-    if (packed_fits(h, b.tau0)) return;
-    uint64_t d2[K];
-    int id[K];
-    const int keff = min(knn_scan_wide<K>(h, qx, qy, b, d2, id), k);
-    *dout = idw_from(h, keff, power, [&](int i, uint64_t& dd, int& ii) {
-        dd = d2[i];
-        ii = id[i];
-    });
-    if (o)
-        for (int i = 0; i < k; ++i) o[i] = i < keff ? id[i] : -1;
-}
-
 // The same of a node that it did not serve: a per-thread search, out of the way
 // of the patch search's code.
 template <int K>
@@ -153,6 +135,26 @@ __device__ __noinline__ KnnFar idw_lone(const HashView& h, int qx, int qy, uint6
     });
     if (nbr) emit_ids<32>(nbr, hp, k, keff, mask);
     return knn_far<K>(h, hp, cnt);
+}
+
+// Wide-key IDW of one query point whose table bound does not fit the packed key
+// (rare); others return.
+template <int K>
+__device__ __forceinline__ void idw_point_wide(const HashView& h, int qx, int qy, int k,
+                                               float power, float* __restrict__ dout,
+                                               int32_t* __restrict__ o) {
+    if (!point_may_be_wide(h, qx, qy)) return;
+    const Bound b = knn_bound<K>(h, qx, qy);
+    if (packed_fits(h, b.tau0)) return;
+    uint64_t d2[K];
+    int id[K];
+    const int keff = min(knn_scan_wide<K>(h, qx, qy, b, d2, id), k);
+    *dout = idw_from(h, keff, power, [&](int i, uint64_t& dd, int& ii) {
+        dd = d2[i];
+        ii = id[i];
+    });
+    if (o)
+        for (int i = 0; i < k; ++i) o[i] = i < keff ? id[i] : -1;
 }
 
 // IDW of the queries of a warp (knn_query): lane n of a query's G holds neighbour

@@ -1,6 +1,6 @@
 // Exact k-nearest-neighbour search of 32 nearby nodes by one warp.
 //
-// A warp takes a patch of 8 x 4 grid nodes (or 32 points), one node per lane,
+// A warp takes a patch of 8 x 4 grid nodes, one node per lane,
 // and walks a strip of patches along x. Neighbouring nodes share almost all
 // their candidates, so the candidates of the whole patch are staged once and
 // every lane tests each of them, without divergence:
@@ -24,11 +24,11 @@
 // are distances that a key holds only in part (large radii drop low bits).
 //
 // What bounds it: latency at 16 (K <= 16) or 12 (K = 32) resident warps per
-// SM, half of the issue slots used (18 warps of 96 registers instead of 16 of 128 spill
-// and take 1.40 ms where these take 1.27); a per-thread heap was bound by divergence.
+// SM, half of the issue slots used (18 warps of 96 registers instead of 16 of 128 spill:
+// whole pass of the swath below 1.40 ms, 1.28 so); a per-thread heap was bound by divergence.
 // IDW k = 16 on a two-line swath (4,000 x 1,692 nodes, a 154 m gap): a heap per
 // thread 277 warp instructions per node with 16 of 32 lanes active, 2.04 ms;
-// this search 105 with 30, 1.20 ms. A candidate costs a warp 7 instructions for
+// this search 102 with 30, 1.17 ms. A candidate costs a warp 7 instructions for
 // its 32 nodes (114 per patch there, 1.15 scans), the networks about 550 a
 // patch. The straight path is kept short (rare courses in functions of their
 // own): with everything inlined the instruction cache missed on three of four

@@ -53,7 +53,8 @@
 // the factor, at K = 32, where on-chip memory holds only one of the two
 // triangles, in the threads' local memory (1.3 KB a thread, 50 MB over the
 // device's resident systems: L2 holds them but for 0.4 KB a system that is
-// written back, 6 % of the DRAM's bandwidth with the ids), read one tile ahead.
+// written back, 6 % of the DRAM's bandwidth with the ids), read one tile ahead. CUDA
+// takes 82 MB for it at the first launch, beside what the context counts.
 // The correction reuses the factor. The weight sum closes in FP64: lambda_0 = 1 -
 // sum(lambda'). Outputs:
 //     zhat    = z_0 + sum_a lambda_a (z_a - z_0)          (= sum lambda_i z_i)
@@ -143,8 +144,9 @@ __device__ __forceinline__ float sqrt_approx(float x) {
 // nodes of that interval (off by 1.3e-9 at most); then (1 - s) + s (1 - exp(-r)), s
 // = 2^-n, which does not cancel at short range. Errors, 2e6 draws in each of nine
 // intervals: 0.89 ulp at most, 0.22 to 0.34 rms (-expm1f: 1.13, 0.22 to 0.50; with
-// q of degree 4 1.01, 0.22 to 0.35 and 2 us less, but the variances of some ranges
-// 3 % further off than with the library call; so 1 to 6 % nearer).
+// q of degree 4 1.01, 0.22 to 0.35 and 2 us less). Variances against 64 bits, relative rms
+// error over 14 random tiles (k 8 to 32, ranges 20 to 76 m): 1.02e-7, with -expm1f 1.04e-7;
+// of one tile between 0.83 and 1.04 times the latter.
 __device__ __forceinline__ u64 one_minus_exp2(u64 t) {
     const u64 magic = dup2(12582912.0f);  // 1.5 * 2^23: the low bits of a sum hold the integer
     const u64 y = fma2(t, dup2(1.44269504f), magic);
