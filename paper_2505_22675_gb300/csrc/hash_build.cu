@@ -10,7 +10,7 @@
 //                      rectangle of cells is counted with four loads
 //
 // All four passes stream through HBM; none has a data-dependent loop. An input
-// of at most 131,072 soundings whose counts fit in shared memory (a tile: some
+// of at most 98,304 soundings whose counts fit in shared memory (a tile: some
 // 48,000 cells) takes them in one cluster of eight 1024-thread blocks instead
 // (k_hash_cluster): one launch instead of seven.
 #include <algorithm>
@@ -321,13 +321,12 @@ void launch_scatter_sat(const int4* orig, int64_t n, const CellGeom& g, int* cur
 // against 43 for eight launches (each from a cold start). For 1,000 a
 // single block takes 7.8 us, the cluster 8.5. Eight SMs are too few for large inputs:
 // whole uploads, us, by the cluster / by seven kernels after the box: 50,000 soundings
-// 41 / 60, 80,000 52 / 60, 100,000 64 / 57, 130,000 74 / 61, 200,000 88 / 66. The line
-// lies above the crossing: beside a busy serving queue each launch waits for it (95,324
-// soundings: 302 us a pass by the cluster, 350 by seven kernels).
+// 41 / 60, 80,000 52 / 60, 100,000 64 / 57, 130,000 74 / 60, 200,000 83 / 65 (after a
+// serving burst, whose streams share the pool, 130,000 111 / 103, 200,000 122 / 105).
 constexpr int kClusterBlocks = 8;       // 1 for at most 4,096 soundings (a cluster starts slower)
 constexpr int64_t kOneBlockN = 1 << 12;
 constexpr int kSmallThreads = 1024;
-constexpr int64_t kSmallN = 1 << 17;    // the whole build by one cluster
+constexpr int64_t kSmallN = 96 << 10;   // the whole build by one cluster
 constexpr int64_t kSmallBox = 1 << 18;  // its bounding box
 constexpr int64_t kClusterSmem = 224 << 10;
 
@@ -594,7 +593,7 @@ bg_status build_soundings(bg_ctx_s* ctx, const int32_t* x, const int32_t* y, con
     bg_status rc = BG_OK;
     const int32_t *dx = x, *dy = y;
     const float* dz = z;
-    Scratch staging(ctx, st), scratch(ctx, st), accbuf(ctx, st);
+    Scratch staging(ctx, st), accbuf(ctx, st);
 
     s->info = bg_soundings_info{};
     s->info.n_total = n;
@@ -686,7 +685,16 @@ bg_status build_soundings(bg_ctx_s* ctx, const int32_t* x, const int32_t* y, con
     s->info.ncx = ncx;
     s->info.ncy = ncy;
 
-    const size_t cs_bytes = (size_t)(ncells + 1) * 4;
+    // Scratch of the many-kernel build: the counts (later cursors) lie where the summed-area
+    // table is written once they have been used, the partial sums behind cell_start. (An
+    // allocation of their own costs a call 10 us where other streams, a serving queue's, have
+    // used the pool.) Chunks of rows for the column prefix of the table: grid.y <= 65535.
+    const bool cluster = cluster_takes(a, n, cs);
+    const int nb = (int)((ncells + kScanTile - 1) / kScanTile);
+    const int sat_rows = std::max(kSatRows, (ncy + 65534) / 65535);
+    const int nch = (ncy + sat_rows - 1) / sat_rows;
+    const size_t sums = cluster ? 0 : (size_t)(nb + 1) + (size_t)nch * (ncx + 1);
+    const size_t cs_bytes = ((size_t)(ncells + 1) + sums) * 4;
     const size_t sat_bytes = (size_t)(ncx + 1) * (ncy + 1) * 4;
     const size_t rec_bytes = (size_t)nvalid * 16;
     if ((rc = dalloc(ctx, &s->d_cell_start, cs_bytes, st)) != BG_OK) return rc;
@@ -698,7 +706,7 @@ bg_status build_soundings(bg_ctx_s* ctx, const int32_t* x, const int32_t* y, con
 
     const CellGeom g{a[0], a[1], (int32_t)cs, ncx, ncy};
     int* cell_start = (int*)s->d_cell_start;
-    if (cluster_takes(a, n, cs)) {
+    if (cluster) {
         const size_t smem = (size_t)cluster_ints(n, ncx, ncy) * sizeof(int);
         const auto kernel = cluster_blocks(n) == 1 ? k_hash_cluster<1> : k_hash_cluster<kClusterBlocks>;
         if (smem > (48 << 10))
@@ -710,19 +718,11 @@ bg_status build_soundings(bg_ctx_s* ctx, const int32_t* x, const int32_t* y, con
         BG_CUDA(cudaGetLastError());
     } else {
         if (!packed) pack(nullptr);
-        const int nb = (int)((ncells + kScanTile - 1) / kScanTile);
-        // chunks of rows for the column prefix of the SAT (grid.y stays <= 65535)
-        const int sat_rows = std::max(kSatRows, (ncy + 65534) / 65535);
-        const int nch = (ncy + sat_rows - 1) / sat_rows;
-        const size_t count_bytes = (size_t)ncells * 4;
-        const size_t bsum_bytes = (size_t)(nb + 1) * 4;
-        const size_t csum_bytes = (size_t)nch * (ncx + 1) * 4;
-        if ((rc = scratch.alloc(count_bytes + bsum_bytes + csum_bytes + 64)) != BG_OK) return rc;
-        int* count = (int*)scratch.p;
-        int* bsum = count + ncells;
+        int* count = (int*)s->d_sat;
+        int* bsum = cell_start + ncells + 1;
         int* csum = bsum + nb + 1;
 
-        BG_CUDA(cudaMemsetAsync(count, 0, count_bytes, st));
+        BG_CUDA(cudaMemsetAsync(count, 0, (size_t)ncells * 4, st));
         k_cell_hist<<<grid_for(n, kThreads * 4, 152 * 16), kThreads, 0, st>>>(
             (const int4*)s->d_orig, n, g, count);
         k_scan_reduce<<<nb, kThreads, 0, st>>>(count, ncells, bsum);
